@@ -13,8 +13,9 @@ gradient), so that the backward does not reload the coefficients, counts its
 bins from 4 bytes per point and needs no rebinding.  ``LumiFn`` does the same
 for the fused luminosity workload, L = (1/n) sum_e sum_a f_a(x1) f_-a(x2).
 
-The coefficients live in ONE table per PDF handle, rebuilt by every forward and
-backward call from the values tensor it is given: two differentiable
+The coefficients live in ONE table per PDF handle, rebuilt by every forward
+call, and every backward call that reads them, from the values tensor it is
+given: two differentiable
 evaluations with different values on one handle, from two streams at once,
 race on that table.  Use one handle per stream (or order the streams).
 """
@@ -113,7 +114,8 @@ class LumiFn(torch.autograd.Function):
         from .lumi import luminosity_backward
         (values,) = ctx.saved_tensors
         pdf = ctx.pdf
-        pdf.bind_values(values)
+        if ctx.saved is None:                 # saved factors hold all that the backward needs of the values
+            pdf.bind_values(values)
         gvals = torch.zeros_like(values)
         gslice = gvals[ctx.member] if values.dim() == 4 else gvals
         luminosity_backward(pdf, ctx.events, float(gL.item()), gslice, ctx.member, saved_p=ctx.saved)

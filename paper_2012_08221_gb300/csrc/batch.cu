@@ -23,14 +23,16 @@
 #include <vector>
 
 #include "pdf_internal.h"
+#include "warp_eval.cuh"
 
 using namespace pdfgpu;
 
 namespace {
 
 constexpr int kMaxReqPids = 16;
-constexpr int kStageX = 256;      // x cells that fit the staged tables
-constexpr int kStageQ = 64;       // Q cells that fit the staged tables
+constexpr size_t kStageMax = 48 * 1024;   // coordinate tables of larger grids stay global
+constexpr int kWarpBytes = kWarpBuf + kQueue * 8;
+static_assert(32 * 8 * kMaxReqPids <= kWarpBuf, "a warp's output rows fit its buffer");
 
 struct BatchReq {
     int grid;
@@ -44,26 +46,19 @@ struct BatchReq {
     int64_t tile0;
 };
 
-__device__ __forceinline__ double qnan() { return __longlong_as_double(0x7FF8000000000000ll); }
-
-struct StageTables {
-    LogEntry logtab[kLogTab];
-    uint64_t xbits[kStageX];
-    double2 xcell[kStageX];
-    uint64_t qbits[kStageQ];
-    double2 qcell[kStageQ];
-};
-
-template <int QPT, bool STAGE, bool CONT>
+template <int QPT, bool STAGE>
 __global__ void k_batch(const GridDev *__restrict__ grids, const BatchReq *__restrict__ reqs, int nreq,
-                        int64_t ntiles, unsigned long long *ticket, int out_stride)
+                        int64_t ntiles, unsigned long long *ticket)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    double *sout = reinterpret_cast<double *>(smem);
-    StageTables *st = reinterpret_cast<StageTables *>(smem + (size_t)blockDim.x * out_stride * sizeof(double));
+    extern __shared__ __align__(128) unsigned char smem[];
     __shared__ GridDev sg;
     __shared__ BatchReq sr;
     __shared__ long long s_tile;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned char *mine = smem + (size_t)wid * kWarpBytes;
+    unsigned char *tabs = smem + (size_t)(blockDim.x >> 5) * kWarpBytes;
+    WarpBufs B{reinterpret_cast<uint4 *>(mine), reinterpret_cast<int64_t *>(mine + kWarpBuf), 0};
+    CoordTabs T{};
     int cur = -1;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -88,96 +83,45 @@ __global__ void k_batch(const GridDev *__restrict__ grids, const BatchReq *__res
             cur = sr.grid;
             if (threadIdx.x == 0) sg = grids[cur];
             __syncthreads();
-            if (STAGE && sg.nxc <= kStageX && sg.nqc <= kStageQ) {
-                for (int k = threadIdx.x; k < kLogTab; k += blockDim.x) st->logtab[k] = sg.logtab[k];
-                for (int k = threadIdx.x; k < sg.nxc; k += blockDim.x) {
-                    st->xbits[k] = sg.xbits[k];
-                    st->xcell[k] = sg.xcell[k];
-                }
-                for (int k = threadIdx.x; k < sg.nqc; k += blockDim.x) {
-                    st->qbits[k] = sg.qbits[k];
-                    st->qcell[k] = sg.qcell[k];
-                }
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    sg.logtab = st->logtab;
-                    sg.xbits = st->xbits;
-                    sg.xcell = st->xcell;
-                    sg.qbits = st->qbits;
-                    sg.qcell = st->qcell;
-                }
-            }
+            T = STAGE && coord_tab_bytes(sg) <= (int)kStageMax ? stage_tabs(sg, tabs) : grid_tabs(sg);
             __syncthreads();
         }
         const GridDev &g = sg;
-        const int npid = sr.npid;
-        const int64_t n = sr.n;
-        const size_t cell_stride = (size_t)g.nflav * 16;
-        const double *cm = g.coef + (size_t)sr.member * g.nqc * g.nxc * cell_stride;
+        const size_t patches = (size_t)sr.member * g.nqc * g.nxc * g.nflav;
+        const Query Y{sr.cols, sr.npid, 0, sr.npid, g.coef + patches * 16,
+                      g.fcoef ? reinterpret_cast<const unsigned char *>(g.fcoef) + patches * 128 : nullptr,
+                      sr.x, sr.q2, sr.n, sr.out, nullptr, nullptr};
         const int64_t p0 = (int64_t)(t - sr.tile0) * ((int64_t)blockDim.x * QPT);
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        double *wbuf = sout + (size_t)wid * 32 * out_stride;
 #pragma unroll 1
         for (int qq = 0; qq < QPT; ++qq) {
             // this warp's 32 consecutive points of the tile
             const int64_t base = p0 + (int64_t)qq * blockDim.x + 32 * wid;
-            if (base >= n) break;
-            const int64_t i = base + lane;
-            const bool live = i < n;
-            double xi = live ? sr.x[i] : 0.5;
-            double qi = live ? sr.q2[i] : 10.0;
-            bool bad = live && !(x_ok(dbits(xi)) && q2_ok(dbits(qi)));
-            flag_status(g, bad);
-            if (bad) {
-                xi = 0.5;
-                qi = 10.0;
-            }
-            double u, w;
-            Axis X = axis_x(g, xi, &u);
-            Axis Q = axis_q2(g, qi, &w);
-            const bool oor = live && out_of_range(g, X, Q);
-            flag_status(g, oor, PDF_S_RANGE);
-            bad |= oor;
-            const double *cell = cm + ((size_t)Q.cell * g.nxc + X.cell) * cell_stride;
-            double *srow = wbuf + lane * npid;
-            for (int a = 0; a < npid; ++a) {
-                int col = sr.cols[a];
-                if (col >= 0) col = checked_index(g.status, col, g.nflav);
-                double v = col >= 0 ? patch_any<CONT>(g, cell + col * 16, X, Q) : 0.0;
-                srow[a] = bad ? qnan() : v;
-            }
-            __syncwarp();
-            const int rows = (int)min((int64_t)32, n - base);
-            const int cnt = rows * npid;
-            double *dst = sr.out + base * npid;
-            for (int k = lane; k < cnt; k += 32) dst[k] = wbuf[k];
-            __syncwarp();
+            if (base >= Y.n) break;
+            eval_points<false, false, false, true>(g, T, Y, B, base, lane);
         }
+        while (B.qn) drain_queue(g, Y, false, B, lane);
         __syncthreads();   // everyone is done with sr/s_tile before thread 0 refills them
     }
+    if (lane == 0) bulk_wait_all();
 }
 
 struct Shape {
     int block, qpt, stage;
 };
 
-using KernelFn = void (*)(const GridDev *, const BatchReq *, int, int64_t, unsigned long long *, int);
+using KernelFn = void (*)(const GridDev *, const BatchReq *, int, int64_t, unsigned long long *);
 
-template <bool CONT>
-KernelFn kernel_for_t(const Shape &s)
+KernelFn kernel_for(const Shape &s)
 {
     if (s.stage) {
-        if (s.qpt == 1) return k_batch<1, true, CONT>;
-        if (s.qpt == 2) return k_batch<2, true, CONT>;
-        return k_batch<4, true, CONT>;
+        if (s.qpt == 1) return k_batch<1, true>;
+        if (s.qpt == 2) return k_batch<2, true>;
+        return k_batch<4, true>;
     }
-    if (s.qpt == 1) return k_batch<1, false, CONT>;
-    if (s.qpt == 2) return k_batch<2, false, CONT>;
-    return k_batch<4, false, CONT>;
+    if (s.qpt == 1) return k_batch<1, false>;
+    if (s.qpt == 2) return k_batch<2, false>;
+    return k_batch<4, false>;
 }
-
-// `cont`: some grid of the launch uses the continuation extrapolation.
-KernelFn kernel_for(const Shape &s, bool cont) { return cont ? kernel_for_t<true>(s) : kernel_for_t<false>(s); }
 
 // ---------------------------------------------------------- tune cache (JSON)
 // One entry per line: "signature": {"block": B, "qpt": Q, "stage": S, "ms": T}
@@ -234,9 +178,9 @@ struct pdfgpu_batch {
     unsigned long long *d_ticket = nullptr;
     int nreq = 0;
     int out_stride = 1;
+    size_t tab_bytes = 0;               // the largest staged grid's coordinate tables
     int64_t ntiles = 0;
     Shape shape{256, 2, 1};
-    bool cont = false;                  // some grid uses the continuation extrapolation
     int ctas = 0;
     size_t smem = 0;
     float tuned_ms = 0;
@@ -246,8 +190,7 @@ struct pdfgpu_batch {
 
 static size_t shape_smem(const pdfgpu_batch *b, const Shape &s)
 {
-    size_t out = (size_t)s.block * b->out_stride * sizeof(double);
-    return out + (s.stage ? sizeof(StageTables) : 0);
+    return (size_t)(s.block / 32) * kWarpBytes + (s.stage ? b->tab_bytes : 0);
 }
 
 // Fill tile offsets for a shape and upload the request table.
@@ -261,7 +204,7 @@ static int configure(pdfgpu_batch *b, const Shape &s, cudaStream_t st)
     b->ntiles = acc;
     PDF_CUDA(cudaMemcpyAsync(b->d_reqs, b->host_reqs.data(), b->host_reqs.size() * sizeof(BatchReq),
                              cudaMemcpyHostToDevice, st));
-    KernelFn k = kernel_for(s, b->cont);
+    KernelFn k = kernel_for(s);
     size_t smem = shape_smem(b, s);
     int rc = allow_dynamic_smem((const void *)k, smem);
     if (rc) return rc;
@@ -274,9 +217,8 @@ static int configure(pdfgpu_batch *b, const Shape &s, cudaStream_t st)
 static int enqueue(pdfgpu_batch *b, cudaStream_t st)
 {
     PDF_CUDA(cudaMemsetAsync(b->d_ticket, 0, sizeof(unsigned long long), st));
-    KernelFn k = kernel_for(b->shape, b->cont);
-    k<<<b->ctas, b->shape.block, b->smem, st>>>(b->d_grids, b->d_reqs, b->nreq, b->ntiles, b->d_ticket,
-                                                 b->out_stride);
+    KernelFn k = kernel_for(b->shape);
+    k<<<b->ctas, b->shape.block, b->smem, st>>>(b->d_grids, b->d_reqs, b->nreq, b->ntiles, b->d_ticket);
     PDF_CUDA(cudaGetLastError());
     return PDF_OK;
 }
@@ -349,7 +291,8 @@ extern "C" int pdf_batch_prepare(const pdfgpu_batch_desc *descs, int32_t n_desc,
             gi = (int)b->grid_handles.size();
             b->grid_handles.push_back(D.grid);
             gd.push_back(D.grid->d);
-            if (D.grid->d.extrap == PDF_EXTRAP_CONTINUATION) b->cont = true;
+            const size_t tab = (size_t)coord_tab_bytes(D.grid->d);
+            if (tab <= kStageMax) b->tab_bytes = std::max(b->tab_bytes, tab);
         }
         Cols cols;
         int rc2 = resolve_cols(D.grid, D.pids, D.n_pid, &cols);
@@ -579,9 +522,7 @@ extern "C" int pdf_batch_run_noalloc(const pdfgpu_batch_desc *descs, int32_t n_d
     std::lock_guard<std::mutex> lock(g_noalloc_mu);
     NoAllocHead &H = g_noalloc_head;
     int ngrids = 0;
-    bool cont = false;                  // some grid uses the continuation extrapolation
     pdfgpu_grid_t handles[kNoAllocMaxGrids];
-    int out_stride = 1;
     const int block = 256, qpt = 2;
     const int64_t tile = (int64_t)block * qpt;
     // first pass: validate every request and build the grid table
@@ -601,13 +542,11 @@ extern "C" int pdf_batch_run_noalloc(const pdfgpu_batch_desc *descs, int32_t n_d
                 return fail(PDF_E_RANGE, "pdf_batch_run_noalloc takes at most 32 distinct grids");
             gi = ngrids++;
             handles[gi] = D.grid;
-            if (D.grid->d.extrap == PDF_EXTRAP_CONTINUATION) cont = true;
             H.grids[gi] = D.grid->d;
         }
         Cols cols;
         rc = resolve_cols(D.grid, D.pids, D.n_pid, &cols);
         if (rc) return rc;
-        out_stride = std::max(out_stride, (int)D.n_pid);
     }
     H.ngrids = ngrids;
     if (!g_noalloc_dev_addr[dev]) {
@@ -652,14 +591,14 @@ extern "C" int pdf_batch_run_noalloc(const pdfgpu_batch_desc *descs, int32_t n_d
         PDF_CUDA(cudaGetLastError());
     }
     if (ntiles == 0) return PDF_OK;
-    KernelFn k = kernel_for(Shape{block, qpt, 0}, cont);
-    size_t smem = (size_t)block * out_stride * sizeof(double);
+    KernelFn k = kernel_for(Shape{block, qpt, 0});
+    const size_t smem = (size_t)(block / 32) * kWarpBytes;
     int rc = allow_dynamic_smem((const void *)k, smem);
     if (rc) return rc;
     int sms = 0;
     PDF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     int ctas = sms * occupancy((const void *)k, block, smem);
-    k<<<ctas, block, smem, st>>>(S->grids, S->reqs, n_desc, ntiles, &S->ticket, out_stride);
+    k<<<ctas, block, smem, st>>>(S->grids, S->reqs, n_desc, ntiles, &S->ticket);
     PDF_CUDA(cudaGetLastError());
     return PDF_OK;
 }

@@ -114,9 +114,8 @@ __global__ void __launch_bounds__(kBlock) k_bwd(GridDev g, Cols cols, int npid, 
                 if (gq) gq[i] = qnan();
                 continue;
             }
-            double u, w;
-            X = axis_x(g, xi, &u);
-            Q = axis_q2(g, qi, &w);
+            X = axis_x(g, xi);
+            Q = axis_q2(g, qi);
             if (out_of_range(g, X, Q)) {
                 if (gx) gx[i] = qnan();
                 if (gq) gq[i] = qnan();
@@ -225,9 +224,8 @@ __global__ void __launch_bounds__(kBlock) k_bwd_axes(GridDev g, const double *__
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
         const double xi = x[i0 + k], qi = q2[i0 + k];
         bool bad = !(x_ok(dbits(xi)) && q2_ok(dbits(qi)));
-        double u, w;
-        Axis X = axis_x(g, bad ? 0.5 : xi, &u);
-        Axis Q = axis_q2(g, bad ? 10.0 : qi, &w);
+        Axis X = axis_x(g, bad ? 0.5 : xi);
+        Axis Q = axis_q2(g, bad ? 10.0 : qi);
         bad |= out_of_range(g, X, Q);
         tape_put(tape, k, X, Q, bad);
     }

@@ -1,0 +1,197 @@
+// Fixed-point evaluation of the interpolant.
+//
+// The FP64 pipe of this GPU issues 2 FMAs per clock and SM; IMAD.WIDE (32 x
+// 32 + 64 bits) issues 64.  Inside the knot range a patch is therefore
+// evaluated in 64-bit integers: the 16 monomial coefficients of the patch
+// about the cell's centre, scaled by the power of two above the largest of
+// them (a block exponent), against the 16 products of the powers of the two
+// local coordinates tc = t - 1/2 in [-1/2, 1/2].  A 64-bit by 64-bit product
+// costs three IMAD.WIDE (the low x low digit product is below the last bit
+// kept), and sums need no normalisation.
+//
+// Formats.  A "Dig" is a 64-bit integer h 2^32 + l with SIGNED l, so that
+// digit products are plain signed 32 x 32 multiplies.
+//   coordinates and their products (weights)  value 2^62
+//   coefficients                              value 2^(61 - E), |.| <= 2^61,
+//                                             E: max |coefficient| < 2^E
+//   sums of coefficient x weight              value 2^(59 - E)
+//   logarithms                                value 2^60 modulo 16
+// Errors: a patch value is within about 2^-57 of the largest coefficient
+// (FP64 Horner: several roundings of 2^-53), a logarithm within about 2^-59
+// absolute (FP64: 2^-49 at |ln x| = 16 ... 32), so results are closer to the
+// exact interpolant than in FP64.  Integer sums do not depend on their order:
+// every kernel gives the same bits however it splits a patch over lanes.
+// Everything else (points outside the knots, patches whose scale the block
+// exponent cannot hold, cells too narrow or too wide for the logarithm's
+// format) takes the FP64 path.
+#pragma once
+
+// Included by pdf_common.cuh, after the bit helpers it uses.
+
+namespace pdfgpu {
+
+struct Dig {
+    int h, l;
+};
+
+PDF_HD Dig fix_split(int64_t v)
+{
+    const uint32_t lo = (uint32_t)v;
+    return {(int)(uint32_t)((uint64_t)v >> 32) + (int)(lo >> 31), (int)lo};
+}
+
+PDF_HD int64_t wide(int a, int b) { return (int64_t)a * (int64_t)b; }
+PDF_HD int64_t wide(int a, int b, int64_t c) { return (int64_t)a * (int64_t)b + c; }
+PDF_HD int fix_hi(int64_t v) { return (int)(uint32_t)((uint64_t)v >> 32); }
+
+// Product of two values of at most 1/2 (2^61), in the format of the factors.
+PDF_HD int64_t fix_mul(Dig a, Dig b)
+{
+    const int64_t cr = wide(a.l, b.h, wide(a.h, b.l, (int64_t)1 << 29));
+    return wide(2 * a.h, 2 * b.h) + (int)(cr >> 30);
+}
+
+// ln 2 in 2^-60, and its next 32 bits.
+constexpr int64_t kLn2Fix = 799144290325165978ll;
+constexpr uint32_t kLn2Low = 3164486457u;
+
+// ln of a positive normal double from its bits, value 2^60 modulo 2^64.
+//   x = 2^e m; j = top 10 bits of m; inv = 1/c_j in 2^-31 (c_j the middle of
+//   the table interval), r = m inv - 1 exact to 2^-62, |r| <= 2^-11;
+//   ln(1 + r) = r - r^2/2 + r^3 (1/3 - r/4 + r^2/5)  (next term < 2^-68);
+//   tab holds -ln(inv).  Host tables and kernels call this same routine, so
+//   a point on a knot gets the knot's own logarithm.
+PDF_HD int64_t fix_log(uint64_t bits, const uint32_t *inv, const int64_t *tab)
+{
+    const uint32_t hw = (uint32_t)(bits >> 32);
+    const int e = (int)(hw >> 20) - 1023;
+    const uint32_t j = (hw >> (20 - kLogBits)) & (kLogTab - 1);
+    const uint64_t M = (bits << 11) | ((uint64_t)1 << 63);
+    const uint32_t I = inv[j];
+    const uint64_t lo = (uint64_t)(uint32_t)M * I;
+    const uint64_t P = (uint64_t)(uint32_t)(M >> 32) * I + (lo >> 32);
+    const int64_t R = (int64_t)(P - ((uint64_t)1 << 62));       // r 2^62
+    const int rh = (int)(R >> 21), rl = (int)((uint32_t)R & 0x1FFFFFu), rs = (int)(R >> 30);
+    const int64_t sq = wide(rh, rh);                            // r^2 2^82
+    const int64_t r2 = sq + (wide(rh, rl) >> 20);
+    int z = fix_hi(wide(rs, 429496730, -((int64_t)536870912 << 32)));  // -1/4 + r/5, in 2^-31
+    z = fix_hi(wide(rs, z, (int64_t)715827883 << 32));                 // 1/3 + r z
+    const int c = fix_hi(wide(fix_hi(sq), rh));                        // r^3 2^59
+    const int tail = (int)(wide(c, z, 1 << 29) >> 30);                 // in 2^-60
+    const int64_t head = (R - (r2 >> 21) + 2) >> 2;
+    const int64_t el = (int64_t)e * kLn2Fix + (((int64_t)e * kLn2Low + ((int64_t)1 << 31)) >> 32);
+    return (int64_t)((uint64_t)head + (uint64_t)tab[j] + (uint64_t)el) + tail;
+}
+
+// One cell's logarithm of the lower knot and 2^126 / (width << s), with the
+// normalising shift s in the low 6 bits (width << s in [2^62, 2^63)); K = 0
+// marks a cell that the format cannot serve.
+struct FixCell {
+    int64_t U;
+    uint64_t K;
+};
+
+// Local coordinate t of a logarithm in its cell, value 2^62.
+PDF_HD int64_t fix_coord(int64_t u, const FixCell &c)
+{
+    int64_t v = (int64_t)((uint64_t)u - (uint64_t)c.U);
+    v = v < 0 ? 0 : v;                      // a unit of the logarithm's error below the knot
+    const uint64_t vv = (uint64_t)v << (c.K & 63);
+    const uint32_t vh = (uint32_t)(vv >> 32), vl = (uint32_t)vv, kh = (uint32_t)(c.K >> 32), kl = (uint32_t)c.K;
+    return (int64_t)((uint64_t)vh * kh + (((uint64_t)vh * kl) >> 32) + (((uint64_t)vl * kh) >> 32));
+}
+
+constexpr int64_t kFixHalf = (int64_t)1 << 61;
+
+#ifdef __CUDACC__
+// The same t as a double.
+__device__ __forceinline__ double fix_t(int64_t t) { return __ll2double_rn(t) * 2.168404344971009e-19; /* 2^-62 */ }
+#endif
+
+// The 16 weights tq^n tx^m of a point (index 4 n + m) from tc = t - 1/2.
+PDF_HD void fix_weights(int64_t tcx, int64_t tcq, Dig w[16])
+{
+    w[0] = {1 << 30, 0};
+    w[1] = fix_split(tcx);
+    w[2] = fix_split(fix_mul(w[1], w[1]));
+    w[3] = fix_split(fix_mul(w[2], w[1]));
+    w[4] = fix_split(tcq);
+    w[8] = fix_split(fix_mul(w[4], w[4]));
+    w[12] = fix_split(fix_mul(w[8], w[4]));
+#pragma unroll
+    for (int n = 4; n <= 12; n += 4)
+#pragma unroll
+        for (int m = 1; m < 4; ++m) w[n + m] = fix_split(fix_mul(w[n], w[m]));
+}
+
+// Sum of four coefficients (l, h pairs) against four weights: the high
+// products, and the upper word of the cross products' rounded sum, which is
+// below 2^63 in size (4 x 2^29 x 2^31 + 2^31 x 2^30 (1 + 1/2 + 1/4 + 1/8)).
+PDF_HD int64_t fix_row(const int c[8], const Dig w[4])
+{
+    int64_t hh = 0, cr = (int64_t)1 << 31;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        hh = wide(c[2 * m + 1], w[m].h, hh);
+        cr = wide(c[2 * m + 1], w[m].l, cr);
+        cr = wide(c[2 * m], w[m].h, cr);
+    }
+    return hh + fix_hi(cr);
+}
+
+// Block exponent: the low byte of a row's last coefficient is E + kFixBias;
+// kFixNone marks a patch that the format cannot hold.
+constexpr int kFixBias = 160;
+constexpr int kFixNone = 255;
+
+#ifdef __CUDACC__
+__device__ __forceinline__ bool fix_none(int last) { return (last & 255) == kFixNone; }
+__device__ __forceinline__ double fix_value(int64_t s, int last)
+{
+    return __ll2double_rn(s) * __hiloint2double((last & 255) * (1 << 20) + ((1023 - 59 - kFixBias) << 20), 0);
+}
+
+// Eight 32-bit words (one row of a fixed-point patch) in one 32-byte load.
+__device__ __forceinline__ void fix_ld(const unsigned char *p, int c[8])
+{
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(c[0]), "=r"(c[1]), "=r"(c[2]), "=r"(c[3]), "=r"(c[4]), "=r"(c[5]), "=r"(c[6]), "=r"(c[7])
+        : "l"(p));
+}
+#endif
+
+// Packs `rows` x 4 centred coefficients into the table's words: `big` is the
+// part of the constant term that is added exactly, the patch's value at its
+// lower corner (t = 0 on both axes), about which the FP64 form expands.  The
+// fixed-point error follows the patch's largest coefficient, the FP64 error
+// next to the lower edges follows the values there: a patch whose lower
+// corner is 2^12 below its largest coefficient (a flavour that sets in at a
+// threshold knot, say) keeps FP64.
+PDF_HD void fix_pack(const double *c, int rows, double big, uint32_t *out)
+{
+    double top = fabs(c[0] + big);
+    for (int k = 1; k < 4 * rows; ++k) top = fabs(c[k]) > top || !(fabs(c[k]) <= 1e300) ? fabs(c[k]) : top;
+    int e = 0;
+    double scale = 0.0;
+    bool ok = top <= 1e300 && fabs(big) <= 1e300;
+    if (ok && top > 0.0) {
+        const int E = (int)((dbits(top) >> 52) & 0x7FF) - 1022;
+        e = E + kFixBias;
+        ok = e >= 0 && e < kFixNone && fabs(big) >= dfrom((uint64_t)(E - 12 + 1023) << 52);
+        if (ok) scale = dfrom((uint64_t)(61 - E + 1023) << 52);
+    }
+    if (!ok) e = kFixNone;
+    for (int k = 0; k < 4 * rows; ++k) {
+        int64_t v = 0;
+        if (ok) {
+            v = (int64_t)rint(c[k] * scale);
+            if (k == 0) v += (int64_t)rint(big * scale);
+        }
+        if ((k & 3) == 3) v = ((v - e + 128) & ~(int64_t)255) | e;
+        const Dig d = fix_split(v);
+        out[2 * k] = (uint32_t)d.l;
+        out[2 * k + 1] = (uint32_t)d.h;
+    }
+}
+
+}  // namespace pdfgpu

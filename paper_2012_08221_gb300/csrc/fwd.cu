@@ -10,198 +10,199 @@
 
 #include "pdf_internal.h"
 #include "sort_acc.cuh"
+#include "warp_eval.cuh"
 
 using namespace pdfgpu;
 
 namespace {
 
 constexpr int kBlock = 256;
-__device__ __forceinline__ double qnan() { return __longlong_as_double(0x7FF8000000000000ll); }
 
-// One point per thread; each warp takes 32 consecutive points at a time
-// (grid-stride over warps).  A warp's results are staged in its own slice of
-// shared memory and leave as one contiguous run of 32 * npid doubles (the
-// output is [n][npid] row-major): one bulk copy issued by lane 0 when the run
-// is 16-byte aligned and a multiple of 16 bytes long, else coalesced stores
-// by the whole warp.  Only warp-level synchronisation, no block barriers in
-// the loop.  With TAPE each point's adjoint tape record is written as well;
-// with AS alpha_s at the point's Q^2 goes to as_out[i], from the same Q
-// search and logarithm as the PDFs (a point whose x alone is out of the
+// Matrix form.  A warp's task is 32 consecutive points and one group of `per`
+// consecutive columns (all of them, one group, in long queries), taken
+// grid-stride; the work of a task is eval_points (warp_eval.cuh).  With all
+// columns in one group the rows of 32 points leave as one contiguous run.
+// STAGE: the block first copies the coordinate tables into shared memory.
+// TAPE: each point's adjoint tape record is written as well; AS: alpha_s at
+// the point's Q^2 goes to as_out[i] (a point whose x alone is out of the
 // domain still gets its alpha_s, as alphasQ2 would give it).
-template <bool Q_IS_Q, bool CONT, bool TAPE, bool AS = false>
-__global__ void __launch_bounds__(kBlock) k_xfxq2(GridDev g, Cols cols, int npid, int member,
-                                                  const double *__restrict__ x,
-                                                  const double *__restrict__ q,
-                                                  int64_t n, double *__restrict__ out,
-                                                  double *__restrict__ tape, double *__restrict__ as_out = nullptr)
+template <bool Q_IS_Q, bool TAPE, bool AS, bool STAGE, bool WHOLE>
+__global__ void __launch_bounds__(kBlock, WHOLE ? 3 : 2) k_xfxq2(const __grid_constant__ GridDev g,
+                                                     const __grid_constant__ Cols cols, int npid, int per, int groups,
+                                                     int member, const double *__restrict__ x,
+                                                     const double *__restrict__ q, int64_t n,
+                                                     double *__restrict__ out, double *__restrict__ tape,
+                                                     double *__restrict__ as_out, int tab_bytes, int warp_bytes)
 {
-    extern __shared__ __align__(16) double sout[];
-    __shared__ signed char scol[PDF_MAX_PIDS];
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < PDF_MAX_PIDS; ++k) scol[k] = cols.c[k];
-    }
+    extern __shared__ __align__(128) unsigned char smem[];
+    const CoordTabs T = STAGE ? stage_tabs(g, smem) : grid_tabs(g);
     __syncthreads();
-    const size_t cell_stride = (size_t)g.nflav * 16;
-    const double *cm = g.coef + (size_t)member * g.nqc * g.nxc * cell_stride;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double *wbuf = sout + (size_t)wid * 32 * npid;
-    const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5) * 32;
-    for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + wid) * 32; base < n; base += wstride) {
-        int64_t i = base + lane;
-        bool live = i < n;
-        double xi = live ? x[i] : 0.5;
-        double qi = live ? q[i] : 10.0;
-        if (Q_IS_Q) qi = qi * qi;
-        const bool qbad = !q2_ok(dbits(qi));
-        bool bad = live && !(x_ok(dbits(xi)) && !qbad);
-        flag_status(g, bad);
-        if (bad) {
-            xi = 0.5;
-            if (!AS || qbad) qi = 10.0;
+    unsigned char *mine = smem + tab_bytes + (size_t)wid * warp_bytes;
+    WarpBufs B{reinterpret_cast<uint4 *>(mine), reinterpret_cast<int64_t *>(mine + warp_bytes - kQueue * 8), 0};
+    const size_t patches = (size_t)member * g.nqc * g.nxc * g.nflav;
+    Query Y{cols.c, npid, 0, npid, g.coef + patches * 16,
+            g.fcoef ? reinterpret_cast<const unsigned char *>(g.fcoef) + patches * 128 : nullptr,
+            x, q, n, out, tape, as_out};
+    const int64_t tasks = (n + 31) / 32 * groups;
+    const int64_t stride = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + wid; t < tasks; t += stride) {
+        int64_t base = t * 32;
+        if (!WHOLE) {
+            const int64_t blk = t / groups;
+            Y.a0 = (int)(t - blk * groups) * per;
+            Y.a1 = min(npid, Y.a0 + per);
+            base = blk * 32;
         }
-        double u, w;
-        Axis X = axis_x(g, xi, &u);
-        Axis Q = axis_q2(g, qi, &w);
-        const bool oor = live && out_of_range(g, X, Q);
-        flag_status(g, oor, PDF_S_RANGE);
-        bad |= oor;
-        if (TAPE && live) tape_put(tape, i, X, Q, bad);
-        if (AS && live) {
-            const double a = alphas_any(g, ld4(g.acoef + (size_t)Q.cell * 4), Q);
-            as_out[i] = (qbad || (g.extrap == PDF_EXTRAP_ERROR && !Q.in)) ? qnan() : a;
-        }
-        const double *cell = cm + ((size_t)Q.cell * g.nxc + X.cell) * cell_stride;
-        double *srow = wbuf + lane * npid;
-        warp_run_reuse(lane);                 // the previous run has left the slice
-        for (int a = 0; a < npid; ++a) {
-            int col = scol[a];
-            if (col >= 0) col = checked_index(g.status, col, g.nflav);
-            double v = col >= 0 ? patch_any<CONT>(g, cell + col * 16, X, Q) : 0.0;
-            srow[a] = bad ? qnan() : v;
-        }
-        const int rows = (int)min((int64_t)32, n - base);
-        warp_run_store(out + base * npid, wbuf, rows * npid, lane);
+        eval_points<Q_IS_Q, TAPE, AS, WHOLE>(g, T, Y, B, base, lane);
+        if (!WHOLE && B.qn) drain_queue(g, Y, Q_IS_Q, B, lane);
     }
+    if (WHOLE)
+        while (B.qn) drain_queue(g, Y, Q_IS_Q, B, lane);
     if (lane == 0) bulk_wait_all();
-}
-
-// Small queries (at most kPairMax point-flavour pairs): one thread per pair,
-// so that a few thousand points still spread over every SM and each thread's
-// dependent chain is one flavour long; the coordinates are recomputed for
-// every flavour of a point.  Outputs are written in pair order, which is the
-// row-major [n][npid] layout.
-constexpr int64_t kPairMax = 1 << 18;
-
-template <bool Q_IS_Q, bool CONT, bool TAPE>
-__global__ void __launch_bounds__(kBlock) k_xfxq2_pairs(GridDev g, Cols cols, int npid, int member,
-                                                        const double *__restrict__ x,
-                                                        const double *__restrict__ q,
-                                                        int64_t n, double *__restrict__ out,
-                                                        double *__restrict__ tape)
-{
-    __shared__ signed char scol[PDF_MAX_PIDS];
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < PDF_MAX_PIDS; ++k) scol[k] = cols.c[k];
-    }
-    __syncthreads();
-    const size_t cell_stride = (size_t)g.nflav * 16;
-    const double *cm = g.coef + (size_t)member * g.nqc * g.nxc * cell_stride;
-    const int64_t total = n * npid;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < total;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = p / npid;
-        const int a = (int)(p - i * npid);
-        double xi = x[i], qi = q[i];
-        if (Q_IS_Q) qi = qi * qi;
-        bool bad = !(x_ok(dbits(xi)) && q2_ok(dbits(qi)));
-        flag_status(g, bad);
-        if (bad) {
-            xi = 0.5;
-            qi = 10.0;
-        }
-        double u, w;
-        Axis X = axis_x(g, xi, &u);
-        Axis Q = axis_q2(g, qi, &w);
-        const bool oor = out_of_range(g, X, Q);
-        flag_status(g, oor, PDF_S_RANGE);
-        bad |= oor;
-        if (TAPE && a == 0) tape_put(tape, i, X, Q, bad);
-        int col = scol[a];
-        double v = 0.0;
-        if (col >= 0) {
-            col = checked_index(g.status, col, g.nflav);
-            v = patch_any<CONT>(g, cm + ((size_t)Q.cell * g.nxc + X.cell) * cell_stride + col * 16, X, Q);
-        }
-        out[p] = bad ? qnan() : v;
-    }
 }
 
 // DT (with TAPE): also keep each point's patch derivatives in t_x and t_q,
 // computed with the value (patch_vd: the value's bits are unchanged), in
 // dtape[i] = (dP/dtx, dP/dtq) (zeros for an absent pid), and the point's bin
 // in the pointwise sorted adjoint in dbins[i] (-1 for none).
-template <bool CONT, bool TAPE, bool DT = false>
-__global__ void __launch_bounds__(kBlock) k_xfxq2_pw(GridDev g, int member,
-                                                     const int *__restrict__ pid,
-                                                     const double *__restrict__ x,
-                                                     const double *__restrict__ q2,
-                                                     int64_t n, double *__restrict__ out,
-                                                     double *__restrict__ tape, double *__restrict__ dtape,
-                                                     int *__restrict__ dbins, int nbins)
+__device__ __noinline__ void slow_point_pw(const GridDev &g, const double *cm, int col, double xi, double qi, int64_t i,
+                                           double *out, double *tape, double *dtape, int *dbins, int nbins)
 {
-    const size_t cell_stride = (size_t)g.nflav * 16;
-    const double *cm = g.coef + (size_t)member * g.nqc * g.nxc * cell_stride;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        double xi = x[i], qi = q2[i];
-        int col = pid_col(g, pid[i]);
-        bool bad = !(x_ok(dbits(xi)) && q2_ok(dbits(qi)));
-        flag_status(g, bad);
-        if (bad) {
-            xi = 0.5;
-            qi = 10.0;
-        }
-        double u, w;
-        Axis X = axis_x(g, xi, &u);
-        Axis Q = axis_q2(g, qi, &w);
-        const bool oor = out_of_range(g, X, Q);
-        flag_status(g, oor, PDF_S_RANGE);
-        bad |= oor;
-        if (TAPE) tape_put(tape, i, X, Q, bad);
-        double v = 0.0;
-        if (DT) {
-            double dtx = 0.0, dtq = 0.0;
-            if (col >= 0) v = patch_vd(cm + ((size_t)Q.cell * g.nxc + X.cell) * cell_stride + col * 16, X, Q, &dtx, &dtq);
-            reinterpret_cast<double2 *>(dtape)[i] = make_double2(dtx, dtq);
-            dbins[i] = sorted_bin(g, X, Q, bad, col, half_pair(X, Q), nbins);
-        } else if (col >= 0) {
-            v = patch_any<CONT>(g, cm + ((size_t)Q.cell * g.nxc + X.cell) * cell_stride + col * 16, X, Q);
-        }
-        out[i] = bad ? qnan() : v;
+    bool bad = !(x_ok(dbits(xi)) && q2_ok(dbits(qi)));
+    flag_status(g, bad);
+    if (bad) {
+        xi = 0.5;
+        qi = 10.0;
     }
+    const Axis X = axis_x(g, xi), Q = axis_q2(g, qi);
+    const bool oor = out_of_range(g, X, Q);
+    flag_status(g, oor, PDF_S_RANGE);
+    bad |= oor;
+    if (tape) tape_put(tape, i, X, Q, bad);
+    const double *C = cm + (((size_t)Q.cell * g.nxc + X.cell) * g.nflav + (col >= 0 ? col : 0)) * 16;
+    double v = 0.0;
+    if (dtape) {
+        double dtx = 0.0, dtq = 0.0;
+        if (col >= 0) v = patch_vd(C, X, Q, &dtx, &dtq);
+        reinterpret_cast<double2 *>(dtape)[i] = make_double2(dtx, dtq);
+        dbins[i] = sorted_bin(g, X, Q, bad, col, half_pair(X, Q), nbins);
+    } else if (col >= 0) {
+        v = patch_any<true>(g, C, X, Q);
+    }
+    out[i] = bad ? dnan() : v;
 }
 
-template <bool Q_IS_Q>
-__global__ void __launch_bounds__(kBlock) k_alphas(GridDev g, const double *__restrict__ q,
-                                                   int64_t n, double *__restrict__ out)
+template <bool TAPE, bool DT>
+__global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ GridDev g, int member,
+                                                        const int *__restrict__ pid,
+                                                        const double *__restrict__ x,
+                                                        const double *__restrict__ q2,
+                                                        int64_t n, double *__restrict__ out,
+                                                        double *__restrict__ tape, double *__restrict__ dtape,
+                                                        int *__restrict__ dbins, int nbins, int tab_bytes)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        double qi = q[i];
-        if (Q_IS_Q) qi = qi * qi;
-        bool bad = !q2_ok(dbits(qi));
-        flag_status(g, bad);
-        if (bad) qi = 10.0;
-        double w;
-        Axis Q = axis_q2(g, qi, &w);
-        const bool oor = g.extrap == PDF_EXTRAP_ERROR && !Q.in;
-        flag_status(g, oor, PDF_S_RANGE);
-        bad |= oor;
-        double v = alphas_any(g, ld4(g.acoef + (size_t)Q.cell * 4), Q);
-        out[i] = bad ? qnan() : v;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const CoordTabs T = tab_bytes ? stage_tabs(g, smem) : grid_tabs(g);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned char *mine = smem + tab_bytes + (size_t)wid * (kWarpBuf + kQueue * 8);
+    WarpBufs B{reinterpret_cast<uint4 *>(mine), reinterpret_cast<int64_t *>(mine + kWarpBuf), 0};
+    const size_t patches = (size_t)member * g.nqc * g.nxc * g.nflav;
+    const double *cm = g.coef + patches * 16;
+    const unsigned char *fm = g.fcoef ? reinterpret_cast<const unsigned char *>(g.fcoef) + patches * 128 : nullptr;
+    auto drain = [&]() {
+        const int64_t i = next_queued(B, lane);
+        if (i >= 0)
+            slow_point_pw(g, cm, pid_col(g, pid[i]), x[i], q2[i], i, out, tape, dtape, dbins, nbins);
+        __syncwarp();
+    };
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + wid) * 32; base < n; base += stride) {
+        const int64_t i = base + lane;
+        const bool live = i < n;
+        const double xi = live ? x[i] : 0.5, qi = live ? q2[i] : 10.0;
+        const int col = live ? pid_col(g, pid[i]) : -1;
+        const FixAxis X = fix_axis_x(g, T, dbits(xi)), Q = fix_axis_q2(g, T, dbits(qi));
+        bool fast = live && X.ok && Q.ok && x_ok(dbits(xi)) && q2_ok(dbits(qi)) && fm;
+        if (__any_sync(kAll, fast)) {
+            const uint32_t patch0 =
+                fast ? (uint32_t)(Q.cell * g.nxc + X.cell) * (uint32_t)g.nflav + (col >= 0 ? col : 0) : 0u;
+            uint32_t off[4];
+            quad_offsets(patch0 * 128u, lane, off);
+            Dig W[4][4];
+            quad_weights(B.buf, lane, fast ? X.t : kFixHalf, fast ? Q.t : kFixHalf, W);
+            int c[4][8], last;
+            quad_load(fm, off, c);
+            const int64_t s = quad_patch(c, W, quad_pos(lane), last);
+            fast &= col < 0 || !fix_none(last);
+            if (fast) {
+                out[i] = col >= 0 ? fix_value(s, last) : 0.0;
+                if (TAPE) {
+                    Axis AX, AQ;
+                    AX.cell = X.cell;
+                    AQ.cell = Q.cell;
+                    AX.in = AQ.in = true;
+                    AX.below = AQ.below = false;
+                    make_basis(AX, fix_t(X.t), g.extrap);
+                    make_basis(AQ, fix_t(Q.t), g.extrap);
+                    tape_put(tape, i, AX, AQ, false);
+                    if (DT) {
+                        double dtx = 0.0, dtq = 0.0;
+                        if (col >= 0) patch_vd(cm + (size_t)patch0 * 16, AX, AQ, &dtx, &dtq);
+                        reinterpret_cast<double2 *>(dtape)[i] = make_double2(dtx, dtq);
+                        dbins[i] = sorted_bin(g, AX, AQ, false, col, half_pair(AX, AQ), nbins);
+                    }
+                }
+            }
+        }
+        push_queue(B, live && !fast, i, lane);
+        if (B.qn >= 32) drain();
     }
+    if (B.qn) drain();
+}
+
+// alpha_s, one point per lane (fix_alphas): 1e7 points 286 -> 120 us (FP64
+// pipe 82 % busy before; now integer issue of the logarithm and the table
+// look-ups in shared memory); points outside the Q range or the
+// domain are queued per warp and evaluated 32 at a time.
+template <bool Q_IS_Q>
+__global__ void __launch_bounds__(kBlock) k_alphas(const __grid_constant__ GridDev g, const double *__restrict__ q,
+                                                   int64_t n, double *__restrict__ out, int tab_bytes)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ int64_t squeue[kBlock / 32][kQueue];
+    const CoordTabs T = tab_bytes ? stage_tabs(g, smem) : grid_tabs(g);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    WarpBufs B{nullptr, squeue[wid], 0};
+    auto drain = [&]() {
+        const int64_t i = next_queued(B, lane);
+        if (i >= 0) {
+            double qi = q[i];
+            if (Q_IS_Q) qi = qi * qi;
+            const bool bad = !q2_ok(dbits(qi));
+            flag_status(g, bad);
+            bool oor;
+            const double v = alphas_at(g, grid_tabs(g), bad ? 10.0 : qi, &oor);
+            flag_status(g, oor && !bad, PDF_S_RANGE);
+            out[i] = bad ? dnan() : v;
+        }
+        __syncwarp();
+    };
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + wid) * 32; base < n; base += stride) {
+        const int64_t i = base + lane;
+        const bool live = i < n;
+        double qi = live ? q[i] : 10.0;
+        if (Q_IS_Q) qi = qi * qi;
+        const FixAxis Q = fix_axis_q2(g, T, dbits(qi));
+        const bool fast = live && Q.ok && q2_ok(dbits(qi));
+        if (fast) out[i] = fix_alphas(g, Q);
+        push_queue(B, live && !fast, i, lane);
+        if (B.qn >= 32) drain();
+    }
+    if (B.qn) drain();
 }
 
 // alpha_s and d alpha_s / d Q^2 = (da/dtq) / dW / Q^2 (zero across a frozen edge).
@@ -214,13 +215,12 @@ __global__ void __launch_bounds__(kBlock) k_alphas_grad(GridDev g, const double 
         bool bad = !q2_ok(dbits(qi));
         flag_status(g, bad);
         if (bad) qi = 10.0;
-        double w;
-        Axis Q = axis_q2(g, qi, &w);
-        const bool oor = g.extrap == PDF_EXTRAP_ERROR && !Q.in;
+        const Axis Q = axis_q2(g, qi);
+        bool oor;
+        const double v = alphas_at(g, grid_tabs(g), qi, &oor);
         flag_status(g, oor, PDF_S_RANGE);
         bad |= oor;
         const D4 a = ld4(g.acoef + (size_t)Q.cell * 4);
-        double v = alphas_any(g, a, Q);
         double d2 = Q.in ? 2.0 * Q.t : 1.0, d3 = Q.in ? 3.0 * Q.t * Q.t : 1.0;
         double dt = fma(d3, a.w, fma(d2, a.z, a.y));
         if (!Q.in && g.extrap == PDF_EXTRAP_FREEZE) dt = 0.0;
@@ -229,8 +229,8 @@ __global__ void __launch_bounds__(kBlock) k_alphas_grad(GridDev g, const double 
             const double y0 = a.x, y1 = a.x + a.y + a.z + a.w;
             dt = (y0 > kContMin && y1 > kContMin) ? v * log(y1 / y0) : y1 - y0;
         }
-        if (out) out[i] = bad ? qnan() : v;
-        dq2[i] = bad ? qnan() : dt * g.qcell[Q.cell].y * __drcp_rn(qi);
+        if (out) out[i] = bad ? dnan() : v;
+        dq2[i] = bad ? dnan() : dt * g.qcell[Q.cell].y * __drcp_rn(qi);
     }
 }
 
@@ -241,9 +241,8 @@ __global__ void k_cells(GridDev g, const double *__restrict__ x, const double *_
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        double u, w;
-        xc[i] = axis_x(g, x[i], &u).cell;
-        qc[i] = axis_q2(g, q2[i], &w).cell;
+        xc[i] = axis_x(g, x[i]).cell;
+        qc[i] = axis_q2(g, q2[i]).cell;
     }
 }
 
@@ -266,6 +265,53 @@ int check_tape(const pdfgpu_grid *g, const double *tape)
     return PDF_OK;
 }
 
+// The matrix form's launch.  A long query gives each warp all the columns of
+// 32 points.  A short one splits the columns into groups until there are
+// about kShortWarps warps per SM: below that the SMs wait for one warp's
+// chain of loads, and the coordinates computed once per group are cheaper
+// than idle SMs (1e5 points x 11 flavours with alpha_s: 35 us; 43 us in FP64).
+constexpr int kShortWarps = 16;
+// Points per SM from which copying the coordinate tables into shared memory
+// pays (the copy is about 20 KB per block).
+constexpr int64_t kStagePoints = 256;
+constexpr size_t kStageMax = 48 * 1024;      // the tables of larger grids stay global
+
+template <bool Q_IS_Q, bool TAPE, bool AS>
+int launch_points(pdfgpu_grid *g, int32_t member, const Cols &cols, int n_pid, const double *x, const double *q,
+                  int64_t n, double *out, double *tape, double *alphas, cudaStream_t s)
+{
+    using Kern = void (*)(const GridDev, const Cols, int, int, int, int, const double *, const double *, int64_t,
+                          double *, double *, double *, int, int);
+    const int64_t blocks32 = (n + 31) / 32;
+    int groups = 1, per = n_pid;
+    if (blocks32 < (int64_t)kShortWarps * g->sm_count) {
+        groups = (int)std::min<int64_t>(n_pid, (int64_t)kShortWarps * g->sm_count / blocks32);
+        per = (n_pid + groups - 1) / groups;
+        groups = (n_pid + per - 1) / per;
+    }
+    int tab = coord_tab_bytes(g->d);
+    const bool stage = n >= kStagePoints * g->sm_count && (size_t)tab <= kStageMax;
+    if (!stage) tab = 0;
+    const Kern k = groups > 1 ? (stage ? k_xfxq2<Q_IS_Q, TAPE, AS, true, false>
+                                       : k_xfxq2<Q_IS_Q, TAPE, AS, false, false>)
+                              : (stage ? k_xfxq2<Q_IS_Q, TAPE, AS, true, true>
+                                       : k_xfxq2<Q_IS_Q, TAPE, AS, false, true>);
+    const int warp_bytes = (groups > 1 ? kWarpBuf : std::max(kWarpBuf, 32 * 8 * n_pid)) + kQueue * 8;
+    // 256-thread blocks share one copy of the tables; a short query or wide
+    // rows take smaller blocks, which spread more evenly over the SMs
+    int block = kBlock;
+    while (block > 32 && ((size_t)tab + (size_t)(block / 32) * warp_bytes > 75 * 1024 ||
+                          (!stage && blocks32 * groups < (int64_t)(block / 32) * 2 * g->sm_count)))
+        block /= 2;
+    const size_t smem = (size_t)tab + (size_t)(block / 32) * warp_bytes;
+    int rc = allow_dynamic_smem((const void *)k, smem);
+    if (rc) return rc;
+    const int grid = wave_grid(g, (const void *)k, block, smem, blocks32 * groups * 32);
+    k<<<grid, block, smem, s>>>(g->d, cols, n_pid, per, groups, member, x, q, n, out, tape, alphas, tab, warp_bytes);
+    PDF_CUDA(cudaGetLastError());
+    return PDF_OK;
+}
+
 int launch_matrix(pdfgpu_grid *g, int32_t member, const int32_t *pids, int32_t n_pid,
                   const double *x, const double *q, int64_t n, double *out, double *tape, cudaStream_t s,
                   bool q_is_q)
@@ -282,45 +328,13 @@ int launch_matrix(pdfgpu_grid *g, int32_t member, const int32_t *pids, int32_t n
     if (rc) return rc;
     if (n == 0) return PDF_OK;
     if (!x || !q || !out) return fail(PDF_E_ARG, "null array");
-    using PairKern = void (*)(GridDev, Cols, int, int, const double *, const double *, int64_t, double *, double *);
-    using Kern = void (*)(GridDev, Cols, int, int, const double *, const double *, int64_t, double *, double *,
-                          double *);
-    const bool cont = g->d.extrap == PDF_EXTRAP_CONTINUATION;
-    if (n * n_pid <= kPairMax) {
-        PairKern k = tape ? k_xfxq2_pairs<false, false, true>
-                 : q_is_q ? (cont ? k_xfxq2_pairs<true, true, false> : k_xfxq2_pairs<true, false, false>)
-                          : (cont ? k_xfxq2_pairs<false, true, false> : k_xfxq2_pairs<false, false, false>);
-        int grid = wave_grid(g, (const void *)k, kBlock, 0, n * n_pid);
-        k<<<grid, kBlock, 0, s>>>(g->d, cols, n_pid, member, x, q, n, out, tape);
-        PDF_CUDA(cudaGetLastError());
-        return PDF_OK;
-    }
-    size_t smem = (size_t)kBlock * n_pid * sizeof(double);
-    Kern k = tape ? k_xfxq2<false, false, true>
-             : q_is_q ? (cont ? k_xfxq2<true, true, false> : k_xfxq2<true, false, false>)
-                      : (cont ? k_xfxq2<false, true, false> : k_xfxq2<false, false, false>);
-    rc = allow_dynamic_smem((const void *)k, smem);
-    if (rc) return rc;
-    // A query shorter than one wave runs in the smallest CTAs (32, 64 or 128
-    // threads) whose grid still fits in one wave, so that the CTAs spread
-    // evenly over the SMs: in 256-thread CTAs a short query leaves some SMs
-    // a whole CTA (8 warps of points) more than others.
-    int block = kBlock;
-    for (int b : {32, 64, 128}) {
-        const size_t sb = (size_t)b * n_pid * sizeof(double);
-        if ((n + b - 1) / b <= (int64_t)g->sm_count * occupancy((const void *)k, b, sb)) {
-            block = b;
-            smem = sb;
-            break;
-        }
-    }
-    int grid = wave_grid(g, (const void *)k, block, smem, n);
-    k<<<grid, block, smem, s>>>(g->d, cols, n_pid, member, x, q, n, out, tape, nullptr);
-    PDF_CUDA(cudaGetLastError());
-    return PDF_OK;
+    auto launch = tape     ? launch_points<false, true, false>
+                  : q_is_q ? launch_points<true, false, false>
+                           : launch_points<false, false, false>;
+    return launch(g, member, cols, n_pid, x, q, n, out, tape, nullptr, s);
 }
 
-// x*f and alpha_s at the same points in one launch of the per-point kernel.
+// x*f and alpha_s at the same points in one launch.
 int launch_xf_alphas(pdfgpu_grid *g, int32_t member, const int32_t *pids, int32_t n_pid, const double *x,
                      const double *q2, int64_t n, double *out, double *alphas, cudaStream_t s)
 {
@@ -335,24 +349,7 @@ int launch_xf_alphas(pdfgpu_grid *g, int32_t member, const int32_t *pids, int32_
     if (rc) return rc;
     if (n == 0) return PDF_OK;
     if (!x || !q2 || !out || !alphas) return fail(PDF_E_ARG, "null array");
-    const bool cont = g->d.extrap == PDF_EXTRAP_CONTINUATION;
-    auto k = cont ? k_xfxq2<false, true, false, true> : k_xfxq2<false, false, false, true>;
-    size_t smem = (size_t)kBlock * n_pid * sizeof(double);
-    rc = allow_dynamic_smem((const void *)k, smem);
-    if (rc) return rc;
-    int block = kBlock;
-    for (int b : {32, 64, 128}) {
-        const size_t sb = (size_t)b * n_pid * sizeof(double);
-        if ((n + b - 1) / b <= (int64_t)g->sm_count * occupancy((const void *)k, b, sb)) {
-            block = b;
-            smem = sb;
-            break;
-        }
-    }
-    int grid = wave_grid(g, (const void *)k, block, smem, n);
-    k<<<grid, block, smem, s>>>(g->d, cols, n_pid, member, x, q2, n, out, nullptr, alphas);
-    PDF_CUDA(cudaGetLastError());
-    return PDF_OK;
+    return launch_points<false, false, true>(g, member, cols, n_pid, x, q2, n, out, nullptr, alphas, s);
 }
 
 int launch_alphas(pdfgpu_grid *g, const double *q, int64_t n, double *out, cudaStream_t s, bool q_is_q)
@@ -365,11 +362,13 @@ int launch_alphas(pdfgpu_grid *g, const double *q, int64_t n, double *out, cudaS
     if (n == 0) return PDF_OK;
     if (!q || !out) return fail(PDF_E_ARG, "null array");
     const void *kern = q_is_q ? (const void *)k_alphas<true> : (const void *)k_alphas<false>;
-    int grid = wave_grid(g, kern, kBlock, 0, n);
+    int tab = coord_tab_bytes(g->d);
+    if (n < kStagePoints * g->sm_count || (size_t)tab > kStageMax) tab = 0;
+    int grid = wave_grid(g, kern, kBlock, tab, n);
     if (q_is_q)
-        k_alphas<true><<<grid, kBlock, 0, s>>>(g->d, q, n, out);
+        k_alphas<true><<<grid, kBlock, tab, s>>>(g->d, q, n, out, tab);
     else
-        k_alphas<false><<<grid, kBlock, 0, s>>>(g->d, q, n, out);
+        k_alphas<false><<<grid, kBlock, tab, s>>>(g->d, q, n, out, tab);
     PDF_CUDA(cudaGetLastError());
     return PDF_OK;
 }
@@ -390,13 +389,16 @@ int launch_pw(pdfgpu_grid *g, int32_t member, const int32_t *pid, const double *
     if (dtape && nbins64 >= (int64_t)1 << 30) return fail(PDF_E_RANGE, "grid too large for the derivative tape");
     if (n == 0) return PDF_OK;
     if (!pid || !x || !q2 || !out) return fail(PDF_E_ARG, "null array");
-    auto k = dtape  ? k_xfxq2_pw<false, true, true>
-             : tape ? k_xfxq2_pw<false, true>
-             : g->d.extrap == PDF_EXTRAP_CONTINUATION ? k_xfxq2_pw<true, false> : k_xfxq2_pw<false, false>;
-    int grid = wave_grid(g, (const void *)k, kBlock, 0, n);
+    auto k = dtape ? k_xfxq2_pw<true, true> : tape ? k_xfxq2_pw<true, false> : k_xfxq2_pw<false, false>;
+    int tab = coord_tab_bytes(g->d);
+    if (n < kStagePoints * g->sm_count || (size_t)tab > kStageMax) tab = 0;
+    const size_t smem = (size_t)tab + (kBlock / 32) * (kWarpBuf + kQueue * 8);
+    rc = allow_dynamic_smem((const void *)k, smem);
+    if (rc) return rc;
+    int grid = wave_grid(g, (const void *)k, kBlock, smem, n);
     int *dbins = dtape ? reinterpret_cast<int *>(dtape + 2 * n) : nullptr;
-    k<<<grid, kBlock, 0, s>>>(g->d, member, pid, x, q2, n, out, tape, dtape, dbins,
-                              (int)std::min<int64_t>(nbins64, (int64_t)1 << 30));
+    k<<<grid, kBlock, smem, s>>>(g->d, member, pid, x, q2, n, out, tape, dtape, dbins,
+                                 (int)std::min<int64_t>(nbins64, (int64_t)1 << 30), tab);
     PDF_CUDA(cudaGetLastError());
     return PDF_OK;
 }

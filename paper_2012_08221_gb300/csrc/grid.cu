@@ -122,26 +122,34 @@ int resolve_cols(const pdfgpu_grid *g, const int32_t *pids, int32_t n_pid, Cols 
 // Tables of the log routine: (1/c_j, -ln(1/c_j) as high + low parts) with
 // c_j = 1 + (j + 1/2)/1024 (c_0 = 1, c_1023 = 2), and e ln 2 as high + low
 // parts for every biased exponent; long double for the logs.
-static void make_log_tables(std::vector<LogEntry> &tab, std::vector<double2> &etab)
+struct LogTables {
+    std::vector<LogEntry> tab = std::vector<LogEntry>(kLogTab);
+    std::vector<double2> etab = std::vector<double2>(2048);
+    LogTables()
+    {
+        for (int j = 0; j < kLogTab; ++j) {
+            double c = 1.0 + (j + 0.5) / (double)kLogTab;     // exact
+            if (j == 0) c = 1.0;
+            if (j == kLogTab - 1) c = 2.0;
+            double inv = 1.0 / c;                              // correctly rounded
+            long double L = -logl((long double)inv);
+            double hi = (double)L;
+            double lo = (double)(L - (long double)hi);
+            tab[j] = LogEntry{inv, hi, lo, 0.0};
+        }
+        const long double ln2 = 0.693147180559945309417232121458176568L;
+        for (int e = 0; e < 2048; ++e) {
+            long double v = (long double)(e - 1023) * ln2;
+            double hi = (double)v;
+            etab[e] = make_double2(hi, (double)(v - (long double)hi));
+        }
+    }
+};
+
+static const LogTables &log_tables()   // made once per process
 {
-    tab.resize(kLogTab);
-    for (int j = 0; j < kLogTab; ++j) {
-        double c = 1.0 + (j + 0.5) / (double)kLogTab;     // exact
-        if (j == 0) c = 1.0;
-        if (j == kLogTab - 1) c = 2.0;
-        double inv = 1.0 / c;                              // correctly rounded
-        long double L = -logl((long double)inv);
-        double hi = (double)L;
-        double lo = (double)(L - (long double)hi);
-        tab[j] = LogEntry{inv, hi, lo, 0.0};
-    }
-    etab.resize(2048);
-    const long double ln2 = 0.693147180559945309417232121458176568L;
-    for (int e = 0; e < 2048; ++e) {
-        long double v = (long double)(e - 1023) * ln2;
-        double hi = (double)v;
-        etab[e] = make_double2(hi, (double)(v - (long double)hi));
-    }
+    static const LogTables t;
+    return t;
 }
 
 // Finite-difference coefficients of cell k on knots z[0..n-1]:
@@ -207,38 +215,97 @@ static void cell_matrix(const double *z, int n, int k, double M[16], bool linear
 // Guide table of a cell search over ascending lower keys (see
 // find_cell_guided): the widest bucket width 2^shift, at most kGuideMax
 // buckets from the first key to key_hi, for which no bucket holds more than
-// kGuideRun further lower keys (the last bucket counts every cell above it,
-// since keys beyond key_hi fall into it).  Left empty when no width
-// qualifies (knots clustered far more densely in one place than another);
-// the kernels then search by bisection.
+// one further lower key, else more than kGuideRun (the last bucket counts
+// every cell above it, since keys beyond key_hi fall into it).  Left empty
+// when no width qualifies (knots clustered far more densely in one place
+// than another); the kernels then search by bisection.
 static constexpr uint64_t kGuideMax = 4096;
 
-static void build_guide(const std::vector<uint64_t> &keys, uint64_t key_hi, std::vector<int> &guide, int *shift)
+static void build_guide(const std::vector<uint64_t> &keys, uint64_t key_hi, std::vector<uint16_t> &guide, int *shift,
+                        int *run)
 {
     guide.clear();
     *shift = 0;
+    *run = kGuideRun;
     const int ncell = (int)keys.size();
+    if (ncell > 65536) return;               // the table holds 16-bit cells
     const uint64_t key0 = keys[0];
-    auto cell_of = [&](uint64_t key) {   // largest c with keys[c] <= key (key >= key0)
-        return (int)(std::upper_bound(keys.begin(), keys.end(), key) - keys.begin()) - 1;
-    };
-    std::vector<int> gd;
-    for (int s = 63; s >= 0; --s) {
-        const uint64_t nb = ((key_hi - key0) >> s) + 1;
-        if (nb > kGuideMax) return;
-        gd.assign(nb, 0);
-        bool ok = true;
-        for (uint64_t b = 0; b < nb && ok; ++b) {
-            const uint64_t first = key0 + (b << s);
-            gd[b] = cell_of(first);
-            const int last = b + 1 < nb ? cell_of(first + ((((uint64_t)1) << s) - 1)) : ncell - 1;
-            ok = last - gd[b] <= kGuideRun;
+    std::vector<uint16_t> gd;
+    for (int most : {1, kGuideRun})
+        for (int s = 63; s >= 0; --s) {
+            const uint64_t nb = ((key_hi - key0) >> s) + 1;
+            if (nb > kGuideMax) break;
+            gd.assign(nb, 0);
+            bool ok = true;
+            int c = 0;                       // largest cell whose key is <= the bucket's first
+            for (uint64_t b = 0; b < nb && ok; ++b) {
+                gd[b] = (uint16_t)c;
+                const int c0 = c;
+                int last = ncell - 1;        // the bucket's last cell
+                if (b + 1 < nb) {
+                    const uint64_t next = key0 + ((b + 1) << s);
+                    while (c + 1 < ncell && keys[c + 1] <= next) ++c;
+                    last = c > c0 && keys[c] == next ? c - 1 : c;
+                }
+                ok = last - c0 <= most;
+            }
+            if (ok) {
+                guide.swap(gd);
+                *shift = s;
+                *run = most;
+                return;
+            }
         }
-        if (ok) {
-            guide.swap(gd);
-            *shift = s;
-            return;
+}
+
+// Tables of fix_log: 1/c_j in 2^-31, c_j = 1 + (j + 1/2)/1024, and minus the
+// logarithm of that rounded reciprocal in 2^-60.
+struct FixLogTables {
+    std::vector<uint32_t> inv = std::vector<uint32_t>(kLogTab);
+    std::vector<int64_t> log = std::vector<int64_t>(kLogTab);
+    FixLogTables()
+    {
+        for (int j = 0; j < kLogTab; ++j) {
+            const long double c = 1.0L + (j + 0.5L) / kLogTab;
+            inv[j] = (uint32_t)llrintl(2147483648.0L / c);
+            log[j] = llrintl(-logl((long double)inv[j] / 2147483648.0L) * 1152921504606846976.0L);
         }
+    }
+};
+
+static const FixLogTables &fix_log_tables()   // made once per process
+{
+    static const FixLogTables t;
+    return t;
+}
+
+// Fixed-point cell between two knots (bits of positive normal doubles).  A
+// cell wider than half the logarithm's format or so narrow that the
+// logarithm's 2^-59 is more than 2^-45 of it keeps FP64 (K = 0).
+static FixCell fix_cell(double z0, double z1, const uint32_t *inv, const int64_t *tab)
+{
+    FixCell c{0, 0};
+    if (!(z0 >= 2.2250738585072014e-308) || !(log(z1 / z0) < 7.99)) return c;
+    c.U = fix_log(dbits(z0), inv, tab);
+    const uint64_t d = (uint64_t)fix_log(dbits(z1), inv, tab) - (uint64_t)c.U;
+    if (d < ((uint64_t)1 << 46) || (d >> 63)) return c;
+    int s = 0;
+    while (!((d << s) >> 62)) ++s;
+    const unsigned __int128 q = ((unsigned __int128)1 << 126) / (d << s);
+    c.K = (q >> 64) ? ~(uint64_t)0 : (uint64_t)q;
+    c.K = (c.K & ~(uint64_t)63) | (uint64_t)s;
+    return c;
+}
+
+// The rows of a cell matrix in powers of t - 1/2.
+static void centre_matrix(const double M[16], double Mc[16])
+{
+    for (int i = 0; i < 4; ++i) {
+        const long double c0 = M[i], c1 = M[4 + i], c2 = M[8 + i], c3 = M[12 + i];
+        Mc[i] = (double)(c0 + c1 / 2 + c2 / 4 + c3 / 8);
+        Mc[4 + i] = (double)(c1 + c2 + 0.75L * c3);
+        Mc[8 + i] = (double)(c2 + 1.5L * c3);
+        Mc[12 + i] = (double)c3;
     }
 }
 
@@ -257,8 +324,44 @@ static int largest_pow2_below(int n)
 // One thread per (member, Q cell, x cell, flavour): expand the bicubic patch
 // C[n][m] = sum_r Mq[n][r] sum_i Mx[m][i] v[row r][knot i] over the 4x4
 // stencil (rows outside the cell's subgrid and knots outside the x axis have
-// zero weight and are not read).
-__global__ void k_build_coef(GridDev g, const double *__restrict__ values, double *__restrict__ coef)
+// zero weight and are not read).  The same patch about the
+// cell's centre (in powers of t - 1/2, from the centred matrices) goes to the
+// fixed-point table; the interpolation of a constant being the constant, its
+// sums run over the differences to the cell's first corner, so that their
+// rounding is that of the differences.
+// MONO: the matrices are in powers of t, whose first row is (0, 1, 0, 0) and
+// whose second ends in 0 (those products are left out: 88 FMAs, not 128).
+template <bool MONO>
+__device__ __forceinline__ void stencil_to_patch(const double *__restrict__ Mx, const double *__restrict__ Mq,
+                                                 const double d[4][4], double C[16])
+{
+    double cx[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            double s = 0.0;
+            if (MONO && m == 0) s = d[r][1];
+            else
+#pragma unroll
+                for (int i = 0; i < (MONO && m == 1 ? 3 : 4); ++i) s = fma(Mx[m * 4 + i], d[r][i], s);
+            cx[r][m] = s;
+        }
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            double s = 0.0;
+            if (MONO && n == 0) s = cx[1][m];
+            else
+#pragma unroll
+                for (int r = 0; r < (MONO && n == 1 ? 3 : 4); ++r) s = fma(Mq[n * 4 + r], cx[r][m], s);
+            C[n * 4 + m] = s;
+        }
+}
+
+__global__ void k_build_coef(GridDev g, const double *__restrict__ values, double *__restrict__ coef,
+                             uint32_t *__restrict__ fcoef)
 {
     int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t total = (int64_t)g.nmem * g.nqc * g.nxc * g.nflav;
@@ -269,32 +372,37 @@ __global__ void k_build_coef(GridDev g, const double *__restrict__ values, doubl
     r /= g.nxc;
     int c = (int)(r % g.nqc);
     int mem = (int)(r / g.nqc);
-    const double *Mx = g.mx + (size_t)ix * 16;
-    const double *Mq = g.mq + (size_t)c * 16;
     int qmask = g.qmask[c];
     int row0 = g.qrow[c] - 1;
     const double *vm = values + (size_t)mem * g.nrows * g.nx * g.nflav;
-    double cx[4][4];
-    for (int rr = 0; rr < 4; ++rr) {
-        double gi[4];
+    double v[4][4], C[16];
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr)
+#pragma unroll
         for (int i = 0; i < 4; ++i) {
             int k = ix - 1 + i;
             bool ok = ((qmask >> rr) & 1) && k >= 0 && k < g.nx;
-            gi[i] = ok ? vm[((size_t)(row0 + rr) * g.nx + k) * g.nflav + a] : 0.0;
+            v[rr][i] = ok ? vm[((size_t)(row0 + rr) * g.nx + k) * g.nflav + a] : 0.0;
         }
-        for (int m = 0; m < 4; ++m) {
-            double s = 0.0;
-            for (int i = 0; i < 4; ++i) s = fma(Mx[m * 4 + i], gi[i], s);
-            cx[rr][m] = s;
-        }
-    }
+    stencil_to_patch<true>(g.mx + (size_t)ix * 16, g.mq + (size_t)c * 16, v, C);
     double *out = coef + (size_t)tid * 16;
-    for (int n = 0; n < 4; ++n)
-        for (int m = 0; m < 4; ++m) {
-            double s = 0.0;
-            for (int rr = 0; rr < 4; ++rr) s = fma(Mq[n * 4 + rr], cx[rr][m], s);
-            out[n * 4 + m] = s;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) out[k] = C[k];
+    if (!fcoef) return;
+    const double ref = v[1][1];
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int k = ix - 1 + i;
+            v[rr][i] = ((qmask >> rr) & 1) && k >= 0 && k < g.nx ? v[rr][i] - ref : 0.0;
         }
+    stencil_to_patch<false>(g.mxc + (size_t)ix * 16, g.mqc + (size_t)c * 16, v, C);
+    uint32_t w[32];
+    fix_pack(C, 4, ref, w);
+    uint4 *fo = reinterpret_cast<uint4 *>(fcoef + (size_t)tid * 32);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) fo[k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
 }
 
 namespace pdfgpu {
@@ -304,7 +412,8 @@ int build_coefficients(pdfgpu_grid *g, const double *dev_values, cudaStream_t s)
     int64_t total = (int64_t)g->d.nmem * g->d.nqc * g->d.nxc * g->d.nflav;
     int block = 128;
     int64_t blocks = (total + block - 1) / block;
-    k_build_coef<<<(unsigned)blocks, block, 0, s>>>(g->d, dev_values, const_cast<double *>(g->d.coef));
+    k_build_coef<<<(unsigned)blocks, block, 0, s>>>(g->d, dev_values, const_cast<double *>(g->d.coef),
+                                                    const_cast<uint32_t *>(g->d.fcoef));
     PDF_CUDA(cudaGetLastError());
     g->bound = true;
     return PDF_OK;
@@ -333,18 +442,30 @@ static void release_grid(pdfgpu_grid *g)
     delete g;
 }
 
-template <typename T>
-static int dev_upload(pdfgpu_grid *g, const T *host, size_t count, const T **dst)
-{
-    void *p = nullptr;
-    size_t bytes = std::max<size_t>(count * sizeof(T), 16);
-    int rc = dev_malloc(&p, bytes, "grid table");
-    if (rc) return rc;
-    g->blocks.push_back(p);
-    if (count) PDF_CUDA(cudaMemcpy(p, host, count * sizeof(T), cudaMemcpyHostToDevice));
-    *dst = (const T *)p;
-    return PDF_OK;
-}
+// The grid's tables, collected on the host and uploaded as one block.
+struct TableUpload {
+    std::vector<char> host;
+    std::vector<std::pair<const void **, size_t>> dst;
+
+    template <typename T>
+    void add(const T *src, size_t count, const T **to)
+    {
+        const size_t at = (host.size() + 255) & ~(size_t)255;
+        host.resize(at + std::max<size_t>(count * sizeof(T), 16));
+        if (count) memcpy(host.data() + at, src, count * sizeof(T));
+        dst.push_back({reinterpret_cast<const void **>(to), at});
+    }
+    int upload(pdfgpu_grid *g)
+    {
+        void *p = nullptr;
+        int rc = dev_malloc(&p, host.size(), "grid table");
+        if (rc) return rc;
+        g->blocks.push_back(p);
+        PDF_CUDA(cudaMemcpy(p, host.data(), host.size(), cudaMemcpyHostToDevice));
+        for (auto &d : dst) *d.first = (const char *)p + d.second;
+        return PDF_OK;
+    }
+};
 
 #define TRY(x)                          \
     do {                                \
@@ -415,9 +536,8 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
     g->n_q.assign(D.n_q, D.n_q + D.n_sub);
     for (int a = 0; a < D.n_flav; ++a) g->pids.push_back(D.pids[a] == 21 ? 0 : D.pids[a]);
 
-    std::vector<LogEntry> ltab;
-    std::vector<double2> etab;
-    make_log_tables(ltab, etab);
+    const std::vector<LogEntry> &ltab = log_tables().tab;
+    const std::vector<double2> &etab = log_tables().etab;
     const int nx = D.n_x, nxc = nx - 1;
     g->U.resize(nx);
     for (int k = 0; k < nx; ++k) g->U[k] = tlog(D.x_knots[k], ltab.data(), etab.data());
@@ -479,6 +599,9 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
         }
     }
     const int nqc = (int)qbits.size();
+    std::vector<double> mxc(mx.size()), mqc(mq.size());
+    for (int k = 0; k < nxc; ++k) centre_matrix(&mx[(size_t)k * 16], &mxc[(size_t)k * 16]);
+    for (int c = 0; c < nqc; ++c) centre_matrix(&mq[(size_t)c * 16], &mqc[(size_t)c * 16]);
     for (int c = 1; c < nqc; ++c)
         if (!(qbits[c] > qbits[c - 1])) {
             delete g;
@@ -502,9 +625,14 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
     d.nmem = D.n_members;
     d.xstep = largest_pow2_below(nxc);
     d.qstep = largest_pow2_below(nqc);
-    std::vector<int> xguide, qguide;
-    build_guide(xbits, dbits(D.x_knots[nx - 1]), xguide, &d.xgshift);
-    build_guide(qbits, dbits(Q2[rows - 1]), qguide, &d.qgshift);
+    std::vector<uint16_t> xguide, qguide;
+    build_guide(xbits, dbits(D.x_knots[nx - 1]), xguide, &d.xgshift, &d.xgrun);
+    build_guide(qbits, dbits(Q2[rows - 1]), qguide, &d.qgshift, &d.qgrun);
+    const std::vector<uint32_t> &finv = fix_log_tables().inv;
+    const std::vector<int64_t> &flog = fix_log_tables().log;
+    std::vector<FixCell> xfix(nxc), qfix(nqc);
+    for (int k = 0; k < nxc; ++k) xfix[k] = fix_cell(D.x_knots[k], D.x_knots[k + 1], finv.data(), flog.data());
+    for (int c = 0; c < nqc; ++c) qfix[c] = fix_cell(Q2[qrow[c]], Q2[qrow[c] + 1], finv.data(), flog.data());
     d.nxg = (int)xguide.size();
     d.nqg = (int)qguide.size();
     d.xlo = dbits(D.x_knots[0]);
@@ -517,31 +645,37 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
     d.whi = dkey(g->W[rows - 1]);
     d.extrap = D.extrap;
 
-    TRY(dev_upload(g, xbits.data(), xbits.size(), &d.xbits));
-    TRY(dev_upload(g, ukey.data(), ukey.size(), &d.ukey));
-    TRY(dev_upload(g, xcell.data(), xcell.size(), &d.xcell));
-    TRY(dev_upload(g, qbits.data(), qbits.size(), &d.qbits));
-    if (d.nxg) TRY(dev_upload(g, xguide.data(), xguide.size(), &d.xguide));
-    if (d.nqg) TRY(dev_upload(g, qguide.data(), qguide.size(), &d.qguide));
-    TRY(dev_upload(g, wkey.data(), wkey.size(), &d.wkey));
-    TRY(dev_upload(g, qcell.data(), qcell.size(), &d.qcell));
-    TRY(dev_upload(g, ltab.data(), ltab.size(), &d.logtab));
-    TRY(dev_upload(g, etab.data(), etab.size(), &d.etab));
-    TRY(dev_upload(g, mx.data(), mx.size(), &d.mx));
-    TRY(dev_upload(g, mq.data(), mq.size(), &d.mq));
-    TRY(dev_upload(g, mxs.data(), mxs.size(), &d.mxs));
-    TRY(dev_upload(g, mqs.data(), mqs.size(), &d.mqs));
-    TRY(dev_upload(g, qrow.data(), qrow.size(), &d.qrow));
-    TRY(dev_upload(g, qmask.data(), qmask.size(), &d.qmask));
-    TRY(dev_upload(g, pidmap.data(), pidmap.size(), &d.pidmap));
+    TableUpload up;
+    up.add(xbits.data(), xbits.size(), &d.xbits);
+    up.add(ukey.data(), ukey.size(), &d.ukey);
+    up.add(xcell.data(), xcell.size(), &d.xcell);
+    up.add(qbits.data(), qbits.size(), &d.qbits);
+    if (d.nxg) up.add(xguide.data(), xguide.size(), &d.xguide);
+    if (d.nqg) up.add(qguide.data(), qguide.size(), &d.qguide);
+    up.add(xfix.data(), xfix.size(), &d.xfix);
+    up.add(qfix.data(), qfix.size(), &d.qfix);
+    up.add(finv.data(), finv.size(), &d.finv);
+    up.add(flog.data(), flog.size(), &d.flog);
+    up.add(wkey.data(), wkey.size(), &d.wkey);
+    up.add(qcell.data(), qcell.size(), &d.qcell);
+    up.add(ltab.data(), ltab.size(), &d.logtab);
+    up.add(etab.data(), etab.size(), &d.etab);
+    up.add(mx.data(), mx.size(), &d.mx);
+    up.add(mq.data(), mq.size(), &d.mq);
+    up.add(mxs.data(), mxs.size(), &d.mxs);
+    up.add(mqs.data(), mqs.size(), &d.mqs);
+    up.add(mxc.data(), mxc.size(), &d.mxc);
+    up.add(mqc.data(), mqc.size(), &d.mqc);
+    up.add(qrow.data(), qrow.size(), &d.qrow);
+    up.add(qmask.data(), qmask.size(), &d.qmask);
+    up.add(pidmap.data(), pidmap.size(), &d.pidmap);
     {
         const uint32_t zero = 0;
-        const uint32_t *st;
-        TRY(dev_upload(g, &zero, 1, &st));
-        d.status = const_cast<uint32_t *>(st);
+        up.add(&zero, 1, const_cast<const uint32_t **>(&d.status));
     }
     if (D.alphas) {
         std::vector<double> ac((size_t)nqc * 4);
+        std::vector<uint32_t> fac((size_t)nqc * 8);
         for (int c = 0; c < nqc; ++c) {
             const double *M = &mq[(size_t)c * 16];
             for (int nn = 0; nn < 4; ++nn) {
@@ -552,10 +686,20 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
                 }
                 ac[(size_t)c * 4 + nn] = s;
             }
+            // the same cubic about the cell's centre, from the differences to its first knot
+            const double ref = D.alphas[qrow[c]];
+            double cc[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int nn = 0; nn < 4; ++nn)
+                for (int rr = 0; rr < 4; ++rr)
+                    if ((qmask[c] >> rr) & 1)
+                        cc[nn] = fma(mqc[(size_t)c * 16 + nn * 4 + rr], D.alphas[qrow[c] - 1 + rr] - ref, cc[nn]);
+            fix_pack(cc, 1, ref, &fac[(size_t)c * 8]);
         }
-        TRY(dev_upload(g, ac.data(), ac.size(), &d.acoef));
+        up.add(fac.data(), fac.size(), &d.facoef);
+        up.add(ac.data(), ac.size(), &d.acoef);
         g->has_alphas = true;
     }
+    TRY(up.upload(g));
     // coefficient storage
     size_t ncoef = (size_t)D.n_members * nqc * nxc * D.n_flav * 16;
     {
@@ -566,6 +710,16 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
         }
         g->blocks.push_back(p);
         d.coef = (const double *)p;
+        // the fixed-point patches, as large again; without the memory for
+        // them, or with members beyond 32-bit byte offsets, every point
+        // takes the FP64 path
+        if (ncoef / D.n_members * sizeof(double) < ((size_t)1 << 32) &&
+            dev_malloc(&p, ncoef * sizeof(double), "fixed-point coefficient table") == PDF_OK) {
+            g->blocks.push_back(p);
+            d.fcoef = (const uint32_t *)p;
+        } else {
+            clear_error();
+        }
     }
     if (D.values) {
         size_t nval = (size_t)D.n_members * rows * nx * D.n_flav;

@@ -97,6 +97,12 @@ PDF_HD double tlog(double x, const LogEntry *tab, const double2 *etab)
     return hi + lo;
 }
 
+}  // namespace pdfgpu
+
+#include "fix.cuh"
+
+namespace pdfgpu {
+
 // Device view of one loaded grid (passed by value to kernels).
 struct GridDev {
     int nx, nxc;          // x knots, x cells (nx - 1)
@@ -105,6 +111,7 @@ struct GridDev {
     int xstep, qstep;     // search start steps (largest power of two < cells)
     int nxg, nqg;         // guide-table buckets per axis (0: no guide, binary search)
     int xgshift, qgshift; // log2 of the guide buckets' width in key units
+    int xgrun, qgrun;     // lower keys a bucket may hold beyond its first cell's
     uint64_t xlo, xhi;    // bit patterns of the first / last x knot
     uint64_t qlo, qhi;    // bit patterns of the first / last Q^2 knot
     int64_t ulo, uhi;     // order keys of ln(first / last x knot)
@@ -113,8 +120,14 @@ struct GridDev {
     const int64_t *ukey;     // [nxc] order keys of each x cell's lower ln x
     const double2 *xcell;    // [nxc] (U_k, 1/dU_k)
     const uint64_t *qbits;   // [nqc] bits of each Q cell's lower Q^2 knot
-    const int *xguide;       // [nxg] first cell of each x guide bucket
-    const int *qguide;       // [nqg] the same for Q^2
+    const uint16_t *xguide;  // [nxg] first cell of each x guide bucket
+    const uint16_t *qguide;  // [nqg] the same for Q^2
+    const FixCell *xfix;     // [nxc] the cells of the fixed-point coordinates
+    const FixCell *qfix;     // [nqc]
+    const uint32_t *finv;    // [kLogTab] tables of fix_log
+    const int64_t *flog;     // [kLogTab]
+    const uint32_t *fcoef;   // [nmem][nqc][nxc][nflav][4][8] fixed-point patches, or null
+    const uint32_t *facoef;  // [nqc][8] fixed-point alpha_s cubics, or null
     const int64_t *wkey;     // [nqc] order keys of each Q cell's lower ln Q^2
     const double2 *qcell;    // [nqc] (W_c, 1/dW_c)
     const LogEntry *logtab;  // [kLogTab]
@@ -125,6 +138,8 @@ struct GridDev {
     const double *mq;        // [nqc][16]
     const double *mxs;       // [nxc][16] the same in powers of s = 1 - t
     const double *mqs;       // [nqc][16]
+    const double *mxc;       // [nxc][16] the same in powers of t - 1/2
+    const double *mqc;       // [nqc][16]
     const int *qrow;         // [nqc] grid row of each Q cell's lower knot
     const int *qmask;        // [nqc] bit i (0..3): stencil row i-1 exists
     const signed char *pidmap;  // [129] column of pid in [-64, 64], -1 absent
@@ -148,24 +163,26 @@ __device__ __forceinline__ int find_cell(const K *keys, int ncell, int step, K k
 // The same search through a guide table: bucket b covers the keys
 // key0 + [b 2^shift, (b + 1) 2^shift) (the last bucket also everything
 // above) and holds the largest cell whose lower key is <= the bucket's first
-// key; the host builds the table so that no bucket holds more than
-// kGuideRun further lower keys.  The cell of a key is then the bucket's cell
-// plus the number of the next kGuideRun lower keys that are <= it (the keys
-// ascend): one table load and kGuideRun independent key loads, instead of a
-// chain of log2(cells) dependent ones.  Without a table (nguide == 0) the
-// binary search.
+// key; the host builds the table so that no bucket holds more than `run`
+// (1 to kGuideRun) further lower keys.  The cell of a key is then the
+// bucket's cell plus the number of the next `run` lower keys that are <= it
+// (the keys ascend): one table load and `run` independent key loads, instead
+// of a chain of log2(cells) dependent ones.  Without a table (nguide == 0)
+// the binary search.
 constexpr int kGuideRun = 3;
 
-__device__ __forceinline__ int find_cell_guided(const uint64_t *keys, int ncell, int step, const int *guide,
-                                                int nguide, int shift, uint64_t key0, uint64_t key)
+__device__ __forceinline__ int find_cell_guided(const uint64_t *keys, int ncell, int step, const uint16_t *guide,
+                                                int nguide, int shift, int run, uint64_t key0, uint64_t key)
 {
     if (nguide == 0) return find_cell<uint64_t>(keys, ncell, step, key);
     if (key < key0) return 0;
     const uint64_t off = (key - key0) >> shift;
-    const int c = __ldg(guide + (off < (uint64_t)nguide ? (int)off : nguide - 1));
-    int add = 0;
+    const int c = guide[off < (uint64_t)nguide ? (int)off : nguide - 1];
+    int add = (c + 1 < ncell && keys[c + 1] <= key) ? 1 : 0;
+    if (run > 1) {
 #pragma unroll
-    for (int r = 1; r <= kGuideRun; ++r) add += (c + r < ncell && keys[c + r] <= key) ? 1 : 0;
+        for (int r = 2; r <= kGuideRun; ++r) add += (c + r < ncell && keys[c + r] <= key) ? 1 : 0;
+    }
     return c + add;
 }
 
@@ -231,19 +248,89 @@ __device__ __forceinline__ double dlog(const GridDev &g, double v)
     return tlog(v, g.logtab, g.etab);
 }
 
-// x axis from x (bit search on x), returns u = ln x in *u.
-__device__ __forceinline__ Axis axis_x(const GridDev &g, double x, double *u)
+// The tables of the coordinate searches and logarithms: the grid's own, or a
+// block's copies in shared memory.
+struct CoordTabs {
+    const uint32_t *inv;
+    const int64_t *log;
+    const uint64_t *xbits, *qbits;
+    const uint16_t *xguide, *qguide;
+    const FixCell *xfix, *qfix;
+};
+
+__device__ __forceinline__ CoordTabs grid_tabs(const GridDev &g)
 {
-    uint64_t b = dbits(x);
+    return {g.finv, g.flog, g.xbits, g.qbits, g.xguide, g.qguide, g.xfix, g.qfix};
+}
+
+// Cell and fixed-point local coordinate (value 2^62) of one axis; ok: inside
+// the knot range and in a cell that the format serves.
+struct FixAxis {
+    int cell;
+    int64_t t;
+    bool ok;
+};
+
+__device__ __forceinline__ FixAxis fix_axis_x(const GridDev &g, const CoordTabs &T, uint64_t b)
+{
+    FixAxis A;
+    A.cell = checked_index(g.status, find_cell_guided(T.xbits, g.nxc, g.xstep, T.xguide, g.nxg, g.xgshift, g.xgrun,
+                                                      g.xlo, b), g.nxc);
+    const FixCell c = T.xfix[A.cell];
+    A.ok = (b >= g.xlo) & (b <= g.xhi) & (c.K != 0);
+    A.t = fix_coord(fix_log(b, T.inv, T.log), c);
+    return A;
+}
+
+__device__ __forceinline__ FixAxis fix_axis_q2(const GridDev &g, const CoordTabs &T, uint64_t b)
+{
+    FixAxis A;
+    A.cell = checked_index(g.status, find_cell_guided(T.qbits, g.nqc, g.qstep, T.qguide, g.nqg, g.qgshift, g.qgrun,
+                                                      g.qlo, b), g.nqc);
+    const FixCell c = T.qfix[A.cell];
+    A.ok = (b >= g.qlo) & (b <= g.qhi) & (c.K != 0);
+    A.t = fix_coord(fix_log(b, T.inv, T.log), c);
+    return A;
+}
+
+// The axes in FP64 (adjoints, points outside the knots): inside the knot
+// range t is the fixed-point coordinate, so that every kernel places a point
+// at the same t; elsewhere it comes from the FP64 logarithm.
+__device__ __forceinline__ Axis axis_x(const GridDev &g, double x)
+{
+    const uint64_t b = dbits(x);
+    const FixAxis f = fix_axis_x(g, grid_tabs(g), b);
     Axis A;
-    A.cell = checked_index(g.status, find_cell_guided(g.xbits, g.nxc, g.xstep, g.xguide, g.nxg, g.xgshift, g.xlo, b),
-                           g.nxc);
+    A.cell = f.cell;
     A.in = (b >= g.xlo) & (b <= g.xhi);
     A.below = b < g.xlo;
-    double uu = dlog(g, x);
-    double2 c = g.xcell[A.cell];
-    make_basis(A, (uu - c.x) * c.y, g.extrap);
-    *u = uu;
+    double t;
+    if (f.ok) {
+        t = fix_t(f.t);
+    } else {
+        const double2 c = g.xcell[A.cell];
+        t = (dlog(g, x) - c.x) * c.y;
+    }
+    make_basis(A, t, g.extrap);
+    return A;
+}
+
+__device__ __forceinline__ Axis axis_q2(const GridDev &g, double q2)
+{
+    const uint64_t b = dbits(q2);
+    const FixAxis f = fix_axis_q2(g, grid_tabs(g), b);
+    Axis A;
+    A.cell = f.cell;
+    A.in = (b >= g.qlo) & (b <= g.qhi);
+    A.below = b < g.qlo;
+    double t;
+    if (f.ok) {
+        t = fix_t(f.t);
+    } else {
+        const double2 c = g.qcell[A.cell];
+        t = (dlog(g, q2) - c.x) * c.y;
+    }
+    make_basis(A, t, g.extrap);
     return A;
 }
 
@@ -257,21 +344,6 @@ __device__ __forceinline__ Axis axis_u(const GridDev &g, double u)
     A.below = k < g.ulo;
     double2 c = g.xcell[A.cell];
     make_basis(A, (u - c.x) * c.y, g.extrap);
-    return A;
-}
-
-__device__ __forceinline__ Axis axis_q2(const GridDev &g, double q2, double *w)
-{
-    uint64_t b = dbits(q2);
-    Axis A;
-    A.cell = checked_index(g.status, find_cell_guided(g.qbits, g.nqc, g.qstep, g.qguide, g.nqg, g.qgshift, g.qlo, b),
-                           g.nqc);
-    A.in = (b >= g.qlo) & (b <= g.qhi);
-    A.below = b < g.qlo;
-    double ww = dlog(g, q2);
-    double2 c = g.qcell[A.cell];
-    make_basis(A, (ww - c.x) * c.y, g.extrap);
-    *w = ww;
     return A;
 }
 
