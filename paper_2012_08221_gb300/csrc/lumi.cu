@@ -8,6 +8,7 @@
 #include <algorithm>
 
 #include "pdf_internal.h"
+#include "lumi_eval.cuh"
 #include "sort_acc.cuh"
 
 using namespace pdfgpu;
@@ -49,10 +50,49 @@ __device__ __forceinline__ Event event(int64_t e, const double *ln_tau, const do
     return E;
 }
 
-// At most 64 registers (4 CTAs per SM): with the 32-byte coefficient loads
-// the unbounded build takes 80 and runs 1 % slower at 3 CTAs per SM.
-template <bool SAVE, bool CONT>
-__global__ void __launch_bounds__(kBlock, 4) k_lumi(GridDev g, Cols anti, int member,
+// One event in FP64 (a parton or the scale outside the knots, a patch that the
+// fixed-point format does not hold): its sum, NaN for a bad event.
+__device__ __forceinline__ double slow_event(const GridDev &g, const signed char *anti, const double *cm, Event E,
+                                             int64_t e, double *as, double *save_p, bool report)
+{
+    const Axis Q = axis_w(g, E.w), X1 = axis_u(g, E.u1), X2 = axis_u(g, E.u2);
+    const bool oor = !E.bad && (out_of_range(g, X1, Q) || out_of_range(g, X2, Q));
+    flag_status(g, report && E.bad);
+    flag_status(g, report && oor, PDF_S_RANGE);
+    E.bad |= oor;
+    const size_t cell_stride = (size_t)g.nflav * 16;
+    const double *c1 = cm + ((size_t)Q.cell * g.nxc + X1.cell) * cell_stride;
+    const double *c2 = cm + ((size_t)Q.cell * g.nxc + X2.cell) * cell_stride;
+    double s = 0.0;
+    for (int a = 0; a < g.nflav; ++a) {
+        const int b = anti[a];
+        if (b < 0) continue;
+        const double p1 = patch_any<true>(g, c1 + a * 16, X1, Q);
+        const double p2 = patch_any<true>(g, c2 + b * 16, X2, Q);
+        s = fma(p1, p2, s);
+        if (save_p) {
+            double *pe = save_p + (size_t)e * 2 * g.nflav;
+            pe[a] = p1;
+            pe[g.nflav + b] = p2;
+        }
+    }
+    if (as) {
+        const double v = alphas_any(g, ld4(g.acoef + (size_t)Q.cell * 4), Q);
+        as[e] = E.bad ? qnan() : v;
+    }
+    return E.bad ? qnan() : s;
+}
+
+// Per event the luminosity (lumi_quads), alpha_s at its scale, and with SAVE
+// both partons' values, the partner factors the adjoint needs, in save_p
+// [event][parton][flavour] (the rows of 32 events leave as one run).  Without
+// `partials` (the adjoint's recomputation) no status bit is set either.  2e7
+// events x 26 patches, 5 % of the events outside the knots: 13.9 ms in FP64
+// (pipe 96 % busy), 6.1 ms here (integer issue, and the tail in FP64).  Three
+// blocks per SM at 80 registers; with the wider rows of SAVE two are faster.
+template <bool SAVE>
+__global__ void __launch_bounds__(kBlock, SAVE ? 2 : 3) k_lumi(const __grid_constant__ GridDev g,
+                                                    const __grid_constant__ Cols anti, int member,
                                                     const double *__restrict__ ln_tau,
                                                     const double *__restrict__ y,
                                                     const uint8_t *__restrict__ flags,
@@ -60,57 +100,64 @@ __global__ void __launch_bounds__(kBlock, 4) k_lumi(GridDev g, Cols anti, int me
                                                     const double *__restrict__ ln_x1, double ln_s,
                                                     int64_t n, double *__restrict__ lum,
                                                     double *__restrict__ as, double *__restrict__ partials,
-                                                    double *__restrict__ save_p)
+                                                    double *__restrict__ save_p, int tab_bytes)
 {
-    __shared__ signed char santi[PDF_MAX_PIDS];
+    extern __shared__ __align__(128) unsigned char smem[];
     __shared__ double red[kBlock / 32];
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < PDF_MAX_PIDS; ++k) santi[k] = anti.c[k];
-    }
+    const LogTabs T = tab_bytes ? stage_log_tabs(g, smem) : grid_log_tabs(g);
     __syncthreads();
-    const size_t cell_stride = (size_t)g.nflav * 16;
-    const double *cm = g.coef + (size_t)member * g.nqc * g.nxc * cell_stride;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int row = SAVE ? 2 * g.nflav : g.nflav;
+    unsigned char *mine = smem + tab_bytes + (size_t)wid * lumi_warp_bytes(row);
+    double *rows = reinterpret_cast<double *>(mine + kWarpBuf);
+    WarpBufs B{reinterpret_cast<uint4 *>(mine), reinterpret_cast<int64_t *>(rows + 32 * row), 0};
+    const size_t patches = (size_t)member * g.nqc * g.nxc * g.nflav;
+    const double *cm = g.coef + patches * 16;
+    const unsigned char *fm = g.fcoef ? reinterpret_cast<const unsigned char *>(g.fcoef) + patches * 128 : nullptr;
     double acc = 0.0;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        Event E = event(e, ln_tau, y, flags, ln_mu2, ln_x1, ln_s);
-        flag_status(g, E.bad);
-        Axis Q = axis_w(g, E.w);
-        Axis X1 = axis_u(g, E.u1);
-        Axis X2 = axis_u(g, E.u2);
-        const bool oor = !E.bad && (out_of_range(g, X1, Q) || out_of_range(g, X2, Q));
-        flag_status(g, oor, PDF_S_RANGE);
-        E.bad |= oor;
-        const double *c1 = cm + ((size_t)Q.cell * g.nxc + X1.cell) * cell_stride;
-        const double *c2 = cm + ((size_t)Q.cell * g.nxc + X2.cell) * cell_stride;
-        double s = 0.0;
-        for (int a = 0; a < g.nflav; ++a) {
-            int b = santi[a];
-            if (b < 0) continue;
-            double p1 = patch_any<CONT>(g, c1 + a * 16, X1, Q);
-            double p2 = patch_any<CONT>(g, c2 + b * 16, X2, Q);
-            s = fma(p1, p2, s);
+    auto drain = [&]() {
+        if (SAVE && lane == 0) bulk_wait_all();       // the rows staged for these events have been written
+        const int64_t e = next_queued(B, lane);
+        if (e >= 0) {
+            const Event E = event(e, ln_tau, y, flags, ln_mu2, ln_x1, ln_s);
+            const double s = slow_event(g, anti.c, cm, E, e, as, SAVE ? save_p : nullptr, partials != nullptr);
+            if (lum) lum[e] = s;
+            acc += s;
+        }
+        __syncwarp();
+    };
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + wid) * 32; base < n; base += stride) {
+        const int64_t e = base + lane;
+        const bool live = e < n;
+        const Event E = event(live ? e : n - 1, ln_tau, y, flags, ln_mu2, ln_x1, ln_s);
+        const FixAxis Q = fix_axis_log(g, T.wkey, T.qcell, g.nqc, g.qstep, g.wlo, g.whi, E.w);
+        const FixAxis X1 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, g.ulo, g.uhi, E.u1);
+        const FixAxis X2 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, g.ulo, g.uhi, E.u2);
+        bool fast = live && fm && !E.bad && Q.ok && X1.ok && X2.ok;
+        if (__any_sync(kAll, fast)) {
+            if (SAVE) warp_run_reuse(lane);           // the previous run has left the rows
+            const double s = lumi_quads<SAVE>(g, anti.c, fm, B.buf, rows, row, lane, X1, X2, Q, fast);
+            if (fast) {
+                if (lum) lum[e] = s;
+                if (as) as[e] = fix_alphas(g, Q);
+                acc += s;
+            }
             if (SAVE) {
-                // the partner factors the adjoint needs: [event][parton][flavour]
-                double *pe = save_p + (size_t)e * 2 * g.nflav;
-                pe[a] = p1;
-                pe[g.nflav + b] = p2;
+                const int m = (int)min((int64_t)32, n - base);
+                warp_run_store(save_p + base * row, rows, m * row, lane);
             }
         }
-        if (E.bad) s = qnan();
-        if (lum) lum[e] = s;
-        acc += s;
-        if (as) {
-            double v = alphas_any(g, ld4(g.acoef + (size_t)Q.cell * 4), Q);
-            as[e] = E.bad ? qnan() : v;
-        }
+        push_queue(B, live && !fast, e, lane);
+        if (B.qn >= 32) drain();
     }
+    if (B.qn) drain();
+    if (SAVE && lane == 0) bulk_wait_all();
     // fixed-order block reduction of the per-thread sums
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && partials) {
         double t = 0.0;
         for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[k];
         partials[blockIdx.x] = t;
@@ -138,8 +185,9 @@ __global__ void k_lumi_final(const double *__restrict__ partials, int nb, double
 //                         Wq_j(p) Wx_i(p) f_{-b}(other parton)
 // over each parton's 4x4 stencil.  Instead of 16 x F global atomics per
 // parton, partons are grouped by grid cell and accumulated in registers:
-//   1. k_lumi_rec: per event the two partons' F values (the partner factors)
-//      and, per parton, its bin key, local coordinates and range flags;
+//   1. k_lumi (with save_p) where the caller has not kept them: per event the
+//      two partons' F values (the partner factors); k_lumi_rec: per parton its
+//      bin key, local coordinates and range flags;
 //   2. key_histogram: a histogram of the keys; exclusive_scan: bin offsets;
 //      k_scatter_tiled: parton ids in bin order;
 //   3. k_lumi_accum: each half-warp walks half of a warp's run of sorted
@@ -169,8 +217,7 @@ __device__ __forceinline__ int parton_kind(const Axis &X, const Axis &Q)
     return (upper_half(X.t) ? 1 : 0) | (upper_half(Q.t) ? 2 : 0);
 }
 
-template <bool PATCHES>
-__global__ void __launch_bounds__(kBlock) k_lumi_rec(GridDev g, int member,
+__global__ void __launch_bounds__(kBlock) k_lumi_rec(GridDev g,
                                                      const double *__restrict__ ln_tau,
                                                      const double *__restrict__ y,
                                                      const uint8_t *__restrict__ flags,
@@ -178,11 +225,8 @@ __global__ void __launch_bounds__(kBlock) k_lumi_rec(GridDev g, int member,
                                                      const double *__restrict__ ln_x1, double ln_s,
                                                      int64_t e0, int m, int *__restrict__ key,
                                                      double *__restrict__ tx, double *__restrict__ tq,
-                                                     uint8_t *__restrict__ fin, double *__restrict__ P)
+                                                     uint8_t *__restrict__ fin)
 {
-    const int F = g.nflav;
-    const size_t cell_stride = (size_t)F * 16;
-    const double *cm = g.coef + (size_t)member * g.nqc * g.nxc * cell_stride;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
         Event E = event(e0 + i, ln_tau, y, flags, ln_mu2, ln_x1, ln_s);
         if (E.bad) {
@@ -197,16 +241,6 @@ __global__ void __launch_bounds__(kBlock) k_lumi_rec(GridDev g, int member,
             key[2 * i] = -1;
             key[2 * i + 1] = -1;
             continue;
-        }
-        const double *c1 = cm + ((size_t)Q.cell * g.nxc + X1.cell) * cell_stride;
-        const double *c2 = cm + ((size_t)Q.cell * g.nxc + X2.cell) * cell_stride;
-        if (PATCHES) {
-            double *p1 = P + (size_t)i * 2 * F;
-            double *p2 = p1 + F;
-            for (int a = 0; a < F; ++a) {
-                p1[a] = patch(c1 + a * 16, X1, Q);
-                p2[a] = patch(c2 + a * 16, X2, Q);
-            }
         }
         const int cq = Q.cell * g.nxc;
         key[2 * i] = (cq + X1.cell) * kKinds + parton_kind(X1, Q);
@@ -420,6 +454,36 @@ int lumi_common(pdfgpu_grid *g, int32_t member, const double *ln_tau, const doub
     return PDF_OK;
 }
 
+// The forward kernel; with `sum` the block sums go to g->partials (grown on
+// demand) and their number to *blocks.
+constexpr size_t kLogStageMax = 16 * 1024;   // coordinate tables of larger grids stay global
+
+int launch_lumi(pdfgpu_grid *g, const Cols &anti, int member, const double *ln_tau, const double *y,
+                const uint8_t *flags, const double *ln_mu2, const double *ln_x1, double ln_s, int64_t n, double *lum,
+                double *alphas, bool sum, double *save_p, cudaStream_t s, int *blocks)
+{
+    auto k = save_p ? k_lumi<true> : k_lumi<false>;
+    int tab = log_tab_bytes(g->d);
+    if ((size_t)tab > kLogStageMax) tab = 0;
+    const size_t smem = (size_t)tab + (kBlock / 32) * lumi_warp_bytes((save_p ? 2 : 1) * g->d.nflav);
+    int rc = allow_dynamic_smem((const void *)k, smem);
+    if (rc) return rc;
+    const int grid = wave_grid(g, (const void *)k, kBlock, smem, n);
+    if (sum && g->partials_cap < grid) {
+        if (g->partials) cudaFree(g->partials);
+        g->partials = nullptr;
+        g->partials_cap = 0;
+        rc = dev_malloc((void **)&g->partials, (size_t)grid * sizeof(double), "luminosity partial sums");
+        if (rc) return rc;
+        g->partials_cap = grid;
+    }
+    k<<<grid, kBlock, smem, s>>>(g->d, anti, member, ln_tau, y, flags, ln_mu2, ln_x1, ln_s, n, lum, alphas,
+                                 sum ? g->partials : nullptr, save_p, tab);
+    PDF_CUDA(cudaGetLastError());
+    if (blocks) *blocks = grid;
+    return PDF_OK;
+}
+
 }  // namespace
 
 extern "C" int pdf_lumi(pdfgpu_grid_t g, int32_t member, const double *ln_tau, const double *y,
@@ -439,23 +503,9 @@ extern "C" int pdf_lumi(pdfgpu_grid_t g, int32_t member, const double *ln_tau, c
         return PDF_OK;
     }
     if (alphas && !g->has_alphas) alphas = nullptr;
-    using Kern = void (*)(GridDev, Cols, int, const double *, const double *, const uint8_t *, const double *,
-                          const double *, double, int64_t, double *, double *, double *, double *);
-    const bool cont = g->d.extrap == PDF_EXTRAP_CONTINUATION;
-    Kern k = save_p ? (cont ? k_lumi<true, true> : k_lumi<true, false>)
-                    : (cont ? k_lumi<false, true> : k_lumi<false, false>);
-    int grid = wave_grid(g, (const void *)k, kBlock, 0, n);
-    if (g->partials_cap < grid) {
-        if (g->partials) cudaFree(g->partials);
-        g->partials = nullptr;
-        g->partials_cap = 0;
-        rc = dev_malloc((void **)&g->partials, (size_t)grid * sizeof(double), "luminosity partial sums");
-        if (rc) return rc;
-        g->partials_cap = grid;
-    }
-    k<<<grid, kBlock, 0, s>>>(g->d, anti, member, ln_tau, y, flags, ln_mu2, ln_x1, ln_s, n, lum, alphas,
-                              g->partials, save_p);
-    PDF_CUDA(cudaGetLastError());
+    int grid = 0;
+    rc = launch_lumi(g, anti, member, ln_tau, y, flags, ln_mu2, ln_x1, ln_s, n, lum, alphas, true, save_p, s, &grid);
+    if (rc) return rc;
     k_lumi_final<<<1, 256, 0, s>>>(g->partials, grid, 1.0 / (double)n, L);
     PDF_CUDA(cudaGetLastError());
     return PDF_OK;
@@ -511,20 +561,20 @@ extern "C" int pdf_lumi_backward(pdfgpu_grid_t g, int32_t member, const double *
     int *cursor = (int *)(base += bbins);
     const double scale = dL / (double)n;
     const size_t hsmem = nbins <= kScatterSmemBins ? (size_t)nbins * sizeof(int) : 0;
-    const void *krec = saved_p ? (const void *)k_lumi_rec<false> : (const void *)k_lumi_rec<true>;
     rc = allow_dynamic_smem((const void *)k_scatter_tiled, hsmem);
     if (rc) return rc;
     for (int64_t e0 = 0; e0 < n; e0 += chunk) {
         const int m = (int)std::min(chunk, n - e0);
         PDF_CUDA(cudaMemsetAsync(hist, 0, (size_t)(nbins + 1) * sizeof(int), st));
-        int grid = wave_grid(g, krec, kBlock, 0, m);
         const double *Pc = saved_p ? saved_p + (size_t)e0 * 2 * F : P;
-        if (saved_p)
-            k_lumi_rec<false><<<grid, kBlock, 0, st>>>(g->d, member, ln_tau, y, flags, ln_mu2, ln_x1, ln_s,
-                                                       e0, m, key, tx, tq, fin, nullptr);
-        else
-            k_lumi_rec<true><<<grid, kBlock, 0, st>>>(g->d, member, ln_tau, y, flags, ln_mu2, ln_x1, ln_s,
-                                                      e0, m, key, tx, tq, fin, P);
+        if (!saved_p) {
+            auto at = [&](auto *p) { return p ? p + e0 : p; };
+            rc = launch_lumi(g, anti, member, ln_tau + e0, y + e0, at(flags), at(ln_mu2), at(ln_x1), ln_s, m, nullptr,
+                             nullptr, false, P, st, nullptr);
+            if (rc) return rc;
+        }
+        k_lumi_rec<<<wave_grid(g, (const void *)k_lumi_rec, kBlock, 0, m), kBlock, 0, st>>>(
+            g->d, ln_tau, y, flags, ln_mu2, ln_x1, ln_s, e0, m, key, tx, tq, fin);
         PDF_CUDA(cudaGetLastError());
         rc = key_histogram(key, 2 * (int64_t)m, hist, nbins, g->d.status, g->sm_count, st);
         if (rc) return rc;

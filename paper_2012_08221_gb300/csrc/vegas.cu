@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "lumi_eval.cuh"
 #include "pdf_internal.h"
 
 using namespace pdfgpu;
@@ -29,61 +30,116 @@ namespace {
 constexpr int kBlock = 256;
 constexpr int kMaxBins = 1024;
 
-template <bool CONT>
-__global__ void __launch_bounds__(kBlock) k_vegas(GridDev g, Cols anti, int member, double ln_tau_min,
-                                                  double ln_s, int n_bins, const double *__restrict__ edges,
-                                                  const double *__restrict__ v, int64_t n, double shift,
-                                                  double *__restrict__ partials, double *__restrict__ bins)
+// One point's logarithms through the map: ln Q^2, ln x1, ln x2, the weight
+// without the luminosity, and the two bins.
+struct VegasPoint {
+    double w, u1, u2, factor;
+    int bin[2];
+};
+
+__device__ __forceinline__ VegasPoint vegas_point(double2 vv, const double *edges, int n_bins, double ln_tau_min,
+                                                  double ln_s)
 {
-    extern __shared__ double sbin[];          // [2][n_bins] sums of w^2
-    __shared__ signed char santi[PDF_MAX_PIDS];
-    __shared__ double red[2][kBlock / 32];
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < PDF_MAX_PIDS; ++k) santi[k] = anti.c[k];
-    }
-    for (int k = threadIdx.x; k < 2 * n_bins; k += blockDim.x) sbin[k] = 0.0;
-    __syncthreads();
-    const size_t cell_stride = (size_t)g.nflav * 16;
-    const double *cm = g.coef + (size_t)member * g.nqc * g.nxc * cell_stride;
     const double nb = (double)n_bins;
-    double s1 = 0.0, s2 = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const double2 vv = reinterpret_cast<const double2 *>(v)[i];
-        double r[2], jac = 1.0;
-        int bin[2];
+    VegasPoint P;
+    double r[2], jac = 1.0;
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {
-            const double *e = edges + (size_t)d * (n_bins + 1);
-            double vn = (d ? vv.y : vv.x) * nb;
-            int b = min(max((int)vn, 0), n_bins - 1);    // uniforms outside [0, 1) stay in range
-            double lo = __ldg(e + b), width = __ldg(e + b + 1) - lo;
-            r[d] = fma(vn - (double)b, width, lo);
-            jac *= nb * width;
-            bin[d] = b;
-        }
-        const double ln_tau = (1.0 - r[0]) * ln_tau_min;
-        const double h = 0.5 * ln_tau;
-        const double y = (2.0 * r[1] - 1.0) * (-h);
-        Axis Q = axis_w(g, ln_tau + ln_s);
-        Axis X1 = axis_u(g, h + y);
-        Axis X2 = axis_u(g, h - y);
-        const double *c1 = cm + ((size_t)Q.cell * g.nxc + X1.cell) * cell_stride;
-        const double *c2 = cm + ((size_t)Q.cell * g.nxc + X2.cell) * cell_stride;
-        double lum = 0.0;
-        for (int a = 0; a < g.nflav; ++a) {
-            int b = santi[a];
-            if (b < 0) continue;
-            lum = fma(patch_any<CONT>(g, c1 + a * 16, X1, Q), patch_any<CONT>(g, c2 + b * 16, X2, Q), lum);
-        }
-        const double w = (-ln_tau_min) * (-ln_tau) * lum * jac;
+    for (int d = 0; d < 2; ++d) {
+        const double *e = edges + (size_t)d * (n_bins + 1);
+        const double vn = (d ? vv.y : vv.x) * nb;
+        const int b = min(max((int)vn, 0), n_bins - 1);    // uniforms outside [0, 1) stay in range
+        const double lo = __ldg(e + b), width = __ldg(e + b + 1) - lo;
+        r[d] = fma(vn - (double)b, width, lo);
+        jac *= nb * width;
+        P.bin[d] = b;
+    }
+    const double ln_tau = (1.0 - r[0]) * ln_tau_min;
+    const double h = 0.5 * ln_tau;
+    const double y = (2.0 * r[1] - 1.0) * (-h);
+    P.w = ln_tau + ln_s;
+    P.u1 = h + y;
+    P.u2 = h - y;
+    P.factor = (-ln_tau_min) * (-ln_tau) * jac;
+    return P;
+}
+
+// A point with a parton or the scale outside the knots (or a patch that the
+// fixed-point format does not hold), in FP64.
+__device__ __forceinline__ double slow_lumi(const GridDev &g, const signed char *anti, const double *cm,
+                                            const VegasPoint &P)
+{
+    const Axis Q = axis_w(g, P.w), X1 = axis_u(g, P.u1), X2 = axis_u(g, P.u2);
+    const size_t cell_stride = (size_t)g.nflav * 16;
+    const double *c1 = cm + ((size_t)Q.cell * g.nxc + X1.cell) * cell_stride;
+    const double *c2 = cm + ((size_t)Q.cell * g.nxc + X2.cell) * cell_stride;
+    double lum = 0.0;
+    for (int a = 0; a < g.nflav; ++a) {
+        const int b = anti[a];
+        if (b < 0) continue;
+        lum = fma(patch_any<true>(g, c1 + a * 16, X1, Q), patch_any<true>(g, c2 + b * 16, X2, Q), lum);
+    }
+    return lum;
+}
+
+__global__ void __launch_bounds__(kBlock, 3) k_vegas(const __grid_constant__ GridDev g,
+                                                     const __grid_constant__ Cols anti, int member, double ln_tau_min,
+                                                     double ln_s, int n_bins, const double *__restrict__ edges,
+                                                     const double *__restrict__ v, int64_t n, double shift,
+                                                     double *__restrict__ partials, double *__restrict__ bins,
+                                                     int tab_bytes)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ double red[2][kBlock / 32];
+    double *sbin = reinterpret_cast<double *>(smem + tab_bytes);          // [2][n_bins] sums of w^2
+    for (int k = threadIdx.x; k < 2 * n_bins; k += blockDim.x) sbin[k] = 0.0;
+    const LogTabs T = tab_bytes ? stage_log_tabs(g, smem) : grid_log_tabs(g);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int row = g.nflav;
+    unsigned char *mine = smem + tab_bytes + (((size_t)2 * n_bins * 8 + 127) & ~(size_t)127) +
+                          (size_t)wid * lumi_warp_bytes(row);
+    double *rows = reinterpret_cast<double *>(mine + kWarpBuf);
+    WarpBufs B{reinterpret_cast<uint4 *>(mine), reinterpret_cast<int64_t *>(rows + 32 * row), 0};
+    const size_t patches = (size_t)member * g.nqc * g.nxc * g.nflav;
+    const double *cm = g.coef + patches * 16;
+    const unsigned char *fm = g.fcoef ? reinterpret_cast<const unsigned char *>(g.fcoef) + patches * 128 : nullptr;
+    double s1 = 0.0, s2 = 0.0;
+    auto add = [&](const VegasPoint &P, double lum) {
+        const double w = P.factor * lum;
         const double dw = w - shift;
         s1 += w;
         s2 = fma(dw, dw, s2);
-        atomicAdd(&sbin[bin[0]], w * w);
-        atomicAdd(&sbin[n_bins + bin[1]], w * w);
+        atomicAdd(&sbin[P.bin[0]], w * w);
+        atomicAdd(&sbin[n_bins + P.bin[1]], w * w);
+    };
+    auto point = [&](int64_t i) {
+        return vegas_point(reinterpret_cast<const double2 *>(v)[i], edges, n_bins, ln_tau_min, ln_s);
+    };
+    auto drain = [&]() {
+        const int64_t i = next_queued(B, lane);
+        if (i >= 0) {
+            const VegasPoint P = point(i);
+            add(P, slow_lumi(g, anti.c, cm, P));
+        }
+        __syncwarp();
+    };
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + wid) * 32; base < n; base += stride) {
+        const int64_t i = base + lane;
+        const bool live = i < n;
+        const VegasPoint P = point(live ? i : n - 1);
+        const FixAxis Q = fix_axis_log(g, T.wkey, T.qcell, g.nqc, g.qstep, g.wlo, g.whi, P.w);
+        const FixAxis X1 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, g.ulo, g.uhi, P.u1);
+        const FixAxis X2 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, g.ulo, g.uhi, P.u2);
+        bool fast = live && fm && Q.ok && X1.ok && X2.ok;
+        if (__any_sync(kAll, fast)) {
+            const double lum = lumi_quads<false>(g, anti.c, fm, B.buf, rows, row, lane, X1, X2, Q, fast);
+            if (fast) add(P, lum);
+        }
+        push_queue(B, live && !fast, i, lane);
+        if (B.qn >= 32) drain();
     }
+    if (B.qn) drain();
     for (int o = 16; o > 0; o >>= 1) {
         s1 += __shfl_down_sync(0xffffffffu, s1, o);
         s2 += __shfl_down_sync(0xffffffffu, s2, o);
@@ -267,8 +323,11 @@ extern "C" int pdf_vegas_lumi_iteration(pdfgpu_grid_t g, int32_t member, double 
     cudaStream_t s = (cudaStream_t)stream;
     PDF_CUDA(cudaMemsetAsync(sums, 0, (2 + 2 * (size_t)n_bins) * sizeof(double), s));
     if (n == 0) return PDF_OK;
-    size_t smem = 2 * (size_t)n_bins * sizeof(double);
-    auto k = g->d.extrap == PDF_EXTRAP_CONTINUATION ? k_vegas<true> : k_vegas<false>;
+    int tab = log_tab_bytes(g->d);
+    if (tab > 16 * 1024) tab = 0;            // the tables of larger grids stay global
+    const size_t smem = (size_t)tab + ((2 * (size_t)n_bins * sizeof(double) + 127) & ~(size_t)127) +
+                        (size_t)(kBlock / 32) * lumi_warp_bytes(g->d.nflav);
+    const auto k = k_vegas;
     rc = allow_dynamic_smem((const void *)k, smem);
     if (rc) return rc;
     int grid = wave_grid(g, (const void *)k, kBlock, smem, n);
@@ -281,7 +340,7 @@ extern "C" int pdf_vegas_lumi_iteration(pdfgpu_grid_t g, int32_t member, double 
         g->partials_cap = 2 * grid;
     }
     k<<<grid, kBlock, smem, s>>>(g->d, anti, member, ln_tau_min, ln_s, n_bins, edges, v, n, shift,
-                                 g->partials, sums + 2);
+                                 g->partials, sums + 2, tab);
     PDF_CUDA(cudaGetLastError());
     k_vegas_final<<<1, 256, 0, s>>>(g->partials, grid, sums);
     PDF_CUDA(cudaGetLastError());

@@ -83,3 +83,40 @@ def test_values_at_the_format_limits(odd, extrap, n, outside):
         for k, c in enumerate(cols):
             want = got[:, c] if c < 8 else np.where(np.isnan(got[:, 0]), np.nan, 0.0)
             assert np.array_equal(few[:, k], want, equal_nan=True)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 2000, 60_001])
+def test_luminosity_with_flavours_that_set_in_at_a_threshold(n):
+    """Events (5 % of them outside the knots) on a grid whose b quarks are zero
+    up to their threshold knot, so that the patches above it keep FP64, with
+    an unpaired flavour: lum and alpha_s per event, the saved partner
+    factors, and the VEGAS sums of the same luminosity."""
+    from oracle.oracle import vegas_sums
+    from paper_2012_08221_gb300.lumi import DeviceEvents, luminosity
+    from paper_2012_08221_gb300.pdf import PDF
+    from paper_2012_08221_gb300.vegas import VegasLumi
+    from tests.test_gpu_lumi import _as_kappa, _event_logs, _lum_kappa
+    g = synth.grid_nnpdf(seeds=(83, 84))
+    rows = np.asarray(g.q_knots) <= 4.92
+    g.values[:, rows, :, 1] = g.values[:, rows, :, 11] = 0.0
+    pdf, o = PDF.from_grid(g), OracleGrid.from_synth(g)
+    ev = synth.events_lhc(n, seed=85)
+    d = DeviceEvents.from_host(ev)
+    save = torch.full((n, 2, g.n_flav), 7.0, dtype=torch.float64, device="cuda")
+    L, lum, a_s = luminosity(pdf, d, member=1, save_p=save)
+    L2, lum2, _ = luminosity(pdf, d, member=1)
+    _, lumr, asr = o.lumi(ev, member=1)
+    kap = _lum_kappa(g, o, ev, n, member=1)
+    parity.check(lum.cpu().numpy(), lumr, kap, what="lum")
+    parity.check(a_s.cpu().numpy(), asr, _as_kappa(o, ev, n), what="alpha_s")
+    assert torch.equal(lum, lum2) and abs(L.item() - L2.item()) <= 1e-12 * kap.sum() / n
+    u1, u2, w = _event_logs(ev, n)
+    for k, u in enumerate((u1, u2)):            # exp() of the logarithms: the parity rule's scale covers its rounding
+        x, q2 = np.exp(u), np.exp(w)
+        parity.check(save[:, k].cpu().numpy(), o.xfxq2_batch(g.pids, x, q2, member=1),
+                     o.kappa(g.pids, x, q2, member=1), what=f"saved parton {k}")
+    v = np.random.default_rng(86).uniform(0, 1, (n, 2))
+    vg = VegasLumi(pdf, np.log(1e-6), 2 * np.log(13000.0), n_bins=20, member=1)
+    _, _, s = vg.iteration(torch.as_tensor(v, device="cuda"), refine=False)
+    ref = vegas_sums(o, 1, np.log(1e-6), 2 * np.log(13000.0), np.tile(np.linspace(0, 1, 21), (2, 1)), v)
+    assert np.all(np.abs(s - ref) <= 1e-11 * np.abs(ref) + 1e-300)
