@@ -34,26 +34,59 @@ struct Dig {
     int h, l;
 };
 
+// The two words of a 64-bit value.  On the device they are split off in PTX:
+// from a plain cast the compiler remembers the 64-bit value and widens the
+// products below to 64 x 64 bits (279 instructions per alpha_s, not 150).
+PDF_HD int fix_hi(int64_t v)
+{
+#ifdef __CUDA_ARCH__
+    int hi;
+    asm("{.reg .b32 lo; mov.b64 {lo, %0}, %1;}" : "=r"(hi) : "l"(v));
+    return hi;
+#else
+    return (int)(uint32_t)((uint64_t)v >> 32);
+#endif
+}
+PDF_HD int fix_lo(int64_t v)
+{
+#ifdef __CUDA_ARCH__
+    int lo;
+    asm("{.reg .b32 hi; mov.b64 {%0, hi}, %1;}" : "=r"(lo) : "l"(v));
+    return lo;
+#else
+    return (int)(uint32_t)(uint64_t)v;
+#endif
+}
+// Bits [n, n + 32) of a value, 0 < n < 32 (one funnel shift).
+PDF_HD int fix_bits(int64_t v, int n)
+{
+#ifdef __CUDA_ARCH__
+    return (int)__funnelshift_r((unsigned)fix_lo(v), (unsigned)fix_hi(v), n);
+#else
+    return (int)(uint32_t)((uint64_t)v >> n);
+#endif
+}
+
 PDF_HD Dig fix_split(int64_t v)
 {
-    const uint32_t lo = (uint32_t)v;
-    return {(int)(uint32_t)((uint64_t)v >> 32) + (int)(lo >> 31), (int)lo};
+    const int lo = fix_lo(v);
+    return {fix_hi(v) + (int)((uint32_t)lo >> 31), lo};
 }
 
 PDF_HD int64_t wide(int a, int b) { return (int64_t)a * (int64_t)b; }
 PDF_HD int64_t wide(int a, int b, int64_t c) { return (int64_t)a * (int64_t)b + c; }
-PDF_HD int fix_hi(int64_t v) { return (int)(uint32_t)((uint64_t)v >> 32); }
+PDF_HD uint64_t wide(uint32_t a, uint32_t b) { return (uint64_t)a * (uint64_t)b; }
+PDF_HD uint64_t wide(uint32_t a, uint32_t b, uint64_t c) { return (uint64_t)a * (uint64_t)b + c; }
 
 // Product of two values of at most 1/2 (2^61), in the format of the factors.
 PDF_HD int64_t fix_mul(Dig a, Dig b)
 {
     const int64_t cr = wide(a.l, b.h, wide(a.h, b.l, (int64_t)1 << 29));
-    return wide(2 * a.h, 2 * b.h) + (int)(cr >> 30);
+    return wide(2 * a.h, 2 * b.h) + fix_bits(cr, 30);
 }
 
-// ln 2 in 2^-60, and its next 32 bits.
-constexpr int64_t kLn2Fix = 799144290325165978ll;
-constexpr uint32_t kLn2Low = 3164486457u;
+// ln 2 in 2^-92, in signed 32-bit digits.
+constexpr int kLn2Top = 186065279, kLn2Mid = 2099050395, kLn2Low = -1130480839;
 
 // ln of a positive normal double from its bits, value 2^60 modulo 2^64.
 //   x = 2^e m; j = top 10 bits of m; inv = 1/c_j in 2^-31 (c_j the middle of
@@ -63,24 +96,24 @@ constexpr uint32_t kLn2Low = 3164486457u;
 //   a point on a knot gets the knot's own logarithm.
 PDF_HD int64_t fix_log(uint64_t bits, const uint32_t *inv, const int64_t *tab)
 {
-    const uint32_t hw = (uint32_t)(bits >> 32);
+    const uint32_t hw = (uint32_t)fix_hi((int64_t)bits);
     const int e = (int)(hw >> 20) - 1023;
     const uint32_t j = (hw >> (20 - kLogBits)) & (kLogTab - 1);
-    const uint64_t M = (bits << 11) | ((uint64_t)1 << 63);
+    const uint32_t mh = (uint32_t)fix_bits((int64_t)bits, 21) | 0x80000000u, ml = (uint32_t)fix_lo((int64_t)bits) << 11;
     const uint32_t I = inv[j];
-    const uint64_t lo = (uint64_t)(uint32_t)M * I;
-    const uint64_t P = (uint64_t)(uint32_t)(M >> 32) * I + (lo >> 32);
+    const uint64_t P = wide(mh, I, (uint64_t)(uint32_t)fix_hi((int64_t)wide(ml, I)));
     const int64_t R = (int64_t)(P - ((uint64_t)1 << 62));       // r 2^62
-    const int rh = (int)(R >> 21), rl = (int)((uint32_t)R & 0x1FFFFFu), rs = (int)(R >> 30);
+    const int rh = fix_bits(R, 21), rl = fix_lo(R) & 0x1FFFFF, rs = fix_bits(R, 30);
     const int64_t sq = wide(rh, rh);                            // r^2 2^82
     const int64_t r2 = sq + (wide(rh, rl) >> 20);
     int z = fix_hi(wide(rs, 429496730, -((int64_t)536870912 << 32)));  // -1/4 + r/5, in 2^-31
     z = fix_hi(wide(rs, z, (int64_t)715827883 << 32));                 // 1/3 + r z
     const int c = fix_hi(wide(fix_hi(sq), rh));                        // r^3 2^59
-    const int tail = (int)(wide(c, z, 1 << 29) >> 30);                 // in 2^-60
+    const int64_t tail = wide(c, z, 1 << 29) >> 30;                    // in 2^-60
     const int64_t head = (R - (r2 >> 21) + 2) >> 2;
-    const int64_t el = (int64_t)e * kLn2Fix + (((int64_t)e * kLn2Low + ((int64_t)1 << 31)) >> 32);
-    return (int64_t)((uint64_t)head + (uint64_t)tab[j] + (uint64_t)el) + tail;
+    // e ln 2: the upper 32 bits of the constant times e, the lower ones, and 32 more
+    const int64_t el = wide(e, kLn2Mid, (int64_t)((uint64_t)(uint32_t)(e * kLn2Top) << 32)) + fix_hi(wide(e, kLn2Low, (int64_t)1 << 31));
+    return (int64_t)((uint64_t)head + (uint64_t)tab[j] + (uint64_t)el + (uint64_t)tail);
 }
 
 // One cell's logarithm of the lower knot and 2^126 / (width << s), with the
@@ -97,8 +130,10 @@ PDF_HD int64_t fix_coord(int64_t u, const FixCell &c)
     int64_t v = (int64_t)((uint64_t)u - (uint64_t)c.U);
     v = v < 0 ? 0 : v;                      // a unit of the logarithm's error below the knot
     const uint64_t vv = (uint64_t)v << (c.K & 63);
-    const uint32_t vh = (uint32_t)(vv >> 32), vl = (uint32_t)vv, kh = (uint32_t)(c.K >> 32), kl = (uint32_t)c.K;
-    return (int64_t)((uint64_t)vh * kh + (((uint64_t)vh * kl) >> 32) + (((uint64_t)vl * kh) >> 32));
+    const uint32_t vh = (uint32_t)fix_hi((int64_t)vv), vl = (uint32_t)fix_lo((int64_t)vv);
+    const uint32_t kh = (uint32_t)fix_hi((int64_t)c.K), kl = (uint32_t)fix_lo((int64_t)c.K);
+    const uint64_t a = (uint32_t)fix_hi((int64_t)wide(vh, kl)), b = (uint32_t)fix_hi((int64_t)wide(vl, kh));
+    return (int64_t)(wide(vh, kh, a) + b);
 }
 
 constexpr int64_t kFixHalf = (int64_t)1 << 61;

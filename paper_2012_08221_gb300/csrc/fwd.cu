@@ -93,7 +93,7 @@ __device__ __noinline__ void slow_point_pw(const GridDev &g, const double *cm, i
     out[i] = bad ? dnan() : v;
 }
 
-template <bool TAPE, bool DT>
+template <bool TAPE, bool DT, bool STAGE>
 __global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ GridDev g, int member,
                                                         const int *__restrict__ pid,
                                                         const double *__restrict__ x,
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ 
                                                         int *__restrict__ dbins, int nbins, int tab_bytes)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    const CoordTabs T = tab_bytes ? stage_tabs(g, smem) : grid_tabs(g);
+    const CoordTabs T = STAGE ? stage_tabs(g, smem) : grid_tabs(g);
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned char *mine = smem + tab_bytes + (size_t)wid * (kWarpBuf + kQueue * 8);
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ 
         const double xi = live ? x[i] : 0.5, qi = live ? q2[i] : 10.0;
         const int col = live ? pid_col(g, pid[i]) : -1;
         const FixAxis X = fix_axis_x(g, T, dbits(xi)), Q = fix_axis_q2(g, T, dbits(qi));
-        bool fast = live && X.ok && Q.ok && x_ok(dbits(xi)) && q2_ok(dbits(qi)) && fm;
+        bool fast = live && X.ok && Q.ok && fm;      // inside the knots, so inside the domain
         if (__any_sync(kAll, fast)) {
             const uint32_t patch0 =
                 fast ? (uint32_t)(Q.cell * g.nxc + X.cell) * (uint32_t)g.nflav + (col >= 0 ? col : 0) : 0u;
@@ -162,18 +162,42 @@ __global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ 
     if (B.qn) drain();
 }
 
-// alpha_s, one point per lane (fix_alphas): 1e7 points 286 -> 120 us (FP64
+// alpha_s, one point per lane (fix_alphas): 1e7 points 286 -> 94 us (FP64
 // pipe 82 % busy before; now integer issue of the logarithm and the table
 // look-ups in shared memory); points outside the Q range or the
 // domain are queued per warp and evaluated 32 at a time.
-template <bool Q_IS_Q>
+// STAGE: the block's copy of the Q tables and of the cubics (as chunks of 16
+// bytes, the first of all cells before the second) in shared memory.
+__host__ __device__ inline int alphas_tab_bytes(const GridDev &g)
+{
+    return (g.nqc * 56 + kGuideRun * 8 + kLogTab * 12 + g.nqg * 2 + 127) & ~127;
+}
+
+template <bool Q_IS_Q, bool STAGE>
 __global__ void __launch_bounds__(kBlock) k_alphas(const __grid_constant__ GridDev g, const double *__restrict__ q,
-                                                   int64_t n, double *__restrict__ out, int tab_bytes)
+                                                   int64_t n, double *__restrict__ out)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int64_t squeue[kBlock / 32][kQueue];
-    const CoordTabs T = tab_bytes ? stage_tabs(g, smem) : grid_tabs(g);
-    __syncthreads();
+    uint4 *rows = reinterpret_cast<uint4 *>(smem);
+    FixCell *cells = reinterpret_cast<FixCell *>(rows + 2 * g.nqc);
+    int64_t *logs = reinterpret_cast<int64_t *>(cells + g.nqc);
+    uint64_t *keys = reinterpret_cast<uint64_t *>(logs + kLogTab);
+    uint32_t *invs = reinterpret_cast<uint32_t *>(keys + g.nqc + kGuideRun);
+    uint16_t *guide = reinterpret_cast<uint16_t *>(invs + kLogTab);
+    if (STAGE) {
+        for (int k = threadIdx.x; k < 2 * g.nqc; k += blockDim.x)
+            rows[(k & 1) * g.nqc + (k >> 1)] = reinterpret_cast<const uint4 *>(g.facoef)[k];
+        for (int k = threadIdx.x; k < g.nqc; k += blockDim.x) cells[k] = g.qfix[k];
+        for (int k = threadIdx.x; k < g.nqc + kGuideRun; k += blockDim.x) keys[k] = g.qbits[k];
+        for (int k = threadIdx.x; k < g.nqg; k += blockDim.x) guide[k] = g.qguide[k];
+        for (int k = threadIdx.x; k < kLogTab; k += blockDim.x) {
+            logs[k] = g.flog[k];
+            invs[k] = g.finv[k];
+        }
+        __syncthreads();
+    }
+    const CoordTabs T = STAGE ? CoordTabs{invs, logs, nullptr, keys, nullptr, guide, nullptr, cells} : grid_tabs(g);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     WarpBufs B{nullptr, squeue[wid], 0};
     auto drain = [&]() {
@@ -197,8 +221,18 @@ __global__ void __launch_bounds__(kBlock) k_alphas(const __grid_constant__ GridD
         double qi = live ? q[i] : 10.0;
         if (Q_IS_Q) qi = qi * qi;
         const FixAxis Q = fix_axis_q2(g, T, dbits(qi));
-        const bool fast = live && Q.ok && q2_ok(dbits(qi));
-        if (fast) out[i] = fix_alphas(g, Q);
+        bool fast = live && Q.ok;                    // inside the knots, so inside the domain
+        int c[8];
+        if (STAGE) {
+            const uint4 a = rows[Q.cell], b = rows[g.nqc + Q.cell];
+            c[0] = a.x, c[1] = a.y, c[2] = a.z, c[3] = a.w, c[4] = b.x, c[5] = b.y, c[6] = b.z, c[7] = b.w;
+        } else {
+            fix_ld(reinterpret_cast<const unsigned char *>(g.facoef) + (size_t)Q.cell * 32, c);
+        }
+        bool none;
+        const double v = fix_alphas(c, Q.t, none);
+        fast &= !none;
+        if (fast) out[i] = v;
         push_queue(B, live && !fast, i, lane);
         if (B.qn >= 32) drain();
     }
@@ -361,14 +395,12 @@ int launch_alphas(pdfgpu_grid *g, const double *q, int64_t n, double *out, cudaS
     if (n < 0) return fail(PDF_E_ARG, "negative n");
     if (n == 0) return PDF_OK;
     if (!q || !out) return fail(PDF_E_ARG, "null array");
-    const void *kern = q_is_q ? (const void *)k_alphas<true> : (const void *)k_alphas<false>;
-    int tab = coord_tab_bytes(g->d);
-    if (n < kStagePoints * g->sm_count || (size_t)tab > kStageMax) tab = 0;
-    int grid = wave_grid(g, kern, kBlock, tab, n);
-    if (q_is_q)
-        k_alphas<true><<<grid, kBlock, tab, s>>>(g->d, q, n, out, tab);
-    else
-        k_alphas<false><<<grid, kBlock, tab, s>>>(g->d, q, n, out, tab);
+    int tab = alphas_tab_bytes(g->d);
+    const bool stage = n >= kStagePoints * g->sm_count && (size_t)tab <= 32 * 1024;
+    if (!stage) tab = 0;
+    auto k = q_is_q ? (stage ? k_alphas<true, true> : k_alphas<true, false>)
+                    : (stage ? k_alphas<false, true> : k_alphas<false, false>);
+    k<<<wave_grid(g, (const void *)k, kBlock, tab, n), kBlock, tab, s>>>(g->d, q, n, out);
     PDF_CUDA(cudaGetLastError());
     return PDF_OK;
 }
@@ -389,9 +421,12 @@ int launch_pw(pdfgpu_grid *g, int32_t member, const int32_t *pid, const double *
     if (dtape && nbins64 >= (int64_t)1 << 30) return fail(PDF_E_RANGE, "grid too large for the derivative tape");
     if (n == 0) return PDF_OK;
     if (!pid || !x || !q2 || !out) return fail(PDF_E_ARG, "null array");
-    auto k = dtape ? k_xfxq2_pw<true, true> : tape ? k_xfxq2_pw<true, false> : k_xfxq2_pw<false, false>;
     int tab = coord_tab_bytes(g->d);
-    if (n < kStagePoints * g->sm_count || (size_t)tab > kStageMax) tab = 0;
+    const bool stage = n >= kStagePoints * g->sm_count && (size_t)tab <= kStageMax;
+    if (!stage) tab = 0;
+    auto k = dtape  ? (stage ? k_xfxq2_pw<true, true, true> : k_xfxq2_pw<true, true, false>)
+             : tape ? (stage ? k_xfxq2_pw<true, false, true> : k_xfxq2_pw<true, false, false>)
+                    : (stage ? k_xfxq2_pw<false, false, true> : k_xfxq2_pw<false, false, false>);
     const size_t smem = (size_t)tab + (kBlock / 32) * (kWarpBuf + kQueue * 8);
     rc = allow_dynamic_smem((const void *)k, smem);
     if (rc) return rc;

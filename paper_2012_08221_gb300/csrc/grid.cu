@@ -213,10 +213,10 @@ static void cell_matrix(const double *z, int n, int k, double M[16], bool linear
 }
 
 // Guide table of a cell search over ascending lower keys (see
-// find_cell_guided): the widest bucket width 2^shift, at most kGuideMax
-// buckets from the first key to key_hi, for which no bucket holds more than
-// one further lower key, else more than kGuideRun (the last bucket counts
-// every cell above it, since keys beyond key_hi fall into it).  Left empty
+// find_cell_guided): the widest bucket width 2^shift in the upper words, at
+// most kGuideMax buckets from the first key to key_hi, for which no bucket
+// holds more than one further lower key, else more than kGuideRun (the last
+// bucket counts every cell above it, since keys beyond key_hi fall into it).  Left empty
 // when no width qualifies (knots clustered far more densely in one place
 // than another); the kernels then search by bisection.
 static constexpr uint64_t kGuideMax = 4096;
@@ -229,11 +229,11 @@ static void build_guide(const std::vector<uint64_t> &keys, uint64_t key_hi, std:
     *run = kGuideRun;
     const int ncell = (int)keys.size();
     if (ncell > 65536) return;               // the table holds 16-bit cells
-    const uint64_t key0 = keys[0];
+    const uint32_t h0 = (uint32_t)(keys[0] >> 32), span = (uint32_t)(key_hi >> 32) - h0;
     std::vector<uint16_t> gd;
     for (int most : {1, kGuideRun})
-        for (int s = 63; s >= 0; --s) {
-            const uint64_t nb = ((key_hi - key0) >> s) + 1;
+        for (int s = 31; s >= 0; --s) {
+            const uint64_t nb = (span >> s) + 1;
             if (nb > kGuideMax) break;
             gd.assign(nb, 0);
             bool ok = true;
@@ -243,7 +243,7 @@ static void build_guide(const std::vector<uint64_t> &keys, uint64_t key_hi, std:
                 const int c0 = c;
                 int last = ncell - 1;        // the bucket's last cell
                 if (b + 1 < nb) {
-                    const uint64_t next = key0 + ((b + 1) << s);
+                    const uint64_t next = ((uint64_t)h0 + ((b + 1) << s)) << 32;
                     while (c + 1 < ncell && keys[c + 1] <= next) ++c;
                     last = c > c0 && keys[c] == next ? c - 1 : c;
                 }
@@ -646,6 +646,8 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
     d.extrap = D.extrap;
 
     TableUpload up;
+    xbits.insert(xbits.end(), kGuideRun, ~(uint64_t)0);
+    qbits.insert(qbits.end(), kGuideRun, ~(uint64_t)0);
     up.add(xbits.data(), xbits.size(), &d.xbits);
     up.add(ukey.data(), ukey.size(), &d.ukey);
     up.add(xcell.data(), xcell.size(), &d.xcell);

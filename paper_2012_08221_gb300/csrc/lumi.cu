@@ -139,8 +139,12 @@ __global__ void __launch_bounds__(kBlock, SAVE ? 2 : 3) k_lumi(const __grid_cons
             if (SAVE) warp_run_reuse(lane);           // the previous run has left the rows
             const double s = lumi_quads<SAVE>(g, anti.c, fm, B.buf, rows, row, lane, X1, X2, Q, fast);
             if (fast) {
+                bool none = false;
+                if (as) as[e] = fix_alphas(g, Q, none);
+                fast = !none;
+            }
+            if (fast) {
                 if (lum) lum[e] = s;
-                if (as) as[e] = fix_alphas(g, Q);
                 acc += s;
             }
             if (SAVE) {

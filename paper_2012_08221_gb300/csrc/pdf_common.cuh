@@ -110,16 +110,16 @@ struct GridDev {
     int nrows, nsub, nflav, nmem;
     int xstep, qstep;     // search start steps (largest power of two < cells)
     int nxg, nqg;         // guide-table buckets per axis (0: no guide, binary search)
-    int xgshift, qgshift; // log2 of the guide buckets' width in key units
+    int xgshift, qgshift; // log2 of the guide buckets' width in units of the keys' upper words
     int xgrun, qgrun;     // lower keys a bucket may hold beyond its first cell's
     uint64_t xlo, xhi;    // bit patterns of the first / last x knot
     uint64_t qlo, qhi;    // bit patterns of the first / last Q^2 knot
     int64_t ulo, uhi;     // order keys of ln(first / last x knot)
     int64_t wlo, whi;     // order keys of ln(first / last Q^2 knot)
-    const uint64_t *xbits;   // [nxc] bits of each x cell's lower knot
+    const uint64_t *xbits;   // [nxc + kGuideRun] bits of each x cell's lower knot
     const int64_t *ukey;     // [nxc] order keys of each x cell's lower ln x
     const double2 *xcell;    // [nxc] (U_k, 1/dU_k)
-    const uint64_t *qbits;   // [nqc] bits of each Q cell's lower Q^2 knot
+    const uint64_t *qbits;   // [nqc + kGuideRun] bits of each Q cell's lower Q^2 knot
     const uint16_t *xguide;  // [nxg] first cell of each x guide bucket
     const uint16_t *qguide;  // [nqg] the same for Q^2
     const FixCell *xfix;     // [nxc] the cells of the fixed-point coordinates
@@ -160,28 +160,28 @@ __device__ __forceinline__ int find_cell(const K *keys, int ncell, int step, K k
     return lo;
 }
 
-// The same search through a guide table: bucket b covers the keys
-// key0 + [b 2^shift, (b + 1) 2^shift) (the last bucket also everything
-// above) and holds the largest cell whose lower key is <= the bucket's first
-// key; the host builds the table so that no bucket holds more than `run`
-// (1 to kGuideRun) further lower keys.  The cell of a key is then the
-// bucket's cell plus the number of the next `run` lower keys that are <= it
-// (the keys ascend): one table load and `run` independent key loads, instead
-// of a chain of log2(cells) dependent ones.  Without a table (nguide == 0)
-// the binary search.
+// The same search through a guide table over the keys' upper words: bucket b
+// covers the upper words h0 + [b 2^shift, (b + 1) 2^shift), h0 that of the
+// first key (the last bucket also everything above), and holds the largest
+// cell whose lower key is <= the bucket's first key (the first cell in bucket
+// 0); the host builds the table so that no bucket holds more than `run` (1 to
+// kGuideRun) further lower keys, and ends the keys with kGuideRun largest
+// ones.  The cell of a key is then the bucket's cell plus the number of the
+// next `run` lower keys that are <= it (the keys ascend): one table load and
+// `run` independent key loads, instead of a chain of log2(cells) dependent
+// ones.  Without a table (nguide == 0) the binary search.
 constexpr int kGuideRun = 3;
 
 __device__ __forceinline__ int find_cell_guided(const uint64_t *keys, int ncell, int step, const uint16_t *guide,
                                                 int nguide, int shift, int run, uint64_t key0, uint64_t key)
 {
     if (nguide == 0) return find_cell<uint64_t>(keys, ncell, step, key);
-    if (key < key0) return 0;
-    const uint64_t off = (key - key0) >> shift;
-    const int c = guide[off < (uint64_t)nguide ? (int)off : nguide - 1];
-    int add = (c + 1 < ncell && keys[c + 1] <= key) ? 1 : 0;
+    const uint32_t h0 = (uint32_t)(key0 >> 32), h = max((uint32_t)(key >> 32), h0);
+    const int c = guide[min((h - h0) >> shift, (uint32_t)(nguide - 1))];
+    int add = keys[c + 1] <= key ? 1 : 0;
     if (run > 1) {
 #pragma unroll
-        for (int r = 2; r <= kGuideRun; ++r) add += (c + r < ncell && keys[c + r] <= key) ? 1 : 0;
+        for (int r = 2; r <= kGuideRun; ++r) add += keys[c + r] <= key ? 1 : 0;
     }
     return c + add;
 }

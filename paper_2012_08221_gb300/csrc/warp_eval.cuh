@@ -34,7 +34,7 @@ __device__ __forceinline__ double dnan() { return __longlong_as_double(0x7FF8000
 // Bytes of a block's copies of the coordinate tables (0: they stay global).
 __host__ __device__ inline int coord_tab_bytes(const GridDev &g)
 {
-    const int b = (g.nxc + g.nqc) * 24 + kLogTab * 12 + (g.nxg + g.nqg) * 2;
+    const int b = (g.nxc + g.nqc) * 24 + 2 * kGuideRun * 8 + kLogTab * 12 + (g.nxg + g.nqg) * 2;
     return (b + 127) & ~127;
 }
 
@@ -44,21 +44,17 @@ __device__ __forceinline__ CoordTabs stage_tabs(const GridDev &g, unsigned char 
 {
     FixCell *xf = reinterpret_cast<FixCell *>(buf), *qf = xf + g.nxc;
     int64_t *lg = reinterpret_cast<int64_t *>(qf + g.nqc);
-    uint64_t *xb = reinterpret_cast<uint64_t *>(lg + kLogTab), *qb = xb + g.nxc;
-    uint32_t *iv = reinterpret_cast<uint32_t *>(qb + g.nqc);
+    uint64_t *xb = reinterpret_cast<uint64_t *>(lg + kLogTab), *qb = xb + g.nxc + kGuideRun;
+    uint32_t *iv = reinterpret_cast<uint32_t *>(qb + g.nqc + kGuideRun);
     uint16_t *xg = reinterpret_cast<uint16_t *>(iv + kLogTab), *qg = xg + g.nxg;
     for (int k = threadIdx.x; k < kLogTab; k += blockDim.x) {
         lg[k] = g.flog[k];
         iv[k] = g.finv[k];
     }
-    for (int k = threadIdx.x; k < g.nxc; k += blockDim.x) {
-        xf[k] = g.xfix[k];
-        xb[k] = g.xbits[k];
-    }
-    for (int k = threadIdx.x; k < g.nqc; k += blockDim.x) {
-        qf[k] = g.qfix[k];
-        qb[k] = g.qbits[k];
-    }
+    for (int k = threadIdx.x; k < g.nxc; k += blockDim.x) xf[k] = g.xfix[k];
+    for (int k = threadIdx.x; k < g.nqc; k += blockDim.x) qf[k] = g.qfix[k];
+    for (int k = threadIdx.x; k < g.nxc + kGuideRun; k += blockDim.x) xb[k] = g.xbits[k];
+    for (int k = threadIdx.x; k < g.nqc + kGuideRun; k += blockDim.x) qb[k] = g.qbits[k];
     for (int k = threadIdx.x; k < g.nxg; k += blockDim.x) xg[k] = g.xguide[k];
     for (int k = threadIdx.x; k < g.nqg; k += blockDim.x) qg[k] = g.qguide[k];
     return {iv, lg, xb, qb, xg, qg, xf, qf};
@@ -137,35 +133,34 @@ __device__ __forceinline__ void quad_offsets(uint32_t own, int lane, uint32_t of
     for (int j = 0; j < 4; ++j) off[j] = __shfl_sync(kAll, own, (lane & ~3) | j) + (lane & 3) * 32;
 }
 
-// alpha_s inside the Q range at a fixed-point coordinate.
-__device__ __forceinline__ double fix_alphas(const GridDev &g, const FixAxis &Q)
+// alpha_s inside the Q range at a fixed-point coordinate, from the row of its
+// cell; `none` is set where the cell's cubic needs FP64.
+__device__ __forceinline__ double fix_alphas(const int c[8], int64_t t, bool &none)
+{
+    Dig w[4];
+    w[0] = {1 << 30, 0};
+    w[1] = fix_split(t - kFixHalf);
+    w[2] = fix_split(fix_mul(w[1], w[1]));
+    w[3] = fix_split(fix_mul(w[2], w[1]));
+    none = fix_none(c[6]);
+    return fix_value(fix_row(c, w), c[6]);
+}
+__device__ __forceinline__ double fix_alphas(const GridDev &g, const FixAxis &Q, bool &none)
 {
     int c[8];
     fix_ld(reinterpret_cast<const unsigned char *>(g.facoef) + (size_t)Q.cell * 32, c);
-    Dig w[4];
-    w[0] = {1 << 30, 0};
-    w[1] = fix_split(Q.t - kFixHalf);
-    w[2] = fix_split(fix_mul(w[1], w[1]));
-    w[3] = fix_split(fix_mul(w[2], w[1]));
-    if (fix_none(c[6])) {
-        Axis A;
-        A.cell = Q.cell;
-        A.in = true;
-        A.below = false;
-        make_basis(A, fix_t(Q.t), g.extrap);
-        const D4 a = ld4(g.acoef + (size_t)Q.cell * 4);
-        return horner(A, a.x, a.y, a.z, a.w);
-    }
-    return fix_value(fix_row(c, w), c[6]);
+    return fix_alphas(c, Q.t, none);
 }
 
-// alpha_s at any Q^2 > 0 in FP64 arithmetic outside the knots.
+// alpha_s at any Q^2 > 0; FP64 arithmetic outside the knots.
 __device__ __forceinline__ double alphas_at(const GridDev &g, const CoordTabs &T, double q2, bool *oor)
 {
     const FixAxis f = fix_axis_q2(g, T, dbits(q2));
+    *oor = false;
     if (f.ok) {
-        *oor = false;
-        return fix_alphas(g, f);
+        bool none;
+        const double a = fix_alphas(g, f, none);
+        if (!none) return a;
     }
     const Axis Q = axis_q2(g, q2);
     *oor = g.extrap == PDF_EXTRAP_ERROR && !Q.in;
@@ -277,7 +272,7 @@ __device__ __forceinline__ void eval_points(const GridDev &g, const CoordTabs &T
     double qi = live ? Y.q[i] : 10.0;
     if (Q_IS_Q) qi = qi * qi;
     const FixAxis X = fix_axis_x(g, T, dbits(xi)), Q = fix_axis_q2(g, T, dbits(qi));
-    const bool fast = live && X.ok && Q.ok && x_ok(dbits(xi)) && q2_ok(dbits(qi)) && Y.fm;
+    const bool fast = live && X.ok && Q.ok && Y.fm;      // inside the knots, so inside the domain
     push_queue(B, live && !fast, i, lane);
     if (__any_sync(kAll, fast)) {
         if (TAPE && fast) {
@@ -290,7 +285,8 @@ __device__ __forceinline__ void eval_points(const GridDev &g, const CoordTabs &T
             AQ.t = fix_t(Q.t);
             tape_put(Y.tape, i, AX, AQ, false);
         }
-        if (AS && fast) Y.alphas[i] = fix_alphas(g, Q);
+        bool none = false;                    // a patch or cubic that the format does not hold
+        if (AS && fast) Y.alphas[i] = fix_alphas(g, Q, none);
         const uint32_t cell = fast ? (uint32_t)(Q.cell * g.nxc + X.cell) : 0u;
         uint32_t off[4];
         quad_offsets(cell * ((uint32_t)g.nflav * 128u), lane, off);
@@ -299,7 +295,6 @@ __device__ __forceinline__ void eval_points(const GridDev &g, const CoordTabs &T
         quad_weights(B.buf, lane, fast ? X.t : kFixHalf, fast ? Q.t : kFixHalf, W);
         double *srow = reinterpret_cast<double *>(B.buf) + lane * Y.npid;
         const QuadPos pos = quad_pos(lane);
-        bool none = false;                    // a patch that the format does not hold
         for (int a = Y.a0; a < Y.a1; ++a) {
             int col = Y.scol[a];
             double v = 0.0;
