@@ -195,38 +195,157 @@ __device__ __forceinline__ void fix_ld(const unsigned char *p, int c[8])
 }
 #endif
 
-// Packs `rows` x 4 centred coefficients into the table's words: `big` is the
-// part of the constant term that is added exactly, the patch's value at its
-// lower corner (t = 0 on both axes), about which the FP64 form expands.  The
-// fixed-point error follows the patch's largest coefficient, the FP64 error
-// next to the lower edges follows the values there: a patch whose lower
-// corner is 2^12 below its largest coefficient (a flavour that sets in at a
-// threshold knot, say) keeps FP64.
-PDF_HD void fix_pack(const double *c, int rows, double big, uint32_t *out)
+// A patch whose lower corner (t = 0 on both axes, about which the FP64 form
+// expands) is 2^12 below its largest coefficient keeps FP64: the fixed-point
+// error follows the largest coefficient, the FP64 error next to the lower
+// edges follows the values there (a flavour that sets in at a threshold knot).
+PDF_HD bool fix_corner_ok(double corner, int E)
+{
+    return fabs(corner) >= dfrom((uint64_t)(E - 12 + 1023) << 52);
+}
+
+// The table's words of one coefficient (value 2^(61 - E)); the last of a row
+// carries the block exponent.
+PDF_HD void fix_words(int64_t v, bool last, int e8, uint32_t *out)
+{
+    if (last) v = ((v - e8 + 128) & ~(int64_t)255) | e8;
+    const Dig d = fix_split(v);
+    out[0] = (uint32_t)d.l;
+    out[1] = (uint32_t)d.h;
+}
+
+// Packs a centred cubic (alpha_s): `big` is the part of the constant term
+// that is added exactly, its value at the lower knot.
+PDF_HD void fix_pack_cubic(const double c[4], double big, uint32_t out[8])
 {
     double top = fabs(c[0] + big);
-    for (int k = 1; k < 4 * rows; ++k) top = fabs(c[k]) > top || !(fabs(c[k]) <= 1e300) ? fabs(c[k]) : top;
-    int e = 0;
+    for (int k = 1; k < 4; ++k) top = fabs(c[k]) > top || !(fabs(c[k]) <= 1e300) ? fabs(c[k]) : top;
+    int e8 = 0;
     double scale = 0.0;
     bool ok = top <= 1e300 && fabs(big) <= 1e300;
     if (ok && top > 0.0) {
         const int E = (int)((dbits(top) >> 52) & 0x7FF) - 1022;
-        e = E + kFixBias;
-        ok = e >= 0 && e < kFixNone && fabs(big) >= dfrom((uint64_t)(E - 12 + 1023) << 52);
+        e8 = E + kFixBias;
+        ok = e8 >= 0 && e8 < kFixNone && fix_corner_ok(big, E);
         if (ok) scale = dfrom((uint64_t)(61 - E + 1023) << 52);
     }
-    if (!ok) e = kFixNone;
-    for (int k = 0; k < 4 * rows; ++k) {
+    if (!ok) e8 = kFixNone;
+    for (int k = 0; k < 4; ++k) {
         int64_t v = 0;
-        if (ok) {
-            v = (int64_t)rint(c[k] * scale);
-            if (k == 0) v += (int64_t)rint(big * scale);
-        }
-        if ((k & 3) == 3) v = ((v - e + 128) & ~(int64_t)255) | e;
-        const Dig d = fix_split(v);
-        out[2 * k] = (uint32_t)d.l;
-        out[2 * k + 1] = (uint32_t)d.h;
+        if (ok) v = (int64_t)rint(c[k] * scale) + (k == 0 ? (int64_t)rint(big * scale) : 0);
+        fix_words(v, k == 3, e8, out + 2 * k);
     }
+}
+
+// A cell's centred matrix in fixed point: row m holds its four entries times
+// 2^(61 - k[m]), the sum of their sizes at most 2^k[m]; k[0] < 0 marks a cell
+// whose entries are too large (very uneven knots), which keeps FP64.
+struct FixMatrix {
+    Dig d[4][4];
+    int k[4];
+};
+
+// Sum over i of M[i] v_i / 2^61 (|v_i| <= 2^61): one entry of a matrix product.
+PDF_HD int64_t fix_dot(const Dig M[4], Dig v0, Dig v1, Dig v2, Dig v3)
+{
+    int64_t hh = wide(M[0].h, v0.h), cr = wide(M[0].h, v0.l, (int64_t)1 << 28);
+    cr = wide(M[0].l, v0.h, cr);
+    hh = wide(M[1].h, v1.h, hh), cr = wide(M[1].h, v1.l, cr), cr = wide(M[1].l, v1.h, cr);
+    hh = wide(M[2].h, v2.h, hh), cr = wide(M[2].h, v2.l, cr), cr = wide(M[2].l, v2.h, cr);
+    hh = wide(M[3].h, v3.h, hh), cr = wide(M[3].h, v3.l, cr), cr = wide(M[3].l, v3.h, cr);
+    return (int64_t)((uint64_t)hh << 3) + (cr >> 29);
+}
+
+// A double as an integer times 2^-s, rounded; zero below.
+PDF_HD int64_t fix_from(double v, int s)
+{
+    const uint64_t b = dbits(v);
+    const int e = (int)(b >> 52) & 0x7FF, n = e - 1075 + s;
+    const uint64_t m = e ? (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull : 0;
+    const uint64_t r = n >= 0 ? m << (n & 63) : n > -54 ? (m + ((uint64_t)1 << (-n - 1))) >> -n : 0;
+    return (int64_t)b < 0 ? -(int64_t)r : (int64_t)r;
+}
+
+PDF_HD int fix_clz(uint64_t v)
+{
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)v);
+#else
+    return v ? __builtin_clzll(v) : 64;
+#endif
+}
+PDF_HD int64_t fix_shift(int64_t v, int n)   // v 2^n, rounded
+{
+    if (n >= 0) return (int64_t)((uint64_t)v << (n & 63));
+    return n > -63 ? (v + ((int64_t)1 << (-n - 1))) >> -n : 0;
+}
+
+// The fixed-point patch of a 4 x 4 stencil v (rows of Q, columns of x; ok bits
+// 4 r + i of `mask`), from its cells' matrices: all in integers, so that the
+// coefficients keep about 2^-58 of the stencil's largest value (an FP64 sum
+// keeps 2^-53) and the FP64 pipe stays free.  The interpolation of a constant
+// being the constant, the sums run over the differences to the lower corner.
+PDF_HD void fix_patch(const double v[4][4], unsigned mask, const FixMatrix &X, const FixMatrix &Q, uint32_t out[32])
+{
+    int emax = 0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if ((mask >> (4 * r + i)) & 1) {
+                const int e = (int)(dbits(v[r][i]) >> 52) & 0x7FF;
+                emax = e > emax ? e : emax;
+            }
+    const int Ev = emax - 1022;                      // |v| < 2^Ev
+    bool ok = emax != 0x7FF && X.k[0] >= 0 && Q.k[0] >= 0;
+    const int64_t ref = fix_from(v[1][1], 60 - Ev);
+    int64_t cx[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        Dig d[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            d[i] = fix_split((mask >> (4 * r + i)) & 1 ? fix_from(v[r][i], 60 - Ev) - ref : 0);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) cx[r][m] = fix_dot(X.d[m], d[0], d[1], d[2], d[3]);
+    }
+    int64_t C[4][4];
+    int E = -100000;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        const Dig c0 = fix_split(cx[0][m]), c1 = fix_split(cx[1][m]), c2 = fix_split(cx[2][m]), c3 = fix_split(cx[3][m]);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            C[n][m] = fix_dot(Q.d[n], c0, c1, c2, c3);
+            const int k = X.k[m] + Q.k[n];
+            const int64_t t = n + m ? C[n][m] : C[0][0] + (ref >> (k & 63));
+            const int e = 4 - fix_clz((uint64_t)(t < 0 ? -t : t)) + k + Ev;
+            if (t && e > E) E = e;
+        }
+    }
+    int e8 = 0;
+    if (emax == 0) {                                 // zeros (subnormal values keep FP64)
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) ok = ok && (!((mask >> (4 * r + i)) & 1) || v[r][i] == 0.0);
+    } else {
+        e8 = E + kFixBias;
+        ok = ok && e8 >= 0 && e8 < kFixNone && fix_corner_ok(v[1][1], E);
+    }
+    if (!ok) e8 = kFixNone;
+    const bool fill = ok && emax != 0;
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            int64_t c = 0;
+            if (fill) {
+                c = fix_shift(C[n][m], 1 - E + X.k[m] + Q.k[n] + Ev);
+                if (n + m == 0) c += fix_shift(ref, 1 + Ev - E);
+            }
+            fix_words(c, m == 3, e8, out + 2 * (4 * n + m));
+        }
 }
 
 }  // namespace pdfgpu

@@ -112,8 +112,9 @@ __global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ 
     const double *cm = g.coef + patches * 16;
     const unsigned char *fm = g.fcoef ? reinterpret_cast<const unsigned char *>(g.fcoef) + patches * 128 : nullptr;
     auto drain = [&]() {
-        const int64_t i = next_queued(B, lane);
-        if (i >= 0)
+        const Queued e = next_queued(B, lane);
+        const int64_t i = e.i;
+        if (i >= 0 && e.sub == 0)
             slow_point_pw(g, cm, pid_col(g, pid[i]), x[i], q2[i], i, out, tape, dtape, dbins, nbins);
         __syncwarp();
     };
@@ -201,8 +202,9 @@ __global__ void __launch_bounds__(kBlock) k_alphas(const __grid_constant__ GridD
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     WarpBufs B{nullptr, squeue[wid], 0};
     auto drain = [&]() {
-        const int64_t i = next_queued(B, lane);
-        if (i >= 0) {
+        const Queued e = next_queued(B, lane);
+        const int64_t i = e.i;
+        if (i >= 0 && e.sub == 0) {
             double qi = q[i];
             if (Q_IS_Q) qi = qi * qi;
             const bool bad = !q2_ok(dbits(qi));

@@ -169,46 +169,47 @@ static const LogTables &log_tables()   // made once per process
 // so that its constant and linear rows are exact (e_k+1 and -Q): near the
 // upper knot the weights that vanish there come out of small powers of s,
 // not of a cancellation between the rows of M.
-static void cell_matrix(const double *z, int n, int k, double M[16], bool linear, double Ms[16])
+template <typename T>
+static void cell_matrix(const T *z, int n, int k, T M[16], bool linear, T Ms[16])
 {
     if (linear) {
         // straight line between the interval's two knots: c0 = g_k, c1 = g_{k+1} - g_k
-        const double m[16] = {0.0, 1.0, 0.0, 0.0, 0.0, -1.0, 1.0, 0.0,
-                              0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        const T m[16] = {T(0.0), T(1.0), T(0.0), T(0.0), T(0.0), -T(1.0), T(1.0), T(0.0),
+                              T(0.0), T(0.0), T(0.0), T(0.0), T(0.0), T(0.0), T(0.0), T(0.0)};
         // in s: g_{k+1} + s (g_k - g_{k+1})
-        const double ms[16] = {0.0, 0.0, 1.0, 0.0, 0.0, 1.0, -1.0, 0.0,
-                               0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        const T ms[16] = {T(0.0), T(0.0), T(1.0), T(0.0), T(0.0), T(1.0), -T(1.0), T(0.0),
+                               T(0.0), T(0.0), T(0.0), T(0.0), T(0.0), T(0.0), T(0.0), T(0.0)};
         memcpy(M, m, sizeof(m));
         memcpy(Ms, ms, sizeof(ms));
         return;
     }
-    double dz = z[k + 1] - z[k];
-    double p0, p1, p2, q0, q1, q2;
+    T dz = z[k + 1] - z[k];
+    T p0, p1, p2, q0, q1, q2;
     if (k == 0) {
-        p0 = 0.0; p1 = -1.0; p2 = 1.0;
+        p0 = T(0.0); p1 = -T(1.0); p2 = T(1.0);
     } else {
-        double rho = dz / (z[k] - z[k - 1]);
-        p0 = -0.5 * rho; p1 = 0.5 * rho - 0.5; p2 = 0.5;
+        T rho = dz / (z[k] - z[k - 1]);
+        p0 = -T(0.5) * rho; p1 = T(0.5) * rho - T(0.5); p2 = T(0.5);
     }
     if (k + 1 == n - 1) {
-        q0 = -1.0; q1 = 1.0; q2 = 0.0;
+        q0 = -T(1.0); q1 = T(1.0); q2 = T(0.0);
     } else {
-        double sig = dz / (z[k + 2] - z[k + 1]);
-        q0 = -0.5; q1 = 0.5 - 0.5 * sig; q2 = 0.5 * sig;
+        T sig = dz / (z[k + 2] - z[k + 1]);
+        q0 = -T(0.5); q1 = T(0.5) - T(0.5) * sig; q2 = T(0.5) * sig;
     }
-    const double m[16] = {
-        0.0, 1.0, 0.0, 0.0,
-        p0, p1, p2, 0.0,
-        -2.0 * p0, -3.0 - 2.0 * p1 - q0, 3.0 - 2.0 * p2 - q1, -q2,
-        p0, 2.0 + p1 + q0, -2.0 + p2 + q1, q2};
+    const T m[16] = {
+        T(0.0), T(1.0), T(0.0), T(0.0),
+        p0, p1, p2, T(0.0),
+        -T(2.0) * p0, -T(3.0) - T(2.0) * p1 - q0, T(3.0) - T(2.0) * p2 - q1, -q2,
+        p0, T(2.0) + p1 + q0, -T(2.0) + p2 + q1, q2};
     memcpy(M, m, sizeof(m));
     // h00(s) = 1 - 3s^2 + 2s^3, h01(s) = 3s^2 - 2s^3, h10(s) = s - 2s^2 + s^3,
     // h11(s) = -s^2 + s^3
-    const double ms[16] = {
-        0.0, 0.0, 1.0, 0.0,
-        0.0, -q0, -q1, -q2,
-        p0, 3.0 + p1 + 2.0 * q0, -3.0 + p2 + 2.0 * q1, 2.0 * q2,
-        -p0, -2.0 - p1 - q0, 2.0 - p2 - q1, -q2};
+    const T ms[16] = {
+        T(0.0), T(0.0), T(1.0), T(0.0),
+        T(0.0), -q0, -q1, -q2,
+        p0, T(3.0) + p1 + T(2.0) * q0, -T(3.0) + p2 + T(2.0) * q1, T(2.0) * q2,
+        -p0, -T(2.0) - p1 - q0, T(2.0) - p2 - q1, -q2};
     memcpy(Ms, ms, sizeof(ms));
 }
 
@@ -297,16 +298,35 @@ static FixCell fix_cell(double z0, double z1, const uint32_t *inv, const int64_t
     return c;
 }
 
-// The rows of a cell matrix in powers of t - 1/2.
-static void centre_matrix(const double M[16], double Mc[16])
+// The rows of a cell matrix in powers of t - 1/2, and the same in fixed point
+// (see FixMatrix).
+static void centre_matrix(const long double M[16], long double Mc[16])
 {
     for (int i = 0; i < 4; ++i) {
         const long double c0 = M[i], c1 = M[4 + i], c2 = M[8 + i], c3 = M[12 + i];
-        Mc[i] = (double)(c0 + c1 / 2 + c2 / 4 + c3 / 8);
-        Mc[4 + i] = (double)(c1 + c2 + 0.75L * c3);
-        Mc[8 + i] = (double)(c2 + 1.5L * c3);
-        Mc[12 + i] = (double)c3;
+        Mc[i] = c0 + c1 / 2 + c2 / 4 + c3 / 8;
+        Mc[4 + i] = c1 + c2 + 0.75L * c3;
+        Mc[8 + i] = c2 + 1.5L * c3;
+        Mc[12 + i] = c3;
     }
+}
+
+static FixMatrix fix_matrix(const long double Mc[16])
+{
+    FixMatrix F{};
+    for (int m = 0; m < 4; ++m) {
+        long double sum = 0;
+        for (int i = 0; i < 4; ++i) sum += fabsl(Mc[4 * m + i]);
+        int k = 0;
+        while (k < 16 && sum > (long double)(1 << k)) ++k;
+        F.k[m] = k;
+        if (!(sum <= (long double)(1 << k))) F.k[0] = -1;
+        for (int i = 0; i < 4; ++i)
+            F.d[m][i] = fix_split(sum <= (long double)(1 << k) ? llrintl(ldexpl(Mc[4 * m + i], 61 - k)) : 0);
+    }
+    for (int m = 1; m < 4; ++m)
+        if (F.k[m] < 0) F.k[0] = -1;
+    return F;
 }
 
 static int largest_pow2_below(int n)
@@ -325,13 +345,11 @@ static int largest_pow2_below(int n)
 // C[n][m] = sum_r Mq[n][r] sum_i Mx[m][i] v[row r][knot i] over the 4x4
 // stencil (rows outside the cell's subgrid and knots outside the x axis have
 // zero weight and are not read).  The same patch about the
-// cell's centre (in powers of t - 1/2, from the centred matrices) goes to the
-// fixed-point table; the interpolation of a constant being the constant, its
-// sums run over the differences to the cell's first corner, so that their
-// rounding is that of the differences.
-// MONO: the matrices are in powers of t, whose first row is (0, 1, 0, 0) and
-// whose second ends in 0 (those products are left out: 88 FMAs, not 128).
-template <bool MONO>
+// cell's centre, in fixed point, comes from integer sums (fix_patch): the
+// kernel takes 33 us for the 116610 patches of the 196 x 50 grid with 13
+// flavours (with FP64 sums for both forms 72 us, the FP64 form alone 31 us).
+// The matrices' first row is (0, 1, 0, 0) and their second ends in 0: those
+// products are left out (88 FMAs, not 128).
 __device__ __forceinline__ void stencil_to_patch(const double *__restrict__ Mx, const double *__restrict__ Mq,
                                                  const double d[4][4], double C[16])
 {
@@ -340,22 +358,18 @@ __device__ __forceinline__ void stencil_to_patch(const double *__restrict__ Mx, 
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            double s = 0.0;
-            if (MONO && m == 0) s = d[r][1];
-            else
+            double s = m ? 0.0 : d[r][1];
 #pragma unroll
-                for (int i = 0; i < (MONO && m == 1 ? 3 : 4); ++i) s = fma(Mx[m * 4 + i], d[r][i], s);
+            for (int i = 0; i < (m == 0 ? 0 : m == 1 ? 3 : 4); ++i) s = fma(Mx[m * 4 + i], d[r][i], s);
             cx[r][m] = s;
         }
 #pragma unroll
     for (int n = 0; n < 4; ++n)
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            double s = 0.0;
-            if (MONO && n == 0) s = cx[1][m];
-            else
+            double s = n ? 0.0 : cx[1][m];
 #pragma unroll
-                for (int r = 0; r < (MONO && n == 1 ? 3 : 4); ++r) s = fma(Mq[n * 4 + r], cx[r][m], s);
+            for (int r = 0; r < (n == 0 ? 0 : n == 1 ? 3 : 4); ++r) s = fma(Mq[n * 4 + r], cx[r][m], s);
             C[n * 4 + m] = s;
         }
 }
@@ -384,22 +398,21 @@ __global__ void k_build_coef(GridDev g, const double *__restrict__ values, doubl
             bool ok = ((qmask >> rr) & 1) && k >= 0 && k < g.nx;
             v[rr][i] = ok ? vm[((size_t)(row0 + rr) * g.nx + k) * g.nflav + a] : 0.0;
         }
-    stencil_to_patch<true>(g.mx + (size_t)ix * 16, g.mq + (size_t)c * 16, v, C);
+    stencil_to_patch(g.mx + (size_t)ix * 16, g.mq + (size_t)c * 16, v, C);
     double *out = coef + (size_t)tid * 16;
 #pragma unroll
     for (int k = 0; k < 16; ++k) out[k] = C[k];
     if (!fcoef) return;
-    const double ref = v[1][1];
+    unsigned mask = 0;
 #pragma unroll
     for (int rr = 0; rr < 4; ++rr)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int k = ix - 1 + i;
-            v[rr][i] = ((qmask >> rr) & 1) && k >= 0 && k < g.nx ? v[rr][i] - ref : 0.0;
+            if (((qmask >> rr) & 1) && k >= 0 && k < g.nx) mask |= 1u << (4 * rr + i);
         }
-    stencil_to_patch<false>(g.mxc + (size_t)ix * 16, g.mqc + (size_t)c * 16, v, C);
     uint32_t w[32];
-    fix_pack(C, 4, ref, w);
+    fix_patch(v, mask, g.mxf[ix], g.mqf[c], w);
     uint4 *fo = reinterpret_cast<uint4 *>(fcoef + (size_t)tid * 32);
 #pragma unroll
     for (int k = 0; k < 8; ++k) fo[k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
@@ -599,9 +612,30 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
         }
     }
     const int nqc = (int)qbits.size();
-    std::vector<double> mxc(mx.size()), mqc(mq.size());
-    for (int k = 0; k < nxc; ++k) centre_matrix(&mx[(size_t)k * 16], &mxc[(size_t)k * 16]);
-    for (int c = 0; c < nqc; ++c) centre_matrix(&mq[(size_t)c * 16], &mqc[(size_t)c * 16]);
+    // the centred matrices from knot logarithms to 64 bits and more
+    std::vector<FixMatrix> mxf(nxc), mqf(nqc);
+    std::vector<double> mqc((size_t)nqc * 16);
+    {
+        std::vector<long double> U(nx), W(rows);
+        long double M[16], Ms[16], Mc[16];
+        for (int k = 0; k < nx; ++k) U[k] = logl((long double)D.x_knots[k]);
+        for (int r = 0; r < rows; ++r) W[r] = logl((long double)Q2[r]);
+        for (int k = 0; k < nxc; ++k) {
+            cell_matrix<long double>(U.data(), nx, k, M, x_linear, Ms);
+            centre_matrix(M, Mc);
+            mxf[k] = fix_matrix(Mc);
+        }
+        int c = 0, r0 = 0;
+        for (int s = 0; s < D.n_sub; r0 += D.n_q[s++])
+            for (int j = 0; j + 1 < D.n_q[s]; ++j, ++c) {
+                const bool q_linear = D.interp == PDF_INTERP_LOGBILINEAR ||
+                                      (D.interp == PDF_INTERP_LOGBICUBIC_SMALL_LINEAR && D.n_q[s] < 4);
+                cell_matrix<long double>(W.data() + r0, D.n_q[s], j, M, q_linear, Ms);
+                centre_matrix(M, Mc);
+                mqf[c] = fix_matrix(Mc);
+                for (int e = 0; e < 16; ++e) mqc[(size_t)c * 16 + e] = (double)Mc[e];
+            }
+    }
     for (int c = 1; c < nqc; ++c)
         if (!(qbits[c] > qbits[c - 1])) {
             delete g;
@@ -666,8 +700,8 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
     up.add(mq.data(), mq.size(), &d.mq);
     up.add(mxs.data(), mxs.size(), &d.mxs);
     up.add(mqs.data(), mqs.size(), &d.mqs);
-    up.add(mxc.data(), mxc.size(), &d.mxc);
-    up.add(mqc.data(), mqc.size(), &d.mqc);
+    up.add(mxf.data(), mxf.size(), &d.mxf);
+    up.add(mqf.data(), mqf.size(), &d.mqf);
     up.add(qrow.data(), qrow.size(), &d.qrow);
     up.add(qmask.data(), qmask.size(), &d.qmask);
     up.add(pidmap.data(), pidmap.size(), &d.pidmap);
@@ -695,7 +729,7 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
                 for (int rr = 0; rr < 4; ++rr)
                     if ((qmask[c] >> rr) & 1)
                         cc[nn] = fma(mqc[(size_t)c * 16 + nn * 4 + rr], D.alphas[qrow[c] - 1 + rr] - ref, cc[nn]);
-            fix_pack(cc, 1, ref, &fac[(size_t)c * 8]);
+            fix_pack_cubic(cc, ref, &fac[(size_t)c * 8]);
         }
         up.add(fac.data(), fac.size(), &d.facoef);
         up.add(ac.data(), ac.size(), &d.acoef);

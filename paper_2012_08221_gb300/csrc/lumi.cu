@@ -51,10 +51,12 @@ __device__ __forceinline__ Event event(int64_t e, const double *ln_tau, const do
 }
 
 // One event in FP64 (a parton or the scale outside the knots, a patch that the
-// fixed-point format does not hold): its sum, NaN for a bad event.
+// fixed-point format does not hold): this lane's share of its sum, NaN for a
+// bad event.
 __device__ __forceinline__ double slow_event(const GridDev &g, const signed char *anti, const double *cm, Event E,
-                                             int64_t e, double *as, double *save_p, bool report)
+                                             Queued q, double *as, double *save_p, bool report)
 {
+    const int64_t e = q.i;
     const Axis Q = axis_w(g, E.w), X1 = axis_u(g, E.u1), X2 = axis_u(g, E.u2);
     const bool oor = !E.bad && (out_of_range(g, X1, Q) || out_of_range(g, X2, Q));
     flag_status(g, report && E.bad);
@@ -64,7 +66,7 @@ __device__ __forceinline__ double slow_event(const GridDev &g, const signed char
     const double *c1 = cm + ((size_t)Q.cell * g.nxc + X1.cell) * cell_stride;
     const double *c2 = cm + ((size_t)Q.cell * g.nxc + X2.cell) * cell_stride;
     double s = 0.0;
-    for (int a = 0; a < g.nflav; ++a) {
+    for (int a = q.sub; a < g.nflav; a += q.count) {
         const int b = anti[a];
         if (b < 0) continue;
         const double p1 = patch_any<true>(g, c1 + a * 16, X1, Q);
@@ -76,7 +78,7 @@ __device__ __forceinline__ double slow_event(const GridDev &g, const signed char
             pe[g.nflav + b] = p2;
         }
     }
-    if (as) {
+    if (as && q.sub == 0) {
         const double v = alphas_any(g, ld4(g.acoef + (size_t)Q.cell * 4), Q);
         as[e] = E.bad ? qnan() : v;
     }
@@ -117,11 +119,16 @@ __global__ void __launch_bounds__(kBlock, SAVE ? 2 : 3) k_lumi(const __grid_cons
     double acc = 0.0;
     auto drain = [&]() {
         if (SAVE && lane == 0) bulk_wait_all();       // the rows staged for these events have been written
-        const int64_t e = next_queued(B, lane);
-        if (e >= 0) {
-            const Event E = event(e, ln_tau, y, flags, ln_mu2, ln_x1, ln_s);
-            const double s = slow_event(g, anti.c, cm, E, e, as, SAVE ? save_p : nullptr, partials != nullptr);
-            if (lum) lum[e] = s;
+        const Queued q = next_queued(B, lane);
+        double s = 0.0;
+        if (q.i >= 0) {
+            const Event E = event(q.i, ln_tau, y, flags, ln_mu2, ln_x1, ln_s);
+            s = slow_event(g, anti.c, cm, E, q, as, SAVE ? save_p : nullptr, partials != nullptr);
+        }
+        __syncwarp();
+        for (int o = 1; o < q.count; o <<= 1) s += __shfl_xor_sync(kAll, s, o);
+        if (q.i >= 0 && q.sub == 0) {
+            if (lum) lum[q.i] = s;
             acc += s;
         }
         __syncwarp();

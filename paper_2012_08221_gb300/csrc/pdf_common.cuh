@@ -138,8 +138,8 @@ struct GridDev {
     const double *mq;        // [nqc][16]
     const double *mxs;       // [nxc][16] the same in powers of s = 1 - t
     const double *mqs;       // [nqc][16]
-    const double *mxc;       // [nxc][16] the same in powers of t - 1/2
-    const double *mqc;       // [nqc][16]
+    const FixMatrix *mxf;    // [nxc] the same in powers of t - 1/2, in fixed point
+    const FixMatrix *mqf;    // [nqc]
     const int *qrow;         // [nqc] grid row of each Q cell's lower knot
     const int *qmask;        // [nqc] bit i (0..3): stencil row i-1 exists
     const signed char *pidmap;  // [129] column of pid in [-64, 64], -1 absent

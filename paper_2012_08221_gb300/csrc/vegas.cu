@@ -64,16 +64,16 @@ __device__ __forceinline__ VegasPoint vegas_point(double2 vv, const double *edge
 }
 
 // A point with a parton or the scale outside the knots (or a patch that the
-// fixed-point format does not hold), in FP64.
+// fixed-point format does not hold), in FP64: this lane's share of its sum.
 __device__ __forceinline__ double slow_lumi(const GridDev &g, const signed char *anti, const double *cm,
-                                            const VegasPoint &P)
+                                            const VegasPoint &P, Queued q)
 {
     const Axis Q = axis_w(g, P.w), X1 = axis_u(g, P.u1), X2 = axis_u(g, P.u2);
     const size_t cell_stride = (size_t)g.nflav * 16;
     const double *c1 = cm + ((size_t)Q.cell * g.nxc + X1.cell) * cell_stride;
     const double *c2 = cm + ((size_t)Q.cell * g.nxc + X2.cell) * cell_stride;
     double lum = 0.0;
-    for (int a = 0; a < g.nflav; ++a) {
+    for (int a = q.sub; a < g.nflav; a += q.count) {
         const int b = anti[a];
         if (b < 0) continue;
         lum = fma(patch_any<true>(g, c1 + a * 16, X1, Q), patch_any<true>(g, c2 + b * 16, X2, Q), lum);
@@ -116,11 +116,12 @@ __global__ void __launch_bounds__(kBlock, 3) k_vegas(const __grid_constant__ Gri
         return vegas_point(reinterpret_cast<const double2 *>(v)[i], edges, n_bins, ln_tau_min, ln_s);
     };
     auto drain = [&]() {
-        const int64_t i = next_queued(B, lane);
-        if (i >= 0) {
-            const VegasPoint P = point(i);
-            add(P, slow_lumi(g, anti.c, cm, P));
-        }
+        const Queued q = next_queued(B, lane);
+        const VegasPoint P = point(max(q.i, (int64_t)0));
+        double lum = q.i >= 0 ? slow_lumi(g, anti.c, cm, P, q) : 0.0;
+        __syncwarp();
+        for (int o = 1; o < q.count; o <<= 1) lum += __shfl_xor_sync(kAll, lum, o);
+        if (q.i >= 0 && q.sub == 0) add(P, lum);
         __syncwarp();
     };
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
