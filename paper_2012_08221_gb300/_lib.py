@@ -51,16 +51,16 @@ SIGNATURES = {
     "pdf_bind_values": [c_grid, _VP, _VP],
     "pdf_free_grid": [c_grid],
     "pdf_grid_info": [c_grid, _I, _I, _I, _I, _I],
-    "xfxQ2": [c_grid, C.c_int32, _I, C.c_int32, _VP, _VP, C.c_int64, _VP, _VP],
-    "xfxQ": [c_grid, C.c_int32, _I, C.c_int32, _VP, _VP, C.c_int64, _VP, _VP],
+    "xfxQ2": [c_grid, C.c_int32, _VP, C.c_int32, _VP, _VP, C.c_int64, _VP, _VP],
+    "xfxQ": [c_grid, C.c_int32, _VP, C.c_int32, _VP, _VP, C.c_int64, _VP, _VP],
     "xfxQ2_pw": [c_grid, C.c_int32, _VP, _VP, _VP, C.c_int64, _VP, _VP],
-    "xfxQ2_alphasQ2": [c_grid, C.c_int32, _I, C.c_int32, _VP, _VP, C.c_int64, _VP, _VP, _VP],
-    "xfxQ2_tape": [c_grid, C.c_int32, _I, C.c_int32, _VP, _VP, C.c_int64, _VP, _VP, _VP],
+    "xfxQ2_alphasQ2": [c_grid, C.c_int32, _VP, C.c_int32, _VP, _VP, C.c_int64, _VP, _VP, _VP],
+    "xfxQ2_tape": [c_grid, C.c_int32, _VP, C.c_int32, _VP, _VP, C.c_int64, _VP, _VP, _VP],
     "xfxQ2_pw_tape": [c_grid, C.c_int32, _VP, _VP, _VP, C.c_int64, _VP, _VP, _VP, _VP],
     "alphasQ2": [c_grid, _VP, C.c_int64, _VP, _VP],
     "alphasQ": [c_grid, _VP, C.c_int64, _VP, _VP],
     "alphasQ2_grad": [c_grid, _VP, C.c_int64, _VP, _VP, _VP],
-    "xfxQ2_host": [c_grid, C.c_int32, _I, C.c_int32, _VP, _VP, C.c_int64, _VP],
+    "xfxQ2_host": [c_grid, C.c_int32, _VP, C.c_int32, _VP, _VP, C.c_int64, _VP],
     "xfxQ2_backward": [c_grid, C.c_int32, _VP, C.c_int32, C.c_int32, _VP, _VP, C.c_int64,
                        _VP, _VP, _VP, _VP, _VP],
     "xfxQ2_backward_tape": [c_grid, C.c_int32, _VP, C.c_int32, C.c_int32, _VP, _VP, C.c_int64,
@@ -98,6 +98,8 @@ def path() -> str:
 def lib():
     """The loaded library (raises if it was never built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             p = path()
