@@ -47,7 +47,7 @@ struct BatchReq {
 };
 
 template <int QPT, bool STAGE>
-__global__ void k_batch(const GridDev *__restrict__ grids, const BatchReq *__restrict__ reqs, int nreq,
+__global__ void __launch_bounds__(256, 3) k_batch(const GridDev *__restrict__ grids, const BatchReq *__restrict__ reqs, int nreq,
                         int64_t ntiles, unsigned long long *ticket)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -58,7 +58,7 @@ __global__ void k_batch(const GridDev *__restrict__ grids, const BatchReq *__res
     unsigned char *mine = smem + (size_t)wid * kWarpBytes;
     unsigned char *tabs = smem + (size_t)(blockDim.x >> 5) * kWarpBytes;
     WarpBufs B{reinterpret_cast<uint4 *>(mine), reinterpret_cast<int64_t *>(mine + kWarpBuf), 0};
-    CoordTabs T{};
+    bool staged = false;
     int cur = -1;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -83,7 +83,8 @@ __global__ void k_batch(const GridDev *__restrict__ grids, const BatchReq *__res
             cur = sr.grid;
             if (threadIdx.x == 0) sg = grids[cur];
             __syncthreads();
-            T = STAGE && coord_tab_bytes(sg) <= (int)kStageMax ? stage_tabs(sg, tabs) : grid_tabs(sg);
+            staged = STAGE && coord_tab_bytes(sg) <= (int)kStageMax;
+            if (staged) stage_tabs(sg, tabs);
             __syncthreads();
         }
         const GridDev &g = sg;
@@ -92,13 +93,18 @@ __global__ void k_batch(const GridDev *__restrict__ grids, const BatchReq *__res
                       g.fcoef ? reinterpret_cast<const unsigned char *>(g.fcoef) + patches * 128 : nullptr,
                       sr.x, sr.q2, sr.n, sr.out, nullptr, nullptr};
         const int64_t p0 = (int64_t)(t - sr.tile0) * ((int64_t)blockDim.x * QPT);
+        // this warp's 32 consecutive points of each pass over the tile; two copies
+        // of the loop, so that the tables' address space is known in each
+        auto pass = [&](const CoordTabs &T) {
 #pragma unroll 1
-        for (int qq = 0; qq < QPT; ++qq) {
-            // this warp's 32 consecutive points of the tile
-            const int64_t base = p0 + (int64_t)qq * blockDim.x + 32 * wid;
-            if (base >= Y.n) break;
-            eval_points<false, false, false, true>(g, T, Y, B, base, lane);
-        }
+            for (int qq = 0; qq < QPT; ++qq) {
+                const int64_t base = p0 + (int64_t)qq * blockDim.x + 32 * wid;
+                if (base >= Y.n) break;
+                eval_points<false, false, false, true>(g, T, Y, B, base, lane);
+            }
+        };
+        if (STAGE && staged) pass(staged_tabs(g, tabs));
+        else pass(grid_tabs(g));
         while (B.qn) drain_queue(g, Y, false, B, lane);
         __syncthreads();   // everyone is done with sr/s_tile before thread 0 refills them
     }
@@ -345,17 +351,17 @@ extern "C" int pdf_batch_prepare(const pdfgpu_batch_desc *descs, int32_t n_desc,
     Shape best{256, 2, 1};
     float best_ms = 0.0f;
     auto hit = cache.find(sig);
-    if (hit != cache.end()) {
+    if (hit != cache.end() && hit->second.first.block <= 256) {
         best = hit->second.first;
         best_ms = hit->second.second;
     } else if (autotune) {
-        const int blocks[3] = {128, 256, 512};
+        const int blocks[2] = {128, 256};
         const int qpts[3] = {1, 2, 4};
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
         best_ms = 1e30f;
-        for (int bi = 0; bi < 3; ++bi)
+        for (int bi = 0; bi < 2; ++bi)
             for (int qi = 0; qi < 3; ++qi)
                 for (int s = 0; s < 2; ++s) {
                     Shape sh{blocks[bi], qpts[qi], s};

@@ -38,15 +38,26 @@ __host__ __device__ inline int coord_tab_bytes(const GridDev &g)
     return (b + 127) & ~127;
 }
 
-// Copies the tables into shared memory (whole block; 16-byte aligned buffer).
-// The caller synchronises the block afterwards.
-__device__ __forceinline__ CoordTabs stage_tabs(const GridDev &g, unsigned char *buf)
+// Where a block's copies of the tables lie in its buffer (16-byte aligned).
+__device__ __forceinline__ CoordTabs staged_tabs(const GridDev &g, unsigned char *buf)
 {
     FixCell *xf = reinterpret_cast<FixCell *>(buf), *qf = xf + g.nxc;
     int64_t *lg = reinterpret_cast<int64_t *>(qf + g.nqc);
     uint64_t *xb = reinterpret_cast<uint64_t *>(lg + kLogTab), *qb = xb + g.nxc + kGuideRun;
     uint32_t *iv = reinterpret_cast<uint32_t *>(qb + g.nqc + kGuideRun);
     uint16_t *xg = reinterpret_cast<uint16_t *>(iv + kLogTab), *qg = xg + g.nxg;
+    return {iv, lg, xb, qb, xg, qg, xf, qf};
+}
+
+// Makes the copies (whole block); the caller synchronises the block afterwards.
+__device__ __forceinline__ CoordTabs stage_tabs(const GridDev &g, unsigned char *buf)
+{
+    const CoordTabs T = staged_tabs(g, buf);
+    uint32_t *iv = const_cast<uint32_t *>(T.inv);
+    int64_t *lg = const_cast<int64_t *>(T.log);
+    uint64_t *xb = const_cast<uint64_t *>(T.xbits), *qb = const_cast<uint64_t *>(T.qbits);
+    uint16_t *xg = const_cast<uint16_t *>(T.xguide), *qg = const_cast<uint16_t *>(T.qguide);
+    FixCell *xf = const_cast<FixCell *>(T.xfix), *qf = const_cast<FixCell *>(T.qfix);
     for (int k = threadIdx.x; k < kLogTab; k += blockDim.x) {
         lg[k] = g.flog[k];
         iv[k] = g.finv[k];
@@ -57,7 +68,7 @@ __device__ __forceinline__ CoordTabs stage_tabs(const GridDev &g, unsigned char 
     for (int k = threadIdx.x; k < g.nqc + kGuideRun; k += blockDim.x) qb[k] = g.qbits[k];
     for (int k = threadIdx.x; k < g.nxg; k += blockDim.x) xg[k] = g.xguide[k];
     for (int k = threadIdx.x; k < g.nqg; k += blockDim.x) qg[k] = g.qguide[k];
-    return {iv, lg, xb, qb, xg, qg, xf, qf};
+    return T;
 }
 
 // Weights of the quad's four points for this lane's row, from every lane's
