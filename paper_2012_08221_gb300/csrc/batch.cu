@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(256, 3) k_batch(const GridDev *__restrict__ gr
     __shared__ GridDev sg;
     __shared__ BatchReq sr;
     __shared__ long long s_tile;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = lane_id(), wid = threadIdx.x >> 5;
     unsigned char *mine = smem + (size_t)wid * kWarpBytes;
     unsigned char *tabs = smem + (size_t)(blockDim.x >> 5) * kWarpBytes;
     WarpBufs B{reinterpret_cast<uint4 *>(mine), reinterpret_cast<int64_t *>(mine + kWarpBuf), 0};

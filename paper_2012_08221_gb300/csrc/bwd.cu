@@ -40,6 +40,7 @@
 
 #include "pdf_internal.h"
 #include "sort_acc.cuh"
+#include "warp_eval.cuh"
 
 using namespace pdfgpu;
 
@@ -49,6 +50,14 @@ constexpr int kBlock = 256;
 constexpr size_t kSmemGradMax = 200 * 1024;
 
 __device__ __forceinline__ double qnan() { return __longlong_as_double(0x7FF8000000000000ll); }
+
+// A cell's fixed-point patches, or null.
+__device__ __forceinline__ const unsigned char *fixed_patches(const GridDev &g, int member, int qc, int xc)
+{
+    if (!g.fcoef) return nullptr;
+    return reinterpret_cast<const unsigned char *>(g.fcoef) +
+           (((size_t)member * g.nqc + qc) * g.nxc + xc) * g.nflav * 128;
+}
 
 // Chain rule from the local coordinates to x and Q^2: given sx = g dP/dtx
 // and sq = g dP/dtq, dL/dx = sx (1/dU) / x and dL/dQ^2 = sq (1/dW) / Q^2,
@@ -127,6 +136,7 @@ __global__ void __launch_bounds__(kBlock) k_bwd(GridDev g, Cols cols, int npid, 
         const bool fzx = !X.in && g.extrap == PDF_EXTRAP_FREEZE;
         const bool fzq = !Q.in && g.extrap == PDF_EXTRAP_FREEZE;
         const double *cell = cm + ((size_t)Q.cell * g.nxc + X.cell) * cell_stride;
+        const unsigned char *fcell = fixed_patches(g, member, Q.cell, X.cell);
         double Wx[4], Wq[4];
         int qmask = 0, r0 = 0, k0 = 0;
         if (gval) {
@@ -149,7 +159,7 @@ __global__ void __launch_bounds__(kBlock) k_bwd(GridDev g, Cols cols, int npid, 
                 dtx = d.x;
                 dtq = d.y;
             } else {
-                patch_vd(cell + col * 16, X, Q, &dtx, &dtq);
+                patch_d(cell + col * 16, fcell ? fcell + col * 128 : nullptr, X, Q, &dtx, &dtq);
             }
             if (fzx) dtx = 0.0;
             if (fzq) dtq = 0.0;
@@ -298,7 +308,7 @@ __global__ void __launch_bounds__(kCountBlock) k_bwd_count(GridDev g, const int 
 // the monomial basis the two knots that carry no weight would receive
 // rounding-sized terms instead of zeros).
 template <bool DT>
-__global__ void __launch_bounds__(kBlock, 5) k_bwd_rec(GridDev g, int member, const int *__restrict__ pid,
+__global__ void __launch_bounds__(kBlock, DT ? 5 : 2) k_bwd_rec(GridDev g, int member, const int *__restrict__ pid,
                                                     const double *__restrict__ x,
                                                     const double *__restrict__ q2, int64_t i0, int m,
                                                     const double *__restrict__ tape,
@@ -333,7 +343,9 @@ __global__ void __launch_bounds__(kBlock, 5) k_bwd_rec(GridDev g, int member, co
                 dtx = d.x;
                 dtq = d.y;
             } else {
-                patch_vd(cm + ((size_t)Q.cell * g.nxc + X.cell) * cell_stride + col * 16, X, Q, &dtx, &dtq);
+                const unsigned char *F = fixed_patches(g, member, Q.cell, X.cell);
+                patch_d(cm + ((size_t)Q.cell * g.nxc + X.cell) * cell_stride + col * 16, F ? F + col * 128 : nullptr,
+                        X, Q, &dtx, &dtq);
             }
             if (!X.in && g.extrap == PDF_EXTRAP_FREEZE) dtx = 0.0;
             if (!Q.in && g.extrap == PDF_EXTRAP_FREEZE) dtq = 0.0;
@@ -456,104 +468,148 @@ __global__ void __launch_bounds__(kAccWarps * 32) k_bwd_accum(GridDev g, const d
 
 constexpr int kMaxSortedPids = 16;
 
-// Derivatives of a patch held in registers (as patch_vd).
-__device__ __forceinline__ void patch_d_regs(const double C[16], const Axis &X, const Axis &Q, double *dtx,
-                                             double *dtq)
+// One point of the matrix form in FP64 or lane by lane (patch_d): its
+// derivatives, and outside the knot range its exact extrapolation weights
+// per column, added to the gradient with global atomics.
+__device__ __noinline__ void slow_rec_m(const GridDev &g, const signed char *scol, int npid, int member,
+                                        const Axis &X, const Axis &Q, double xi, double qi, int64_t i,
+                                        const double *go, double *gx, double *gq, double *gval)
 {
-    D4 r[4];
+    const size_t cell_stride = (size_t)g.nflav * 16;
+    const double *cell =
+        g.coef + ((size_t)member * g.nqc * g.nxc + (size_t)Q.cell * g.nxc + X.cell) * cell_stride;
+    if (gx || gq) {
+        const unsigned char *F = fixed_patches(g, member, Q.cell, X.cell);
+        double sx = 0.0, sq = 0.0;
+        for (int a = 0; a < npid; ++a) {
+            int col = scol[a];
+            if (col < 0) continue;
+            col = checked_index(g.status, col, g.nflav);
+            double dtx, dtq;
+            patch_d(cell + col * 16, F ? F + col * 128 : nullptr, X, Q, &dtx, &dtq);
+            sx = fma(go[a], dtx, sx);
+            sq = fma(go[a], dtq, sq);
+        }
+        if (!X.in && g.extrap == PDF_EXTRAP_FREEZE) sx = 0.0;
+        if (!Q.in && g.extrap == PDF_EXTRAP_FREEZE) sq = 0.0;
+        chain_rule(sx, sq, g.xcell[X.cell].y, g.qcell[Q.cell].y, xi, qi, gx, gq, i);
+    }
+    if (X.in && Q.in) return;
+    double Wx[4], Wq[4];
+    stencil_weights(g.mx + (size_t)X.cell * 16, g.mxs + (size_t)X.cell * 16, X, Wx);
+    stencil_weights(g.mq + (size_t)Q.cell * 16, g.mqs + (size_t)Q.cell * 16, Q, Wq);
+    const int qmask = g.qmask[Q.cell], r0 = g.qrow[Q.cell] - 1, k0 = X.cell - 1;
+    for (int a = 0; a < npid; ++a) {
+        int col = scol[a];
+        if (col < 0) continue;
+        col = checked_index(g.status, col, g.nflav);
+        const double ga = go[a];
 #pragma unroll
-    for (int n = 0; n < 4; ++n) r[n] = D4{C[4 * n], C[4 * n + 1], C[4 * n + 2], C[4 * n + 3]};
-    patch_vd_rows(r, X, Q, dtx, dtq);
+        for (int j = 0; j < 4; ++j) {
+            if (!((qmask >> j) & 1)) continue;
+            const double gj = ga * Wq[j];
+            const int row = checked_index(g.status, r0 + j, g.nrows);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int kk = k0 + c;
+                const double t = gj * Wx[c];
+                if (kk >= 0 && kk < g.nx && (dbits(t) << 1))
+                    atomicAdd(gval + ((size_t)row * g.nx + kk) * g.nflav + col, t);
+            }
+        }
+    }
 }
 
-// Per point: dL/dx and dL/dQ^2 from the combined patch, and the point's
-// record (t_x, t_q, bits of cell | x inside << 32 | Q inside << 33, point
-// index) placed in its cell's range; points outside the knot range add
-// their exact extrapolation weights per column with global atomics.
-__global__ void __launch_bounds__(kBlock) k_bwd_rec_m(GridDev g, Cols cols, int npid, int member,
-                                                      const double *__restrict__ x,
-                                                      const double *__restrict__ q2, int64_t i0, int m,
-                                                      const double *__restrict__ tape,
-                                                      const double *__restrict__ gout,
-                                                      double *__restrict__ gx, double *__restrict__ gq,
-                                                      double *__restrict__ gval, int nbins,
-                                                      int *__restrict__ cursor, double *__restrict__ rec)
+// Per point: the record (t_x, t_q, bits of cell | x inside << 32 | Q inside <<
+// 33, point index) placed in its cell's range, and dL/dx and dL/dQ^2 = sum_a
+// g_a times the derivative of patch a.  A warp takes 32 points; the quads
+// evaluate both derivatives of each column in fixed point (quad_patch_d), the
+// gout rows of the 32 points come through shared memory; what that does not
+// serve is queued (slow_rec_m).  1e6 points x 13 columns: 440 us with the
+// combined patch sum_a g_a C_a in FP64 (16 FMA per column, pipe 95 % busy).
+constexpr int kRecWarpBytes = kWarpBuf + 32 * 8 * kMaxSortedPids + kQueue * 8;
+
+__global__ void __launch_bounds__(kBlock, 2) k_bwd_rec_m(const __grid_constant__ GridDev g,
+                                                         const __grid_constant__ Cols cols, int npid, int member,
+                                                         const double *__restrict__ x,
+                                                         const double *__restrict__ q2, int64_t i0, int m,
+                                                         const double *__restrict__ tape,
+                                                         const double *__restrict__ gout,
+                                                         double *__restrict__ gx, double *__restrict__ gq,
+                                                         double *__restrict__ gval, int nbins,
+                                                         int *__restrict__ cursor, double *__restrict__ rec)
 {
-    __shared__ signed char scol[PDF_MAX_PIDS];
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < PDF_MAX_PIDS; ++k) scol[k] = cols.c[k];
-    }
-    __syncthreads();
-    const size_t cell_stride = (size_t)g.nflav * 16;
-    const double *cm = g.coef + (size_t)member * g.nqc * g.nxc * cell_stride;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = lane_id(), wid = threadIdx.x >> 5;
+    unsigned char *mine = smem + (size_t)wid * kRecWarpBytes;
+    double *rows = reinterpret_cast<double *>(mine + kWarpBuf);
+    WarpBufs B{reinterpret_cast<uint4 *>(mine), reinterpret_cast<int64_t *>(rows + 32 * kMaxSortedPids), 0};
+    const unsigned char *fm = fixed_patches(g, member, 0, 0);
+    const bool deriv = gx || gq;
+    auto drain = [&]() {
+        const Queued e = next_queued(B, lane);
+        if (e.i >= 0 && e.sub == 0) {
+            Axis X, Q;
+            tape_get(g, tape, e.i, X, Q);
+            const int64_t i = i0 + e.i;
+            slow_rec_m(g, cols.c, npid, member, X, Q, x[i], q2[i], i, gout + (size_t)i * npid, gx, gq, gval);
+        }
+        __syncwarp();
+    };
+    const int stride = gridDim.x * blockDim.x;
+    for (int base = (blockIdx.x * (blockDim.x >> 5) + wid) * 32; base < m; base += stride) {
+        const int k = base + lane;
+        const bool live = k < m;
         const int64_t i = i0 + k;
         Axis X, Q;
-        if (tape_get(g, tape, k, X, Q)) {
+        const bool bad = !live || tape_get(g, tape, k, X, Q);
+        if (live && bad) {
             if (gx) gx[i] = qnan();
             if (gq) gq[i] = qnan();
-            continue;
         }
-        const double *cell = cm + ((size_t)Q.cell * g.nxc + X.cell) * cell_stride;
-        const double *go = gout + (size_t)i * npid;
-        if (gx || gq) {
-            double C[16];
-#pragma unroll
-            for (int c = 0; c < 16; ++c) C[c] = 0.0;
+        const bool inside = !bad && X.in && Q.in;
+        if (inside) {
+            const int b = sorted_cell(g, X, Q, false, half_pair(X, Q), nbins);
+            const int pos = atomicAdd(&cursor[b], 1);
+            const uint64_t bits = (uint64_t)(uint32_t)b | ((uint64_t)X.in << 32) | ((uint64_t)Q.in << 33);
+            double2 *d = reinterpret_cast<double2 *>(rec + 4 * (size_t)pos);
+            d[0] = make_double2(near_coord(X.t), near_coord(Q.t));
+            d[1] = make_double2(dfrom(bits), dfrom((uint64_t)i));
+        }
+        bool fast = inside && fm && fixed_derivative(X, Q);
+        if (deriv && __any_sync(kAll, fast)) {
+            const int count = min(32, m - base) * npid;
+            const double *go = gout + (size_t)(i0 + base) * npid;
+            for (int e = lane; e < count; e += 32) rows[e] = go[e];
+            uint32_t off[4];
+            quad_offsets(fast ? (uint32_t)(Q.cell * g.nxc + X.cell) * ((uint32_t)g.nflav * 128u) : 0u, lane, off);
+            Dig W[4][4];
+            quad_weights(B.buf, lane, fast ? X.f : kFixHalf, fast ? Q.f : kFixHalf, W);
+            const QuadPos pos = quad_pos(lane);
+            bool none = false;
+            double sx = 0.0, sq = 0.0;
             for (int a = 0; a < npid; ++a) {
-                int col = scol[a];
-                if (col < 0) continue;
+                int col = cols.c[a];
+                if (col < 0) continue;               // the same for the whole warp
                 col = checked_index(g.status, col, g.nflav);
-                const double ga = go[a];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const D4 v = ld4(cell + col * 16 + 4 * r);
-                    C[4 * r] = fma(ga, v.x, C[4 * r]);
-                    C[4 * r + 1] = fma(ga, v.y, C[4 * r + 1]);
-                    C[4 * r + 2] = fma(ga, v.z, C[4 * r + 2]);
-                    C[4 * r + 3] = fma(ga, v.w, C[4 * r + 3]);
-                }
+                int c[4][8];
+                quad_load(fm + col * 128, off, c);
+                const int last = quad_last(c, pos);
+                int64_t dx, dq;
+                quad_patch_d(c, W, B.buf, lane, pos, dx, dq);
+                const double ga = rows[lane * npid + a];
+                sx = fma(ga, fix_value(dx, last), sx);
+                sq = fma(ga, fix_value(dq, last), sq);
+                none |= fix_none(last);
             }
-            double dtx, dtq;
-            patch_d_regs(C, X, Q, &dtx, &dtq);
-            if (!X.in && g.extrap == PDF_EXTRAP_FREEZE) dtx = 0.0;
-            if (!Q.in && g.extrap == PDF_EXTRAP_FREEZE) dtq = 0.0;
-            chain_rule(dtx, dtq, g.xcell[X.cell].y, g.qcell[Q.cell].y, x[i], q2[i], gx, gq, i);
+            __syncwarp();                            // the buffers may be refilled
+            fast = fast && !none;
+            if (fast) chain_rule(sx, sq, g.xcell[X.cell].y, g.qcell[Q.cell].y, x[i], q2[i], gx, gq, i);
         }
-        if (!(X.in && Q.in)) {
-            double Wx[4], Wq[4];
-            stencil_weights(g.mx + (size_t)X.cell * 16, g.mxs + (size_t)X.cell * 16, X, Wx);
-            stencil_weights(g.mq + (size_t)Q.cell * 16, g.mqs + (size_t)Q.cell * 16, Q, Wq);
-            const int qmask = g.qmask[Q.cell], r0 = g.qrow[Q.cell] - 1, k0 = X.cell - 1;
-            for (int a = 0; a < npid; ++a) {
-                int col = scol[a];
-                if (col < 0) continue;
-                col = checked_index(g.status, col, g.nflav);
-                const double ga = go[a];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (!((qmask >> j) & 1)) continue;
-                    const double gj = ga * Wq[j];
-                    const int row = checked_index(g.status, r0 + j, g.nrows);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const int kk = k0 + c;
-                        const double t = gj * Wx[c];
-                        if (kk >= 0 && kk < g.nx && (dbits(t) << 1))
-                            atomicAdd(gval + ((size_t)row * g.nx + kk) * g.nflav + col, t);
-                    }
-                }
-            }
-            continue;
-        }
-        const int b = sorted_cell(g, X, Q, false, half_pair(X, Q), nbins);
-        const int pos = atomicAdd(&cursor[b], 1);
-        const uint64_t bits = (uint64_t)(uint32_t)b | ((uint64_t)X.in << 32) | ((uint64_t)Q.in << 33);
-        double2 *d = reinterpret_cast<double2 *>(rec + 4 * (size_t)pos);
-        d[0] = make_double2(near_coord(X.t), near_coord(Q.t));
-        d[1] = make_double2(dfrom(bits), dfrom((uint64_t)i));
+        push_queue(B, !bad && (!inside || (deriv && !fast)), k, lane);
+        if (B.qn >= 32) drain();
     }
+    if (B.qn) drain();
 }
 
 // Accumulation over the cell-sorted records of the matrix form: as
@@ -838,7 +894,10 @@ int backward_sorted(pdfgpu_grid *g, int member, const Cols &cols, int npid, cons
             PDF_CUDA(cudaGetLastError());
             k_bwd_accum<<<blocks, kAccWarps * 32, 0, st>>>(g->d, rec, offs, nbins, gval);
         } else {
-            k_bwd_rec_m<<<wave_grid(g, (const void *)k_bwd_rec_m, kBlock, 0, m), kBlock, 0, st>>>(
+            const size_t rsmem = (size_t)(kBlock / 32) * kRecWarpBytes;
+            rc = allow_dynamic_smem((const void *)k_bwd_rec_m, rsmem);
+            if (rc) return rc;
+            k_bwd_rec_m<<<wave_grid(g, (const void *)k_bwd_rec_m, kBlock, rsmem, m), kBlock, rsmem, st>>>(
                 g->d, cols, npid, member, x, q2, i0, m, tv, gout, gx, gq, gval, nbins, cursor, rec);
             PDF_CUDA(cudaGetLastError());
             if (npid >= 5)

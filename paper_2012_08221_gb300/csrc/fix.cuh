@@ -174,6 +174,22 @@ PDF_HD int64_t fix_row(const int c[8], const Dig w[4])
     return hh + fix_hi(cr);
 }
 
+// The same row differentiated in t of the x axis, c1 w0 + 2 c2 w1 + 3 c3 w2
+// (the weights w_m = tq^n tx^m serve for their own derivatives).
+PDF_HD int64_t fix_row_dx(const int c[8], const Dig w[4])
+{
+    int64_t h3 = wide(c[7], w[2].h), r3 = wide(c[6], w[2].h, wide(c[7], w[2].l, (int64_t)1 << 31));
+    const int64_t s3 = h3 + fix_hi(r3);
+    const int64_t h2 = wide(c[5], w[1].h, h3), r2 = wide(c[4], w[1].h, wide(c[5], w[1].l, r3));
+    const int64_t s2 = h2 + fix_hi(r2);              // c2 w1 + c3 w2
+    const int64_t h1 = wide(c[3], w[0].h), r1 = wide(c[2], w[0].h, wide(c[3], w[0].l, (int64_t)1 << 31));
+    return (h1 + fix_hi(r1)) + 2 * s2 + s3;
+}
+
+// Coordinates that round to a knot as doubles: there a derivative may be zero
+// by exact cancellation, which FP64 from the knot's own expansion keeps.
+PDF_HD bool fix_at_knot(int64_t t) { return t <= 0 || t >= ((int64_t)1 << 62) - 256; }
+
 // Block exponent: the low byte of a row's last coefficient is E + kFixBias;
 // kFixNone marks a patch that the format cannot hold.
 constexpr int kFixBias = 160;

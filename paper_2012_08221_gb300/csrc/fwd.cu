@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kBlock, WHOLE ? 3 : 2) k_xfxq2(const __grid_co
     extern __shared__ __align__(128) unsigned char smem[];
     const CoordTabs T = STAGE ? stage_tabs(g, smem) : grid_tabs(g);
     __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = lane_id(), wid = threadIdx.x >> 5;
     unsigned char *mine = smem + tab_bytes + (size_t)wid * warp_bytes;
     WarpBufs B{reinterpret_cast<uint4 *>(mine), reinterpret_cast<int64_t *>(mine + warp_bytes - kQueue * 8), 0};
     const size_t patches = (size_t)member * g.nqc * g.nxc * g.nflav;
@@ -63,11 +63,11 @@ __global__ void __launch_bounds__(kBlock, WHOLE ? 3 : 2) k_xfxq2(const __grid_co
 }
 
 // DT (with TAPE): also keep each point's patch derivatives in t_x and t_q,
-// computed with the value (patch_vd: the value's bits are unchanged), in
+// computed with the value from the same rows (quad_patch_d), in
 // dtape[i] = (dP/dtx, dP/dtq) (zeros for an absent pid), and the point's bin
 // in the pointwise sorted adjoint in dbins[i] (-1 for none).
-__device__ __noinline__ void slow_point_pw(const GridDev &g, const double *cm, int col, double xi, double qi, int64_t i,
-                                           double *out, double *tape, double *dtape, int *dbins, int nbins)
+__device__ __forceinline__ void slow_point_pw(const GridDev &g, const double *cm, const unsigned char *fm, int col,
+                                           double xi, double qi, int64_t i, double *out, double *tape, double *dtape, int *dbins, int nbins)
 {
     bool bad = !(x_ok(dbits(xi)) && q2_ok(dbits(qi)));
     flag_status(g, bad);
@@ -80,11 +80,15 @@ __device__ __noinline__ void slow_point_pw(const GridDev &g, const double *cm, i
     flag_status(g, oor, PDF_S_RANGE);
     bad |= oor;
     if (tape) tape_put(tape, i, X, Q, bad);
-    const double *C = cm + (((size_t)Q.cell * g.nxc + X.cell) * g.nflav + (col >= 0 ? col : 0)) * 16;
+    const size_t p = ((size_t)Q.cell * g.nxc + X.cell) * g.nflav + (col >= 0 ? col : 0);
+    const double *C = cm + p * 16;
     double v = 0.0;
     if (dtape) {
         double dtx = 0.0, dtq = 0.0;
-        if (col >= 0) v = patch_vd(C, X, Q, &dtx, &dtq);
+        if (col >= 0) {
+            v = patch(C, X, Q);
+            patch_d(C, fm ? fm + p * 128 : nullptr, X, Q, &dtx, &dtq);
+        }
         reinterpret_cast<double2 *>(dtape)[i] = make_double2(dtx, dtq);
         dbins[i] = sorted_bin(g, X, Q, bad, col, half_pair(X, Q), nbins);
     } else if (col >= 0) {
@@ -105,7 +109,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ 
     extern __shared__ __align__(128) unsigned char smem[];
     const CoordTabs T = STAGE ? stage_tabs(g, smem) : grid_tabs(g);
     __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = lane_id(), wid = threadIdx.x >> 5;
     unsigned char *mine = smem + tab_bytes + (size_t)wid * (kWarpBuf + kQueue * 8);
     WarpBufs B{reinterpret_cast<uint4 *>(mine), reinterpret_cast<int64_t *>(mine + kWarpBuf), 0};
     const size_t patches = (size_t)member * g.nqc * g.nxc * g.nflav;
@@ -115,7 +119,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ 
         const Queued e = next_queued(B, lane);
         const int64_t i = e.i;
         if (i >= 0 && e.sub == 0)
-            slow_point_pw(g, cm, pid_col(g, pid[i]), x[i], q2[i], i, out, tape, dtape, dbins, nbins);
+            slow_point_pw(g, cm, fm, pid_col(g, pid[i]), x[i], q2[i], i, out, tape, dtape, dbins, nbins);
         __syncwarp();
     };
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -139,21 +143,25 @@ __global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ 
             fast &= col < 0 || !fix_none(last);
             if (fast) {
                 out[i] = col >= 0 ? fix_value(s, last) : 0.0;
-                if (TAPE) {
+                if (TAPE) tape_put(tape, i, X, Q);
+            }
+            if (DT) {
+                int64_t dx, dq;
+                quad_patch_d(c, W, B.buf, lane, quad_pos(lane), dx, dq);
+                double dtx = col >= 0 ? fix_value(dx, last) : 0.0, dtq = col >= 0 ? fix_value(dq, last) : 0.0;
+                const bool knot = fast && col >= 0 && (fix_at_knot(X.t) || fix_at_knot(Q.t));
+                if (__any_sync(kAll, knot) && knot) {            // rare: the derivatives at a knot in FP64 (patch_d)
                     Axis AX, AQ;
-                    AX.cell = X.cell;
-                    AQ.cell = Q.cell;
                     AX.in = AQ.in = true;
                     AX.below = AQ.below = false;
                     make_basis(AX, fix_t(X.t), g.extrap);
                     make_basis(AQ, fix_t(Q.t), g.extrap);
-                    tape_put(tape, i, AX, AQ, false);
-                    if (DT) {
-                        double dtx = 0.0, dtq = 0.0;
-                        if (col >= 0) patch_vd(cm + (size_t)patch0 * 16, AX, AQ, &dtx, &dtq);
-                        reinterpret_cast<double2 *>(dtape)[i] = make_double2(dtx, dtq);
-                        dbins[i] = sorted_bin(g, AX, AQ, false, col, half_pair(AX, AQ), nbins);
-                    }
+                    patch_vd(cm + (size_t)patch0 * 16, AX, AQ, &dtx, &dtq);
+                }
+                if (fast) {
+                    reinterpret_cast<double2 *>(dtape)[i] = make_double2(dtx, dtq);
+                    const int halves = (upper_half(X.t) ? 1 : 0) | (upper_half(Q.t) ? 2 : 0);
+                    dbins[i] = col < 0 ? -1 : checked_index(g.status, (int)patch0 * 4 + halves, nbins);   // sorted_bin's
                 }
             }
         }
@@ -199,7 +207,7 @@ __global__ void __launch_bounds__(kBlock) k_alphas(const __grid_constant__ GridD
         __syncthreads();
     }
     const CoordTabs T = STAGE ? CoordTabs{invs, logs, nullptr, keys, nullptr, guide, nullptr, cells} : grid_tabs(g);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = lane_id(), wid = threadIdx.x >> 5;
     WarpBufs B{nullptr, squeue[wid], 0};
     auto drain = [&]() {
         const Queued e = next_queued(B, lane);

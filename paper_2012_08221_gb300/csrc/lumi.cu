@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(kBlock, SAVE ? 2 : 3) k_lumi(const __grid_cons
     __shared__ double red[kBlock / 32];
     const LogTabs T = tab_bytes ? stage_log_tabs(g, smem) : grid_log_tabs(g);
     __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = lane_id(), wid = threadIdx.x >> 5;
     const int row = SAVE ? 2 * g.nflav : g.nflav;
     unsigned char *mine = smem + tab_bytes + (size_t)wid * lumi_warp_bytes(row);
     double *rows = reinterpret_cast<double *>(mine + kWarpBuf);

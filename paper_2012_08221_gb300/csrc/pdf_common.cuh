@@ -209,6 +209,7 @@ struct Axis {
     double h;             // Horner factor: t inside, 1 outside
     bool in;              // inside the knot range
     bool below;           // below the first knot
+    int64_t f;            // fixed-point t (value 2^62), or -1 where FP64 serves
 };
 
 // Basis of the patch polynomial along one axis.  Inside the knot range
@@ -305,6 +306,7 @@ __device__ __forceinline__ Axis axis_x(const GridDev &g, double x)
     A.in = (b >= g.xlo) & (b <= g.xhi);
     A.below = b < g.xlo;
     double t;
+    A.f = f.ok ? f.t : -1;
     if (f.ok) {
         t = fix_t(f.t);
     } else {
@@ -324,6 +326,7 @@ __device__ __forceinline__ Axis axis_q2(const GridDev &g, double q2)
     A.in = (b >= g.qlo) & (b <= g.qhi);
     A.below = b < g.qlo;
     double t;
+    A.f = f.ok ? f.t : -1;
     if (f.ok) {
         t = fix_t(f.t);
     } else {
@@ -340,6 +343,7 @@ __device__ __forceinline__ Axis axis_u(const GridDev &g, double u)
     int64_t k = dkey(u);
     Axis A;
     A.cell = checked_index(g.status, find_cell<int64_t>(g.ukey, g.nxc, g.xstep, k), g.nxc);
+    A.f = -1;
     A.in = (k >= g.ulo) & (k <= g.uhi);
     A.below = k < g.ulo;
     double2 c = g.xcell[A.cell];
@@ -352,6 +356,7 @@ __device__ __forceinline__ Axis axis_w(const GridDev &g, double w)
     int64_t k = dkey(w);
     Axis A;
     A.cell = checked_index(g.status, find_cell<int64_t>(g.wkey, g.nqc, g.qstep, k), g.nqc);
+    A.f = -1;
     A.in = (k >= g.wlo) & (k <= g.whi);
     A.below = k < g.wlo;
     double2 c = g.qcell[A.cell];
@@ -466,9 +471,7 @@ __device__ __forceinline__ VD horner_vd(const Axis &A, double c0, double c1, dou
 // coefficient rows: each row's value i_n and t_x-derivative j_n, then the
 // value and the t_q-derivative from the i_n and the t_x-derivative by
 // Horner's rule over the j_n.  The value is patch()'s, bit for bit; the
-// two derivatives cost 13 FMAs beyond it (28 in all).  Every adjoint takes
-// its patch derivatives from here, so that derivatives kept by a forward
-// pass and derivatives recomputed later are the same bits.
+// two derivatives cost 13 FMAs beyond it (28 in all).
 __device__ __forceinline__ double patch_vd_rows(const D4 r[4], const Axis &X, const Axis &Q, double *dtx,
                                                 double *dtq)
 {
@@ -486,6 +489,40 @@ __device__ __forceinline__ double patch_vd(const double *__restrict__ C, const A
 {
     const D4 r[4] = {ld4(C), ld4(C + 4), ld4(C + 8), ld4(C + 12)};
     return patch_vd_rows(r, X, Q, dtx, dtq);
+}
+
+// Derivatives of a patch in t_x and t_q: from its fixed-point form F (null:
+// none) where the point has fixed-point coordinates away from the knots, else
+// in FP64 from its coefficients C.  Every adjoint and the derivative tape take
+// them by this rule, and integer sums do not depend on how a warp splits
+// them, so derivatives kept and derivatives recomputed are the same bits.
+__device__ __forceinline__ bool fixed_derivative(const Axis &X, const Axis &Q)
+{
+    return X.f >= 0 && Q.f >= 0 && !fix_at_knot(X.f) && !fix_at_knot(Q.f);
+}
+__device__ __forceinline__ void patch_d(const double *__restrict__ C, const unsigned char *__restrict__ F, const Axis &X,
+                                        const Axis &Q, double *dtx, double *dtq)
+{
+    if (F && fixed_derivative(X, Q)) {
+        Dig w[16];
+        fix_weights(X.f - kFixHalf, Q.f - kFixHalf, w);
+        int64_t dx = 0, dq = 0;
+        int last = 0;
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            int c[8];
+            fix_ld(F + 32 * n, c);
+            dx += fix_row_dx(c, w + 4 * n);
+            if (n) dq += n * fix_row(c, w + 4 * (n - 1));
+            last = c[6];
+        }
+        if (!fix_none(last)) {
+            *dtx = fix_value(dx, last);
+            *dtq = fix_value(dq, last);
+            return;
+        }
+    }
+    patch_vd(C, X, Q, dtx, dtq);
 }
 
 // Stencil weights of one axis (i <-> knot cell-1+i): W_i = sum_m M[m][i] t^m
@@ -567,11 +604,12 @@ __device__ __forceinline__ bool out_of_range(const GridDev &g, const Axis &X, co
 // Adjoint tape: 32 bytes per point that a forward pass keeps for the adjoint
 // of the same points, so that the adjoint skips the domain checks, both knot
 // searches and both logarithms.  Layout (four doubles, 32-byte aligned):
-//   [0] t of the x axis, [1] t of the Q axis (after make_basis),
+//   [0] t of the x axis, [1] t of the Q axis (after make_basis; as fixed-point
+//       integers with bit 128),
 //   [2] bits: x cell (low 32) and Q cell (high 32),
 //   [3] bits: 1 x inside, 2 x below, 4 Q inside, 8 Q below, 16 bad point
 //       (domain error, or outside the grid under the error option), 32 t of
-//       the x axis above 1/2, 64 t of the Q axis above 1/2.
+//       the x axis above 1/2, 64 t of the Q axis above 1/2, 128 fixed-point t.
 // It depends on the points, the knots and the extrapolation option only (not
 // on the member or the values), so it stays valid across pdf_bind_values.
 constexpr unsigned kTapeBad = 16u;
@@ -580,15 +618,33 @@ constexpr unsigned kTapeBad = 16u;
 // its bit pattern (which keeps the FP64 pipe free).
 __device__ __forceinline__ bool upper_half(double t) { return dbits(t) > 0x3FE0000000000000ull; }
 
+// The same of a fixed-point t, as its double would say (which rounds 2^61 +
+// 2^8 down to 1/2).
+__device__ __forceinline__ bool upper_half(int64_t t) { return t > kFixHalf + 256; }
+
+__device__ __forceinline__ void tape_words(double *__restrict__ tape, int64_t i, uint64_t tx, uint64_t tq, int xcell,
+                                           int qcell, unsigned f)
+{
+    ulonglong2 *d = reinterpret_cast<ulonglong2 *>(tape + 4 * i);
+    d[0] = make_ulonglong2(tx, tq);
+    d[1] = make_ulonglong2((uint64_t)(uint32_t)xcell | ((uint64_t)(uint32_t)qcell << 32), (uint64_t)f);
+}
+
+// A point inside the knots with fixed-point coordinates.
+__device__ __forceinline__ void tape_put(double *__restrict__ tape, int64_t i, const FixAxis &X, const FixAxis &Q)
+{
+    tape_words(tape, i, (uint64_t)X.t, (uint64_t)Q.t, X.cell, Q.cell,
+               1u | 4u | 128u | (upper_half(X.t) ? 32u : 0u) | (upper_half(Q.t) ? 64u : 0u));
+}
+
 __device__ __forceinline__ void tape_put(double *__restrict__ tape, int64_t i, const Axis &X, const Axis &Q,
                                          bool bad)
 {
+    const bool fixed = X.f >= 0 && Q.f >= 0;
     const unsigned f = (X.in ? 1u : 0u) | (X.below ? 2u : 0u) | (Q.in ? 4u : 0u) | (Q.below ? 8u : 0u) |
-                       (bad ? kTapeBad : 0u) | (upper_half(X.t) ? 32u : 0u) | (upper_half(Q.t) ? 64u : 0u);
-    double2 *d = reinterpret_cast<double2 *>(tape + 4 * i);
-    d[0] = make_double2(X.t, Q.t);
-    d[1] = make_double2(dfrom((uint64_t)(uint32_t)X.cell | ((uint64_t)(uint32_t)Q.cell << 32)),
-                        dfrom((uint64_t)f));
+                       (bad ? kTapeBad : 0u) | (upper_half(X.t) ? 32u : 0u) | (upper_half(Q.t) ? 64u : 0u) |
+                       (fixed ? 128u : 0u);
+    tape_words(tape, i, fixed ? (uint64_t)X.f : dbits(X.t), fixed ? (uint64_t)Q.f : dbits(Q.t), X.cell, Q.cell, f);
 }
 
 // A cell read back from a tape: range-checked (and flagged) in checked
@@ -634,9 +690,11 @@ __device__ __forceinline__ bool tape_get(const GridDev &g, const double *__restr
                                          Axis &Q)
 {
     const D4 r = ld4(tape + 4 * i);
-    const bool bad = tape_decode(g, r.z, r.w, X, Q);
-    make_basis(X, r.x, g.extrap);
-    make_basis(Q, r.y, g.extrap);
+    const bool bad = tape_decode(g, r.z, r.w, X, Q), fixed = (unsigned)dbits(r.w) & 128u;
+    X.f = fixed ? (int64_t)dbits(r.x) : -1;
+    Q.f = fixed ? (int64_t)dbits(r.y) : -1;
+    make_basis(X, fixed ? fix_t(X.f) : r.x, g.extrap);
+    make_basis(Q, fixed ? fix_t(Q.f) : r.y, g.extrap);
     return bad;
 }
 

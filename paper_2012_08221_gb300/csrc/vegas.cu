@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_vegas(const __grid_constant__ Gri
     for (int k = threadIdx.x; k < 2 * n_bins; k += blockDim.x) sbin[k] = 0.0;
     const LogTabs T = tab_bytes ? stage_log_tabs(g, smem) : grid_log_tabs(g);
     __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = lane_id(), wid = threadIdx.x >> 5;
     const int row = g.nflav;
     unsigned char *mine = smem + tab_bytes + (((size_t)2 * n_bins * 8 + 127) & ~(size_t)127) +
                           (size_t)wid * lumi_warp_bytes(row);

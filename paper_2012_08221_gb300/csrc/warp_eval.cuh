@@ -29,6 +29,15 @@ constexpr int kWarpBuf = 4096;            // bytes of the weights buffer of one 
 constexpr int kQueue = 64;                // slots of a warp's queue
 constexpr unsigned kAll = 0xffffffffu;
 
+// This thread's lane, as a value that the compiler keeps instead of reading the
+// thread index again in every loop.
+__device__ __forceinline__ int lane_id()
+{
+    int lane = threadIdx.x & 31;
+    asm volatile("" : "+r"(lane));
+    return lane;
+}
+
 __device__ __forceinline__ double dnan() { return __longlong_as_double(0x7FF8000000000000ll); }
 
 // Bytes of a block's copies of the coordinate tables (0: they stay global).
@@ -124,16 +133,48 @@ __device__ __forceinline__ void quad_load(const unsigned char *base, const uint3
     for (int j = 0; j < 4; ++j) fix_ld(base + off[j], c[j]);
 }
 
-// The fixed-point value of this lane's own point, and in `last` the low word
-// of its patch's last coefficient (the block exponent).
-__device__ __forceinline__ int64_t quad_patch(const int c[4][8], const Dig W[4][4], QuadPos r, int &last)
+// The low word of the last coefficient of this lane's own patch (the block
+// exponent; every row has it).
+__device__ __forceinline__ int quad_last(const int c[4][8], QuadPos r)
 {
     const int lo = r.odd ? c[1][6] : c[0][6], hi = r.odd ? c[3][6] : c[2][6];
-    last = r.up ? hi : lo;
+    return r.up ? hi : lo;
+}
+
+// The fixed-point value of this lane's own point, and in `last` quad_last.
+__device__ __forceinline__ int64_t quad_patch(const int c[4][8], const Dig W[4][4], QuadPos r, int &last)
+{
+    last = quad_last(c, r);
     int64_t s[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) s[j] = fix_row(c[j], W[j]);
     return quad_sum(s, r);
+}
+
+// The two derivatives of the same patch.  A row's derivative in t_q takes the
+// weights of the row before it, which are read again from the buffer that
+// quad_weights left.
+__device__ __forceinline__ void quad_patch_d(const int c[4][8], const Dig W[4][4], const uint4 *buf, int lane,
+                                             QuadPos pos, int64_t &dx, int64_t &dq)
+{
+    const int r = lane & 3, prev = max(r - 1, 0);
+    int64_t sx[4], sq[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        sx[j] = fix_row_dx(c[j], W[j]);
+        const int p = (lane & ~3) | j, sp = weight_swizzle(p);
+        Dig V[4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint4 v = buf[8 * p + ((2 * prev + h) ^ sp)];
+            V[2 * h] = {(int)v.x, (int)v.y};
+            V[2 * h + 1] = {(int)v.z, (int)v.w};
+        }
+        const int64_t t = fix_row(c[j], V);
+        sq[j] = (pos.odd ? t : 0) + (pos.up ? 2 * t : 0);        // r t
+    }
+    dx = quad_sum(sx, pos);
+    dq = quad_sum(sq, pos);
 }
 
 // Byte offsets of this lane's rows of the quad's points, from each lane's own
@@ -302,16 +343,7 @@ __device__ __forceinline__ void eval_points(const GridDev &g, const CoordTabs &T
     const bool fast = live && X.ok && Q.ok && Y.fm;      // inside the knots, so inside the domain
     push_queue(B, live && !fast, i, lane);
     if (__any_sync(kAll, fast)) {
-        if (TAPE && fast) {
-            Axis AX, AQ;
-            AX.cell = X.cell;
-            AQ.cell = Q.cell;
-            AX.in = AQ.in = true;
-            AX.below = AQ.below = false;
-            AX.t = fix_t(X.t);
-            AQ.t = fix_t(Q.t);
-            tape_put(Y.tape, i, AX, AQ, false);
-        }
+        if (TAPE && fast) tape_put(Y.tape, i, X, Q);
         bool none = false;                    // a patch or cubic that the format does not hold
         if (AS && fast) Y.alphas[i] = fix_alphas(g, Q, none);
         const uint32_t cell = fast ? (uint32_t)(Q.cell * g.nxc + X.cell) : 0u;

@@ -120,3 +120,44 @@ def test_luminosity_with_flavours_that_set_in_at_a_threshold(n):
     _, _, s = vg.iteration(torch.as_tensor(v, device="cuda"), refine=False)
     ref = vegas_sums(o, 1, np.log(1e-6), 2 * np.log(13000.0), np.tile(np.linspace(0, 1, 21), (2, 1)), v)
     assert np.all(np.abs(s - ref) <= 1e-11 * np.abs(ref) + 1e-300)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 2000, 30_001])
+def test_derivatives_of_the_matrix_and_the_pointwise_form(n):
+    """dL/dx and dL/dQ^2 of one column through the matrix form (quads of lanes)
+    and the pointwise form with the derivative tape, with the tape and
+    without: the same bits, with points on knots, outside the grid and in
+    patches that keep FP64; against the oracle's derivative."""
+    from paper_2012_08221_gb300.pdf import PDF
+    g = synth.grid_nnpdf(seeds=(87, 88))
+    g.values[:, np.asarray(g.q_knots) <= 4.92, :, 11] = 0.0
+    pdf, o = PDF.from_grid(g), OracleGrid.from_synth(g)
+    x, q2, _ = synth.queries_nnpdf(n, seed=89)
+    x[::7], q2[3::7] = g.x_knots[np.arange(x[::7].size) % 190], 4.92 ** 2
+    x[5::11], q2[6::11] = 3e-11, 1e12
+    X, Q = torch.as_tensor(x, device="cuda"), torch.as_tensor(q2, device="cuda")
+    w = torch.as_tensor(np.random.default_rng(90).standard_normal(n), device="cuda")
+    for pid in (5, -2):
+        col = np.array([pid], np.int32)
+        pids = torch.full((n,), pid, dtype=torch.int32, device="cuda")
+        gv = torch.zeros(g.values.shape[1:], dtype=torch.float64, device="cuda")
+        T, D, TM = pdf.new_tape(n), pdf.new_dtape(n), pdf.new_tape(n)
+        pdf.xfxQ2_pw(pids, X, Q, member=1, tape=T, dtape=D)
+        pdf.xfxQ2(col, X, Q, member=1, tape=TM)
+        a = pdf.xfxQ2_backward(pids, X, Q, w, member=1, pointwise=True, grad_values=gv, tape=T, dtape=D)[:2]
+        others = [pdf.xfxQ2_backward(pids, X, Q, w, member=1, pointwise=True, grad_values=gv, tape=T)[:2],
+                  pdf.xfxQ2_backward(pids, X, Q, w, member=1, pointwise=True)[:2],
+                  pdf.xfxQ2_backward(col, X, Q, w[:, None], member=1, grad_values=gv, tape=TM)[:2],
+                  pdf.xfxQ2_backward(col, X, Q, w[:, None], member=1, grad_values=gv)[:2]]
+        for b in others:
+            assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+        pn = np.full(n, pid, np.int32)
+        rdx, rdq = o.grad_pw(pn, x, q2, member=1)
+        kap = o.kappa(pn, x, q2, member=1, pointwise=True)
+        U, W = np.log(g.x_knots), np.log(g.q_knots ** 2)
+        dW = np.diff(W)
+        wn = w.cpu().numpy()
+        # the suite's gradient rule: 1e-9 of the value's terms over the smallest knot spacing
+        for got, ref, s in ((a[0], rdx, np.min(np.diff(U)) * x), (a[1], rdq, np.min(dW[dW > 0]) * q2)):
+            err = np.abs(got.cpu().numpy() - wn * ref)
+            assert np.all(err <= 1e-9 * np.maximum(np.abs(wn * ref), np.abs(wn) * 4 * kap / s) + 1e-300)
