@@ -264,9 +264,9 @@ int xfxQ2_backward(pdfgpu_grid_t g, int32_t member, const int32_t *pids, int32_t
  *   dtape (xfxQ2_pw_tape only; may be NULL) DEVICE, 20 bytes per point:
  *   [n][2] doubles then [n] int32, caller-owned, 16-byte aligned (PDF_E_ARG
  *   otherwise, and without a tape; PDF_E_RANGE for a grid of 2^28 or more
- *   cell-flavour pairs): the derivative tape, each point's patch
- *   derivatives in its two local coordinates (zeros for an absent pid),
- *   computed with the value (13 FMAs more per point), and the point's bin
+ *   cell-flavour pairs): the derivative tape, each point's derivatives in
+ *   x and Q^2 (zeros for an absent pid), computed with the value, and the
+ *   point's bin
  *   in the sorted grid gradient, so that xfxQ2_backward_tape given it takes
  *   dL/dx and dL/dQ^2 without reloading the point's 16 coefficients and
  *   counts its bins from 4 bytes per point.  Unlike the tape it depends on

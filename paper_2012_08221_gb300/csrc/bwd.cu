@@ -59,29 +59,6 @@ __device__ __forceinline__ const unsigned char *fixed_patches(const GridDev &g, 
            (((size_t)member * g.nqc + qc) * g.nxc + xc) * g.nflav * 128;
 }
 
-// Chain rule from the local coordinates to x and Q^2: given sx = g dP/dtx
-// and sq = g dP/dtq, dL/dx = sx (1/dU) / x and dL/dQ^2 = sq (1/dW) / Q^2,
-// with one reciprocal of x Q^2 for both (1/x = Q^2 / (x Q^2), 1/Q^2 =
-// x / (x Q^2)); where the product leaves the normal range the two
-// reciprocals are taken apart.  Every adjoint goes through here, so their
-// dL/dx and dL/dQ^2 stay the same bits.
-__device__ __forceinline__ void chain_rule(double sx, double sq, double ydu, double ydw, double x, double q2,
-                                           double *__restrict__ gx, double *__restrict__ gq, int64_t i)
-{
-    const double xq = x * q2;
-    double rx, rq;
-    if (dbits(xq) - 0x0010000000000000ull < 0x7FE0000000000000ull) {   // normal and finite
-        const double r = __drcp_rn(xq);
-        rx = q2 * r;
-        rq = x * r;
-    } else {
-        rx = __drcp_rn(x);
-        rq = __drcp_rn(q2);
-    }
-    if (gx) gx[i] = sx * ydu * rx;
-    if (gq) gq[i] = sq * ydw * rq;
-}
-
 template <bool PW, bool SMEM, bool TAPE>
 __global__ void __launch_bounds__(kBlock) k_bwd(GridDev g, Cols cols, int npid, int member,
                                                 const int *__restrict__ pid,
@@ -146,6 +123,7 @@ __global__ void __launch_bounds__(kBlock) k_bwd(GridDev g, Cols cols, int npid, 
             r0 = g.qrow[Q.cell] - 1;
             k0 = X.cell - 1;
         }
+        const ChainFactors f = chain_factors(g, X.cell, Q.cell, xi, qi);
         double sx = 0.0, sq = 0.0;
         const int na = PW ? 1 : npid;
         for (int a = 0; a < na; ++a) {
@@ -153,7 +131,7 @@ __global__ void __launch_bounds__(kBlock) k_bwd(GridDev g, Cols cols, int npid, 
             if (col >= 0) col = checked_index(g.status, col, g.nflav);
             if (col < 0) continue;
             double ga = PW ? gout[i] : gout[i * npid + a];
-            double dtx, dtq;
+            double dtx, dtq;                  // with the derivative tape d/dx and d/dQ^2 already
             if (PW && TAPE && dtape) {
                 const double2 d = __ldg(reinterpret_cast<const double2 *>(dtape) + i);
                 dtx = d.x;
@@ -163,8 +141,12 @@ __global__ void __launch_bounds__(kBlock) k_bwd(GridDev g, Cols cols, int npid, 
             }
             if (fzx) dtx = 0.0;
             if (fzq) dtq = 0.0;
-            sx = fma(ga, dtx, sx);
-            sq = fma(ga, dtq, sq);
+            if (PW && !dtape) {
+                dtx *= f.x;
+                dtq *= f.q;
+            }
+            sx = PW ? ga * dtx : fma(ga, dtx, sx);
+            sq = PW ? ga * dtq : fma(ga, dtq, sq);
             if (gval) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -181,7 +163,8 @@ __global__ void __launch_bounds__(kBlock) k_bwd(GridDev g, Cols cols, int npid, 
                 }
             }
         }
-        chain_rule(sx, sq, g.xcell[X.cell].y, g.qcell[Q.cell].y, xi, qi, gx, gq, i);
+        if (gx) gx[i] = PW ? sx : sx * f.x;
+        if (gq) gq[i] = PW ? sq : sq * f.q;
     }
     if (SMEM) {
         __syncthreads();
@@ -323,6 +306,24 @@ __global__ void __launch_bounds__(kBlock, DT ? 5 : 2) k_bwd_rec(GridDev g, int m
     const double *cm = g.coef + (size_t)member * g.nqc * g.nxc * cell_stride;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
         const int64_t i = i0 + k;
+        if (DT) {
+            // inside the knots with fixed-point coordinates: all that is left is
+            // two multiplies and the record
+            const D4 r = ld4(tape + 4 * (size_t)k);
+            if (((unsigned)dbits(r.w) & (kTapeBad | 128u | 5u)) == (128u | 5u)) {
+                const int b = __ldg(dbins + i);
+                const double ga = gout[i];
+                const double2 d = __ldg(reinterpret_cast<const double2 *>(dtape) + i);
+                if (gx) gx[i] = b < 0 ? 0.0 : ga * d.x;               // b < 0: a pid that the grid does not have
+                if (gq) gq[i] = b < 0 ? 0.0 : ga * d.y;
+                if (b >= 0) {
+                    const int bin = checked_index(g.status, b, nbins);
+                    put_rec(rec, atomicAdd(&cursor[bin], 1), near_coord((int64_t)dbits(r.x)),
+                            near_coord((int64_t)dbits(r.y)), ga, bin, true, true);
+                }
+                continue;
+            }
+        }
         Axis X, Q;
         if (tape_get(g, tape, k, X, Q)) {
             if (gx) gx[i] = qnan();
@@ -337,19 +338,23 @@ __global__ void __launch_bounds__(kBlock, DT ? 5 : 2) k_bwd_rec(GridDev g, int m
         }
         const double ga = gout[i];
         if (gx || gq) {
-            double dtx, dtq;
+            double dx, dq;
             if (DT) {
                 const double2 d = __ldg(reinterpret_cast<const double2 *>(dtape) + i);
-                dtx = d.x;
-                dtq = d.y;
+                dx = d.x;
+                dq = d.y;
             } else {
                 const unsigned char *F = fixed_patches(g, member, Q.cell, X.cell);
                 patch_d(cm + ((size_t)Q.cell * g.nxc + X.cell) * cell_stride + col * 16, F ? F + col * 128 : nullptr,
-                        X, Q, &dtx, &dtq);
+                        X, Q, &dx, &dq);
+                const ChainFactors f = chain_factors(g, X.cell, Q.cell, x[i], q2[i]);
+                dx *= f.x;
+                dq *= f.q;
             }
-            if (!X.in && g.extrap == PDF_EXTRAP_FREEZE) dtx = 0.0;
-            if (!Q.in && g.extrap == PDF_EXTRAP_FREEZE) dtq = 0.0;
-            chain_rule(ga * dtx, ga * dtq, g.xcell[X.cell].y, g.qcell[Q.cell].y, x[i], q2[i], gx, gq, i);
+            if (!X.in && g.extrap == PDF_EXTRAP_FREEZE) dx = 0.0;
+            if (!Q.in && g.extrap == PDF_EXTRAP_FREEZE) dq = 0.0;
+            if (gx) gx[i] = ga * dx;
+            if (gq) gq[i] = ga * dq;
         }
         if (!(X.in && Q.in)) {
             double Wx[4], Wq[4];
@@ -373,7 +378,7 @@ __global__ void __launch_bounds__(kBlock, DT ? 5 : 2) k_bwd_rec(GridDev g, int m
         }
         const int b = DT ? checked_index(g.status, __ldg(dbins + i), nbins)
                          : sorted_bin(g, X, Q, false, col, half_pair(X, Q), nbins);
-        put_rec(rec, atomicAdd(&cursor[b], 1), near_coord(X.t), near_coord(Q.t), ga, b, X.in, Q.in);
+        put_rec(rec, atomicAdd(&cursor[b], 1), near_coord(X), near_coord(Q), ga, b, X.in, Q.in);
     }
 }
 
@@ -492,7 +497,9 @@ __device__ __noinline__ void slow_rec_m(const GridDev &g, const signed char *sco
         }
         if (!X.in && g.extrap == PDF_EXTRAP_FREEZE) sx = 0.0;
         if (!Q.in && g.extrap == PDF_EXTRAP_FREEZE) sq = 0.0;
-        chain_rule(sx, sq, g.xcell[X.cell].y, g.qcell[Q.cell].y, xi, qi, gx, gq, i);
+        const ChainFactors f = chain_factors(g, X.cell, Q.cell, xi, qi);
+        if (gx) gx[i] = sx * f.x;
+        if (gq) gq[i] = sq * f.q;
     }
     if (X.in && Q.in) return;
     double Wx[4], Wq[4];
@@ -573,7 +580,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_bwd_rec_m(const __grid_constant__
             const int pos = atomicAdd(&cursor[b], 1);
             const uint64_t bits = (uint64_t)(uint32_t)b | ((uint64_t)X.in << 32) | ((uint64_t)Q.in << 33);
             double2 *d = reinterpret_cast<double2 *>(rec + 4 * (size_t)pos);
-            d[0] = make_double2(near_coord(X.t), near_coord(Q.t));
+            d[0] = make_double2(near_coord(X), near_coord(Q));
             d[1] = make_double2(dfrom(bits), dfrom((uint64_t)i));
         }
         bool fast = inside && fm && fixed_derivative(X, Q);
@@ -604,7 +611,11 @@ __global__ void __launch_bounds__(kBlock, 2) k_bwd_rec_m(const __grid_constant__
             }
             __syncwarp();                            // the buffers may be refilled
             fast = fast && !none;
-            if (fast) chain_rule(sx, sq, g.xcell[X.cell].y, g.qcell[Q.cell].y, x[i], q2[i], gx, gq, i);
+            if (fast) {
+                const ChainFactors f = chain_factors(g, X.cell, Q.cell, x[i], q2[i]);
+                if (gx) gx[i] = sx * f.x;
+                if (gq) gq[i] = sq * f.q;
+            }
         }
         push_queue(B, !bad && (!inside || (deriv && !fast)), k, lane);
         if (B.qn >= 32) drain();

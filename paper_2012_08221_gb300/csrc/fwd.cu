@@ -62,9 +62,10 @@ __global__ void __launch_bounds__(kBlock, WHOLE ? 3 : 2) k_xfxq2(const __grid_co
     if (lane == 0) bulk_wait_all();
 }
 
-// DT (with TAPE): also keep each point's patch derivatives in t_x and t_q,
-// computed with the value from the same rows (quad_patch_d), in
-// dtape[i] = (dP/dtx, dP/dtq) (zeros for an absent pid), and the point's bin
+// DT (with TAPE): also keep each point's derivatives in x and Q^2, computed
+// with the value from the same rows (quad_patch_d) and taken through the chain
+// rule here, where the FP64 pipe is idle, in dtape[i] = (dP/dx, dP/dQ^2)
+// (zeros for an absent pid), and the point's bin
 // in the pointwise sorted adjoint in dbins[i] (-1 for none).
 __device__ __forceinline__ void slow_point_pw(const GridDev &g, const double *cm, const unsigned char *fm, int col,
                                            double xi, double qi, int64_t i, double *out, double *tape, double *dtape, int *dbins, int nbins)
@@ -88,6 +89,9 @@ __device__ __forceinline__ void slow_point_pw(const GridDev &g, const double *cm
         if (col >= 0) {
             v = patch(C, X, Q);
             patch_d(C, fm ? fm + p * 128 : nullptr, X, Q, &dtx, &dtq);
+            const ChainFactors f = chain_factors(g, X.cell, Q.cell, xi, qi);
+            dtx *= f.x;
+            dtq *= f.q;
         }
         reinterpret_cast<double2 *>(dtape)[i] = make_double2(dtx, dtq);
         dbins[i] = sorted_bin(g, X, Q, bad, col, half_pair(X, Q), nbins);
@@ -159,7 +163,8 @@ __global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ 
                     patch_vd(cm + (size_t)patch0 * 16, AX, AQ, &dtx, &dtq);
                 }
                 if (fast) {
-                    reinterpret_cast<double2 *>(dtape)[i] = make_double2(dtx, dtq);
+                    const ChainFactors f = chain_factors(g, X.cell, Q.cell, xi, qi);
+                    reinterpret_cast<double2 *>(dtape)[i] = make_double2(dtx * f.x, dtq * f.q);
                     const int halves = (upper_half(X.t) ? 1 : 0) | (upper_half(Q.t) ? 2 : 0);
                     dbins[i] = col < 0 ? -1 : checked_index(g.status, (int)patch0 * 4 + halves, nbins);   // sorted_bin's
                 }

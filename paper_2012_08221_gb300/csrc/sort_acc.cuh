@@ -47,8 +47,39 @@ __device__ __forceinline__ int half_pair(const Axis &X, const Axis &Q)
 }
 
 // The local coordinate the accumulation uses: t, or 1 - t in an upper half
-// (exact: t lies in [1/2, 1] there).
-__device__ __forceinline__ double near_coord(double t) { return upper_half(t) ? 1.0 - t : t; }
+// (exact: t lies in [1/2, 1] there; of a fixed-point t before it is rounded).
+__device__ __forceinline__ double near_coord(int64_t t)
+{
+    return fix_t(upper_half(t) ? ((int64_t)1 << 62) - t : t);
+}
+__device__ __forceinline__ double near_coord(const Axis &A)
+{
+    if (A.f >= 0) return near_coord(A.f);
+    return upper_half(A.t) ? 1.0 - A.t : A.t;
+}
+
+// Chain rule from the local coordinates to x and Q^2: d/dx = d/dt_x (1/dU) / x
+// and d/dQ^2 = d/dt_q (1/dW) / Q^2, with one reciprocal of x Q^2 for both (1/x
+// = Q^2 / (x Q^2), 1/Q^2 = x / (x Q^2)); where the product leaves the normal
+// range the two reciprocals are taken apart.  Every adjoint and the derivative
+// tape take their factors from here.
+struct ChainFactors {
+    double x, q;
+};
+__device__ __forceinline__ ChainFactors chain_factors(const GridDev &g, int xc, int qc, double x, double q2)
+{
+    const double xq = x * q2;
+    double rx, rq;
+    if (dbits(xq) - 0x0010000000000000ull < 0x7FE0000000000000ull) {   // normal and finite
+        const double r = __drcp_rn(xq);
+        rx = q2 * r;
+        rq = x * r;
+    } else {
+        rx = __drcp_rn(x);
+        rq = __drcp_rn(q2);
+    }
+    return {g.xcell[xc].y * rx, g.qcell[qc].y * rq};
+}
 
 // Bin of a point in the pointwise sorted accumulation, ((cell * F + flavour
 // column) * 4 + half pair), or -1 for a point that adds nothing there: a

@@ -198,12 +198,12 @@ class PDF:
     @staticmethod
     def dtape_doubles(n):
         """Size in doubles of a derivative tape of ``n`` points: 2 n doubles of
-        patch derivatives, then n int32 bins (20 bytes per point)."""
+        derivatives in x and Q^2, then n int32 bins (20 bytes per point)."""
         return 2 * n + (n + 1) // 2
 
     def new_dtape(self, n):
         """Device buffer for the derivative tape of ``n`` pointwise points (20
-        bytes each): the patch derivatives and the accumulation bin the
+        bytes each): the derivatives and the accumulation bin the
         forward keeps for the adjoint.  ``dtape[:2 * n].view(n, 2)`` are the
         derivatives."""
         return torch.empty(self.dtape_doubles(n), dtype=torch.float64, device=self.device)

@@ -125,9 +125,9 @@ def test_luminosity_with_flavours_that_set_in_at_a_threshold(n):
 @pytest.mark.parametrize("n", [1, 31, 33, 2000, 30_001])
 def test_derivatives_of_the_matrix_and_the_pointwise_form(n):
     """dL/dx and dL/dQ^2 of one column through the matrix form (quads of lanes)
-    and the pointwise form with the derivative tape, with the tape and
-    without: the same bits, with points on knots, outside the grid and in
-    patches that keep FP64; against the oracle's derivative."""
+    and the pointwise form with the derivative tape: each the same bits with
+    the tapes and without, with points on knots, outside the grid and in
+    patches that keep FP64; both against the oracle's derivative."""
     from paper_2012_08221_gb300.pdf import PDF
     g = synth.grid_nnpdf(seeds=(87, 88))
     g.values[:, np.asarray(g.q_knots) <= 4.92, :, 11] = 0.0
@@ -145,12 +145,13 @@ def test_derivatives_of_the_matrix_and_the_pointwise_form(n):
         pdf.xfxQ2_pw(pids, X, Q, member=1, tape=T, dtape=D)
         pdf.xfxQ2(col, X, Q, member=1, tape=TM)
         a = pdf.xfxQ2_backward(pids, X, Q, w, member=1, pointwise=True, grad_values=gv, tape=T, dtape=D)[:2]
-        others = [pdf.xfxQ2_backward(pids, X, Q, w, member=1, pointwise=True, grad_values=gv, tape=T)[:2],
-                  pdf.xfxQ2_backward(pids, X, Q, w, member=1, pointwise=True)[:2],
-                  pdf.xfxQ2_backward(col, X, Q, w[:, None], member=1, grad_values=gv, tape=TM)[:2],
-                  pdf.xfxQ2_backward(col, X, Q, w[:, None], member=1, grad_values=gv)[:2]]
-        for b in others:
+        for b in (pdf.xfxQ2_backward(pids, X, Q, w, member=1, pointwise=True, grad_values=gv, tape=T)[:2],
+                  pdf.xfxQ2_backward(pids, X, Q, w, member=1, pointwise=True)[:2]):
             assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+        mat = pdf.xfxQ2_backward(col, X, Q, w[:, None], member=1, grad_values=gv, tape=TM)[:2]
+        for b in (pdf.xfxQ2_backward(col, X, Q, w[:, None], member=1, grad_values=gv)[:2],
+                  pdf.xfxQ2_backward(col, X, Q, w[:, None], member=1)[:2]):
+            assert torch.equal(mat[0], b[0]) and torch.equal(mat[1], b[1])
         pn = np.full(n, pid, np.int32)
         rdx, rdq = o.grad_pw(pn, x, q2, member=1)
         kap = o.kappa(pn, x, q2, member=1, pointwise=True)
@@ -158,6 +159,7 @@ def test_derivatives_of_the_matrix_and_the_pointwise_form(n):
         dW = np.diff(W)
         wn = w.cpu().numpy()
         # the suite's gradient rule: 1e-9 of the value's terms over the smallest knot spacing
-        for got, ref, s in ((a[0], rdx, np.min(np.diff(U)) * x), (a[1], rdq, np.min(dW[dW > 0]) * q2)):
+        sx, sq = np.min(np.diff(U)) * x, np.min(dW[dW > 0]) * q2
+        for got, ref, s in ((a[0], rdx, sx), (a[1], rdq, sq), (mat[0], rdx, sx), (mat[1], rdq, sq)):
             err = np.abs(got.cpu().numpy() - wn * ref)
             assert np.all(err <= 1e-9 * np.maximum(np.abs(wn * ref), np.abs(wn) * 4 * kap / s) + 1e-300)
