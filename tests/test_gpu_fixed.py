@@ -163,3 +163,27 @@ def test_derivatives_of_the_matrix_and_the_pointwise_form(n):
         for got, ref, s in ((a[0], rdx, sx), (a[1], rdq, sq), (mat[0], rdx, sx), (mat[1], rdq, sq)):
             err = np.abs(got.cpu().numpy() - wn * ref)
             assert np.all(err <= 1e-9 * np.maximum(np.abs(wn * ref), np.abs(wn) * 4 * kap / s) + 1e-300)
+
+
+@pytest.mark.parametrize("power", [0, 1, 9, 10, 11, 12, 60])
+def test_continuation_between_values_of_any_ratio(power):
+    """The power law from edge values whose ratio stays inside the logarithm's
+    format, at its limit (2^10) and beyond.  Two Q knots, the upper row 2^power
+    times the lower: the edge values come out of the patch to full precision
+    (with more rows the patch's own sums lose the smaller one)."""
+    from paper_2012_08221_gb300.pdf import PDF
+    x = np.array([1e-4, 1e-3, 1e-2, 0.1, 0.4])
+    q, nq = synth.subgrid_knots([2.0, 60.0], [2])
+    rng = np.random.default_rng(91 + power)
+    v = rng.uniform(1.0, 1.9, (1, 2, 5, 2))
+    v[:, 1] *= 2.0 ** power
+    a = np.array([0.3, 0.3 * 2.0 ** power])
+    g = synth.Grid(x, nq, q, np.array([1, 2], np.int32), v, a, "ratio")
+    pdf, o = PDF.from_grid(g, extrap="continuation"), OracleGrid.from_synth(g, extrap=3)
+    n = 4003
+    xs = np.minimum(np.exp(rng.uniform(np.log(3e-5), 0.0, n)), 1.0)
+    q2 = np.exp(rng.uniform(2 * np.log(1.2), 2 * np.log(100.0), n))
+    X, Q = torch.as_tensor(xs, device="cuda"), torch.as_tensor(q2, device="cuda")
+    parity.check(pdf.xfxQ2(g.pids, X, Q).cpu().numpy(), o.xfxq2_batch(g.pids, xs, q2), o.kappa(g.pids, xs, q2),
+                 what=f"ratio 2^{power}")
+    parity.check(pdf.alphasQ2(Q).cpu().numpy(), o.alphas_batch(q2), o.alphas_kappa(q2), what="alpha_s")
