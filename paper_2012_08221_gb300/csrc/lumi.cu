@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kAccWarps * 32) k_lumi_accum(GridDev g, Cols a
     __shared__ double sW[kAccWarps][32][17];
     __shared__ double sP[kAccWarps][32][kF + 1];
     __shared__ int sK[kAccWarps][32];
-    __shared__ double sG[kAccWarps][32];                      // map-back slots, 16 per half
+    __shared__ double sG[kAccWarps][2][16 * kMapCols];        // map-back slots of each half
     __shared__ signed char santi[PDF_MAX_PIDS];
     if (threadIdx.x == 0) {
 #pragma unroll
@@ -368,14 +368,18 @@ __global__ void __launch_bounds__(kAccWarps * 32) k_lumi_accum(GridDev g, Cols a
         if (ok) row = checked_index(g.status, row, g.nrows);
         const double *Mq = ((kind & 2) ? g.mqs : g.mq) + (size_t)qc * 16;
         const double *Mx = ((kind & 1) ? g.mxs : g.mx) + (size_t)xc * 16;
-#pragma unroll
-        for (int b = 0; b < kF; ++b) {
-            if (kF == kMaxLumiFlav && b >= F) break;       // the same for the whole warp
-            double v = acc[b];
-            if (kind < 4) v = map_back(v, &sG[wid][row0], Mq, Mx, j, i, hmask);   // the same for the half
+        auto emit = [&](int b, double v) {
             if (ok && santi[b] >= 0 && (dbits(v) << 1))
                 atomicAdd(gval + ((size_t)row * g.nx + col) * F + b, scale * v);
-            acc[b] = 0.0;
+        };
+        if (kind < 4) {                                    // the same for the half
+            map_back_all(acc, F, sG[wid][h], Mq, Mx, j, i, hmask, emit);
+        } else {
+#pragma unroll
+            for (int b = 0; b < kF; ++b) {
+                if (kF < kMaxLumiFlav || b < F) emit(b, acc[b]);
+                acc[b] = 0.0;
+            }
         }
     };
     const int steps = (half + 15) / 16;

@@ -34,6 +34,58 @@ __device__ __forceinline__ double map_back(double g, double *buf, const double *
     return dv;
 }
 
+// The same for a list of accumulators, kMapCols at a time: the matrices' entries
+// are loaded once, and the columns' chains run side by side (one after the
+// other, a flush of 13 columns cost 13 round trips through shared memory and
+// 104 loads while the other half-warp waited).  buf: kMapCols x 16 slots of
+// the half-warp; emit(a, value) gets column a's stencil value of this lane.
+constexpr int kMapCols = 4;
+
+template <int N, typename Emit>
+__device__ __forceinline__ void map_back_all(double (&acc)[N], int n, double *buf, const double *__restrict__ Mq,
+                                             const double *__restrict__ Mx, int sn, int sm, unsigned hmask, Emit emit)
+{
+    double q[4], x[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        q[k] = Mq[4 * k + sn];
+        x[k] = Mx[4 * k + sm];
+    }
+#pragma unroll
+    for (int a0 = 0; a0 < N; a0 += kMapCols) {
+        if (a0 < n) {
+            double t[kMapCols];
+#pragma unroll
+            for (int a = 0; a < kMapCols; ++a)
+                if (a0 + a < N) buf[16 * a + 4 * sn + sm] = acc[a0 + a];
+            __syncwarp(hmask);
+#pragma unroll
+            for (int a = 0; a < kMapCols; ++a) {
+                t[a] = 0.0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (a0 + a < N) t[a] = fma(q[k], buf[16 * a + 4 * k + sm], t[a]);
+            }
+            __syncwarp(hmask);
+#pragma unroll
+            for (int a = 0; a < kMapCols; ++a)
+                if (a0 + a < N) buf[16 * a + 4 * sn + sm] = t[a];
+            __syncwarp(hmask);
+#pragma unroll
+            for (int a = 0; a < kMapCols; ++a)
+                if (a0 + a < N && a0 + a < n) {
+                    double dv = 0.0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) dv = fma(buf[16 * a + 4 * sn + k], x[k], dv);
+                    emit(a0 + a, dv);
+                }
+            __syncwarp(hmask);
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < N; ++a) acc[a] = 0.0;
+}
+
 // Half of a cell a point lies in along each axis: bit 0 set when t_x > 1/2,
 // bit 1 when t_q > 1/2.  In an upper half the accumulation runs in powers of
 // s = 1 - t (and maps back with the cell's matrix in s), so that the weights
