@@ -101,8 +101,12 @@ __device__ __forceinline__ void slow_point_pw(const GridDev &g, const double *cm
     out[i] = bad ? dnan() : v;
 }
 
+// (five blocks of 128 threads per SM: 1351 us per pointwise fit step, two of
+// 256 1364, six of 128 with spills 1385)
+constexpr int kPwBlock = 128;
+
 template <bool TAPE, bool DT, bool STAGE>
-__global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ GridDev g, int member,
+__global__ void __launch_bounds__(kPwBlock, 5) k_xfxq2_pw(const __grid_constant__ GridDev g, int member,
                                                         const int *__restrict__ pid,
                                                         const double *__restrict__ x,
                                                         const double *__restrict__ q2,
@@ -176,7 +180,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_xfxq2_pw(const __grid_constant__ 
     if (B.qn) drain();
 }
 
-// alpha_s, one point per lane (fix_alphas): 1e7 points 286 -> 94 us (FP64
+// alpha_s, one point per lane (fix_alphas): 1e7 points 286 -> 93 us (FP64
 // pipe 82 % busy before; now integer issue of the logarithm and the table
 // look-ups in shared memory); points outside the Q range or the
 // domain are queued per warp and evaluated 32 at a time.
@@ -318,7 +322,7 @@ int check_tape(const pdfgpu_grid *g, const double *tape)
 // 32 points.  A short one splits the columns into groups until there are
 // about kShortWarps warps per SM: below that the SMs wait for one warp's
 // chain of loads, and the coordinates computed once per group are cheaper
-// than idle SMs (1e5 points x 11 flavours with alpha_s: 35 us; 43 us in FP64).
+// than idle SMs (1e5 points x 11 flavours with alpha_s: 22 us; 43 us in FP64).
 constexpr int kShortWarps = 16;
 // Points per SM from which copying the coordinate tables into shared memory
 // pays (the copy is about 20 KB per block).
@@ -442,12 +446,12 @@ int launch_pw(pdfgpu_grid *g, int32_t member, const int32_t *pid, const double *
     auto k = dtape  ? (stage ? k_xfxq2_pw<true, true, true> : k_xfxq2_pw<true, true, false>)
              : tape ? (stage ? k_xfxq2_pw<true, false, true> : k_xfxq2_pw<true, false, false>)
                     : (stage ? k_xfxq2_pw<false, false, true> : k_xfxq2_pw<false, false, false>);
-    const size_t smem = (size_t)tab + (kBlock / 32) * (kWarpBuf + kQueue * 8);
+    const size_t smem = (size_t)tab + (kPwBlock / 32) * (kWarpBuf + kQueue * 8);
     rc = allow_dynamic_smem((const void *)k, smem);
     if (rc) return rc;
-    int grid = wave_grid(g, (const void *)k, kBlock, smem, n);
+    int grid = wave_grid(g, (const void *)k, kPwBlock, smem, n);
     int *dbins = dtape ? reinterpret_cast<int *>(dtape + 2 * n) : nullptr;
-    k<<<grid, kBlock, smem, s>>>(g->d, member, pid, x, q2, n, out, tape, dtape, dbins,
+    k<<<grid, kPwBlock, smem, s>>>(g->d, member, pid, x, q2, n, out, tape, dtape, dbins,
                                  (int)std::min<int64_t>(nbins64, (int64_t)1 << 30), tab);
     PDF_CUDA(cudaGetLastError());
     return PDF_OK;
