@@ -335,6 +335,7 @@ def peaks():
 # FP64 FMA issue rate per SM per clock on GB300: ncu reports a peak of 304
 # DFMA thread-instructions per cycle for 152 SMs.
 DFMA_PER_SM_CLK = 2
+IMAD_WIDE_PER_SM_CLK = 32        # distinct operands, measured
 
 
 def fp64_derived_peak(sm_count):
@@ -449,17 +450,25 @@ def main():
     bytes_launch = npts * work.xfxq2_point_bytes(g.n_flav)
     achieved = flops_launch / (k_ms * 1e-3)
     traffic = measured_traffic("k_xfxq2", npts)
-    roofline = {"bound": "alu", "pipe": "fp64", "kernel": "k_xfxq2",
-                "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
-                "frac": achieved / peak,
+    products = npts * work.xfxq2_point_products(g.n_flav) / (k_ms * 1e-3)
+    peak_products = sms * IMAD_WIDE_PER_SM_CLK * peak_mhz * 1e6
+    roofline = {"bound": "alu", "pipe": "integer multiply (32 x 32 -> 64)", "kernel": "k_xfxq2",
+                "achieved": products / 1e12, "peak": peak_products / 1e12, "unit": "Tproduct/s",
+                "frac": products / peak_products,
+                "products_per_point": work.xfxq2_point_products(g.n_flav),
+                "fp64_achieved_tflops": achieved / 1e12, "fp64_peak_tflops": peak / 1e12,
+                "fp64_frac": achieved / peak,
                 "flops_per_point": work.xfxq2_point_flops(g.n_flav),
                 "frac_matrix_form": flops_matrix / (k_ms * 1e-3) / peak,
                 "flops_per_point_matrix_form": work.xfxq2_point_flops_matrix_form(g.n_flav),
-                "frac_note": "frac counts the flops of the patch form the kernel runs (15 FMA per flavour, "
-                             "table log); frac_matrix_form counts 40 F + 50 flops per point, the separable-"
-                             "weight form (20 FMA per flavour + weights), which does more arithmetic than the "
-                             "kernel and so can exceed 1; the headroom left is 100 - ncu_fp64_pipe_active_pct",
-                "peak_source": f"derived: {sms} SMs x {DFMA_PER_SM_CLK} DFMA/clk x 2 flop x {peak_mhz:.0f} MHz "
+                "frac_note": "the kernel evaluates the patches in 64-bit fixed point on the integer pipes: frac "
+                             "counts the 48 digit products per flavour against the wide multiply's rate (the "
+                             "kernel is bound by instruction issue, of which they are the largest part); "
+                             "fp64_frac counts the method's FP64 flops (15 FMA per flavour, table log) against "
+                             "the FP64 pipe it no longer uses, and frac_matrix_form 40 F + 50 flops per point, "
+                             "the separable-weight form: both exceed 1",
+                "peak_source": f"derived: {sms} SMs x {IMAD_WIDE_PER_SM_CLK} products/clk x {peak_mhz:.0f} MHz; "
+                               f"FP64: {sms} SMs x {DFMA_PER_SM_CLK} DFMA/clk x 2 flop x {peak_mhz:.0f} MHz "
                                f"(max SM clock)",
                 "probe": {"value": probe / 1e12, "unit": "TFLOP/s",
                           "what": "FP64 FMA chains measured in this run (pdf_probe_fp64_peak)"},
@@ -584,7 +593,7 @@ def main():
             "two_calls": {"ms_per_step": ms1_two, "what": "xfxQ2 then alphasQ2 on the same arrays"},
             "fp64_frac": n1 * (work.xfxq2_point_flops(g1.n_flav) + 6) / (ms1 * 1e-3) / peak,
             "l2": "flushed (256 MB write) before every timed step; the step's data fit in L2",
-            "note": "1e5 points occupy about half of one wave of resident threads (152 SMs x 1280): "
+            "note": "1e5 points are less than one wave of resident warps: "
                     "the time is mostly one thread's latency (11 patches after coefficient loads that "
                     "miss the flushed L2)"}
         del flush, graph1
@@ -600,7 +609,7 @@ def main():
         GV = torch.zeros(gs.values.shape[1:], dtype=torch.float64, device=dev)
 
         T3 = p3.new_tape(x3.size)            # the forward's adjoint tape (32 B per point)
-        D3 = p3.new_dtape(x3.size)           # its patch derivatives and bins (20 B per point)
+        D3 = p3.new_dtape(x3.size)           # its derivatives and bins (20 B per point)
 
         def step3():
             p3.bind_values(V3)
@@ -665,7 +674,7 @@ def main():
                            "frac_separable_count": n3 * work.pw_bwd_point_flops_separable() / (kb * 1e-3) / peak},
             "tape": "the forward pass writes 32 bytes per point (cells, local coordinates, flags) that the "
                     "adjoint reads instead of searching the knots and taking logarithms again, and 20 bytes "
-                    "of patch derivatives (computed with the value) and the point's bin, which spare the "
+                    "of derivatives (computed with the value) and the point's bin, which spare the "
                     "adjoint the coefficients and let it count its bins from 4 bytes per point",
             "direct_calls": {"ms_per_step": ms3, "value": world * n3 / (ms3 * 1e-3),
                              "what": "the same two library calls without autograd (no torch "

@@ -8,7 +8,7 @@ into dL/dvalues (the derivative a PDF fit needs).  The forward keeps a
 32-byte adjoint tape per point (cells, local coordinates, flags), so that the
 backward does not search the knots or take logarithms again; in the pointwise
 form, when x or Q^2 needs a gradient, also the 20-byte derivative tape (the
-patch derivatives, computed with the value, and the point's bin in the grid
+derivatives in x and Q^2, computed with the value, and the point's bin in the grid
 gradient), so that the backward does not reload the coefficients, counts its
 bins from 4 bytes per point and needs no rebinding.  ``LumiFn`` does the same
 for the fused luminosity workload, L = (1/n) sum_e sum_a f_a(x1) f_-a(x2).

@@ -13,7 +13,7 @@
 // the adjoint rebuilds each point's cells and local coordinates from it
 // instead of searching the knots and taking the two logarithms again; the
 // arithmetic that follows is the same.  A pointwise forward pass may also
-// keep each point's two patch derivatives (the derivative tape), computed
+// keep each point's derivatives in x and Q^2 (the derivative tape), computed
 // with its value by the same routine the adjoint would use, so that the
 // adjoint reads them instead of reloading the coefficients.
 //
@@ -533,7 +533,8 @@ __device__ __noinline__ void slow_rec_m(const GridDev &g, const signed char *sco
 // evaluate both derivatives of each column in fixed point (quad_patch_d), the
 // gout rows of the 32 points come through shared memory; what that does not
 // serve is queued (slow_rec_m).  1e6 points x 13 columns: 440 us with the
-// combined patch sum_a g_a C_a in FP64 (16 FMA per column, pipe 95 % busy).
+// combined patch sum_a g_a C_a in FP64 (16 FMA per column, pipe 95 % busy),
+// 313 us here (pipe 57 %: the products with g and the conversions).
 constexpr int kRecWarpBytes = kWarpBuf + 32 * 8 * kMaxSortedPids + kQueue * 8;
 
 __global__ void __launch_bounds__(kBlock, 2) k_bwd_rec_m(const __grid_constant__ GridDev g,

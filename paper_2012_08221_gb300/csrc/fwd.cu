@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kPwBlock, 5) k_xfxq2_pw(const __grid_constant_
 }
 
 // alpha_s, one point per lane (fix_alphas): 1e7 points 286 -> 93 us (FP64
-// pipe 82 % busy before; now integer issue of the logarithm and the table
+// pipe 82 % busy before; now 56 % of the issue slots, the logarithm and the table
 // look-ups in shared memory); points outside the Q range or the
 // domain are queued per warp and evaluated 32 at a time.
 // STAGE: the block's copy of the Q tables and of the cubics (as chunks of 16

@@ -90,7 +90,7 @@ __device__ __forceinline__ double slow_event(const GridDev &g, const signed char
 // [event][parton][flavour] (the rows of 32 events leave as one run).  Without
 // `partials` (the adjoint's recomputation) no status bit is set either.  2e7
 // events x 26 patches, 5 % of the events outside the knots: 13.9 ms in FP64
-// (pipe 96 % busy), 6.1 ms here (integer issue, and the tail in FP64).  Three
+// (pipe 96 % busy), 5.9 ms here (57 % of the FP64 pipe, for the pairs and the tail).  Three
 // blocks per SM at 80 registers; with the wider rows of SAVE two are faster.
 template <bool SAVE>
 __global__ void __launch_bounds__(kBlock, SAVE ? 2 : 3) k_lumi(const __grid_constant__ GridDev g,

@@ -5,9 +5,12 @@
 // monomial coefficients C[n][m] of the bicubic patch in the local coordinates
 // tx = (ln x - U_k)/dU_k and tq = (ln Q^2 - W_c)/dW_c.  These are the Hermite
 // cubics with finite-difference knot derivatives, expanded once at load time,
-// so a query costs two table lookups, two knot searches and 15 FP64 FMAs per
+// so a query costs two logarithms, two knot searches and 16 coefficients per
 // flavour:   P = sum_n bq_n sum_m bx_m C[n][m],  b = (1, t, t^2, t^3).
-// Outside the grid the basis becomes (1, t, t, t): that turns the edge patch
+// Inside the knots the kernels evaluate it in 64-bit fixed point (fix.cuh);
+// this file's FP64 form, 15 FMAs by Horner's rule, serves the points outside
+// the knots and the patches and cells that the fixed-point format does not
+// hold.  Outside the grid the basis becomes (1, t, t, t): that turns the edge patch
 // into the linear continuation from its two edge knots (P(0) + t (P(1)-P(0))).
 //
 // The knot searches compare IEEE bit patterns as integers (the FP64 pipe of

@@ -220,7 +220,7 @@ class PDF:
     def xfxQ2_pw(self, pid, x, q2, member=0, out=None, tape=None, dtape=None):
         """One pid per point: ``out[i] = x*f_{pid_i}(x_i, Q^2_i)``; ``tape`` as
         for ``xfxQ2``; ``dtape`` (with ``tape``, from ``new_dtape``) also keeps
-        each point's patch derivatives for ``xfxQ2_backward``."""
+        each point's derivatives in x and Q^2 for ``xfxQ2_backward``."""
         x = _f64_cuda(x, self.device)
         q2 = _f64_cuda(q2, self.device)
         pid = torch.as_tensor(pid, device=self.device).to(torch.int32).contiguous()

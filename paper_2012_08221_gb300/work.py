@@ -10,6 +10,9 @@ Per point of the x*f kernel with F flavours:
   2 logs x 15 flops (1 FMA reduction, 4 FMA series, 1 multiply, 4 adds),
   2 axes x (subtract, multiply) for t, 15 FMA per flavour for the
   16-coefficient patch by Horner's rule:  34 + 30 F flops.
+Inside the knots the kernels do the same arithmetic in 64-bit fixed point:
+16 products per flavour of two digits each, three 32 x 32 -> 64 bit products
+apiece.
 """
 from __future__ import annotations
 
@@ -32,6 +35,12 @@ def xfxq2_point_flops_matrix_form(n_flav: int) -> int:
     precomputed patch coefficients in 15 FMA per flavour, so this count is
     larger than the work they do: a fraction on it can exceed 1."""
     return 40 * n_flav + 50
+
+
+def xfxq2_point_products(n_flav: int) -> int:
+    """32 x 32 -> 64 bit products of the fixed-point patches of one point
+    (coordinates and weights not counted)."""
+    return 48 * n_flav
 
 
 def xfxq2_point_bytes(n_flav: int) -> int:
