@@ -462,8 +462,8 @@ def main():
                 "frac_matrix_form": flops_matrix / (k_ms * 1e-3) / peak,
                 "flops_per_point_matrix_form": work.xfxq2_point_flops_matrix_form(g.n_flav),
                 "frac_note": "the kernel evaluates the patches in 64-bit fixed point on the integer pipes: frac "
-                             "counts the 48 digit products per flavour against the wide multiply's rate (the "
-                             "kernel is bound by instruction issue, of which they are the largest part); "
+                             "counts the 48 digit products per flavour against the wide multiply's rate (beside "
+                             "them the L1's data path is 50 % busy and warps wait for rows from L2); "
                              "fp64_frac counts the method's FP64 flops (15 FMA per flavour, table log) against "
                              "the FP64 pipe it no longer uses, and frac_matrix_form 40 F + 50 flops per point, "
                              "the separable-weight form: both exceed 1",
