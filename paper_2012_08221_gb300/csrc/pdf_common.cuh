@@ -153,7 +153,7 @@ struct GridDev {
 // Largest cell c in [0, ncell) whose lower key is <= key (0 below the grid).
 // Tables are read with generic loads: they may sit in global or shared memory.
 template <typename K>
-__device__ __forceinline__ int find_cell(const K *keys, int ncell, int step, K key)
+PDF_HD int find_cell(const K *keys, int ncell, int step, K key)
 {
     int lo = 0;
     for (int s = step; s > 0; s >>= 1) {
@@ -170,13 +170,14 @@ __device__ __forceinline__ int find_cell(const K *keys, int ncell, int step, K k
 // 0); the host builds the table so that no bucket holds more than `run` (1 to
 // kGuideRun) further lower keys, and ends the keys with kGuideRun largest
 // ones.  The cell of a key is then the bucket's cell plus the number of the
-// next `run` lower keys that are <= it (the keys ascend): one table load and
+// next `run` lower keys that are <= it (the keys ascend), at most the last
+// cell (a NaN of all ones counts the largest keys too): one table load and
 // `run` independent key loads, instead of a chain of log2(cells) dependent
 // ones.  Without a table (nguide == 0) the binary search.
 constexpr int kGuideRun = 3;
 
-__device__ __forceinline__ int find_cell_guided(const uint64_t *keys, int ncell, int step, const uint16_t *guide,
-                                                int nguide, int shift, int run, uint64_t key0, uint64_t key)
+PDF_HD int find_cell_guided(const uint64_t *keys, int ncell, int step, const uint16_t *guide, int nguide, int shift,
+                            int run, uint64_t key0, uint64_t key)
 {
     if (nguide == 0) return find_cell<uint64_t>(keys, ncell, step, key);
     const uint32_t h0 = (uint32_t)(key0 >> 32), h = max((uint32_t)(key >> 32), h0);
@@ -186,7 +187,7 @@ __device__ __forceinline__ int find_cell_guided(const uint64_t *keys, int ncell,
 #pragma unroll
         for (int r = 2; r <= kGuideRun; ++r) add += keys[c + r] <= key ? 1 : 0;
     }
-    return c + add;
+    return min(c + add, ncell - 1);
 }
 
 // Checked builds (-DPDFGPU_CHECKED, the library built with PDFGPU_CHECKED=1):
