@@ -255,10 +255,13 @@ PDF_HD void fix_pack_cubic(const double c[4], double big, uint32_t out[8])
 
 // A cell's centred matrix in fixed point: row m holds its four entries times
 // 2^(61 - k[m]), the sum of their sizes at most 2^k[m]; k[0] < 0 marks a cell
-// whose entries are too large (very uneven knots), which keeps FP64.
+// whose entries are too large (very uneven knots), which keeps FP64.  Bit i of
+// `used`: the stencil's entry i has weight in it (a straight line takes the two
+// knots of its interval only).
 struct FixMatrix {
     Dig d[4][4];
     int k[4];
+    unsigned used;
 };
 
 // Sum over i of M[i] v_i / 2^61 (|v_i| <= 2^61): one entry of a matrix product.
@@ -301,19 +304,27 @@ PDF_HD int64_t fix_shift(int64_t v, int n)   // v 2^n, rounded
 // coefficients keep about 2^-58 of the stencil's largest value (an FP64 sum
 // keeps 2^-53) and the FP64 pipe stays free.  The interpolation of a constant
 // being the constant, the sums run over the differences to the lower corner.
+// The values' common exponent is that of the entries with weight: a straight
+// line's neighbours may be far larger than its own knots (2^30: values off by
+// 1e-9 when they counted; FP64 never mixes them in).
 PDF_HD void fix_patch(const double v[4][4], unsigned mask, const FixMatrix &X, const FixMatrix &Q, uint32_t out[32])
 {
+    unsigned used = 0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) used |= (Q.used >> r) & 1 ? X.used << (4 * r) : 0;
     int emax = 0;
+    bool finite = true;
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if ((mask >> (4 * r + i)) & 1) {
-                const int e = (int)(dbits(v[r][i]) >> 52) & 0x7FF;
-                emax = e > emax ? e : emax;
-            }
+        for (int i = 0; i < 4; ++i) {
+            const int e = (int)(dbits(v[r][i]) >> 52) & 0x7FF;
+            if ((mask >> (4 * r + i)) & 1) finite = finite && e != 0x7FF;
+            if ((mask & used) >> (4 * r + i) & 1) emax = e > emax ? e : emax;
+        }
+    mask &= used;
     const int Ev = emax - 1022;                      // |v| < 2^Ev
-    bool ok = emax != 0x7FF && X.k[0] >= 0 && Q.k[0] >= 0;
+    bool ok = finite && X.k[0] >= 0 && Q.k[0] >= 0;
     const int64_t ref = fix_from(v[1][1], 60 - Ev);
     int64_t cx[4][4];
 #pragma unroll

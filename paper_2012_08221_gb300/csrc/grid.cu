@@ -323,9 +323,9 @@ static FixMatrix fix_matrix(const long double Mc[16])
         if (!(sum <= (long double)(1 << k))) F.k[0] = -1;
         for (int i = 0; i < 4; ++i)
             F.d[m][i] = fix_split(sum <= (long double)(1 << k) ? llrintl(ldexpl(Mc[4 * m + i], 61 - k)) : 0);
+        for (int i = 0; i < 4; ++i)
+            if (Mc[4 * m + i] != 0) F.used |= 1u << i;
     }
-    for (int m = 1; m < 4; ++m)
-        if (F.k[m] < 0) F.k[0] = -1;
     return F;
 }
 

@@ -25,3 +25,51 @@ def test_search_gives_a_cell_for_every_bit_pattern(knots):
     assert np.array_equal(got, np.clip(np.searchsorted(z[:-1], x, side="right") - 1, 0, z.size - 2))
     got, _ = fixed_host.cells(z[:-1], z[-1], NAN_KEYS)
     assert np.array_equal(got, np.full(NAN_KEYS.size, z.size - 2))
+
+
+def _points(x, q2, cell, n, rng):
+    """Points of cell (i, j) in both axes: at its lower knots, near them (down to
+    2^-30 of the cell) on one axis and on both, and anywhere."""
+    i, j = cell
+    tx, tq = rng.uniform(0, 1, n), rng.uniform(0, 1, n)
+    tx[::3] = 2.0 ** -rng.uniform(0, 30, tx[::3].size)
+    tq[::2] = 2.0 ** -rng.uniform(0, 30, tq[::2].size)
+    px = np.clip(x[i] * (x[i + 1] / x[i]) ** tx, x[i], np.nextafter(x[i + 1], 0))
+    pq = np.clip(q2[j] * (q2[j + 1] / q2[j]) ** tq, q2[j], np.nextafter(q2[j + 1], 0))
+    px[:8], pq[4:12] = x[i], q2[j]
+    return px, pq
+
+
+@pytest.mark.parametrize("x_linear,q_linear", [(True, True), (False, True)])
+@pytest.mark.parametrize("power", [0, 10, 20, 40, 60, 200])
+def test_straight_lines_next_to_far_larger_values(power, x_linear, q_linear):
+    """Linear axes read the two knots of their interval only: neighbours 2^power
+    larger leave the cell's value and derivatives alone.  Every coefficient is
+    at most 2^3 here (values in [1, 2)), so that the fixed-point error, 2^-57 of
+    it in the value and four times that in a derivative, and the rounding to a
+    double stay below 2^-52 and 2^-50 of the weighted values."""
+    rng = np.random.default_rng(200 + power)
+    x, q2 = np.exp(-2 + 0.1 * np.arange(4)), np.exp(3 + 0.1 * np.arange(4))
+    v = rng.uniform(1, 2, (4, 4))
+    v[[0, 3]] *= 2.0 ** power
+    if x_linear:
+        v[:, [0, 3]] *= 2.0 ** power
+    px, pq = _points(x, q2, (1, 1), 60, rng)
+    got, t = fixed_host.evaluate(x, q2, v, px, pq, x_linear, q_linear)
+    ref = fixed_host.exact(x, q2, v, px, pq, t, x_linear, q_linear)
+    kap = np.array([float(r[1]) for r in ref])
+    assert np.all(np.isfinite(got))
+    for col, k, tol in ((0, 0, 2.0 ** -52), (2, 2, 2.0 ** -50), (3, 3, 2.0 ** -50)):
+        err = fixed_host.error(got[:, col], [r[k] for r in ref])
+        assert np.all(err <= tol * np.maximum(kap, 1.0)), (col, np.max(err / kap))
+
+
+def test_non_finite_neighbours_of_a_straight_line_keep_fp64():
+    """The FP64 form multiplies them by its zero weights, which gives NaN; the
+    fixed-point form does not serve such a patch."""
+    x, q2 = np.exp(-2 + 0.1 * np.arange(4)), np.exp(3 + 0.1 * np.arange(4))
+    for bad in (np.inf, np.nan):
+        v = np.ones((4, 4))
+        v[0, 1] = bad
+        got, _ = fixed_host.evaluate(x, q2, v, x[1:2], q2[1:2], True, True)
+        assert np.isnan(got[0, 0]) and np.isnan(got[0, 1])

@@ -44,3 +44,37 @@ def test_points_of_all_ones_are_domain_errors(checked):
     r = subprocess.run([sys.executable, "-c", ALL_ONES], cwd=ROOT, capture_output=True, text=True, timeout=600,
                        env=dict(os.environ, PDFGPU_CHECKED=checked, PYTHONPATH=ROOT))
     assert r.returncode == 0, r.stderr[-3000:]
+
+
+@pytest.mark.parametrize("interp", [1, 2])
+def test_straight_lines_next_to_far_larger_values(interp):
+    """Log-bilinear, and straight lines in a short Q subgrid: knots 2^40 above a
+    cell's own on the rows and columns that it does not read.  Values against
+    the oracle, the luminosity's and the derivatives' patches with them."""
+    from oracle.oracle import OracleGrid
+    from paper_2012_08221_gb300 import build
+    from paper_2012_08221_gb300.pdf import PDF
+    from tests import parity
+    build.build()
+    rng = np.random.default_rng(31)
+    x = synth.log_knots(1e-4, 1.0, 12)
+    q, nq = synth.subgrid_knots([1.3, 4.0, 90.0, 500.0], [3, 3, 3])
+    v = rng.uniform(1, 2, (1, q.size, x.size, 3))
+    v[:, ::3] *= 2.0 ** 40                       # the first row of every subgrid; the others beside it
+    if interp == 1:
+        v[:, :, ::3] *= 2.0 ** 40
+    g = synth.Grid(x, nq, q, np.array([-1, 1, 2], np.int32), v, np.full(q.size, 0.2), "steps")
+    pdf, o = PDF.from_grid(g, interp=interp), OracleGrid.from_synth(g, interp=interp)
+    n = 20_011
+    xs, q2 = np.exp(rng.uniform(np.log(1e-4), 0, n)), np.exp(rng.uniform(2 * np.log(1.3), 2 * np.log(500), n))
+    X, Q = torch.as_tensor(xs, device="cuda"), torch.as_tensor(q2, device="cuda")
+    parity.check(pdf.xfxQ2(g.pids, X, Q).cpu().numpy(), o.xfxq2_batch(g.pids, xs, q2), o.kappa(g.pids, xs, q2))
+    pid = np.full(n, 2, np.int32)
+    dx, dq, _ = pdf.xfxQ2_backward(torch.as_tensor(pid, device="cuda"), X, Q,
+                                   torch.ones(n, dtype=torch.float64, device="cuda"), pointwise=True)
+    rdx, rdq = o.grad_pw(pid, xs, q2)
+    kap = o.kappa(pid, xs, q2, pointwise=True)
+    dU, dW = np.min(np.diff(np.log(x))), np.min(np.diff(2 * np.log(np.unique(q))))
+    # the suite's gradient rule: 1e-9 of the value's terms over the smallest knot spacing
+    for got, ref, s in ((dx, rdx, dU * xs), (dq, rdq, dW * q2)):
+        assert np.all(np.abs(got.cpu().numpy() - ref) <= 1e-9 * np.maximum(np.abs(ref), 4 * kap / s))
