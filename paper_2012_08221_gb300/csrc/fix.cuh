@@ -220,6 +220,14 @@ PDF_HD bool fix_corner_ok(double corner, int E)
     return fabs(corner) >= dfrom((uint64_t)(E - 12 + 1023) << 52);
 }
 
+// What the build leaves in a patch is about 2^(Ev - 60 + spreads) for stencil
+// values below 2^Ev: with interval ratios 2^r on both axes that is 2^(2 r),
+// and smooth values have coefficients (2^E) that do not grow with it.  Patches
+// where it passes 2^(E - 53) keep FP64 (ratios from about 2^6 on; a cell
+// 2^12 times its neighbours on both axes was off by 8e-12 of its values'
+// size).  Nor may the stencil be 2^12 above the corner.
+constexpr int kFixBuild = 7;
+
 // The table's words of one coefficient (value 2^(61 - E)); the last of a row
 // carries the block exponent.
 PDF_HD void fix_words(int64_t v, bool last, int e8, uint32_t *out)
@@ -257,10 +265,12 @@ PDF_HD void fix_pack_cubic(const double c[4], double big, uint32_t out[8])
 // 2^(61 - k[m]), the sum of their sizes at most 2^k[m]; k[0] < 0 marks a cell
 // whose entries are too large (very uneven knots), which keeps FP64.  Bit i of
 // `used`: the stencil's entry i has weight in it (a straight line takes the two
-// knots of its interval only).
+// knots of its interval only).  spread = max over the rows of k[m] - m: an error
+// in row m's coefficient counts 2^-m at the cell's edges.
 struct FixMatrix {
     Dig d[4][4];
     int k[4];
+    int spread;
     unsigned used;
 };
 
@@ -358,7 +368,8 @@ PDF_HD void fix_patch(const double v[4][4], unsigned mask, const FixMatrix &X, c
             for (int i = 0; i < 4; ++i) ok = ok && (!((mask >> (4 * r + i)) & 1) || v[r][i] == 0.0);
     } else {
         e8 = E + kFixBias;
-        ok = ok && e8 >= 0 && e8 < kFixNone && fix_corner_ok(v[1][1], E);
+        ok = ok && e8 >= 0 && e8 < kFixNone && fix_corner_ok(v[1][1], E > Ev ? E : Ev) &&
+             Ev + X.spread + Q.spread - E <= kFixBuild;
     }
     if (!ok) e8 = kFixNone;
     const bool fill = ok && emax != 0;

@@ -314,6 +314,7 @@ static void centre_matrix(const long double M[16], long double Mc[16])
 static FixMatrix fix_matrix(const long double Mc[16])
 {
     FixMatrix F{};
+    F.spread = -3;
     for (int m = 0; m < 4; ++m) {
         long double sum = 0;
         for (int i = 0; i < 4; ++i) sum += fabsl(Mc[4 * m + i]);
@@ -321,6 +322,7 @@ static FixMatrix fix_matrix(const long double Mc[16])
         while (k < 16 && sum > (long double)(1 << k)) ++k;
         F.k[m] = k;
         if (!(sum <= (long double)(1 << k))) F.k[0] = -1;
+        if (sum > 0) F.spread = std::max(F.spread, k - m);
         for (int i = 0; i < 4; ++i)
             F.d[m][i] = fix_split(sum <= (long double)(1 << k) ? llrintl(ldexpl(Mc[4 * m + i], 61 - k)) : 0);
         for (int i = 0; i < 4; ++i)

@@ -73,3 +73,35 @@ def test_non_finite_neighbours_of_a_straight_line_keep_fp64():
         v[0, 1] = bad
         got, _ = fixed_host.evaluate(x, q2, v, x[1:2], q2[1:2], True, True)
         assert np.isnan(got[0, 0]) and np.isnan(got[0, 1])
+
+
+def _uneven(r, rng):
+    """Knots whose second interval is 2^r times its lower neighbour."""
+    d = rng.uniform(0.02, 0.4)
+    return -2 + np.array([-d * 2.0 ** -r, 0.0, d, d * rng.uniform(1.3, 4.0)])
+
+
+@pytest.mark.parametrize("r", [0, 3, 5, 6, 8, 10, 12, 14, 15])
+def test_uneven_cells_on_both_axes(r):
+    """Smooth positive values on a cell that is 2^r times its lower neighbour on
+    both axes, at its knots and inside.  Where fixed point serves, what the
+    build leaves is at most 2^(E - 53), E at most 1 above the corner's exponent
+    for values that vary by less than 2 over the cell, and the corner at least
+    half of 2^that: 2^-51 of the values, and 2^-50 with the evaluation's and
+    the rounding's share."""
+    rng = np.random.default_rng(300 + r)
+    served = 0
+    for _ in range(6):
+        u, w = _uneven(r, rng), 5 + _uneven(r, rng)
+        a, b = rng.uniform(-0.5, 0.5), rng.uniform(-0.02, 0.1)
+        v = np.exp(a * u)[None] * (1 + b * w)[:, None]
+        x, q2 = np.exp(u), np.exp(w)
+        px, pq = _points(x, q2, (1, 1), 60, rng)
+        got, t = fixed_host.evaluate(x, q2, v, px, pq)
+        ref = fixed_host.exact(x, q2, v, px, pq, t)
+        kap = np.array([float(k[1]) for k in ref])
+        ok = np.isfinite(got[:, 0])
+        served += ok.sum()
+        err = fixed_host.error(got[:, 0], [k[0] for k in ref])
+        assert np.all(err[ok] <= 2.0 ** -50 * kap[ok]), np.max(err[ok] / kap[ok])
+    assert served == 360 if r <= 4 else True          # ordinary cells stay in fixed point

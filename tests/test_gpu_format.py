@@ -78,3 +78,38 @@ def test_straight_lines_next_to_far_larger_values(interp):
     # the suite's gradient rule: 1e-9 of the value's terms over the smallest knot spacing
     for got, ref, s in ((dx, rdx, dU * xs), (dq, rdq, dW * q2)):
         assert np.all(np.abs(got.cpu().numpy() - ref) <= 1e-9 * np.maximum(np.abs(ref), 4 * kap / s))
+
+
+def test_knots_uneven_on_both_axes():
+    """Intervals of very different widths next to each other in x and in Q^2:
+    the values at every pair of knots, next to them and in between, against
+    the oracle and, at the knots, against the grid's own values."""
+    from oracle.oracle import OracleGrid
+    from paper_2012_08221_gb300 import build
+    from paper_2012_08221_gb300.pdf import PDF
+    from tests import parity
+    build.build()
+    rng = np.random.default_rng(41)
+    steps = 2.0 ** -np.array([2, 8, 2, 10, 3, 13, 3, 5, 2, 12, 2])
+    x = np.exp(np.concatenate([[0.0], np.cumsum(steps)]) - 4.0)
+    w = np.concatenate([[0.0], np.cumsum(steps[::-1])])
+    qa, qb = np.exp(1.0 + w / 2), np.exp(1.0 + w[-1] / 2 + w / 2)
+    qb[0] = qa[-1]
+    q, nq = np.concatenate([qa, qb]), np.array([qa.size, qb.size], np.int32)
+    lx, lq = np.log(x)[None, :, None], 2 * np.log(q)[:, None, None]
+    v = np.exp(lx * np.array([-0.4, 0.3, 0.9])) * (1 + 0.1 * lq)
+    g = synth.Grid(x, nq, q, np.array([-1, 0, 1], np.int32), v[None], 0.3 / (1 + 0.1 * lq[:, 0, 0]), "uneven")
+    pdf, o = PDF.from_grid(g), OracleGrid.from_synth(g)
+    X, Q = (a.ravel() for a in np.meshgrid(x, q * q))
+    pdf.status()
+    at = pdf.xfxQ2(g.pids, torch.as_tensor(X, device="cuda"), torch.as_tensor(Q, device="cuda")).cpu().numpy()
+    parity.check(at, o.xfxq2_batch(g.pids, X, Q), o.kappa(g.pids, X, Q), what="knots")
+    assert np.allclose(at, v.reshape(-1, 3), rtol=1e-12, atol=0)
+    k, j = rng.integers(0, x.size - 1, 20_003), rng.integers(0, q.size - 1, 20_003)
+    tx, tq = (2.0 ** -rng.uniform(0, 40, (2, 20_003)))
+    xs, qs = x[k] * (x[k + 1] / x[k]) ** tx, (q[j] * (q[j + 1] / q[j]) ** tq) ** 2
+    xs, qs = np.clip(xs, x[0], x[-1]), np.clip(qs, q[0] ** 2, q[-1] ** 2)
+    D = [torch.as_tensor(a, device="cuda") for a in (xs, qs)]
+    parity.check(pdf.xfxQ2(g.pids, *D).cpu().numpy(), o.xfxq2_batch(g.pids, xs, qs), o.kappa(g.pids, xs, qs))
+    parity.check(pdf.alphasQ2(D[1]).cpu().numpy(), o.alphas_batch(qs), o.alphas_kappa(qs), what="alpha_s")
+    assert pdf.status() == 0
