@@ -259,6 +259,13 @@ static void build_guide(const std::vector<uint64_t> &keys, uint64_t key_hi, std:
         }
 }
 
+// The table that the search reads, from the lower keys (see find_cell_guided).
+static void search_table(std::vector<uint64_t> &keys)
+{
+    for (uint64_t &k : keys) --k;
+    keys.insert(keys.end(), kGuideRun, ~(uint64_t)0);
+}
+
 // Tables of fix_log: 1/c_j in 2^-31, c_j = 1 + (j + 1/2)/1024, and minus the
 // logarithm of that rounded reciprocal in 2^-60.
 struct FixLogTables {
@@ -682,8 +689,8 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
     d.extrap = D.extrap;
 
     TableUpload up;
-    xbits.insert(xbits.end(), kGuideRun, ~(uint64_t)0);
-    qbits.insert(qbits.end(), kGuideRun, ~(uint64_t)0);
+    search_table(xbits);
+    search_table(qbits);
     up.add(xbits.data(), xbits.size(), &d.xbits);
     up.add(ukey.data(), ukey.size(), &d.ukey);
     up.add(xcell.data(), xcell.size(), &d.xcell);

@@ -119,10 +119,10 @@ struct GridDev {
     uint64_t qlo, qhi;    // bit patterns of the first / last Q^2 knot
     int64_t ulo, uhi;     // order keys of ln(first / last x knot)
     int64_t wlo, whi;     // order keys of ln(first / last Q^2 knot)
-    const uint64_t *xbits;   // [nxc + kGuideRun] bits of each x cell's lower knot
+    const uint64_t *xbits;   // [nxc + kGuideRun] bits of each x cell's lower knot, less one
     const int64_t *ukey;     // [nxc] order keys of each x cell's lower ln x
     const double2 *xcell;    // [nxc] (U_k, 1/dU_k)
-    const uint64_t *qbits;   // [nqc + kGuideRun] bits of each Q cell's lower Q^2 knot
+    const uint64_t *qbits;   // [nqc + kGuideRun] bits of each Q cell's lower Q^2 knot, less one
     const uint16_t *xguide;  // [nxg] first cell of each x guide bucket
     const uint16_t *qguide;  // [nqg] the same for Q^2
     const FixCell *xfix;     // [nxc] the cells of the fixed-point coordinates
@@ -168,26 +168,28 @@ PDF_HD int find_cell(const K *keys, int ncell, int step, K key)
 // first key (the last bucket also everything above), and holds the largest
 // cell whose lower key is <= the bucket's first key (the first cell in bucket
 // 0); the host builds the table so that no bucket holds more than `run` (1 to
-// kGuideRun) further lower keys, and ends the keys with kGuideRun largest
-// ones.  The cell of a key is then the bucket's cell plus the number of the
-// next `run` lower keys that are <= it (the keys ascend), at most the last
-// cell (a NaN of all ones counts the largest keys too): one table load and
-// `run` independent key loads, instead of a chain of log2(cells) dependent
-// ones.  Without a table (nguide == 0) the binary search.
+// kGuideRun) further lower keys.  The cell of a key is then the bucket's cell
+// plus the number of the next `run` lower keys that are <= it (the keys
+// ascend): one table load and `run` independent key loads, instead of a chain
+// of log2(cells) dependent ones.  Without a table (nguide == 0) the binary
+// search.  The table holds the lower keys less one (a lower key is at least 1)
+// and ends with kGuideRun largest values: "below the key" then says the same,
+// and no key is above those, a NaN of all ones included (points are searched
+// before their domain is tested).
 constexpr int kGuideRun = 3;
 
 PDF_HD int find_cell_guided(const uint64_t *keys, int ncell, int step, const uint16_t *guide, int nguide, int shift,
                             int run, uint64_t key0, uint64_t key)
 {
-    if (nguide == 0) return find_cell<uint64_t>(keys, ncell, step, key);
+    if (nguide == 0) return find_cell<uint64_t>(keys, ncell, step, key - (key != 0));
     const uint32_t h0 = (uint32_t)(key0 >> 32), h = max((uint32_t)(key >> 32), h0);
     const int c = guide[min((h - h0) >> shift, (uint32_t)(nguide - 1))];
-    int add = keys[c + 1] <= key ? 1 : 0;
+    int add = keys[c + 1] < key ? 1 : 0;
     if (run > 1) {
 #pragma unroll
-        for (int r = 2; r <= kGuideRun; ++r) add += keys[c + r] <= key ? 1 : 0;
+        for (int r = 2; r <= kGuideRun; ++r) add += keys[c + r] < key ? 1 : 0;
     }
-    return min(c + add, ncell - 1);
+    return c + add;
 }
 
 // Checked builds (-DPDFGPU_CHECKED, the library built with PDFGPU_CHECKED=1):

@@ -45,11 +45,11 @@ extern "C" void host_cells(const uint64_t *lo, int ncell, uint64_t last, const u
     std::vector<uint16_t> guide;
     int shift, run;
     build_guide(keys, last, guide, &shift, &run);
-    keys.insert(keys.end(), kGuideRun, ~(uint64_t)0);
+    search_table(keys);
     *guided = (int)guide.size();
     for (int i = 0; i < n; ++i)
         cell[i] = find_cell_guided(keys.data(), ncell, largest_pow2_below(ncell), guide.data(), (int)guide.size(),
-                                   shift, run, keys[0], key[i]);
+                                   shift, run, lo[0], key[i]);
 }
 
 // n points on one subgrid of nq Q^2 knots (v [nq][nx]): per point the

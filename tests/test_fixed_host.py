@@ -13,6 +13,9 @@ NAN_KEYS = np.array([0x7FF0000000000000, 0x7FF8000000000000, 0x8000000000000000,
 @pytest.mark.parametrize("knots", [[0.1, 1.0], [1e-4, 0.5, 1.0], [1e-9, 1e-3, 0.5, 0.9, 1 - 6e-5, 1 - 2e-5, 1.0],
                                    synth.log_knots(1e-9, 1.0, 196),
                                    np.concatenate([synth.log_knots(1e-5, 0.5, 9), 0.5 + 2.0 ** -40 * np.arange(1, 12),
+                                                   [1.0]]),
+                                   # steps from 2^-12 to 2^-46: no bucket width fits, binary search
+                                   np.concatenate([[1e-6, 0.5], 0.5 + np.cumsum(2.0 ** -np.arange(46.0, 2.0, -2.0)),
                                                    [1.0]])])
 def test_search_gives_a_cell_for_every_bit_pattern(knots):
     """Points are searched before their domain is tested, so infinities,
@@ -23,6 +26,7 @@ def test_search_gives_a_cell_for_every_bit_pattern(knots):
     x = np.concatenate([z, np.nextafter(z, 0), np.nextafter(z, 2), np.exp(rng.uniform(np.log(z[0]) - 5, 1, 2000))])
     got, _ = fixed_host.cells(z[:-1], z[-1], x.view(np.uint64))
     assert np.array_equal(got, np.clip(np.searchsorted(z[:-1], x, side="right") - 1, 0, z.size - 2))
+    assert np.array_equal(fixed_host.cells(z[:-1], z[-1], np.arange(3, dtype=np.uint64))[0], np.zeros(3))
     got, _ = fixed_host.cells(z[:-1], z[-1], NAN_KEYS)
     assert np.array_equal(got, np.full(NAN_KEYS.size, z.size - 2))
 
