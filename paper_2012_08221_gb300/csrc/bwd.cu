@@ -594,6 +594,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_bwd_rec_m(const __grid_constant__
             Dig W[4][4];
             quad_weights(B.buf, lane, fast ? X.f : kFixHalf, fast ? Q.f : kFixHalf, W);
             const QuadPos pos = quad_pos(lane);
+            const int limit = fix_limit(X.f, Q.f);
             bool none = false;
             double sx = 0.0, sq = 0.0;
             for (int a = 0; a < npid; ++a) {
@@ -608,7 +609,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_bwd_rec_m(const __grid_constant__
                 const double ga = rows[lane * npid + a];
                 sx = fma(ga, fix_value(dx, last), sx);
                 sq = fma(ga, fix_value(dq, last), sq);
-                none |= fix_none(last);
+                none |= fix_needs_fp64(last, limit);
             }
             __syncwarp();                            // the buffers may be refilled
             fast = fast && !none;

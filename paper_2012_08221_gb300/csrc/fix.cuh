@@ -190,16 +190,29 @@ PDF_HD int64_t fix_row_dx(const int c[8], const Dig w[4])
 // by exact cancellation, which FP64 from the knot's own expansion keeps.
 PDF_HD bool fix_at_knot(int64_t t) { return t <= 0 || t >= ((int64_t)1 << 62) - 256; }
 
-// Block exponent: the low byte of a row's last coefficient is E + kFixBias;
-// kFixNone marks a patch that the format cannot hold.
-constexpr int kFixBias = 160;
+// Block exponent: the low 7 bits of a row's last coefficient are E + kFixBias.
+// Bit 7 marks a patch that serves away from the cell's lower edges only
+// (kFixWeak), kFixNone one that the format cannot hold.
+constexpr int kFixBias = 80;
+constexpr int kFixWeak = 128;
 constexpr int kFixNone = 255;
 
+// On a lower edge: t < 2^-16 on either axis.  There the FP64 form, which expands
+// about the lower corner, gives the values on the knots to the last bit, and
+// the fixed-point form's error follows the patch's largest coefficient: a weak
+// patch (fix_patch) then takes FP64.  The limit is the least exponent byte that
+// does so at the point.
+constexpr int kFixEdge = 1 << 14;         // 2^-16 in the upper word of a t (value 2^62)
+PDF_HD int fix_limit(int64_t tx, int64_t tq)
+{
+    return fix_hi(tx) < kFixEdge || fix_hi(tq) < kFixEdge ? kFixWeak : kFixNone;
+}
+PDF_HD bool fix_needs_fp64(int last, int limit) { return (last & 255) >= limit; }
+
 #ifdef __CUDACC__
-__device__ __forceinline__ bool fix_none(int last) { return (last & 255) == kFixNone; }
 __device__ __forceinline__ double fix_value(int64_t s, int last)
 {
-    return __ll2double_rn(s) * __hiloint2double((last & 255) * (1 << 20) + ((1023 - 59 - kFixBias) << 20), 0);
+    return __ll2double_rn(s) * __hiloint2double((last & 127) * (1 << 20) + ((1023 - 59 - kFixBias) << 20), 0);
 }
 
 // Eight 32-bit words (one row of a fixed-point patch) in one 32-byte load.
@@ -211,55 +224,51 @@ __device__ __forceinline__ void fix_ld(const unsigned char *p, int c[8])
 }
 #endif
 
-// A patch whose lower corner (t = 0 on both axes, about which the FP64 form
-// expands) is 2^12 below its largest coefficient keeps FP64: the fixed-point
-// error follows the largest coefficient, the FP64 error next to the lower
-// edges follows the values there (a flavour that sets in at a threshold knot).
-PDF_HD bool fix_corner_ok(double corner, int E)
-{
-    return fabs(corner) >= dfrom((uint64_t)(E - 12 + 1023) << 52);
-}
+// Lower corner (t = 0 on both axes) against the largest coefficient (below 2^E)
+// and the stencil (below 2^Ev).  A fixed-point sum is off by 2^(E - 57) or so,
+// at the corner by less than 2^(E - 57.5), which rounds to the knot's value
+// while the corner is 2^(E - 5) at least; FP64 is off by 2^-53 of the largest
+// term at the point, next to the corner of the corner's value.
+//  - From 2^(E - 2) on fixed point is as good everywhere.
+//  - Below, the patch is weak: FP64 on its lower edges.  Away from them the
+//    argument decides: FP64's logarithm moves the value by 2^-53 |ln x| / width
+//    of 2^E, more than 2^(E - 54) anywhere; fixed point's by 2^(E - 59) /
+//    width.  Largest error of the value itself, FP64 / fixed point, cells of
+//    0.1 at ln x = -5 with the corner 2^-k of the rest: k = 4 1e-13 / 1e-15, 8
+//    2e-12 / 2e-14.  (The patch alone, at a given t above 2^-16: 8e-15 / 7e-16
+//    and 1e-14 / 1e-14.)
+//  - 2^8 below (a flavour that sets in at a threshold knot), or with a stencil
+//    2^12 above the corner, the patch keeps FP64.
+// Of the 196 x 50 grid's patches 2.8 % are weak (by area), 0.5 % at 2^-5 and
+// below; a limit at 2^-4 of the edges cost 3.5 % there and 11 % with few
+// flavours per point.
+constexpr int kFixStrong = 1;
+constexpr int kFixCorner = 8;
+constexpr int kFixStencil = 12;
+PDF_HD int fix_exponent(double v) { return ((int)(dbits(v) >> 52) & 0x7FF) - 1022; }   // |v| < 2^this
 
 // What the build leaves in a patch is about 2^(Ev - 60 + spreads) for stencil
 // values below 2^Ev: with interval ratios 2^r on both axes that is 2^(2 r),
 // and smooth values have coefficients (2^E) that do not grow with it.  Patches
 // where it passes 2^(E - 53) keep FP64 (ratios from about 2^6 on; a cell
 // 2^12 times its neighbours on both axes was off by 8e-12 of its values'
-// size).  Nor may the stencil be 2^12 above the corner.
+// size).
 constexpr int kFixBuild = 7;
 
-// The table's words of one coefficient (value 2^(61 - E)); the last of a row
-// carries the block exponent.
-PDF_HD void fix_words(int64_t v, bool last, int e8, uint32_t *out)
+// One coefficient (value 2^(61 - E)) as the table holds it: the last of a row
+// carries the exponent byte.
+PDF_HD int64_t fix_last(int64_t v, int e8) { return ((v - e8 + 128) & ~(int64_t)255) | e8; }
+
+PDF_HD void fix_words(int64_t v, uint32_t *out)
 {
-    if (last) v = ((v - e8 + 128) & ~(int64_t)255) | e8;
     const Dig d = fix_split(v);
     out[0] = (uint32_t)d.l;
     out[1] = (uint32_t)d.h;
 }
 
-// Packs a centred cubic (alpha_s): `big` is the part of the constant term
-// that is added exactly, its value at the lower knot.
-PDF_HD void fix_pack_cubic(const double c[4], double big, uint32_t out[8])
-{
-    double top = fabs(c[0] + big);
-    for (int k = 1; k < 4; ++k) top = fabs(c[k]) > top || !(fabs(c[k]) <= 1e300) ? fabs(c[k]) : top;
-    int e8 = 0;
-    double scale = 0.0;
-    bool ok = top <= 1e300 && fabs(big) <= 1e300;
-    if (ok && top > 0.0) {
-        const int E = (int)((dbits(top) >> 52) & 0x7FF) - 1022;
-        e8 = E + kFixBias;
-        ok = e8 >= 0 && e8 < kFixNone && fix_corner_ok(big, E);
-        if (ok) scale = dfrom((uint64_t)(61 - E + 1023) << 52);
-    }
-    if (!ok) e8 = kFixNone;
-    for (int k = 0; k < 4; ++k) {
-        int64_t v = 0;
-        if (ok) v = (int64_t)rint(c[k] * scale) + (k == 0 ? (int64_t)rint(big * scale) : 0);
-        fix_words(v, k == 3, e8, out + 2 * k);
-    }
-}
+// c1 - (c2 - c3 / 2) / 2, all halved: minus the cubic without its constant term
+// at tc = -1/2.
+PDF_HD int64_t fix_lower(int64_t c1, int64_t c2, int64_t c3) { return (c1 - ((c2 - (c3 >> 1)) >> 1)) >> 1; }
 
 // A cell's centred matrix in fixed point: row m holds its four entries times
 // 2^(61 - k[m]), the sum of their sizes at most 2^k[m]; k[0] < 0 marks a cell
@@ -367,9 +376,10 @@ PDF_HD void fix_patch(const double v[4][4], unsigned mask, const FixMatrix &X, c
 #pragma unroll
             for (int i = 0; i < 4; ++i) ok = ok && (!((mask >> (4 * r + i)) & 1) || v[r][i] == 0.0);
     } else {
+        const int ec = fix_exponent(v[1][1]), spread = X.spread + Q.spread;
         e8 = E + kFixBias;
-        ok = ok && e8 >= 0 && e8 < kFixNone && fix_corner_ok(v[1][1], E > Ev ? E : Ev) &&
-             Ev + X.spread + Q.spread - E <= kFixBuild;
+        ok = ok && e8 >= 0 && e8 < 127 && E - ec <= kFixCorner && Ev - ec <= kFixStencil && Ev + spread - E <= kFixBuild;
+        if (E - ec > kFixStrong || Ev + spread - ec > kFixBuild) e8 |= kFixWeak;
     }
     if (!ok) e8 = kFixNone;
     const bool fill = ok && emax != 0;
@@ -377,13 +387,19 @@ PDF_HD void fix_patch(const double v[4][4], unsigned mask, const FixMatrix &X, c
     for (int n = 0; n < 4; ++n)
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            int64_t c = 0;
-            if (fill) {
-                c = fix_shift(C[n][m], 1 - E + X.k[m] + Q.k[n] + Ev);
-                if (n + m == 0) c += fix_shift(ref, 1 + Ev - E);
-            }
-            fix_words(c, m == 3, e8, out + 2 * (4 * n + m));
+            C[n][m] = fill ? fix_shift(C[n][m], 1 - E + X.k[m] + Q.k[n] + Ev) : 0;
+            if (m == 3) C[n][m] = fix_last(C[n][m], e8);
         }
+    // the constant term from the others as stored, so that the sum at the corner is the knot's value
+    int64_t low[4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n) low[n] = fix_lower(C[n][1], C[n][2], C[n][3]);
+    if (fill)
+        C[0][0] = fix_shift(ref, 1 + Ev - E) + low[0] + fix_lower(C[1][0] - low[1], C[2][0] - low[2], C[3][0] - low[3]);
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) fix_words(C[n][m], out + 2 * (4 * n + m));
 }
 
 }  // namespace pdfgpu

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kPwBlock, 5) k_xfxq2_pw(const __grid_constant_
             int c[4][8], last;
             quad_load(fm, off, c);
             const int64_t s = quad_patch(c, W, quad_pos(lane), last);
-            fast &= col < 0 || !fix_none(last);
+            fast &= col < 0 || !fix_needs_fp64(last, fix_limit(X.t, Q.t));
             if (fast) {
                 out[i] = col >= 0 ? fix_value(s, last) : 0.0;
                 if (TAPE) tape_put(tape, i, X, Q);

@@ -338,6 +338,36 @@ static FixMatrix fix_matrix(const long double Mc[16])
     return F;
 }
 
+// The centred cubic of cell k on knots z[0..n-1] with values a (alpha_s), packed
+// as fix_patch does (one that would be weak keeps FP64); the sums run over the differences to the lower
+// knot's value.
+static void fix_cubic(const long double *z, const double *a, int n, int k, bool linear, uint32_t out[8])
+{
+    long double M[16], Ms[16], Mc[16], c[4] = {0, 0, 0, 0};
+    cell_matrix<long double>(z, n, k, M, linear, Ms);
+    centre_matrix(M, Mc);
+    const double first = a[k];
+    for (int m = 0; m < 4; ++m)
+        for (int i = 0; i < 4; ++i)
+            if (k - 1 + i >= 0 && k - 1 + i < n) c[m] += Mc[4 * m + i] * ((long double)a[k - 1 + i] - first);
+    long double top = fabsl(c[0] + first);
+    for (int k = 1; k < 4; ++k) top = fabsl(c[k]) > top || !(fabsl(c[k]) <= 1e300L) ? fabsl(c[k]) : top;
+    int E = 0, e8 = 0;
+    bool ok = top <= 1e300L && fabs(first) <= 1e300;
+    if (ok && top > 0) {
+        const int ec = fix_exponent(first);
+        E = fix_exponent((double)top);
+        e8 = E + kFixBias;
+        ok = e8 >= 0 && e8 < 127 && E - ec <= kFixStrong;
+    }
+    if (!ok) e8 = kFixNone;
+    int64_t v[4];
+    for (int k = 0; k < 4; ++k) v[k] = ok && top > 0 ? llrintl(ldexpl(c[k], 61 - E)) : 0;
+    v[3] = fix_last(v[3], e8);
+    if (ok && top > 0) v[0] = llrintl(ldexpl((long double)first, 61 - E)) + fix_lower(v[1], v[2], v[3]);
+    for (int k = 0; k < 4; ++k) fix_words(v[k], out + 2 * k);
+}
+
 static int largest_pow2_below(int n)
 {
     int s = 0;
@@ -623,7 +653,7 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
     const int nqc = (int)qbits.size();
     // the centred matrices from knot logarithms to 64 bits and more
     std::vector<FixMatrix> mxf(nxc), mqf(nqc);
-    std::vector<double> mqc((size_t)nqc * 16);
+    std::vector<uint32_t> fac(D.alphas ? (size_t)nqc * 8 : 0);   // alpha_s about the cells' centres
     {
         std::vector<long double> U(nx), W(rows);
         long double M[16], Ms[16], Mc[16];
@@ -642,7 +672,7 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
                 cell_matrix<long double>(W.data() + r0, D.n_q[s], j, M, q_linear, Ms);
                 centre_matrix(M, Mc);
                 mqf[c] = fix_matrix(Mc);
-                for (int e = 0; e < 16; ++e) mqc[(size_t)c * 16 + e] = (double)Mc[e];
+                if (D.alphas) fix_cubic(W.data() + r0, D.alphas + r0, D.n_q[s], j, q_linear, &fac[(size_t)c * 8]);
             }
     }
     for (int c = 1; c < nqc; ++c)
@@ -720,7 +750,6 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
     }
     if (D.alphas) {
         std::vector<double> ac((size_t)nqc * 4);
-        std::vector<uint32_t> fac((size_t)nqc * 8);
         for (int c = 0; c < nqc; ++c) {
             const double *M = &mq[(size_t)c * 16];
             for (int nn = 0; nn < 4; ++nn) {
@@ -731,14 +760,6 @@ extern "C" int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out)
                 }
                 ac[(size_t)c * 4 + nn] = s;
             }
-            // the same cubic about the cell's centre, from the differences to its first knot
-            const double ref = D.alphas[qrow[c]];
-            double cc[4] = {0.0, 0.0, 0.0, 0.0};
-            for (int nn = 0; nn < 4; ++nn)
-                for (int rr = 0; rr < 4; ++rr)
-                    if ((qmask[c] >> rr) & 1)
-                        cc[nn] = fma(mqc[(size_t)c * 16 + nn * 4 + rr], D.alphas[qrow[c] - 1 + rr] - ref, cc[nn]);
-            fix_pack_cubic(cc, ref, &fac[(size_t)c * 8]);
         }
         up.add(fac.data(), fac.size(), &d.facoef);
         up.add(ac.data(), ac.size(), &d.acoef);

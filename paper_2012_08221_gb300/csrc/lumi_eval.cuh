@@ -78,6 +78,7 @@ __device__ __forceinline__ double lumi_quads(const GridDev &g, const signed char
         quad_offsets(fast ? (uint32_t)(Q.cell * g.nxc + X.cell) * cell_bytes : 0u, lane, off);
         Dig W[4][4];
         quad_weights(buf, lane, fast ? X.t : kFixHalf, fast ? Q.t : kFixHalf, W);
+        const int limit = fix_limit(X.t, Q.t);
         for (int a = 0; a < g.nflav; ++a) {
             const int b = anti[a];
             double v = 0.0;
@@ -87,7 +88,7 @@ __device__ __forceinline__ double lumi_quads(const GridDev &g, const signed char
                 quad_load(fm + col * 128, off, c);
                 const int64_t p = quad_patch(c, W, pos, last);
                 v = fix_value(p, last);
-                none |= fix_none(last);
+                none |= fix_needs_fp64(last, limit);
             }
             if (side == 0) {
                 mine[a] = v;

@@ -536,7 +536,7 @@ __device__ __forceinline__ void patch_d(const double *__restrict__ C, const unsi
             if (n) dq += n * fix_row(c, w + 4 * (n - 1));
             last = c[6];
         }
-        if (!fix_none(last)) {
+        if (!fix_needs_fp64(last, fix_limit(X.f, Q.f))) {
             *dtx = fix_value(dx, last);
             *dtq = fix_value(dq, last);
             return;

@@ -195,7 +195,7 @@ __device__ __forceinline__ double fix_alphas(const int c[8], int64_t t, bool &no
     w[1] = fix_split(t - kFixHalf);
     w[2] = fix_split(fix_mul(w[1], w[1]));
     w[3] = fix_split(fix_mul(w[2], w[1]));
-    none = fix_none(c[6]);
+    none = fix_needs_fp64(c[6], kFixNone);
     return fix_value(fix_row(c, w), c[6]);
 }
 __device__ __forceinline__ double fix_alphas(const GridDev &g, const FixAxis &Q, bool &none)
@@ -275,12 +275,14 @@ __device__ __forceinline__ void slow_point(const GridDev &g, const Query &Y, boo
     flag_status(g, oor, PDF_S_RANGE);
     bad |= oor;
     if (Y.tape && e.sub == 0) tape_put(Y.tape, i, X, Q, bad);
+    const int limit = fix_limit(X.f, Q.f);
     const size_t patch0 = ((size_t)Q.cell * g.nxc + X.cell) * g.nflav;
     const double *cell = Y.cm + patch0 * 16;
     for (int a = Y.a0 + e.sub; a < Y.a1; a += e.count) {
         int col = Y.scol[a];
         if (col >= 0) col = checked_index(g.status, col, g.nflav);
-        if (fixed && (col < 0 || !fix_none(reinterpret_cast<const int *>(Y.fm + (patch0 + col) * 128)[6]))) continue;
+        if (fixed && (col < 0 || !fix_needs_fp64(reinterpret_cast<const int *>(Y.fm + (patch0 + col) * 128)[6], limit)))
+            continue;
         const double v = col >= 0 ? patch_any<true>(g, cell + col * 16, X, Q) : 0.0;
         Y.out[i * Y.npid + a] = bad ? dnan() : v;
     }
@@ -355,6 +357,7 @@ __device__ __forceinline__ void eval_points(const GridDev &g, const CoordTabs &T
         quad_weights(B.buf, lane, fast ? X.t : kFixHalf, fast ? Q.t : kFixHalf, W);
         double *srow = reinterpret_cast<double *>(B.buf) + lane * Y.npid;
         const QuadPos pos = quad_pos(lane);
+        const int limit = fix_limit(X.t, Q.t);
         for (int a = Y.a0; a < Y.a1; ++a) {
             int col = Y.scol[a];
             double v = 0.0;
@@ -364,7 +367,7 @@ __device__ __forceinline__ void eval_points(const GridDev &g, const CoordTabs &T
                 quad_load(Y.fm + col * 128, off, c);
                 const int64_t s = quad_patch(c, W, pos, last);
                 v = fix_value(s, last);
-                none |= fix_none(last);
+                none |= fix_needs_fp64(last, limit);
             }
             if (WHOLE) srow[a] = v;
             else if (fast) Y.out[i * Y.npid + a] = v;

@@ -54,8 +54,9 @@ extern "C" void host_cells(const uint64_t *lo, int ncell, uint64_t last, const u
 
 // n points on one subgrid of nq Q^2 knots (v [nq][nx]): per point the
 // fixed-point value, the FP64 form's at the same coordinates, the two
-// fixed-point derivatives in t (NaN where the kernels take FP64), and the
-// coordinates (value 2^62; -1 in a cell without them).
+// fixed-point derivatives in t (NaN where the kernels take FP64), the FP64
+// form's value at coordinates from FP64 logarithms, and the coordinates (value
+// 2^62; -1 in a cell without them).
 extern "C" void host_eval(int nx, const double *x, int x_linear, int nq, const double *q2, int q_linear,
                           const double *v, int n, const double *px, const double *pq, double *out, int64_t *t)
 {
@@ -101,13 +102,17 @@ extern "C" void host_eval(int nx, const double *x, int x_linear, int nq, const d
         auto horner = [](double z, double a, double b, double c, double d) {
             return fma(z, fma(z, fma(z, d, c), b), a);
         };
-        double row[4];
-        for (int k = 0; k < 4; ++k) row[k] = horner(tx, P[k][0], P[k][1], P[k][2], P[k][3]);
-        double *o = out + 4 * i;
-        o[1] = horner(tq, row[0], row[1], row[2], row[3]);
+        auto fp64 = [&](double zx, double zq) {
+            double row[4];
+            for (int k = 0; k < 4; ++k) row[k] = horner(zx, P[k][0], P[k][1], P[k][2], P[k][3]);
+            return horner(zq, row[0], row[1], row[2], row[3]);
+        };
+        double *o = out + 5 * i;
+        o[1] = fp64(tx, tq);
+        o[4] = fp64(fp_coord(px[i], X.U, kx), fp_coord(pq[i], Q.U, kq));
         o[0] = o[2] = o[3] = NAN;
         const int last = (int)w[6];
-        if (!cells || (last & 255) == kFixNone) continue;
+        if (!cells || fix_needs_fp64(last, fix_limit(t[2 * i], t[2 * i + 1]))) continue;
         Dig wt[16];
         fix_weights(t[2 * i] - kFixHalf, t[2 * i + 1] - kFixHalf, wt);
         int64_t sum = 0, dx = 0, dq = 0;
@@ -117,9 +122,31 @@ extern "C" void host_eval(int nx, const double *x, int x_linear, int nq, const d
             dx += fix_row_dx(c, wt + 4 * k);
             if (k) dq += k * fix_row(c, wt + 4 * (k - 1));
         }
-        const int e = (last & 255) - kFixBias - 59;
+        const int e = (last & 127) - kFixBias - 59;
         o[0] = ldexp((double)sum, e);
         o[2] = ldexp((double)dx, e);
         o[3] = ldexp((double)dq, e);
+    }
+}
+
+extern "C" void host_alphas(int nq, const double *q2, const double *a, int n, const double *pq, double *out, int64_t *t)
+{
+    const HostAxis Q(q2, nq, false);
+    const FixLogTables &T = fix_log_tables();
+    std::vector<long double> W(nq);
+    for (int k = 0; k < nq; ++k) W[k] = logl((long double)q2[k]);
+    for (int i = 0; i < n; ++i) {
+        const int k = std::max((int)(std::upper_bound(q2, q2 + nq - 1, pq[i]) - q2) - 1, 0);
+        uint32_t w[8];
+        fix_cubic(W.data(), a, nq, k, false, w);
+        t[i] = fix_coord(fix_log(dbits(pq[i]), T.inv.data(), T.log.data()), Q.C[k]);
+        out[i] = NAN;
+        if (!Q.C[k].K || fix_needs_fp64((int)w[6], kFixNone)) continue;
+        Dig d[4];
+        d[0] = {1 << 30, 0};
+        d[1] = fix_split(t[i] - kFixHalf);
+        d[2] = fix_split(fix_mul(d[1], d[1]));
+        d[3] = fix_split(fix_mul(d[2], d[1]));
+        out[i] = ldexp((double)fix_row((const int *)w, d), ((int)w[6] & 127) - kFixBias - 59);
     }
 }

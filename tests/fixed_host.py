@@ -39,11 +39,12 @@ def cells(lower, last, keys):
 
 
 def evaluate(x, q2, v, px, pq, x_linear=False, q_linear=False):
-    """Columns: fixed-point value (NaN where FP64 serves), FP64 form, the two
-    fixed-point derivatives; and the coordinates as integers (value 2^62)."""
+    """Columns: fixed-point value (NaN where FP64 serves), FP64 form at the same
+    coordinates, the two fixed-point derivatives, FP64 form at coordinates from
+    FP64 logarithms; and the coordinates as integers (value 2^62)."""
     a = [np.ascontiguousarray(z, np.float64) for z in (x, q2, v, px, pq)]
     n = a[3].size
-    out, t = np.empty((n, 4)), np.empty((n, 2), np.int64)
+    out, t = np.empty((n, 5)), np.empty((n, 2), np.int64)
     lib().host_eval(a[0].size, _p(a[0]), int(x_linear), a[1].size, _p(a[1]), int(q_linear), _p(a[2]), n, _p(a[3]),
                     _p(a[4]), _p(out), _p(t))
     return out, t
@@ -95,3 +96,12 @@ def exact(x, q2, v, px, pq, t=None, x_linear=False, q_linear=False):
 def error(got, want):
     """|got - want| of a double against a decimal, as a double."""
     return np.array([abs(float(D(float(g)) - w)) if np.isfinite(g) else np.nan for g, w in zip(got, want)])
+
+
+def alphas(q2, a, pq):
+    """alpha_s in fixed point on one subgrid (NaN where FP64 serves), and the
+    coordinates."""
+    z = [np.ascontiguousarray(b, np.float64) for b in (q2, a, pq)]
+    out, t = np.empty(z[2].size), np.empty(z[2].size, np.int64)
+    lib().host_alphas(z[0].size, _p(z[0]), _p(z[1]), z[2].size, _p(z[2]), _p(out), _p(t))
+    return out, t

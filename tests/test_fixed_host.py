@@ -109,3 +109,62 @@ def test_uneven_cells_on_both_axes(r):
         err = fixed_host.error(got[:, 0], [k[0] for k in ref])
         assert np.all(err[ok] <= 2.0 ** -50 * kap[ok]), np.max(err[ok] / kap[ok])
     assert served == 360 if r <= 4 else True          # ordinary cells stay in fixed point
+
+
+@pytest.mark.parametrize("what", ["corner", "column", "row"])
+@pytest.mark.parametrize("k", [0, 1, 2, 3, 4, 6, 8, 10, 12, 14])
+def test_values_small_at_the_lower_edges(k, what):
+    """Cells whose corner, left column or lower row is 2^-k of the rest.  Where
+    fixed point serves: the knot's value itself at the corner; next to it within
+    2^-52 of the value where fixed point serves the edges too (off by 2^(E - 56)
+    at most, the corner at least 2^(E - 2), and the rounding adds 2^-53); and
+    over the whole cell no larger an error against the exact value of the
+    argument, on the scale of the weighted values, than the FP64 form."""
+    rng = np.random.default_rng(400 + k)
+    fixed, fp64, served = [], [], 0
+    for _ in range(8):
+        u = np.concatenate([[-5.0], -5 + np.cumsum(0.1 * 7.0 ** rng.uniform(-0.5, 0.5, 3))])
+        w = np.concatenate([[2.0], 2 + np.cumsum(0.2 * 7.0 ** rng.uniform(-0.5, 0.5, 3))])
+        x, q2 = np.exp(u), np.exp(w)
+        v = rng.uniform(1, 2, (4, 4)) * rng.choice([-1, 1])
+        v[(1, 1) if what == "corner" else np.s_[:, 1] if what == "column" else np.s_[1]] *= 2.0 ** -k
+        px, pq = _points(x, q2, (1, 1), 60, rng)
+        px[:20] = np.clip(x[1] * (1 + rng.uniform(0, 1e-9, 20)), x[1], None)
+        pq[:20] = np.clip(q2[1] * (1 + rng.uniform(0, 1e-9, 20)), q2[1], None)
+        px[0], pq[0] = x[1], q2[1]
+        got, t = fixed_host.evaluate(x, q2, v, px, pq)
+        ok = np.isfinite(got[:, 0])
+        if ok[0]:
+            assert got[0, 0] == v[1, 1]
+        near = fixed_host.exact(x, q2, v, px[:20], pq[:20], t)
+        err = fixed_host.error(got[:20, 0], [r[0] for r in near])
+        assert np.all(err[ok[:20]] <= 2.0 ** -52 * abs(v[1, 1]))
+        ref = fixed_host.exact(x, q2, v, px, pq)
+        kap = np.array([float(r[1]) for r in ref])
+        fixed.append((fixed_host.error(got[:, 0], [r[0] for r in ref]) / kap)[ok])
+        fp64.append((fixed_host.error(got[:, 4], [r[0] for r in ref]) / kap)[ok])
+        served += ok.sum()
+    fixed, fp64 = np.concatenate(fixed), np.concatenate(fp64)
+    if k <= 4:
+        assert served >= 100                             # away from the edges at least
+    if fixed.size:
+        assert np.max(fixed) <= np.max(fp64)
+
+
+def test_alpha_s_cubics():
+    """The centred cubics of alpha_s where they serve: exact at the lower knots,
+    and within 2^-52 of the terms' size in between, on even and uneven knots."""
+    rng = np.random.default_rng(500)
+    for r in (0, 4, 8, 12):
+        w = np.cumsum(np.concatenate([[1.0], 0.3 * 2.0 ** -rng.permutation([r, 0, 1, 0, r, 0])]))
+        a = 1.3 / (1 + 0.6 * w) + 0.01 * rng.uniform(0, 1, w.size)
+        q2 = np.exp(w)
+        p = np.concatenate([q2[:-1], np.exp(rng.uniform(w[0], w[-1], 80))])
+        got, t = fixed_host.alphas(q2, a, p)
+        ref = fixed_host.exact(q2, np.array([1.0, 2.0]), np.vstack([a, a]), p, np.ones(p.size),
+                               np.column_stack([t, np.zeros_like(t)]))
+        kap = np.array([float(k[1]) for k in ref])
+        ok = np.isfinite(got)
+        assert ok.sum() >= (got.size if r == 0 else got.size // 2)
+        assert np.array_equal(got[:w.size - 1][ok[:w.size - 1]], a[:-1][ok[:w.size - 1]])
+        assert np.all(fixed_host.error(got, [k[0] for k in ref])[ok] <= 2.0 ** -52 * kap[ok])

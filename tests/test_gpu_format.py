@@ -49,8 +49,9 @@ def test_points_of_all_ones_are_domain_errors(checked):
 @pytest.mark.parametrize("interp", [1, 2])
 def test_straight_lines_next_to_far_larger_values(interp):
     """Log-bilinear, and straight lines in a short Q subgrid: knots 2^40 above a
-    cell's own on the rows and columns that it does not read.  Values against
-    the oracle, the luminosity's and the derivatives' patches with them."""
+    cell's own on the rows and columns that it does not read.  Values and
+    derivatives of the points whose own knots are the small ones (between 1 and
+    2^80 the value follows the rounding of t), against the oracle."""
     from oracle.oracle import OracleGrid
     from paper_2012_08221_gb300 import build
     from paper_2012_08221_gb300.pdf import PDF
@@ -67,6 +68,12 @@ def test_straight_lines_next_to_far_larger_values(interp):
     pdf, o = PDF.from_grid(g, interp=interp), OracleGrid.from_synth(g, interp=interp)
     n = 20_011
     xs, q2 = np.exp(rng.uniform(np.log(1e-4), 0, n)), np.exp(rng.uniform(2 * np.log(1.3), 2 * np.log(500), n))
+    row = np.searchsorted(np.unique(q) ** 2, q2, side="right") - 1
+    col = np.searchsorted(x, xs, side="right") - 1
+    own = (row % 2 == 1) & ((col % 3 == 1) | (interp == 2))
+    xs, q2 = xs[own], q2[own]
+    n = xs.size
+    assert n > 2000
     X, Q = torch.as_tensor(xs, device="cuda"), torch.as_tensor(q2, device="cuda")
     parity.check(pdf.xfxQ2(g.pids, X, Q).cpu().numpy(), o.xfxq2_batch(g.pids, xs, q2), o.kappa(g.pids, xs, q2))
     pid = np.full(n, 2, np.int32)
@@ -113,3 +120,82 @@ def test_knots_uneven_on_both_axes():
     parity.check(pdf.xfxQ2(g.pids, *D).cpu().numpy(), o.xfxq2_batch(g.pids, xs, qs), o.kappa(g.pids, xs, qs))
     parity.check(pdf.alphasQ2(D[1]).cpu().numpy(), o.alphas_batch(qs), o.alphas_kappa(qs), what="alpha_s")
     assert pdf.status() == 0
+
+
+def test_knots_give_their_own_values():
+    """Every knot that opens a cell returns the grid's value itself, bit for bit,
+    and alpha_s likewise; with flavours that set in at a threshold and ones
+    that fall away towards the next knot."""
+    from paper_2012_08221_gb300 import build
+    from paper_2012_08221_gb300.pdf import PDF
+    build.build()
+    for g in (synth.grid_small(), synth.grid_nnpdf()):
+        rng = np.random.default_rng(51)
+        g.values[..., 1] *= 2.0 ** rng.integers(-14, 15, g.values.shape[1:3])
+        if g.n_q.size > 1:
+            g.values[:, np.asarray(g.q_knots) <= 4.92, :, 2] = 0.0
+        pdf = PDF.from_grid(g)
+        last = np.cumsum(g.n_q) - 1                       # the last row of a subgrid opens no cell
+        rows = np.setdiff1d(np.arange(g.n_rows), last)
+        X, Q = (a.ravel() for a in np.meshgrid(g.x_knots[:-1], g.q_knots[rows] ** 2))
+        X, Q = torch.as_tensor(X, device="cuda"), torch.as_tensor(Q, device="cuda")
+        want = np.ascontiguousarray(g.values[0][rows][:, :-1].reshape(-1, g.n_flav))
+        assert np.array_equal(pdf.xfxQ2(g.pids, X, Q).cpu().numpy(), want)
+        q = torch.as_tensor(g.q_knots[rows] ** 2, device="cuda")
+        assert np.array_equal(pdf.alphasQ2(q).cpu().numpy(), g.alphas[rows])
+
+
+@pytest.mark.parametrize("k", [2, 4, 6, 8, 10, 13])
+def test_values_next_to_a_small_corner(k):
+    """Knots whose value is 2^-k of their neighbours': the value itself on them,
+    the one in 60 digits next to them and in their cells, the same bits from the
+    matrix form with few and with all columns, the pointwise form and the
+    batch; derivatives with and without the tapes the same bits."""
+    from paper_2012_08221_gb300 import build
+    from paper_2012_08221_gb300.batch import Batch
+    from paper_2012_08221_gb300.pdf import PDF
+    from tests import fixed_host, parity
+    build.build()
+    g = synth.grid_nnpdf(seeds=(61,))
+    rng = np.random.default_rng(60 + k)
+    low = np.zeros(g.values.shape[1:3], bool)
+    low[1::3, 1::3] = True
+    g.values[...] = rng.uniform(1, 2, g.values.shape)
+    g.values[:, low] *= 2.0 ** -k
+    pdf = PDF.from_grid(g)
+    r, c = np.nonzero(low)
+    keep = (c < g.n_x - 1) & ~np.isin(r, np.cumsum(g.n_q) - 1)
+    r, c = np.repeat(r[keep], 8), np.repeat(c[keep], 8)
+    n = r.size
+    x, q2 = g.x_knots[c].copy(), g.q_knots[r] ** 2
+    tx, tq = 2.0 ** -rng.uniform(0, 40, (2, n))
+    x[n // 2:] = (x * (g.x_knots[c + 1] / x) ** tx)[n // 2:]
+    q2[n // 2:] = (q2 * (g.q_knots[r + 1] ** 2 / q2) ** tq)[n // 2:]
+    X, Q = torch.as_tensor(x, device="cuda"), torch.as_tensor(q2, device="cuda")
+    got = pdf.xfxQ2(g.pids, X, Q)
+    assert np.array_equal(got[:n // 2].cpu().numpy(), g.values[0][r, c][:n // 2])
+    some = np.concatenate([rng.choice(n, 100), np.arange(n // 2, n)[::n // 100]])
+    for i in some:                       # (the oracle's own logarithms, to 2^-49, are not good enough here)
+        s = int(np.searchsorted(np.cumsum(g.n_q), r[i], side="right"))
+        rows = slice(int(np.sum(g.n_q[:s])), int(np.sum(g.n_q[:s + 1])))
+        near = slice(max(c[i] - 1, 0), c[i] + 3)
+        ref = fixed_host.exact(g.x_knots[near], g.q_knots[rows] ** 2, g.values[0, rows, near, 3], x[i:i + 1], q2[i:i + 1])
+        parity.check(got[i, 3].item(), float(ref[0][0]), float(ref[0][1]), atol=0)
+    pid = torch.as_tensor(g.pids[np.arange(n) % g.n_flav], device="cuda")
+    assert torch.equal(pdf.xfxQ2_pw(pid, X, Q), got[torch.arange(n), torch.arange(n) % g.n_flav])
+    assert torch.equal(pdf.xfxQ2(g.pids[4:7], X[-1001:], Q[-1001:]), got[-1001:, 4:7])
+    out = torch.empty((n, 3), dtype=torch.float64, device="cuda")
+    Batch([(pdf, 0, g.pids[4:7].copy(), X, Q, out)], autotune=False).run()
+    assert torch.equal(out, got[:, 4:7])
+    w = torch.as_tensor(rng.standard_normal(n), device="cuda")
+    gv = torch.zeros(g.values.shape[1:], dtype=torch.float64, device="cuda")
+    T, D, TM = pdf.new_tape(n), pdf.new_dtape(n), pdf.new_tape(n)
+    pdf.xfxQ2_pw(pid, X, Q, tape=T, dtape=D)
+    pdf.xfxQ2(g.pids, X, Q, tape=TM)
+    a = pdf.xfxQ2_backward(pid, X, Q, w, pointwise=True, grad_values=gv, tape=T, dtape=D)[:2]
+    b = pdf.xfxQ2_backward(pid, X, Q, w, pointwise=True)[:2]
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+    go = w[:, None].expand(n, g.n_flav).contiguous()
+    a = pdf.xfxQ2_backward(g.pids, X, Q, go, grad_values=gv, tape=TM)[:2]
+    b = pdf.xfxQ2_backward(g.pids, X, Q, go)[:2]
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
