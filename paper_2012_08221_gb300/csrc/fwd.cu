@@ -136,9 +136,11 @@ __global__ void __launch_bounds__(kPwBlock, 5) k_xfxq2_pw(const __grid_constant_
         const bool live = i < n;
         const double xi = live ? x[i] : 0.5, qi = live ? q2[i] : 10.0;
         const int col = live ? pid_col(g, pid[i]) : -1;
-        const FixAxis X = fix_axis_x(g, T, dbits(xi)), Q = fix_axis_q2(g, T, dbits(qi));
-        bool fast = live && X.ok && Q.ok && fm;      // inside the knots, so inside the domain
+        // inside the knots, so inside the domain (32 points outside: no coordinates)
+        bool fast = live && in_x(g, dbits(xi)) && in_q2(g, dbits(qi)) && fm;
         if (__any_sync(kAll, fast)) {
+            const FixAxis X = fix_axis_x(g, T, dbits(xi)), Q = fix_axis_q2(g, T, dbits(qi));
+            fast = fast && X.ok && Q.ok;
             const uint32_t patch0 =
                 fast ? (uint32_t)(Q.cell * g.nxc + X.cell) * (uint32_t)g.nflav + (col >= 0 ? col : 0) : 0u;
             uint32_t off[4];
@@ -227,7 +229,7 @@ __global__ void __launch_bounds__(kBlock) k_alphas(const __grid_constant__ GridD
             const bool bad = !q2_ok(dbits(qi));
             flag_status(g, bad);
             bool oor;
-            const double v = alphas_at(g, grid_tabs(g), bad ? 10.0 : qi, &oor);
+            const double v = alphas_at(g, axis_q2(g, bad ? 10.0 : qi), &oor);
             flag_status(g, oor && !bad, PDF_S_RANGE);
             out[i] = bad ? dnan() : v;
         }
@@ -270,7 +272,7 @@ __global__ void __launch_bounds__(kBlock) k_alphas_grad(GridDev g, const double 
         if (bad) qi = 10.0;
         const Axis Q = axis_q2(g, qi);
         bool oor;
-        const double v = alphas_at(g, grid_tabs(g), qi, &oor);
+        const double v = alphas_at(g, Q, &oor);
         flag_status(g, oor, PDF_S_RANGE);
         bad |= oor;
         const D4 a = ld4(g.acoef + (size_t)Q.cell * 4);

@@ -138,16 +138,16 @@ __global__ void __launch_bounds__(kBlock, SAVE ? 2 : 3) k_lumi(const __grid_cons
         const int64_t e = base + lane;
         const bool live = e < n;
         const Event E = event(live ? e : n - 1, ln_tau, y, flags, ln_mu2, ln_x1, ln_s);
-        const FixAxis Q = fix_axis_log(g, T.wkey, T.qcell, g.nqc, g.qstep, g.wlo, g.whi, E.w);
-        const FixAxis X1 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, g.ulo, g.uhi, E.u1);
-        const FixAxis X2 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, g.ulo, g.uhi, E.u2);
-        bool fast = live && fm && !E.bad && Q.ok && X1.ok && X2.ok;
-        if (__any_sync(kAll, fast)) {
+        bool fast = live && fm && !E.bad && in_logs(g, E.u1, E.u2, E.w);
+        if (__any_sync(kAll, fast)) {                 // (32 events outside: no coordinates)
+            const FixAxis Q = fix_axis_log(g, T.wkey, T.qcell, g.nqc, g.qstep, E.w);
+            const FixAxis X1 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, E.u1);
+            const FixAxis X2 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, E.u2);
             if (SAVE) warp_run_reuse(lane);           // the previous run has left the rows
             const double s = lumi_quads<SAVE>(g, anti.c, fm, B.buf, rows, row, lane, X1, X2, Q, fast);
             if (fast) {
                 bool none = false;
-                if (as) as[e] = fix_alphas(g, Q, none);
+                if (as) as[e] = fix_alphas(g, Q.cell, Q.t, none);
                 fast = !none;
             }
             if (fast) {

@@ -39,15 +39,21 @@ __device__ __forceinline__ LogTabs stage_log_tabs(const GridDev &g, unsigned cha
     return {uk, wk, xc, qc};
 }
 
-// Cell and fixed-point coordinate (value 2^62) of a logarithm z; ok: inside
-// the knot range.  The coordinate is the FP64 one of axis_u / axis_w.
-__device__ __forceinline__ FixAxis fix_axis_log(const GridDev &g, const int64_t *keys, const double2 *cells, int ncell,
-                                                int step, int64_t lo, int64_t hi, double z)
+// Whether both partons and the scale lie in the knot range.
+__device__ __forceinline__ bool in_logs(const GridDev &g, double u1, double u2, double w)
 {
-    const int64_t k = dkey(z);
+    const int64_t a = dkey(u1), b = dkey(u2), c = dkey(w);
+    return (a >= g.ulo) & (a <= g.uhi) & (b >= g.ulo) & (b <= g.uhi) & (c >= g.wlo) & (c <= g.whi);
+}
+
+// Cell and fixed-point coordinate (value 2^62) of a logarithm z inside the knot
+// range.  The coordinate is the FP64 one of axis_u / axis_w.
+__device__ __forceinline__ FixAxis fix_axis_log(const GridDev &g, const int64_t *keys, const double2 *cells, int ncell,
+                                                int step, double z)
+{
     FixAxis A;
-    A.cell = checked_index(g.status, find_cell<int64_t>(keys, ncell, step, k), ncell);
-    A.ok = (k >= lo) & (k <= hi);
+    A.cell = checked_index(g.status, find_cell<int64_t>(keys, ncell, step, dkey(z)), ncell);
+    A.ok = true;
     const double2 c = cells[A.cell];
     const int64_t t = __double2ll_rn((z - c.x) * c.y * 4611686018427387904.0 /* 2^62 */);
     A.t = min(max(t, (int64_t)0), (int64_t)1 << 62);

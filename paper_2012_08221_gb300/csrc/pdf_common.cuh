@@ -278,13 +278,28 @@ struct FixAxis {
     bool ok;
 };
 
+// Whether the bits of a value lie in the knot range.
+__device__ __forceinline__ bool in_x(const GridDev &g, uint64_t b) { return (b >= g.xlo) & (b <= g.xhi); }
+__device__ __forceinline__ bool in_q2(const GridDev &g, uint64_t b) { return (b >= g.qlo) & (b <= g.qhi); }
+
+// The cell of a value's bits.
+__device__ __forceinline__ int cell_x(const GridDev &g, const CoordTabs &T, uint64_t b)
+{
+    return checked_index(g.status, find_cell_guided(T.xbits, g.nxc, g.xstep, T.xguide, g.nxg, g.xgshift, g.xgrun,
+                                                    g.xlo, b), g.nxc);
+}
+__device__ __forceinline__ int cell_q2(const GridDev &g, const CoordTabs &T, uint64_t b)
+{
+    return checked_index(g.status, find_cell_guided(T.qbits, g.nqc, g.qstep, T.qguide, g.nqg, g.qgshift, g.qgrun,
+                                                    g.qlo, b), g.nqc);
+}
+
 __device__ __forceinline__ FixAxis fix_axis_x(const GridDev &g, const CoordTabs &T, uint64_t b)
 {
     FixAxis A;
-    A.cell = checked_index(g.status, find_cell_guided(T.xbits, g.nxc, g.xstep, T.xguide, g.nxg, g.xgshift, g.xgrun,
-                                                      g.xlo, b), g.nxc);
+    A.cell = cell_x(g, T, b);
     const FixCell c = T.xfix[A.cell];
-    A.ok = (b >= g.xlo) & (b <= g.xhi) & (c.K != 0);
+    A.ok = in_x(g, b) & (c.K != 0);
     A.t = fix_coord(fix_log(b, T.inv, T.log), c);
     return A;
 }
@@ -292,54 +307,49 @@ __device__ __forceinline__ FixAxis fix_axis_x(const GridDev &g, const CoordTabs 
 __device__ __forceinline__ FixAxis fix_axis_q2(const GridDev &g, const CoordTabs &T, uint64_t b)
 {
     FixAxis A;
-    A.cell = checked_index(g.status, find_cell_guided(T.qbits, g.nqc, g.qstep, T.qguide, g.nqg, g.qgshift, g.qgrun,
-                                                      g.qlo, b), g.nqc);
+    A.cell = cell_q2(g, T, b);
     const FixCell c = T.qfix[A.cell];
-    A.ok = (b >= g.qlo) & (b <= g.qhi) & (c.K != 0);
+    A.ok = in_q2(g, b) & (c.K != 0);
     A.t = fix_coord(fix_log(b, T.inv, T.log), c);
     return A;
 }
 
 // The axes in FP64 (adjoints, points outside the knots): inside the knot
 // range t is the fixed-point coordinate, so that every kernel places a point
-// at the same t; elsewhere it comes from the FP64 logarithm.
+// at the same t; elsewhere it comes from the FP64 logarithm.  Only the one that
+// is needed is taken.
+__device__ __forceinline__ void axis_coord(const GridDev &g, Axis &A, double z, const FixCell &f, double2 c)
+{
+    A.f = -1;
+    double t;
+    if (A.in && f.K != 0) {
+        A.f = fix_coord(fix_log(dbits(z), g.finv, g.flog), f);
+        t = fix_t(A.f);
+    } else {
+        t = (dlog(g, z) - c.x) * c.y;
+    }
+    make_basis(A, t, g.extrap);
+}
+
 __device__ __forceinline__ Axis axis_x(const GridDev &g, double x)
 {
     const uint64_t b = dbits(x);
-    const FixAxis f = fix_axis_x(g, grid_tabs(g), b);
     Axis A;
-    A.cell = f.cell;
-    A.in = (b >= g.xlo) & (b <= g.xhi);
+    A.cell = cell_x(g, grid_tabs(g), b);
+    A.in = in_x(g, b);
     A.below = b < g.xlo;
-    double t;
-    A.f = f.ok ? f.t : -1;
-    if (f.ok) {
-        t = fix_t(f.t);
-    } else {
-        const double2 c = g.xcell[A.cell];
-        t = (dlog(g, x) - c.x) * c.y;
-    }
-    make_basis(A, t, g.extrap);
+    axis_coord(g, A, x, g.xfix[A.cell], g.xcell[A.cell]);
     return A;
 }
 
 __device__ __forceinline__ Axis axis_q2(const GridDev &g, double q2)
 {
     const uint64_t b = dbits(q2);
-    const FixAxis f = fix_axis_q2(g, grid_tabs(g), b);
     Axis A;
-    A.cell = f.cell;
-    A.in = (b >= g.qlo) & (b <= g.qhi);
+    A.cell = cell_q2(g, grid_tabs(g), b);
+    A.in = in_q2(g, b);
     A.below = b < g.qlo;
-    double t;
-    A.f = f.ok ? f.t : -1;
-    if (f.ok) {
-        t = fix_t(f.t);
-    } else {
-        const double2 c = g.qcell[A.cell];
-        t = (dlog(g, q2) - c.x) * c.y;
-    }
-    make_basis(A, t, g.extrap);
+    axis_coord(g, A, q2, g.qfix[A.cell], g.qcell[A.cell]);
     return A;
 }
 

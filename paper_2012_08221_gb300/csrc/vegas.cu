@@ -129,11 +129,11 @@ __global__ void __launch_bounds__(kBlock, 3) k_vegas(const __grid_constant__ Gri
         const int64_t i = base + lane;
         const bool live = i < n;
         const VegasPoint P = point(live ? i : n - 1);
-        const FixAxis Q = fix_axis_log(g, T.wkey, T.qcell, g.nqc, g.qstep, g.wlo, g.whi, P.w);
-        const FixAxis X1 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, g.ulo, g.uhi, P.u1);
-        const FixAxis X2 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, g.ulo, g.uhi, P.u2);
-        bool fast = live && fm && Q.ok && X1.ok && X2.ok;
+        bool fast = live && fm && in_logs(g, P.u1, P.u2, P.w);
         if (__any_sync(kAll, fast)) {
+            const FixAxis Q = fix_axis_log(g, T.wkey, T.qcell, g.nqc, g.qstep, P.w);
+            const FixAxis X1 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, P.u1);
+            const FixAxis X2 = fix_axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, P.u2);
             const double lum = lumi_quads<false>(g, anti.c, fm, B.buf, rows, row, lane, X1, X2, Q, fast);
             if (fast) add(P, lum);
         }

@@ -199,3 +199,44 @@ def test_values_next_to_a_small_corner(k):
     a = pdf.xfxQ2_backward(g.pids, X, Q, go, grad_values=gv, tape=TM)[:2]
     b = pdf.xfxQ2_backward(g.pids, X, Q, go)[:2]
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("extrap", ["linear", "freeze", "error", "continuation"])
+@pytest.mark.parametrize("n", [1, 32, 64, 2016, 70_016])
+def test_blocks_of_points_outside_the_knots(extrap, n):
+    """Runs of 32 points that all lie outside, between runs that lie inside: the
+    same bits for every point as in a shuffled order, in x*f, the pointwise
+    form and alpha_s; the same luminosity but for the order of its sum of 13
+    pairs of values up to about 3 (13 x 2^-53 x 9 each); the same status."""
+    from paper_2012_08221_gb300 import build
+    from paper_2012_08221_gb300.lumi import DeviceEvents, luminosity
+    from paper_2012_08221_gb300.pdf import PDF
+    build.build()
+    g = synth.grid_set_b()
+    pdf = PDF.from_grid(g, extrap=extrap)
+    rng = np.random.default_rng(70 + n)
+    out = (np.arange(n) // 32) % 2 == 0
+    x = np.exp(rng.uniform(np.log(1e-8), 0, n))
+    q2 = np.exp(rng.uniform(2 * np.log(1.65), 2 * np.log(1e5), n))
+    low = out & (np.arange(n) // 64 % 2 == 0)
+    x[low] *= 1e-10
+    q2[out & ~low] = np.where(rng.uniform(size=n) < 0.5, 0.3, 1e13)[out & ~low]
+    perm = rng.permutation(n)
+    pid = torch.as_tensor(g.pids[np.arange(n) % g.n_flav], device="cuda")
+    X, Q, P = (torch.as_tensor(a, device="cuda") for a in (x, q2, perm))
+
+    def same(a, b):
+        return np.array_equal(a[P].cpu().numpy(), b.cpu().numpy(), equal_nan=True)
+    pdf.status()
+    a = (pdf.xfxQ2(g.pids, X, Q), pdf.xfxQ2_pw(pid, X, Q), pdf.alphasQ2(Q), *pdf.xfxQ2_alphasQ2(g.pids[:3], X, Q))
+    first = pdf.status()
+    b = (pdf.xfxQ2(g.pids, X[P], Q[P]), pdf.xfxQ2_pw(pid[P], X[P], Q[P]), pdf.alphasQ2(Q[P]),
+         *pdf.xfxQ2_alphasQ2(g.pids[:3], X[P], Q[P]))
+    assert all(same(u, w) for u, w in zip(a, b)) and first == pdf.status()
+    ev = synth.events_lhc(n, seed=71)
+    ev.flags[:] = np.where(out, ev.flags | 1, ev.flags & 0)
+    d = DeviceEvents.from_host(ev)
+    e = DeviceEvents(d.ln_tau[P], d.y[P], d.flags[P], d.ln_mu2[P], d.ln_x1[P], d.ln_s)
+    (_, l1, a1), (_, l2, a2) = luminosity(pdf, d), luminosity(pdf, e)
+    assert same(a1, a2)                   # (lanes share an event's pairs: the order of its sum may differ)
+    assert torch.allclose(l1[P], l2, rtol=1e-12, atol=1e-13, equal_nan=True)
