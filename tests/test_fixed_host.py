@@ -168,3 +168,33 @@ def test_alpha_s_cubics():
         assert ok.sum() >= (got.size if r == 0 else got.size // 2)
         assert np.array_equal(got[:w.size - 1][ok[:w.size - 1]], a[:-1][ok[:w.size - 1]])
         assert np.all(fixed_host.error(got, [k[0] for k in ref])[ok] <= 2.0 ** -52 * kap[ok])
+
+
+@pytest.mark.parametrize("j", [3, 5, 7, 8, 9, 10, 11, 13])
+@pytest.mark.parametrize("axis", ["x", "q"])
+def test_narrow_cells_next_to_one(j, axis):
+    """Knots 2^-j / 5 apart up to x = 1 (or from Q^2 = 1 on): there the FP64
+    logarithm is accurate to its own size, the fixed-point one to 2^-59, and a
+    narrow cell magnifies both.  Where fixed point serves, its error against the
+    exact value of the argument is no larger than that of FP64."""
+    rng = np.random.default_rng(600 + j)
+    h = 2.0 ** -j
+    near = 1 - h * np.array([1.0, 0.82, 0.58, 0.4, 0.19, 0.0]) if axis == "x" else 1 + h * np.arange(6) / 5
+    far = np.exp(np.arange(5) * 0.3 + (2 if axis == "x" else -3))
+    x, q2 = (near, far) if axis == "x" else (far, near)
+    fixed, fp64 = [], []
+    for smooth in (False, True):
+        v = rng.uniform(1, 2, (q2.size, x.size))
+        if smooth:
+            v = (2 - x)[None] ** 3 * (1 + 0.1 * np.log(q2))[:, None]
+        px, pq = rng.uniform(x[0], x[-1], 250), rng.uniform(q2[0], q2[-1], 250)
+        got, _ = fixed_host.evaluate(x, q2, v, px, pq)
+        ref = fixed_host.exact(x, q2, v, px, pq)
+        kap = np.array([float(r[1]) for r in ref])
+        fixed.append(fixed_host.error(got[:, 0], [r[0] for r in ref]) / kap)
+        fp64.append(fixed_host.error(got[:, 4], [r[0] for r in ref]) / kap)
+    fixed, fp64 = np.concatenate(fixed), np.concatenate(fp64)
+    served = np.isfinite(fixed)
+    assert served.all() if j <= 5 else True
+    if served.any():
+        assert np.max(fixed[served]) <= np.max(fp64)

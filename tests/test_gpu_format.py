@@ -206,8 +206,8 @@ def test_values_next_to_a_small_corner(k):
 def test_blocks_of_points_outside_the_knots(extrap, n):
     """Runs of 32 points that all lie outside, between runs that lie inside: the
     same bits for every point as in a shuffled order, in x*f, the pointwise
-    form and alpha_s; the same luminosity but for the order of its sum of 13
-    pairs of values up to about 3 (13 x 2^-53 x 9 each); the same status."""
+    form and alpha_s; the same luminosity but for the order of its sum of 11
+    pairs of values up to about 3 (11 x 2^-53 x 9 each); the same status."""
     from paper_2012_08221_gb300 import build
     from paper_2012_08221_gb300.lumi import DeviceEvents, luminosity
     from paper_2012_08221_gb300.pdf import PDF
