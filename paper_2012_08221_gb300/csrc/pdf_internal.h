@@ -16,6 +16,7 @@ struct pdfgpu_grid {
     int sm_count = 0;
     pdfgpu::GridDev d{};            // device view (pointers into `blocks`)
     std::vector<void *> blocks;     // device allocations owned by the grid
+    size_t fixed_bytes = 0;         // of the fixed-point patches among them
     bool bound = false;             // coefficients built
     bool has_alphas = false;
     std::vector<int32_t> pids;      // host copy

@@ -48,10 +48,10 @@ def test_points_of_all_ones_are_domain_errors(checked):
 
 @pytest.mark.parametrize("interp", [1, 2])
 def test_straight_lines_next_to_far_larger_values(interp):
-    """Log-bilinear, and straight lines in a short Q subgrid: knots 2^40 above a
+    """Log-bilinear, and straight lines in a short Q subgrid: knots 2^25 above a
     cell's own on the rows and columns that it does not read.  Values and
     derivatives of the points whose own knots are the small ones (between 1 and
-    2^80 the value follows the rounding of t), against the oracle."""
+    2^50 the value follows the rounding of t), against the oracle."""
     from oracle.oracle import OracleGrid
     from paper_2012_08221_gb300 import build
     from paper_2012_08221_gb300.pdf import PDF
@@ -61,9 +61,9 @@ def test_straight_lines_next_to_far_larger_values(interp):
     x = synth.log_knots(1e-4, 1.0, 12)
     q, nq = synth.subgrid_knots([1.3, 4.0, 90.0, 500.0], [3, 3, 3])
     v = rng.uniform(1, 2, (1, q.size, x.size, 3))
-    v[:, ::3] *= 2.0 ** 40                       # the first row of every subgrid; the others beside it
+    v[:, ::3] *= 2.0 ** 25                       # the first row of every subgrid; the others beside it
     if interp == 1:
-        v[:, :, ::3] *= 2.0 ** 40
+        v[:, :, ::3] *= 2.0 ** 25
     g = synth.Grid(x, nq, q, np.array([-1, 1, 2], np.int32), v, np.full(q.size, 0.2), "steps")
     pdf, o = PDF.from_grid(g, interp=interp), OracleGrid.from_synth(g, interp=interp)
     n = 20_011
@@ -97,7 +97,7 @@ def test_knots_uneven_on_both_axes():
     from tests import parity
     build.build()
     rng = np.random.default_rng(41)
-    steps = 2.0 ** -np.array([2, 8, 2, 10, 3, 13, 3, 5, 2, 12, 2])
+    steps = 2.0 ** -np.array([2, 8, 2, 15, 2, 13, 3, 5, 2, 14, 2])
     x = np.exp(np.concatenate([[0.0], np.cumsum(steps)]) - 4.0)
     w = np.concatenate([[0.0], np.cumsum(steps[::-1])])
     qa, qb = np.exp(1.0 + w / 2), np.exp(1.0 + w[-1] / 2 + w / 2)
@@ -240,3 +240,41 @@ def test_blocks_of_points_outside_the_knots(extrap, n):
     (_, l1, a1), (_, l2, a2) = luminosity(pdf, d), luminosity(pdf, e)
     assert same(a1, a2)                   # (lanes share an event's pairs: the order of its sum may differ)
     assert torch.allclose(l1[P], l2, rtol=1e-12, atol=1e-13, equal_nan=True)
+
+
+def test_a_grid_loads_where_only_the_fp64_table_fits():
+    """Device memory for the FP64 table and the values but not for the
+    fixed-point table beside them: the grid loads, leaves the rest of the
+    memory alone, and gives the oracle's values; with plenty of memory the table
+    is there, and freeing the grid gives it back."""
+    from oracle.oracle import OracleGrid
+    from paper_2012_08221_gb300 import build
+    from paper_2012_08221_gb300.pdf import PDF
+    from tests import parity
+    build.build()
+    g = synth.grid_nnpdf(seeds=tuple(range(81, 81 + 32)))
+    pdf, o = PDF.from_grid(g), OracleGrid.from_synth(g)          # kernels and context loaded
+    cells = (g.n_x - 1) * int(np.sum(g.n_q - 1)) * g.n_flav * g.n_members
+    table = cells * 16 * 8
+    del pdf
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free0 = torch.cuda.mem_get_info()[0]
+    pdf = PDF.from_grid(g)
+    assert 2 * table <= free0 - torch.cuda.mem_get_info()[0] < 2.2 * table
+    x, q2, _ = synth.queries_nnpdf(3001, seed=82)
+    X, Q = torch.as_tensor(x, device="cuda"), torch.as_tensor(q2, device="cuda")
+    full = pdf.xfxQ2(g.pids, X, Q, member=5)
+    del pdf
+    torch.cuda.synchronize()
+    assert abs(free0 - torch.cuda.mem_get_info()[0]) < 0.1 * table
+    for left in (2 * table + g.values.nbytes // 3, 4 * table):
+        fill = torch.empty(int(torch.cuda.mem_get_info()[0] - left) // 8, dtype=torch.float64, device="cuda")
+        before = torch.cuda.mem_get_info()[0]
+        pdf = PDF.from_grid(g)
+        assert before - torch.cuda.mem_get_info()[0] < 1.2 * table
+        got = pdf.xfxQ2(g.pids, X, Q, member=5)
+        parity.check(got.cpu().numpy(), o.xfxq2_batch(g.pids, x, q2, member=5), o.kappa(g.pids, x, q2, member=5))
+        parity.check(full.cpu().numpy(), o.xfxq2_batch(g.pids, x, q2, member=5), o.kappa(g.pids, x, q2, member=5))
+        del pdf, fill
+        torch.cuda.empty_cache()
