@@ -278,3 +278,47 @@ def test_a_grid_loads_where_only_the_fp64_table_fits():
         parity.check(full.cpu().numpy(), o.xfxq2_batch(g.pids, x, q2, member=5), o.kappa(g.pids, x, q2, member=5))
         del pdf, fill
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("n", [1, 33, 3001])
+def test_luminosity_with_an_unpaired_flavour(n):
+    """A flavour without an antiflavour next to b quarks that set in at their
+    threshold (patches that keep FP64) and events outside the knots: lum, the
+    saved factors of the paired flavours, and the gradient from the saved and
+    from recomputed factors, which leaves the unpaired flavour alone."""
+    from oracle.oracle import OracleGrid
+    from paper_2012_08221_gb300 import build
+    from paper_2012_08221_gb300.lumi import DeviceEvents, luminosity, luminosity_backward
+    from paper_2012_08221_gb300.pdf import PDF
+    from tests import parity
+    from tests.test_gpu_lumi import _event_logs
+    build.build()
+    full = synth.grid_nnpdf(seeds=(91,))
+    v = np.concatenate([full.values, 0.7 * full.values[..., 3:4]], axis=3)
+    pids = np.append(full.pids, 22).astype(np.int32)
+    v[:, np.asarray(full.q_knots) <= 4.92, :, 1] = v[:, np.asarray(full.q_knots) <= 4.92, :, 11] = 0.0
+    g = synth.Grid(full.x_knots, full.n_q, full.q_knots, pids, v, full.alphas, "unpaired")
+    pdf, o = PDF.from_grid(g), OracleGrid.from_synth(g)
+    ev = synth.events_lhc(n, seed=92, tail=0.2)
+    d = DeviceEvents.from_host(ev)
+    save = torch.full((n, 2, g.n_flav), float("nan"), dtype=torch.float64, device="cuda")
+    L, lum, _ = luminosity(pdf, d, save_p=save)
+    Lr, lumr, _ = o.lumi(ev)
+    u1, u2, w = _event_logs(ev, n)
+    kap, f = [], []
+    for k, u in enumerate((u1, u2)):
+        x, q2 = np.exp(u), np.exp(w)
+        f.append(o.xfxq2_batch(pids, x, q2))
+        kap.append(o.kappa(pids, x, q2))
+        parity.check(save[:, k, :13].cpu().numpy(), f[k][:, :13], kap[k][:, :13], what=f"saved parton {k}")
+    a = slice(0, 13)
+    terms = kap[0][:, a] * np.abs(f[1][:, 12::-1]) + np.abs(f[0][:, a]) * kap[1][:, 12::-1] + \
+        kap[0][:, a] * kap[1][:, 12::-1]
+    parity.check(lum.cpu().numpy(), lumr, terms.sum(1), what="lum")
+    ref = o.lumi_dgrid(ev)
+    tol = 1e-9 * np.maximum(np.abs(ref), o.lumi_dgrid(ev, absval=True)) + 1e-300      # the suite's gradient rule
+    for saved in (save, None):
+        gv = torch.zeros(g.values.shape[1:], dtype=torch.float64, device="cuda")
+        luminosity_backward(pdf, d, 1.0, gv, saved_p=saved)
+        got = gv.cpu().numpy()
+        assert np.all(np.abs(got - ref) <= tol) and not got[..., 13].any()
