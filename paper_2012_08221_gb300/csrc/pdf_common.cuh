@@ -35,7 +35,6 @@ namespace pdfgpu {
 
 constexpr int kLogBits = 10;              // table index: top 10 mantissa bits
 constexpr int kLogTab = 1 << kLogBits;
-constexpr int kMaxStencilRows = 4;
 
 PDF_HD uint64_t dbits(double x)
 {
@@ -211,14 +210,14 @@ __device__ __forceinline__ int checked_index(unsigned *, int i, int) { return i;
 // Per-axis local coordinate and basis of one query.
 struct Axis {
     int cell;
-    double t, b2, b3;     // basis (1, t, b2, b3)
+    double t;
     double h;             // Horner factor: t inside, 1 outside
     bool in;              // inside the knot range
     bool below;           // below the first knot
     int64_t f;            // fixed-point t (value 2^62), or -1 where FP64 serves
 };
 
-// Basis of the patch polynomial along one axis.  Inside the knot range
+// Basis of the patch polynomial along one axis (horner).  Inside the knot range
 // (1, t, t^2, t^3).  Outside: linear continuation (1, t, t, t), i.e.
 // P(0) + t (P(1) - P(0)); frozen at the edge, t becomes 0 (below) or 1
 // (above), the edge knot of the edge cell.  The error mode is handled by the
@@ -227,10 +226,6 @@ __device__ __forceinline__ void make_basis(Axis &A, double t, int extrap)
 {
     if (!A.in && extrap == PDF_EXTRAP_FREEZE) t = A.below ? 0.0 : 1.0;
     A.t = t;
-    double t2 = t * t;
-    double t3 = t2 * t;
-    A.b2 = A.in ? t2 : t;
-    A.b3 = A.in ? t3 : t;
     A.h = A.in ? t : 1.0;
 }
 
