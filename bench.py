@@ -335,7 +335,9 @@ def peaks():
 # FP64 FMA issue rate per SM per clock on GB300: ncu reports a peak of 304
 # DFMA thread-instructions per cycle for 152 SMs.
 DFMA_PER_SM_CLK = 2
-IMAD_WIDE_PER_SM_CLK = 32        # distinct operands, measured
+# 32 x 32 + 64-bit multiply-adds per SM per clock: pdf_probe_wide_multiply
+# measures 63 on chains with operands of their own.
+IMAD_WIDE_PER_SM_CLK = 64
 
 
 def fp64_derived_peak(sm_count):
@@ -374,7 +376,7 @@ def main():
 
     from paper_2012_08221_gb300 import build, synth, work
     build.build()
-    from paper_2012_08221_gb300.pdf import PDF, fp64_mixed, fp64_mma_peak, fp64_peak
+    from paper_2012_08221_gb300.pdf import PDF, fp64_mixed, fp64_mma_peak, fp64_peak, WIDE_MODES, wide_multiply_peak
 
     rank, world, local = env_rank()
     torch.cuda.set_device(local)
@@ -391,6 +393,7 @@ def main():
         return reduce_max(v, world, dev)
 
     probe = fp64_peak()                             # FLOP/s, FMA chains (burst)
+    wide_probe = {m: wide_multiply_peak(m) / 1e12 for m in WIDE_MODES}
     mma_probe = {"m8n8k4_tflops": fp64_mma_peak("m8n8k4") / 1e12,
                  **{k + "_tflops": v / 1e12 for k, v in fp64_mixed().items()}}
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
@@ -470,6 +473,9 @@ def main():
                 "peak_source": f"derived: {sms} SMs x {IMAD_WIDE_PER_SM_CLK} products/clk x {peak_mhz:.0f} MHz; "
                                f"FP64: {sms} SMs x {DFMA_PER_SM_CLK} DFMA/clk x 2 flop x {peak_mhz:.0f} MHz "
                                f"(max SM clock)",
+                "wide_multiply_probe": {**wide_probe, "unit": "Tproduct/s",
+                                        "what": "integer multiply-add chains measured in this run "
+                                                "(pdf_probe_wide_multiply), by how they share operands"},
                 "probe": {"value": probe / 1e12, "unit": "TFLOP/s",
                           "what": "FP64 FMA chains measured in this run (pdf_probe_fp64_peak)"},
                 "fp64_tensor_probe": {**mma_probe,

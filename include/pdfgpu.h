@@ -495,6 +495,14 @@ int pdf_probe_fp64_mma_peak(int32_t shape, double *flops);
  * sum) says the two share one pipe.  Beyond the paper.  Synchronous. */
 int pdf_probe_fp64_mixed(double *dfma_flops, double *dmma_flops, double *mixed_flops);
 
+/* Rate of this GPU's 32 x 32 + 64-bit integer multiply-add in products per
+ * second, from eight independent chains per thread timed with CUDA events.
+ * mode 0: all instructions with the same two operands, 1: every chain with two
+ * of its own, 2: all pairs of eight operands by eight; PDF_E_ARG otherwise.
+ * Beyond the paper: the denominator of the x*f kernel's roofline.
+ * Synchronous. */
+int pdf_probe_wide_multiply(int32_t mode, double *products);
+
 /* (Beyond the paper: a test hook.)  The kernels' natural log (table-driven argument reduction after
  * P. T. P. Tang, ACM TOMS 16 (1990) 378, with a degree-5 series for
  * ln(1+r), |r| <= 2^-11) applied to n DEVICE doubles: out[i] = ln(in[i]) for

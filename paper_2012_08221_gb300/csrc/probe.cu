@@ -293,3 +293,80 @@ extern "C" int pdf_probe_fp64_mixed(double *dfma_flops, double *dmma_flops, doub
     *mixed_flops = 2.0 * half / (ms[2] * 1e-3);
     return PDF_OK;
 }
+
+// ------------------------------------------------- integer multiply-add probe
+//
+// Rate of the 32 x 32 + 64-bit multiply-add that the fixed-point patches are
+// made of, from eight independent chains per thread: all instructions with the
+// same two operands (MODE 0), every chain with two of its own (1), or every
+// pair of eight operands by eight in turn (2: registers meet in all pairings, so
+// that bank conflicts show).
+
+namespace {
+
+template <int MODE>
+__global__ void k_wide_chains(long long *out, int iters, int seed)
+{
+    int a[kChains], b[kChains];
+    long long acc[kChains];
+#pragma unroll
+    for (int k = 0; k < kChains; ++k) {
+        a[k] = seed * (k + 3) + (int)threadIdx.x;
+        b[k] = seed * (k + 5) - (int)threadIdx.x;
+        acc[k] = k;
+    }
+    for (int it = 0; it < iters; ++it) {
+#pragma unroll
+        for (int r = 0; r < kChains; ++r)
+#pragma unroll
+            for (int k = 0; k < kChains; ++k)
+                asm volatile("mad.wide.s32 %0, %1, %2, %0;"
+                             : "+l"(acc[k])
+                             : "r"(a[MODE ? k : 0]),
+                               "r"(b[MODE == 2 ? (k + r) % kChains : MODE ? k : 0]));
+    }
+    long long s = 0;
+#pragma unroll
+    for (int k = 0; k < kChains; ++k) s += acc[k];
+    out[blockIdx.x * blockDim.x + threadIdx.x] = s;
+}
+
+}  // namespace
+
+extern "C" int pdf_probe_wide_multiply(int32_t mode, double *products)
+{
+    PDF_TRACE("pdf_probe_wide_multiply");
+    pdfgpu::clear_error();
+    if (!products) return pdfgpu::fail(PDF_E_ARG, "null output");
+    if (mode < 0 || mode > 2) return pdfgpu::fail(PDF_E_ARG, "mode must be 0..2");
+    int dev = 0, sms = 0;
+    PDF_CUDA(cudaGetDevice(&dev));
+    PDF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int block = 256, per_sm = 4, iters = 2048;
+    const int blocks = sms * per_sm;
+    long long *buf = nullptr;
+    int rc = pdfgpu::dev_malloc((void **)&buf, (size_t)blocks * block * sizeof(long long), "probe buffer");
+    if (rc) return rc;
+    const auto k = mode == 2 ? k_wide_chains<2> : mode == 1 ? k_wide_chains<1> : k_wide_chains<0>;
+    cudaEvent_t e0, e1;
+    cudaEventCreate(&e0);
+    cudaEventCreate(&e1);
+    k<<<blocks, block>>>(buf, 8, 12345);
+    float best = 1e30f;
+    for (int rep = 0; rep < 3; ++rep) {
+        cudaEventRecord(e0);
+        k<<<blocks, block>>>(buf, iters, 12345);
+        cudaEventRecord(e1);
+        cudaEventSynchronize(e1);
+        float ms = 0;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (ms < best) best = ms;
+    }
+    cudaError_t err = cudaGetLastError();
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    cudaFree(buf);
+    if (err != cudaSuccess) return pdfgpu::cuda_fail(err, "probe kernel");
+    *products = (double)kChains * kChains * iters * blocks * block / (best * 1e-3);
+    return PDF_OK;
+}

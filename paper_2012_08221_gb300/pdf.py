@@ -401,3 +401,15 @@ def fp64_mixed() -> dict:
     f, m, x = C.c_double(), C.c_double(), C.c_double()
     check("pdf_probe_fp64_mixed", lib().pdf_probe_fp64_mixed(C.byref(f), C.byref(m), C.byref(x)))
     return {"dfma": f.value, "dmma": m.value, "mixed": x.value}
+
+
+WIDE_MODES = ("shared", "own", "all_pairs")
+
+
+def wide_multiply_peak(mode: str = "own") -> float:
+    """Measured rate of the 32 x 32 + 64-bit integer multiply-add of the current
+    GPU in products per second: all instructions with the same two operands,
+    each chain with its own, or all pairs of eight operands by eight."""
+    v = C.c_double()
+    check("pdf_probe_wide_multiply", lib().pdf_probe_wide_multiply(WIDE_MODES.index(mode), C.byref(v)))
+    return v.value

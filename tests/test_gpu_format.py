@@ -322,3 +322,15 @@ def test_luminosity_with_an_unpaired_flavour(n):
         luminosity_backward(pdf, d, 1.0, gv, saved_p=saved)
         got = gv.cpu().numpy()
         assert np.all(np.abs(got - ref) <= tol) and not got[..., 13].any()
+
+
+def test_wide_multiply_probe():
+    """The rate that the x*f roofline divides by: 64 products per clock and SM
+    (within a tenth on chains with operands of their own, less where all pairs
+    of operands meet), at the largest clock or below it."""
+    from paper_2012_08221_gb300 import build
+    from paper_2012_08221_gb300.pdf import WIDE_MODES, wide_multiply_peak
+    build.build()
+    peak = 64 * 2.07e9 * torch.cuda.get_device_properties(0).multi_processor_count
+    rate = {m: wide_multiply_peak(m) for m in WIDE_MODES}
+    assert 0.5 * peak < rate["all_pairs"] <= rate["own"] <= 1.01 * peak and rate["own"] <= 1.01 * rate["shared"]
