@@ -46,9 +46,12 @@ struct BatchReq {
     int64_t tile0;
 };
 
+// (three blocks of 256 threads per SM at 80 registers; with staged tables 76
+// bytes of them spilled)
 template <int QPT, bool STAGE>
-__global__ void __launch_bounds__(256, 3) k_batch(const GridDev *__restrict__ grids, const BatchReq *__restrict__ reqs, int nreq,
-                        int64_t ntiles, unsigned long long *ticket)
+__global__ void __launch_bounds__(256, 3) k_batch(const GridDev *__restrict__ grids,
+                                                  const BatchReq *__restrict__ reqs, int nreq, int64_t ntiles,
+                                                  unsigned long long *ticket)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ GridDev sg;

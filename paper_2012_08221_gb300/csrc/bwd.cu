@@ -467,9 +467,8 @@ __global__ void __launch_bounds__(kAccWarps * 32) k_bwd_accum(GridDev g, const d
 // The matrix form (a shared list of up to kMaxSortedPids flavour columns,
 // gout [n][npid]) sorts the points by cell only: every column of a point
 // accumulates in the same bin, lane 4n + m of a half-warp keeping
-// G_a[n][m] for every column a.  dL/dx and dL/dQ^2 take the derivative of
-// one combined patch, sum_a g_a C_a (16 FMA per column), instead of one
-// derivative per column (the result is linear in the coefficients).
+// G_a[n][m] for every column a.  dL/dx and dL/dQ^2 sum the columns'
+// derivatives, taken in fixed point from the patches (k_bwd_rec_m).
 
 constexpr int kMaxSortedPids = 16;
 

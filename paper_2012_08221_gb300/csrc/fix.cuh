@@ -1,7 +1,8 @@
 // Fixed-point evaluation of the interpolant.
 //
 // The FP64 pipe of this GPU issues 2 FMAs per clock and SM; IMAD.WIDE (32 x
-// 32 + 64 bits) issues 64.  Inside the knot range a patch is therefore
+// 32 + 64 bits) issues 64 (pdf_probe_wide_multiply: 63, and 57 where all pairs
+// of operands meet).  Inside the knot range a patch is therefore
 // evaluated in 64-bit integers: the 16 monomial coefficients of the patch
 // about the cell's centre, scaled by the power of two above the largest of
 // them (a block exponent), against the 16 products of the powers of the two
@@ -16,14 +17,19 @@
 //                                             E: max |coefficient| < 2^E
 //   sums of coefficient x weight              value 2^(59 - E)
 //   logarithms                                value 2^60 modulo 16
-// Errors: a patch value is within about 2^-57 of the largest coefficient
-// (FP64 Horner: several roundings of 2^-53), a logarithm within about 2^-59
-// absolute (FP64: 2^-49 at |ln x| = 16 ... 32), so results are closer to the
-// exact interpolant than in FP64.  Integer sums do not depend on their order:
-// every kernel gives the same bits however it splits a patch over lanes.
-// Everything else (points outside the knots, patches whose scale the block
-// exponent cannot hold, cells too narrow or too wide for the logarithm's
-// format) takes the FP64 path.
+// Errors: a sum is off by about 2^(E - 57) anywhere in the cell, what the build
+// leaves by at most 2^(E - 53) (uneven cells; 2^(E - 58) on even ones), a
+// logarithm by about 2^-59 absolute.  FP64 is off by several 2^-53 of the terms
+// at the point, and its logarithm by 2^-53 |ln x| (2^-49 at 16 ... 32), which a
+// cell's width magnifies.  What FP64 does better keeps FP64: values on the lower
+// edges of a patch that is small there (fix_patch, fix_limit; knots come out to
+// the last bit in either form), patches that the block exponent or the build
+// cannot hold, cells too wide or too narrow (fix_cell in grid.cu), points
+// outside the knots.  At a given t a weak patch (see kFixStrong) is still less
+// accurate next to its lower edges than the FP64 form would be; at a given x and
+// Q^2 it is more accurate.
+// Integer sums do not depend on their order: every kernel gives the same bits
+// however it splits a patch over lanes.
 #pragma once
 
 // Included by pdf_common.cuh, after the bit helpers it uses.

@@ -62,13 +62,10 @@ __global__ void __launch_bounds__(kBlock, WHOLE ? 3 : 2) k_xfxq2(const __grid_co
     if (lane == 0) bulk_wait_all();
 }
 
-// DT (with TAPE): also keep each point's derivatives in x and Q^2, computed
-// with the value from the same rows (quad_patch_d) and taken through the chain
-// rule here, where the FP64 pipe is idle, in dtape[i] = (dP/dx, dP/dQ^2)
-// (zeros for an absent pid), and the point's bin
-// in the pointwise sorted adjoint in dbins[i] (-1 for none).
+// One point of the pointwise form in FP64.
 __device__ __forceinline__ void slow_point_pw(const GridDev &g, const double *cm, const unsigned char *fm, int col,
-                                           double xi, double qi, int64_t i, double *out, double *tape, double *dtape, int *dbins, int nbins)
+                                              double xi, double qi, int64_t i, double *out, double *tape,
+                                              double *dtape, int *dbins, int nbins)
 {
     bool bad = !(x_ok(dbits(xi)) && q2_ok(dbits(qi)));
     flag_status(g, bad);
@@ -101,8 +98,15 @@ __device__ __forceinline__ void slow_point_pw(const GridDev &g, const double *cm
     out[i] = bad ? dnan() : v;
 }
 
-// (five blocks of 128 threads per SM: 1351 us per pointwise fit step, two of
-// 256 1364, six of 128 with spills 1385)
+// Pointwise form: one flavour per point.  DT (with TAPE): also keep each point's
+// derivatives in x and Q^2, computed with the value from the same rows
+// (quad_patch_d) and taken through the chain rule here, where the FP64 pipe is
+// idle, in dtape[i] = (dP/dx, dP/dQ^2) (zeros for an absent pid), and the
+// point's bin in the pointwise sorted adjoint in dbins[i] (-1 for none).
+// Five blocks of 128 threads per SM, at 96 registers (with both tapes 160 bytes
+// of them spilled, 104 with one, 100 plain): 1351 us per pointwise fit step; two
+// blocks of 256 1364, six of 128, which spill more, 1385.  With the rules of
+// fix_limit 1356.
 constexpr int kPwBlock = 128;
 
 template <bool TAPE, bool DT, bool STAGE>
@@ -182,7 +186,7 @@ __global__ void __launch_bounds__(kPwBlock, 5) k_xfxq2_pw(const __grid_constant_
     if (B.qn) drain();
 }
 
-// alpha_s, one point per lane (fix_alphas): 1e7 points 286 -> 93 us (FP64
+// alpha_s, one point per lane (fix_alphas): 1e7 points 286 -> 94.5 us (FP64
 // pipe 82 % busy before; now 56 % of the issue slots, the logarithm and the table
 // look-ups in shared memory); points outside the Q range or the
 // domain are queued per warp and evaluated 32 at a time.

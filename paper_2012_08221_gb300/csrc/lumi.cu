@@ -1,8 +1,9 @@
 // Fused parton-luminosity workload (PDFFlow Sec. 3.1-3.2: the integrand maps
 // random numbers to x1, x2 and the scale, calls xfxQ2 twice and multiplies
-// the PDFs into the luminosity).  One thread per event does the kinematics
-// in log variables, one Q search shared by both partons and by alpha_s, two
-// x searches, 2 x F patch contractions and the flavour-paired product sum.
+// the PDFs into the luminosity).  A warp takes 32 events: each lane does the
+// kinematics of its own in log variables, one Q search shared by both partons
+// and by alpha_s, and two x searches; quads of lanes evaluate the 2 x F patches
+// of their four events (lumi_eval.cuh).
 #include <math.h>
 
 #include <algorithm>
@@ -90,8 +91,9 @@ __device__ __forceinline__ double slow_event(const GridDev &g, const signed char
 // [event][parton][flavour] (the rows of 32 events leave as one run).  Without
 // `partials` (the adjoint's recomputation) no status bit is set either.  2e7
 // events x 26 patches, 5 % of the events outside the knots: 13.9 ms in FP64
-// (pipe 96 % busy), 5.9 ms here (57 % of the FP64 pipe, for the pairs and the tail).  Three
-// blocks per SM at 80 registers; with the wider rows of SAVE two are faster.
+// (pipe 96 % busy), 5.9 ms here (57 % of the FP64 pipe, for the pairs and the
+// tail).  Three blocks per SM at 80 registers, 176 bytes of them spilled; with
+// the wider rows of SAVE two are faster.
 template <bool SAVE>
 __global__ void __launch_bounds__(kBlock, SAVE ? 2 : 3) k_lumi(const __grid_constant__ GridDev g,
                                                     const __grid_constant__ Cols anti, int member,

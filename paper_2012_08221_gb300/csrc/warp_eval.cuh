@@ -9,17 +9,22 @@
 // reduce-scatter of three exchanges that leaves each lane its own point's
 // patch.  The weights of a point are computed by its own lane and reach the
 // quad through a swizzled 4 KB buffer per warp.
-// What bounds it now is a mix: per flavour and 32 points 48 IMAD.WIDE (4
-// cycles each of a sub-core with distinct operands: 45 % of the time), about
-// 75 other integer instructions (2 cycles each) and 2 FP64 instructions for
-// the conversion of the result; the L1's data path is 50 % busy, and the
-// 24 warps that 80 registers allow wait for the rows from L2 in between.  1e7 points x 13 flavours of the 196 x 50 grid:
-// 3656 us with FP64 Horner patches (FP64 pipe 95 % busy), 1371 us here.
+// What bounds it now is no single unit: per flavour and 32 points 48 IMAD.WIDE
+// (2 cycles each of a sub-core: 22 % of the time), about 75 other integer
+// instructions and 2 FP64 instructions for the conversion of the result (issue
+// slots 42 % busy); the L1's data path is 50 % busy, and the 24 warps that 80
+// registers allow wait for the rows from L2 and for their own chains.  1e7
+// points x 13 flavours of the 196 x 50 grid: 3656 us with FP64 Horner patches
+// (FP64 pipe 95 % busy), 1389 us here (1369 without the rules of fix_limit, whose
+// operand spills 12 bytes).
 //
 // Points outside the knots (or in cells or patches that the format does not
 // hold) are collected in a queue per warp and evaluated 32 at a time in FP64,
 // so that a few of them do not make every warp run both paths (1e6 points x 3
-// flavours with 5 % outside under the continuation: 475 -> 105 us).
+// flavours with 5 % outside under the continuation: 475 -> 103 us).  A query that
+// mostly outside pays for both: it is slower than FP64 alone was from two thirds
+// of the points outside on (1e6 points x 13 flavours 380 -> 451 us at 95 %, 386
+// with all of them outside; alpha_s 36 -> 44; 1e6 events 735 -> 935 and 769).
 #pragma once
 
 #include "pdf_common.cuh"
