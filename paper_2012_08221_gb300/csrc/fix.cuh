@@ -18,8 +18,8 @@
 //   sums of coefficient x weight              value 2^(59 - E)
 //   logarithms                                value 2^60 modulo 16
 // Errors: a sum is off by about 2^(E - 57) anywhere in the cell, what the build
-// leaves by at most 2^(E - 53) (uneven cells; 2^(E - 58) on even ones), a
-// logarithm by about 2^-59 absolute.  FP64 is off by several 2^-53 of the terms
+// leaves by 2^(E - 57) on even cells and up to 2^(E - 53) at the limit of those
+// it serves (kFixBuild), a logarithm by about 2^-59 absolute.  FP64 is off by several 2^-53 of the terms
 // at the point, and its logarithm by 2^-53 |ln x| (2^-49 at 16 ... 32), which a
 // cell's width magnifies.  What FP64 does better keeps FP64: values on the lower
 // edges of a patch that is small there (fix_patch, fix_limit; knots come out to
@@ -203,12 +203,12 @@ constexpr int kFixBias = 80;
 constexpr int kFixWeak = 128;
 constexpr int kFixNone = 255;
 
-// On a lower edge: t < 2^-16 on either axis.  There the FP64 form, which expands
+// On a lower edge: t < 2^-14 on either axis.  There the FP64 form, which expands
 // about the lower corner, gives the values on the knots to the last bit, and
 // the fixed-point form's error follows the patch's largest coefficient: a weak
 // patch (fix_patch) then takes FP64.  The limit is the least exponent byte that
 // does so at the point.
-constexpr int kFixEdge = 1 << 14;         // 2^-16 in the upper word of a t (value 2^62)
+constexpr int kFixEdge = 1 << 16;         // 2^-14 in the upper word of a t (value 2^62)
 PDF_HD int fix_limit(int64_t tx, int64_t tq)
 {
     return fix_hi(tx) < kFixEdge || fix_hi(tq) < kFixEdge ? kFixWeak : kFixNone;
@@ -240,26 +240,32 @@ __device__ __forceinline__ void fix_ld(const unsigned char *p, int c[8])
 //    argument decides: FP64's logarithm moves the value by 2^-53 |ln x| / width
 //    of 2^E, more than 2^(E - 54) anywhere; fixed point's by 2^(E - 59) /
 //    width.  Largest error of the value itself, FP64 / fixed point, cells of
-//    0.1 at ln x = -5 with the corner 2^-k of the rest: k = 4 1e-13 / 1e-15, 8
-//    2e-12 / 2e-14.  (The patch alone, at a given t above 2^-16: 8e-15 / 7e-16
-//    and 1e-14 / 1e-14.)
-//  - 2^8 below (a flavour that sets in at a threshold knot), or with a stencil
+//    0.1 at ln x = -5 with the corner 2^-k of the rest: k = 4 1e-13 / 1e-15, 6
+//    8e-13 / 6e-15.  (The patch alone, at a given t: 8e-15 / 7e-16, 1e-14 /
+//    4e-15.)
+//  - 2^6 below (a flavour that sets in at a threshold knot), or with a stencil
 //    2^12 above the corner, the patch keeps FP64.
-// Of the 196 x 50 grid's patches 2.8 % are weak (by area), 0.5 % at 2^-5 and
-// below; a limit at 2^-4 of the edges cost 3.5 % there and 11 % with few
-// flavours per point.
+// Of the 196 x 50 grid's patches 2.8 % are weak (by area), 0.005 % are 2^6
+// below.  Where the edge ends costs: at 2^-14 nothing that shows, at 2^-10 the
+// matrix-form fit step 3 % and the luminosity 2 % (one point with a weak patch
+// keeps its warp), at 2^-4 x*f 3.5 % and 400 batched requests 11 %.
 constexpr int kFixStrong = 1;
-constexpr int kFixCorner = 8;
+constexpr int kFixCorner = 6;
 constexpr int kFixStencil = 12;
 PDF_HD int fix_exponent(double v) { return ((int)(dbits(v) >> 52) & 0x7FF) - 1022; }   // |v| < 2^this
 
 // What the build leaves in a patch is about 2^(Ev - 60 + spreads) for stencil
 // values below 2^Ev: with interval ratios 2^r on both axes that is 2^(2 r),
-// and smooth values have coefficients (2^E) that do not grow with it.  Patches
-// where it passes 2^(E - 53) keep FP64 (ratios from about 2^6 on; a cell
-// 2^12 times its neighbours on both axes was off by 8e-12 of its values'
-// size).
-constexpr int kFixBuild = 7;
+// and smooth values have coefficients (2^E) that do not grow with it; steep ones
+// have a stencil far above the cell.  Patches where it passes 2^(E - 54) keep
+// FP64 (ratios from about 2^6 on; a cell 2^12 times its neighbours on both axes
+// was off by 8e-12 of its values' size).  The limit lies where ordinary grids
+// have nothing beyond it (196 x 50: 0.21 % of the area from 5 on, 0.007 % from 6,
+// none from 7); with it at 4, 400 batched requests took 10 % longer and the
+// luminosity 25 %.  kFixReach: the same against the corner's size, for a weak
+// patch.
+constexpr int kFixBuild = 6;
+constexpr int kFixReach = 7;
 
 // One coefficient (value 2^(61 - E)) as the table holds it: the last of a row
 // carries the exponent byte.
@@ -289,14 +295,19 @@ struct FixMatrix {
     unsigned used;
 };
 
-// Sum over i of M[i] v_i / 2^61 (|v_i| <= 2^61): one entry of a matrix product.
+// Sum over i of M[i] v_i / 2^61 (|v_i| <= 2^61), rounded: one entry of a matrix
+// product.  The low x low products count here (without them an entry was off by
+// up to 8 units, and the build by 2^4 times what it leaves now).
 PDF_HD int64_t fix_dot(const Dig M[4], Dig v0, Dig v1, Dig v2, Dig v3)
 {
-    int64_t hh = wide(M[0].h, v0.h), cr = wide(M[0].h, v0.l, (int64_t)1 << 28);
-    cr = wide(M[0].l, v0.h, cr);
-    hh = wide(M[1].h, v1.h, hh), cr = wide(M[1].h, v1.l, cr), cr = wide(M[1].l, v1.h, cr);
-    hh = wide(M[2].h, v2.h, hh), cr = wide(M[2].h, v2.l, cr), cr = wide(M[2].l, v2.h, cr);
-    hh = wide(M[3].h, v3.h, hh), cr = wide(M[3].h, v3.l, cr), cr = wide(M[3].l, v3.h, cr);
+    const Dig v[4] = {v0, v1, v2, v3};
+    int64_t hh = 0, cr = (int64_t)1 << 28;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        hh = wide(M[i].h, v[i].h, hh);
+        cr = wide(M[i].h, v[i].l, cr);
+        cr = wide(M[i].l, v[i].h, cr) + fix_hi(wide(M[i].l, v[i].l));
+    }
     return (int64_t)((uint64_t)hh << 3) + (cr >> 29);
 }
 
@@ -385,7 +396,7 @@ PDF_HD void fix_patch(const double v[4][4], unsigned mask, const FixMatrix &X, c
         const int ec = fix_exponent(v[1][1]), spread = X.spread + Q.spread;
         e8 = E + kFixBias;
         ok = ok && e8 >= 0 && e8 < 127 && E - ec <= kFixCorner && Ev - ec <= kFixStencil && Ev + spread - E <= kFixBuild;
-        if (E - ec > kFixStrong || Ev + spread - ec > kFixBuild) e8 |= kFixWeak;
+        if (E - ec > kFixStrong || Ev + spread - ec > kFixReach) e8 |= kFixWeak;
     }
     if (!ok) e8 = kFixNone;
     const bool fill = ok && emax != 0;

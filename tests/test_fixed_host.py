@@ -198,3 +198,37 @@ def test_narrow_cells_next_to_one(j, axis):
     assert served.all() if j <= 5 else True
     if served.any():
         assert np.max(fixed[served]) <= np.max(fp64)
+
+
+@pytest.mark.parametrize("seed", range(8))
+def test_steep_falls_on_uneven_cells(seed):
+    """A function that falls by orders of magnitude over coarse and uneven cells,
+    (1 - x)^b up to x = 1, at points near both ends of the cells: the matrices'
+    row sums, the stencil's range and the cancellation towards the far knot all
+    meet.  Where fixed point serves, its error against the exact value of the
+    argument, on the scale of the weighted values, is no larger than FP64's: root
+    mean square against root mean square, and the largest within twice the
+    largest (of 480 points each, a few of which lie where both cancel)."""
+    rng = np.random.default_rng(700 + seed)
+    fixed, fp64 = [], []
+    for _ in range(4):
+        u = -np.cumsum(np.exp(rng.uniform(-3, 2, 5)))[::-1]
+        x = np.append(np.exp(u - 0.01), 1.0)
+        q2 = np.exp(3 + np.cumsum(0.2 * np.exp(rng.uniform(-1, 1, 5))))
+        v = x[None] ** rng.uniform(-0.5, 1) * np.maximum(1 - x, 0)[None] ** rng.uniform(2, 6) * \
+            (1 + rng.uniform(-0.05, 0.1) * np.log(q2))[:, None]
+        n = 120
+        k, j = rng.integers(0, x.size - 1, n), rng.integers(0, q2.size - 1, n)
+        t, s = 2.0 ** -rng.uniform(0, 10, (2, n))
+        t[::2], s[::4] = 1 - t[::2], 1 - s[::4]
+        px = np.clip(x[k] * (x[k + 1] / x[k]) ** t, x[k], np.nextafter(x[k + 1], 0))
+        pq = np.clip(q2[j] * (q2[j + 1] / q2[j]) ** s, q2[j], np.nextafter(q2[j + 1], 0))
+        got, _ = fixed_host.evaluate(x, q2, v, px, pq)
+        ref = fixed_host.exact(x, q2, v, px, pq)
+        kap = np.array([float(r[1]) for r in ref])
+        ok = np.isfinite(got[:, 0]) & (kap > 0)
+        fixed.append((fixed_host.error(got[:, 0], [r[0] for r in ref])[ok] / kap[ok]))
+        fp64.append((fixed_host.error(got[:, 4], [r[0] for r in ref])[ok] / kap[ok]))
+    fixed, fp64 = np.concatenate(fixed), np.concatenate(fp64)
+    assert fixed.size > 50 and np.max(fixed) <= 2 * np.max(fp64), (np.max(fixed), np.max(fp64))
+    assert np.mean(fixed ** 2) <= np.mean(fp64 ** 2)
