@@ -290,10 +290,10 @@ static const FixLogTables &fix_log_tables()   // made once per process
 // Fixed-point cell between two knots (bits of positive normal doubles).  A
 // cell wider than half the logarithm's format or so narrow that the
 // logarithm's 2^-59 is more than 2^-45 of it keeps FP64 (K = 0).  So does one
-// narrower than 2^-10 where |ln z| < 2^-7: the FP64 logarithm is accurate to
-// its own size there and gives the better coordinate (largest error of the
-// terms' size, cells of 2^-12 below x = 1: 6e-15 in fixed point, 1e-15 in FP64;
-// equal at 2^-10).
+// whose knots lie within 2^-6.5 of ln z = 0: the FP64 logarithm is accurate to
+// its own size (2^-53 |ln z|) there and gives the better coordinate (cells of
+// 2^-12 below x = 1, largest error of the terms' size: 6e-15 in fixed point, 1e-15
+// in FP64).
 static FixCell fix_cell(double z0, double z1, const uint32_t *inv, const int64_t *tab)
 {
     FixCell c{0, 0};
@@ -301,7 +301,7 @@ static FixCell fix_cell(double z0, double z1, const uint32_t *inv, const int64_t
     c.U = fix_log(dbits(z0), inv, tab);
     const uint64_t d = (uint64_t)fix_log(dbits(z1), inv, tab) - (uint64_t)c.U;
     if (d < ((uint64_t)1 << 46) || (d >> 63)) return c;
-    if (d < ((uint64_t)1 << 50) && fmax(fabs(log(z0)), fabs(log(z1))) < 0x1p-7) return c;
+    if (fmax(fabs(log(z0)), fabs(log(z1))) < 0x1.6ap-7) return c;
     int s = 0;
     while (!((d << s) >> 62)) ++s;
     const unsigned __int128 q = ((unsigned __int128)1 << 126) / (d << s);
