@@ -203,12 +203,12 @@ constexpr int kFixBias = 80;
 constexpr int kFixWeak = 128;
 constexpr int kFixNone = 255;
 
-// On a lower edge: t < 2^-14 on either axis.  There the FP64 form, which expands
+// On a lower edge: t < 2^-20 on either axis.  There the FP64 form, which expands
 // about the lower corner, gives the values on the knots to the last bit, and
 // the fixed-point form's error follows the patch's largest coefficient: a weak
 // patch (fix_patch) then takes FP64.  The limit is the least exponent byte that
 // does so at the point.
-constexpr int kFixEdge = 1 << 16;         // 2^-14 in the upper word of a t (value 2^62)
+constexpr int kFixEdge = 1 << 10;         // 2^-20 in the upper word of a t (value 2^62)
 PDF_HD int fix_limit(int64_t tx, int64_t tq)
 {
     return fix_hi(tx) < kFixEdge || fix_hi(tq) < kFixEdge ? kFixWeak : kFixNone;
@@ -241,14 +241,16 @@ __device__ __forceinline__ void fix_ld(const unsigned char *p, int c[8])
 //    of 2^E, more than 2^(E - 54) anywhere; fixed point's by 2^(E - 59) /
 //    width.  Largest error of the value itself, FP64 / fixed point, cells of
 //    0.1 at ln x = -5 with the corner 2^-k of the rest: k = 4 1e-13 / 1e-15, 6
-//    8e-13 / 6e-15.  (The patch alone, at a given t: 8e-15 / 7e-16, 1e-14 /
-//    4e-15.)
+//    8e-13 / 6e-15.  (The patch alone, at a given t: 8e-15 / 9e-16, 1e-14 /
+//    5e-15.)
 //  - 2^6 below (a flavour that sets in at a threshold knot), or with a stencil
 //    2^12 above the corner, the patch keeps FP64.
 // Of the 196 x 50 grid's patches 2.8 % are weak (by area), 0.005 % are 2^6
-// below.  Where the edge ends costs: at 2^-14 nothing that shows, at 2^-10 the
-// matrix-form fit step 3 % and the luminosity 2 % (one point with a weak patch
-// keeps its warp), at 2^-4 x*f 3.5 % and 400 batched requests 11 %.
+// below.  A point that takes FP64 keeps its warp: one in a query of one pass per
+// warp costs 2.5 us and more (1e5 points x 11 flavours 19.3 -> 21.7 us, 54000
+// events 33 -> 37).  So the edge is narrow: with it at 2^-14 every second such
+// query had a point there, with 2^-10 the matrix-form fit step took 3 % longer
+// and the luminosity 2 %, with 2^-4 x*f 3.5 % and 400 batched requests 11 %.
 constexpr int kFixStrong = 1;
 constexpr int kFixCorner = 6;
 constexpr int kFixStencil = 12;
