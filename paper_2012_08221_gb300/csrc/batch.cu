@@ -105,10 +105,10 @@ __global__ void __launch_bounds__(256, 3) k_batch(const GridDev *__restrict__ gr
                 if (base >= Y.n) break;
                 eval_points<false, false, false, true>(g, T, Y, B, base, lane);
             }
+            while (B.qn) drain_queue(g, T, Y, false, B, lane);
         };
         if (STAGE && staged) pass(staged_tabs(g, tabs));
         else pass(grid_tabs(g));
-        while (B.qn) drain_queue(g, Y, false, B, lane);
         __syncthreads();   // everyone is done with sr/s_tile before thread 0 refills them
     }
     if (lane == 0) bulk_wait_all();

@@ -55,10 +55,10 @@ __global__ void __launch_bounds__(kBlock, WHOLE ? 3 : 2) k_xfxq2(const __grid_co
             base = blk * 32;
         }
         eval_points<Q_IS_Q, TAPE, AS, WHOLE>(g, T, Y, B, base, lane);
-        if (!WHOLE && B.qn) drain_queue(g, Y, Q_IS_Q, B, lane);
+        if (!WHOLE && B.qn) drain_queue(g, T, Y, Q_IS_Q, B, lane);
     }
     if (WHOLE)
-        while (B.qn) drain_queue(g, Y, Q_IS_Q, B, lane);
+        while (B.qn) drain_queue(g, T, Y, Q_IS_Q, B, lane);
     if (lane == 0) bulk_wait_all();
 }
 
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kBlock) k_alphas(const __grid_constant__ GridD
             const bool bad = !q2_ok(dbits(qi));
             flag_status(g, bad);
             bool oor;
-            const double v = alphas_at(g, axis_q2(g, bad ? 10.0 : qi), &oor);
+            const double v = alphas_at(g, axis_q2(g, T, bad ? 10.0 : qi), &oor);
             flag_status(g, oor && !bad, PDF_S_RANGE);
             out[i] = bad ? dnan() : v;
         }

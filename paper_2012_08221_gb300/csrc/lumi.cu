@@ -54,11 +54,12 @@ __device__ __forceinline__ Event event(int64_t e, const double *ln_tau, const do
 // One event in FP64 (a parton or the scale outside the knots, a patch that the
 // fixed-point format does not hold): this lane's share of its sum, NaN for a
 // bad event.
-__device__ __forceinline__ double slow_event(const GridDev &g, const signed char *anti, const double *cm, Event E,
-                                             Queued q, double *as, double *save_p, bool report)
+__device__ __forceinline__ double slow_event(const GridDev &g, const LogTabs &T, const signed char *anti,
+                                             const double *cm, Event E, Queued q, double *as, double *save_p,
+                                             bool report)
 {
     const int64_t e = q.i;
-    const Axis Q = axis_w(g, E.w), X1 = axis_u(g, E.u1), X2 = axis_u(g, E.u2);
+    const Axis Q = axis_w(g, T, E.w), X1 = axis_u(g, T, E.u1), X2 = axis_u(g, T, E.u2);
     const bool oor = !E.bad && (out_of_range(g, X1, Q) || out_of_range(g, X2, Q));
     flag_status(g, report && E.bad);
     flag_status(g, report && oor, PDF_S_RANGE);
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(kBlock, SAVE ? 2 : 3) k_lumi(const __grid_cons
         double s = 0.0;
         if (q.i >= 0) {
             const Event E = event(q.i, ln_tau, y, flags, ln_mu2, ln_x1, ln_s);
-            s = slow_event(g, anti.c, cm, E, q, as, SAVE ? save_p : nullptr, partials != nullptr);
+            s = slow_event(g, T, anti.c, cm, E, q, as, SAVE ? save_p : nullptr, partials != nullptr);
         }
         __syncwarp();
         for (int o = 1; o < q.count; o <<= 1) s += __shfl_xor_sync(kAll, s, o);

@@ -39,6 +39,16 @@ __device__ __forceinline__ LogTabs stage_log_tabs(const GridDev &g, unsigned cha
     return {uk, wk, xc, qc};
 }
 
+// The axes of axis_u and axis_w from these tables.
+__device__ __forceinline__ Axis axis_u(const GridDev &g, const LogTabs &T, double u)
+{
+    return axis_log(g, T.ukey, T.xcell, g.nxc, g.xstep, g.ulo, g.uhi, u);
+}
+__device__ __forceinline__ Axis axis_w(const GridDev &g, const LogTabs &T, double w)
+{
+    return axis_log(g, T.wkey, T.qcell, g.nqc, g.qstep, g.wlo, g.whi, w);
+}
+
 // Whether both partons and the scale lie in the knot range.
 __device__ __forceinline__ bool in_logs(const GridDev &g, double u1, double u2, double w)
 {

@@ -313,12 +313,13 @@ __device__ __forceinline__ FixAxis fix_axis_q2(const GridDev &g, const CoordTabs
 // range t is the fixed-point coordinate, so that every kernel places a point
 // at the same t; elsewhere it comes from the FP64 logarithm.  Only the one that
 // is needed is taken.
-__device__ __forceinline__ void axis_coord(const GridDev &g, Axis &A, double z, const FixCell &f, double2 c)
+__device__ __forceinline__ void axis_coord(const GridDev &g, const CoordTabs &T, Axis &A, double z, const FixCell &f,
+                                           double2 c)
 {
     A.f = -1;
     double t;
     if (A.in && f.K != 0) {
-        A.f = fix_coord(fix_log(dbits(z), g.finv, g.flog), f);
+        A.f = fix_coord(fix_log(dbits(z), T.inv, T.log), f);
         t = fix_t(A.f);
     } else {
         t = (dlog(g, z) - c.x) * c.y;
@@ -326,53 +327,54 @@ __device__ __forceinline__ void axis_coord(const GridDev &g, Axis &A, double z, 
     make_basis(A, t, g.extrap);
 }
 
-__device__ __forceinline__ Axis axis_x(const GridDev &g, double x)
+__device__ __forceinline__ Axis axis_x(const GridDev &g, const CoordTabs &T, double x)
 {
     const uint64_t b = dbits(x);
     Axis A;
-    A.cell = cell_x(g, grid_tabs(g), b);
+    A.cell = cell_x(g, T, b);
     A.in = in_x(g, b);
     A.below = b < g.xlo;
-    axis_coord(g, A, x, g.xfix[A.cell], g.xcell[A.cell]);
+    axis_coord(g, T, A, x, T.xfix[A.cell], g.xcell[A.cell]);
     return A;
 }
+__device__ __forceinline__ Axis axis_x(const GridDev &g, double x) { return axis_x(g, grid_tabs(g), x); }
 
-__device__ __forceinline__ Axis axis_q2(const GridDev &g, double q2)
+__device__ __forceinline__ Axis axis_q2(const GridDev &g, const CoordTabs &T, double q2)
 {
     const uint64_t b = dbits(q2);
     Axis A;
-    A.cell = cell_q2(g, grid_tabs(g), b);
+    A.cell = cell_q2(g, T, b);
     A.in = in_q2(g, b);
     A.below = b < g.qlo;
-    axis_coord(g, A, q2, g.qfix[A.cell], g.qcell[A.cell]);
+    axis_coord(g, T, A, q2, T.qfix[A.cell], g.qcell[A.cell]);
+    return A;
+}
+__device__ __forceinline__ Axis axis_q2(const GridDev &g, double q2) { return axis_q2(g, grid_tabs(g), q2); }
+
+// An axis from a logarithm directly (order-key search): the keys and cells of
+// the table, its first and last knot's keys.
+__device__ __forceinline__ Axis axis_log(const GridDev &g, const int64_t *keys, const double2 *cells, int ncell,
+                                         int step, int64_t lo, int64_t hi, double z)
+{
+    const int64_t k = dkey(z);
+    Axis A;
+    A.cell = checked_index(g.status, find_cell<int64_t>(keys, ncell, step, k), ncell);
+    A.f = -1;
+    A.in = (k >= lo) & (k <= hi);
+    A.below = k < lo;
+    const double2 c = cells[A.cell];
+    make_basis(A, (z - c.x) * c.y, g.extrap);
     return A;
 }
 
-// x axis from u = ln x directly (order-key search on u).
+// The x axis from u = ln x, and the Q axis from w = ln Q^2.
 __device__ __forceinline__ Axis axis_u(const GridDev &g, double u)
 {
-    int64_t k = dkey(u);
-    Axis A;
-    A.cell = checked_index(g.status, find_cell<int64_t>(g.ukey, g.nxc, g.xstep, k), g.nxc);
-    A.f = -1;
-    A.in = (k >= g.ulo) & (k <= g.uhi);
-    A.below = k < g.ulo;
-    double2 c = g.xcell[A.cell];
-    make_basis(A, (u - c.x) * c.y, g.extrap);
-    return A;
+    return axis_log(g, g.ukey, g.xcell, g.nxc, g.xstep, g.ulo, g.uhi, u);
 }
-
 __device__ __forceinline__ Axis axis_w(const GridDev &g, double w)
 {
-    int64_t k = dkey(w);
-    Axis A;
-    A.cell = checked_index(g.status, find_cell<int64_t>(g.wkey, g.nqc, g.qstep, k), g.nqc);
-    A.f = -1;
-    A.in = (k >= g.wlo) & (k <= g.whi);
-    A.below = k < g.wlo;
-    double2 c = g.qcell[A.cell];
-    make_basis(A, (w - c.x) * c.y, g.extrap);
-    return A;
+    return axis_log(g, g.wkey, g.qcell, g.nqc, g.qstep, g.wlo, g.whi, w);
 }
 
 // Four consecutive doubles in one 32-byte read-only load (sm_100 and later).

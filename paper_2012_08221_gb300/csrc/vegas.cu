@@ -65,10 +65,10 @@ __device__ __forceinline__ VegasPoint vegas_point(double2 vv, const double *edge
 
 // A point with a parton or the scale outside the knots (or a patch that the
 // fixed-point format does not hold), in FP64: this lane's share of its sum.
-__device__ __forceinline__ double slow_lumi(const GridDev &g, const signed char *anti, const double *cm,
+__device__ __forceinline__ double slow_lumi(const GridDev &g, const LogTabs &T, const signed char *anti, const double *cm,
                                             const VegasPoint &P, Queued q)
 {
-    const Axis Q = axis_w(g, P.w), X1 = axis_u(g, P.u1), X2 = axis_u(g, P.u2);
+    const Axis Q = axis_w(g, T, P.w), X1 = axis_u(g, T, P.u1), X2 = axis_u(g, T, P.u2);
     const size_t cell_stride = (size_t)g.nflav * 16;
     const double *c1 = cm + ((size_t)Q.cell * g.nxc + X1.cell) * cell_stride;
     const double *c2 = cm + ((size_t)Q.cell * g.nxc + X2.cell) * cell_stride;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_vegas(const __grid_constant__ Gri
     auto drain = [&]() {
         const Queued q = next_queued(B, lane);
         const VegasPoint P = point(max(q.i, (int64_t)0));
-        double lum = q.i >= 0 ? slow_lumi(g, anti.c, cm, P, q) : 0.0;
+        double lum = q.i >= 0 ? slow_lumi(g, T, anti.c, cm, P, q) : 0.0;
         __syncwarp();
         for (int o = 1; o < q.count; o <<= 1) lum += __shfl_xor_sync(kAll, lum, o);
         if (q.i >= 0 && q.sub == 0) add(P, lum);

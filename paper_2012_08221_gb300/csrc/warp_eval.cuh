@@ -255,7 +255,7 @@ struct Queued {
 // format does not serve; of a point in a cell that it serves only the patches
 // that the format does not hold (its other flavours keep the bits that any
 // other query gives them).
-__device__ __forceinline__ void slow_point(const GridDev &g, const Query &Y, bool q_is_q, Queued e)
+__device__ __forceinline__ void slow_point(const GridDev &g, const CoordTabs &T, const Query &Y, bool q_is_q, Queued e)
 {
     const int64_t i = e.i;
     double xi = Y.x[i], qi = Y.q[i];
@@ -267,7 +267,7 @@ __device__ __forceinline__ void slow_point(const GridDev &g, const Query &Y, boo
         xi = 0.5;
         if (!Y.alphas || qbad) qi = 10.0;
     }
-    const Axis X = axis_x(g, xi), Q = axis_q2(g, qi);
+    const Axis X = axis_x(g, T, xi), Q = axis_q2(g, T, qi);
     const bool fixed = !bad && Y.fm && X.f >= 0 && Q.f >= 0;
     if (Y.alphas && e.sub == 0) {
         bool oor;
@@ -326,11 +326,12 @@ __device__ __forceinline__ Queued next_queued(WarpBufs &B, int lane)
 
 // The queue's first 32 points in FP64, after the rows staged for them have
 // been written; the lanes that share a point share its columns.
-__device__ __forceinline__ void drain_queue(const GridDev &g, const Query &Y, bool q_is_q, WarpBufs &B, int lane)
+__device__ __forceinline__ void drain_queue(const GridDev &g, const CoordTabs &T, const Query &Y, bool q_is_q, WarpBufs &B,
+                                            int lane)
 {
     if (lane == 0) bulk_wait_all();
     const Queued e = next_queued(B, lane);
-    if (e.i >= 0) slow_point(g, Y, q_is_q, e);
+    if (e.i >= 0) slow_point(g, T, Y, q_is_q, e);
     __syncwarp();
 }
 
@@ -389,7 +390,7 @@ __device__ __forceinline__ void eval_points(const GridDev &g, const CoordTabs &T
         }
         push_queue(B, fast && none, i, lane);
     }
-    if (B.qn >= 32) drain_queue(g, Y, Q_IS_Q, B, lane);
+    if (B.qn >= 32) drain_queue(g, T, Y, Q_IS_Q, B, lane);
 }
 
 }  // namespace pdfgpu
