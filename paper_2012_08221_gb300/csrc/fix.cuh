@@ -243,28 +243,28 @@ __device__ __forceinline__ void fix_ld(const unsigned char *p, int c[8])
 //    0.1 at ln x = -5 with the corner 2^-k of the rest: k = 4 1e-13 / 1e-15, 6
 //    8e-13 / 6e-15.  (The patch alone, at a given t: 8e-15 / 9e-16, 1e-14 /
 //    5e-15.)
-//  - 2^6 below (a flavour that sets in at a threshold knot), or with a stencil
+//  - 2^7 below (a flavour that sets in at a threshold knot), or with a stencil
 //    2^12 above the corner, the patch keeps FP64.
-// Of the 196 x 50 grid's patches 2.8 % are weak (by area), 0.005 % are 2^6
-// below.  A point that takes FP64 keeps its warp: one in a query of one pass per
+// Of the 196 x 50 grid's patches 2.8 % are weak (by area), none is 2^7 below
+// (0.005 % are 2^6 below).  A point that takes FP64 keeps its warp: one in a query of one pass per
 // warp costs 2.5 us and more (1e5 points x 11 flavours 19.3 -> 21.7 us, 54000
 // events 33 -> 37).  So the edge is narrow: with it at 2^-14 every second such
 // query had a point there, with 2^-10 the matrix-form fit step took 3 % longer
 // and the luminosity 2 %, with 2^-4 x*f 3.5 % and 400 batched requests 11 %.
 constexpr int kFixStrong = 1;
-constexpr int kFixCorner = 6;
+constexpr int kFixCorner = 7;
 constexpr int kFixStencil = 12;
 PDF_HD int fix_exponent(double v) { return ((int)(dbits(v) >> 52) & 0x7FF) - 1022; }   // |v| < 2^this
 
-// What the build leaves in a patch is about 2^(Ev - 60 + spreads) for stencil
-// values below 2^Ev: with interval ratios 2^r on both axes that is 2^(2 r),
-// and smooth values have coefficients (2^E) that do not grow with it; steep ones
-// have a stencil far above the cell.  Patches where it passes 2^(E - 54) keep
-// FP64 (ratios from about 2^6 on; a cell 2^12 times its neighbours on both axes
-// was off by 8e-12 of its values' size).  The limit lies where ordinary grids
-// have nothing beyond it (196 x 50: 0.21 % of the area from 5 on, 0.007 % from 6,
-// none from 7); with it at 4, 400 batched requests took 10 % longer and the
-// luminosity 25 %.  kFixReach: the same against the corner's size, for a weak
+// What the build leaves in a patch is at most about 2^(Ev - 60 + spreads) for
+// stencil values below 2^Ev: with interval ratios 2^r on both axes that is 2^(2
+// r), and smooth values have coefficients (2^E) that do not grow with it; steep
+// ones have a stencil far above the cell.  Patches where it passes 2^(E - 54)
+// keep FP64 (ratios from about 2^6 on; a cell 2^12 times its neighbours on both
+// axes was off by 8e-12 of its values' size).  The limit lies where ordinary
+// grids have nothing beyond it (196 x 50: 0.21 % of the area from 5 on, 0.007 %
+// from 6, none from 7); with it at 4, 400 batched requests took 10 % longer and
+// the luminosity 25 %.  kFixReach: the same against the corner's size, for a weak
 // patch.
 constexpr int kFixBuild = 6;
 constexpr int kFixReach = 7;
@@ -297,20 +297,27 @@ struct FixMatrix {
     unsigned used;
 };
 
-// Sum over i of M[i] v_i / 2^61 (|v_i| <= 2^61), rounded: one entry of a matrix
-// product.  The low x low products count here (without them an entry was off by
-// up to 8 units, and the build by 2^4 times what it leaves now).
-PDF_HD int64_t fix_dot(const Dig M[4], Dig v0, Dig v1, Dig v2, Dig v3)
+// Sum over i of M[i] v_i / 2^61 (|v_i| <= 2^61), rounded down, and the next 8 bits
+// in `rest`: one entry of a matrix product.  The low x low products count here
+// (without them an entry was off by up to 8 units, and the build by 2^4 times
+// what it leaves now).
+PDF_HD int64_t fix_dot(const Dig M[4], Dig v0, Dig v1, Dig v2, Dig v3, int &rest)
 {
     const Dig v[4] = {v0, v1, v2, v3};
-    int64_t hh = 0, cr = (int64_t)1 << 28;
+    int64_t hh = 0, cr = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         hh = wide(M[i].h, v[i].h, hh);
         cr = wide(M[i].h, v[i].l, cr);
         cr = wide(M[i].l, v[i].h, cr) + fix_hi(wide(M[i].l, v[i].l));
     }
+    rest = (int)((uint64_t)cr >> 21) & 255;
     return (int64_t)((uint64_t)hh << 3) + (cr >> 29);
+}
+// The entry times 2^s, 0 <= s < 8, rounded.
+PDF_HD int64_t fix_entry(int64_t v, int rest, int s)
+{
+    return (int64_t)((uint64_t)v << s) + ((rest + (128 >> s)) >> (8 - s));
 }
 
 // A double as an integer times 2^-s, rounded; zero below.
@@ -342,6 +349,8 @@ PDF_HD int64_t fix_shift(int64_t v, int n)   // v 2^n, rounded
 // coefficients keep about 2^-58 of the stencil's largest value (an FP64 sum
 // keeps 2^-53) and the FP64 pipe stays free.  The interpolation of a constant
 // being the constant, the sums run over the differences to the lower corner.
+// The first product keeps the bits that the matrix's row sum leaves room for
+// (steep functions have entries far below it, and lost up to 5 of them).
 // The values' common exponent is that of the entries with weight: a straight
 // line's neighbours may be far larger than its own knots (2^30: values off by
 // 1e-9 when they counted; FP64 never mixes them in).
@@ -365,6 +374,7 @@ PDF_HD void fix_patch(const double v[4][4], unsigned mask, const FixMatrix &X, c
     bool ok = finite && X.k[0] >= 0 && Q.k[0] >= 0;
     const int64_t ref = fix_from(v[1][1], 60 - Ev);
     int64_t cx[4][4];
+    int rest[4][4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         Dig d[4];
@@ -372,17 +382,26 @@ PDF_HD void fix_patch(const double v[4][4], unsigned mask, const FixMatrix &X, c
         for (int i = 0; i < 4; ++i)
             d[i] = fix_split((mask >> (4 * r + i)) & 1 ? fix_from(v[r][i], 60 - Ev) - ref : 0);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) cx[r][m] = fix_dot(X.d[m], d[0], d[1], d[2], d[3]);
+        for (int m = 0; m < 4; ++m) cx[r][m] = fix_dot(X.d[m], d[0], d[1], d[2], d[3], rest[r][m]);
     }
     int64_t C[4][4];
-    int E = -100000;
+    int E = -100000, up[4];                          // up[m]: bits that column m gains before the second product
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-        const Dig c0 = fix_split(cx[0][m]), c1 = fix_split(cx[1][m]), c2 = fix_split(cx[2][m]), c3 = fix_split(cx[3][m]);
+        uint64_t any = 0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) any |= (uint64_t)(cx[r][m] < 0 ? -cx[r][m] : cx[r][m]);
+        const int most = m ? 7 : X.k[0] + Q.k[0], room = fix_clz(any) - 4;
+        up[m] = room < 0 ? 0 : room < most ? room : most < 7 ? most : 7;
+        Dig c[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) c[r] = fix_split(fix_entry(cx[r][m], rest[r][m], up[m]));
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
-            C[n][m] = fix_dot(Q.d[n], c0, c1, c2, c3);
-            const int k = X.k[m] + Q.k[n];
+            int low;
+            const int64_t down = fix_dot(Q.d[n], c[0], c[1], c[2], c[3], low);
+            C[n][m] = fix_entry(down, low, 0);
+            const int k = X.k[m] + Q.k[n] - up[m];
             const int64_t t = n + m ? C[n][m] : C[0][0] + (ref >> (k & 63));
             const int e = 4 - fix_clz((uint64_t)(t < 0 ? -t : t)) + k + Ev;
             if (t && e > E) E = e;
@@ -406,7 +425,7 @@ PDF_HD void fix_patch(const double v[4][4], unsigned mask, const FixMatrix &X, c
     for (int n = 0; n < 4; ++n)
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            C[n][m] = fill ? fix_shift(C[n][m], 1 - E + X.k[m] + Q.k[n] + Ev) : 0;
+            C[n][m] = fill ? fix_shift(C[n][m], 1 - E + X.k[m] + Q.k[n] - up[m] + Ev) : 0;
             if (m == 3) C[n][m] = fix_last(C[n][m], e8);
         }
     // the constant term from the others as stored, so that the sum at the corner is the knot's value
