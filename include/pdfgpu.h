@@ -148,7 +148,11 @@ typedef struct {
 
 /* Validate a grid description, upload it and build the interpolation tables
  * on the current CUDA device (PDFFlow Sec. 2.1 `mkPDF`; Sec. 4 grid format).
- * Synchronous.  On success *out owns device memory until pdf_free_grid. */
+ * Synchronous.  On success *out owns device memory until pdf_free_grid: 128
+ * bytes per cell, flavour and member for the FP64 coefficients, and as much
+ * again for the fixed-point ones if that is at most an eighth of the free
+ * memory and all grids together stay within an eighth of the device's (else
+ * every point is evaluated in FP64). */
 int pdf_load_grid(const pdfgpu_grid_desc *desc, pdfgpu_grid_t *out);
 
 /* (Re)build the per-cell bicubic coefficients of ALL members from a DEVICE

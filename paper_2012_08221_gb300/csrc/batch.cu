@@ -46,7 +46,7 @@ struct BatchReq {
     int64_t tile0;
 };
 
-// (three blocks of 256 threads per SM at 80 registers; with staged tables 76
+// (three blocks of 256 threads per SM at 80 registers; with staged tables 24
 // bytes of them spilled)
 template <int QPT, bool STAGE>
 __global__ void __launch_bounds__(256, 3) k_batch(const GridDev *__restrict__ grids,

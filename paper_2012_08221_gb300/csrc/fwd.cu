@@ -106,7 +106,7 @@ __device__ __forceinline__ void slow_point_pw(const GridDev &g, const double *cm
 // Five blocks of 128 threads per SM, at 96 registers (with both tapes 160 bytes
 // of them spilled, 104 with one, 100 plain): 1351 us per pointwise fit step; two
 // blocks of 256 1364, six of 128, which spill more, 1385.  With the rules of
-// fix_limit 1356.
+// fix_limit 1360.
 constexpr int kPwBlock = 128;
 
 template <bool TAPE, bool DT, bool STAGE>
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kPwBlock, 5) k_xfxq2_pw(const __grid_constant_
     if (B.qn) drain();
 }
 
-// alpha_s, one point per lane (fix_alphas): 1e7 points 286 -> 94.5 us (FP64
+// alpha_s, one point per lane (fix_alphas): 1e7 points 286 -> 93 us (FP64
 // pipe 82 % busy before; now 56 % of the issue slots, the logarithm and the table
 // look-ups in shared memory); points outside the Q range or the
 // domain are queued per warp and evaluated 32 at a time.

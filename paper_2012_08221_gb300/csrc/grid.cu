@@ -390,7 +390,7 @@ static int largest_pow2_below(int n)
 // stencil (rows outside the cell's subgrid and knots outside the x axis have
 // zero weight and are not read).  The same patch about the
 // cell's centre, in fixed point, comes from integer sums (fix_patch): the
-// kernel takes 33 us for the 116610 patches of the 196 x 50 grid with 13
+// kernel takes 37 us for the 116610 patches of the 196 x 50 grid with 13
 // flavours (with FP64 sums for both forms 72 us, the FP64 form alone 31 us).
 // The matrices' first row is (0, 1, 0, 0) and their second ends in 0: those
 // products are left out (88 FMAs, not 128).

@@ -15,7 +15,7 @@
 // slots 42 % busy); the L1's data path is 50 % busy, and the 24 warps that 80
 // registers allow wait for the rows from L2 and for their own chains.  1e7
 // points x 13 flavours of the 196 x 50 grid: 3656 us with FP64 Horner patches
-// (FP64 pipe 95 % busy), 1389 us here (1369 without the rules of fix_limit, whose
+// (FP64 pipe 95 % busy), 1392 us here (1369 without the rules of fix_limit, whose
 // operand spills 12 bytes).
 //
 // Points outside the knots (or in cells or patches that the format does not
@@ -23,8 +23,8 @@
 // so that a few of them do not make every warp run both paths (1e6 points x 3
 // flavours with 5 % outside under the continuation: 475 -> 103 us).  A query that
 // mostly outside pays for both: it is slower than FP64 alone was from two thirds
-// of the points outside on (1e6 points x 13 flavours 380 -> 451 us at 95 %, 386
-// with all of them outside; alpha_s 36 -> 44; 1e6 events 735 -> 935 and 769).
+// of the points outside on (1e6 points x 13 flavours 380 -> 451 us at 95 %, 382
+// with all of them outside; alpha_s 36 -> 44; 1e6 events 735 -> 925 and 764).
 #pragma once
 
 #include "pdf_common.cuh"
