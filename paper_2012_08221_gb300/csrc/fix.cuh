@@ -391,8 +391,9 @@ PDF_HD void fix_patch(const double v[4][4], unsigned mask, const FixMatrix &X, c
         uint64_t any = 0;
 #pragma unroll
         for (int r = 0; r < 4; ++r) any |= (uint64_t)(cx[r][m] < 0 ? -cx[r][m] : cx[r][m]);
-        const int most = m ? 7 : X.k[0] + Q.k[0], room = fix_clz(any) - 4;
-        up[m] = room < 0 ? 0 : room < most ? room : most < 7 ? most : 7;
+        const int most = m || X.k[0] + Q.k[0] > 7 ? 7 : X.k[0] + Q.k[0], room = fix_clz(any) - 4;
+        up[m] = room < most ? room : most;
+        up[m] = up[m] < 0 ? 0 : up[m];
         Dig c[4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) c[r] = fix_split(fix_entry(cx[r][m], rest[r][m], up[m]));
